@@ -3,11 +3,9 @@
 // followed by the epilogue of Eq. 2 / Eq. 3: optional GELU-tanh or gate, bf16 rounding, and
 // rows written either compactly or straight into their slots of a [B, N, D] cache.
 //
-// Persistent kernel, one CTA per SM, 128 x 256 output tile, K in steps of 64:
-//   warp 0      TMA producer: A tile (128x64) and W tile (256x64) per stage, 128-byte swizzle
-//   warp 1      MMA issuer:   4 x tcgen05.mma (M128 N256 K16) per stage, commit frees the stage
-//   warps 2..5  epilogue:     tcgen05.ld of the finished accumulator, bias/act, global stores
-// Two 256-column accumulators in TMEM let the epilogue of tile i overlap the MMAs of tile i+1.
+// Two kernels (launch_tc_gemm says which runs when):
+//  * tc_gemm_pair_kernel for problems that fill the chip: persistent CTA pairs on 256-row tiles (cta_group::2);
+//  * tc_gemm_split_kernel for the others: one 128-row tile per CTA, the K loop cut over the CTAs of a cluster.
 #include <cuda.h>
 
 #include <mutex>
@@ -64,19 +62,11 @@ int make_tmap_bf16(CUtensorMap* m, const void* base, int rank, const uint64_t* d
 namespace {
 using namespace tc;
 
-#ifndef HERO_GEMM_BN
-#define HERO_GEMM_BN 256
-#endif
-#ifndef HERO_GEMM_STAGES
-#define HERO_GEMM_STAGES 4
-#endif
-constexpr int kBM = 128, kBN = HERO_GEMM_BN, kBK = 64, kStages = HERO_GEMM_STAGES;
+constexpr int kBM = 128, kBK = 64;                     // rows of A per CTA; K step (one 128-byte swizzle row)
 constexpr int kABytes = kBM * kBK * 2;                 // 16 KB
-constexpr int kBBytes = kBN * kBK * 2;                 // 32 KB
-constexpr int kStageBytes = kABytes + kBBytes;
-constexpr int kGemmThreads = 192;
-constexpr int kTmemCols = 512;                         // two accumulators of 256 fp32 columns
-constexpr size_t kGemmSmem = 1024 /*alignment slack*/ + (size_t)kStages * kStageBytes + 256 /*barriers*/;
+constexpr int kGemmThreads = 320;                      // producer, issuer, eight epilogue warps
+constexpr int kEpiWarps = 8;                           // two per TMEM lane quadrant, each with half of a tile's columns
+constexpr size_t kAlignSlack = 1024, kBarrierBytes = 512;
 
 __device__ __forceinline__ float gelu_tanh_f(float t) {
   // 0.5 t (1 + tanh(sqrt(2/pi) (t + 0.044715 t^3))) with the hardware tanh (one special-function
@@ -90,13 +80,130 @@ __device__ __forceinline__ float gelu_tanh_f(float t) {
   return fmaf(h, th, h);
 }
 
-// Tile order of the persistent CTAs.  Consecutive tile numbers run down kGroupM row tiles before moving
-// to the next column tile, and only then to the next band of rows: the ~148 tiles in flight at any time
-// then cover about 24 x 6 tiles, whose operands (24 row panels of A, 6 of W) stay in L2 and are shared by
-// the CTAs working on them, instead of every CTA streaming its own panel of A from DRAM.  Bands of 16 to 48
-// row tiles time within a percent of each other in the step, 24 slightly ahead (12: 1 % slower, 6: 3 %, one
-// band over all rows: 3 %).
-constexpr int kGroupM = 24;
+// Where one accumulator row goes.
+struct RowOut {
+  bool ok;                 // the row exists
+  int m, b;                // row of the compact operand, its batch item
+  long long scat;          // its row in a [B, n_rows] destination
+};
+__device__ __forceinline__ RowOut row_out(const GemmOut& out, int m, int M) {
+  RowOut r;
+  r.ok = m < M;
+  r.m = m; r.b = 0; r.scat = 0;
+  if (r.ok) {
+    r.b = m / out.n_sel;
+    const int li = m - r.b * out.n_sel;
+    r.scat = (long long)r.b * out.n_rows + (out.idx ? __ldg(out.idx + li) : li);
+  }
+  return r;
+}
+
+__device__ __forceinline__ void st_global_v8(void* p, const uint32_t* w) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+               "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
+}
+
+// Finish NC accumulator columns [n0, n0 + NC) of one row, all of one segment: bias (fp32, staged in shared memory),
+// activation, scale or gate, bf16, full 32-byte sectors per lane (16-byte stores where the destination is not 32-byte
+// aligned or ends inside the columns).
+template <int NC>
+__device__ __forceinline__ void emit(const uint32_t (&acc)[NC], const float* s_bias, int n0, int Nout, const GemmOut& out,
+                                     const RowOut& row) {
+  float2 f[NC / 2];
+#pragma unroll
+  for (int v = 0; v < NC / 4; ++v) {
+    const float4 b4 = *reinterpret_cast<const float4*>(s_bias + v * 4);
+    f[2 * v] = __fadd2_rn(make_float2(__uint_as_float(acc[4 * v]), __uint_as_float(acc[4 * v + 1])), make_float2(b4.x, b4.y));
+    f[2 * v + 1] = __fadd2_rn(make_float2(__uint_as_float(acc[4 * v + 2]), __uint_as_float(acc[4 * v + 3])), make_float2(b4.z, b4.w));
+  }
+  // (segments are selected, not indexed or divided for: at most three, and a parameter indexed at run time would be
+  // copied to local memory)
+  const bool s1 = n0 >= out.seg_cols, s2 = n0 >= 2 * out.seg_cols;        // warp-uniform
+  const int col0 = n0 - (s2 ? 2 * out.seg_cols : (s1 ? out.seg_cols : 0));
+  if (out.act == 1) {
+#pragma unroll
+    for (int i = 0; i < NC / 2; ++i) f[i] = make_float2(gelu_tanh_f(f[i].x), gelu_tanh_f(f[i].y));
+  }
+  if (out.seg0_scale != 0.f && !s1) {
+#pragma unroll
+    for (int i = 0; i < NC / 2; ++i) f[i] = __fmul2_rn(f[i], make_float2(out.seg0_scale, out.seg0_scale));
+  }
+  if (!row.ok) return;
+  if (out.gate) {
+    const float* gate = out.gate + (long long)row.b * out.gate_ld + col0;
+#pragma unroll
+    for (int i = 0; i < NC / 2; ++i)
+      if (n0 + 2 * i < Nout) f[i] = __fmul2_rn(f[i], __ldg(reinterpret_cast<const float2*>(gate + 2 * i)));
+  }
+  uint32_t packed[NC / 2];
+#pragma unroll
+  for (int i = 0; i < NC / 2; ++i) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(f[i].x, f[i].y);
+    packed[i] = *reinterpret_cast<const uint32_t*>(&p);
+  }
+  void* const base = s2 ? out.ptr[2] : (s1 ? out.ptr[1] : out.ptr[0]);
+  const long long ld = s2 ? out.ld[2] : (s1 ? out.ld[1] : out.ld[0]);
+  const int scatter = s2 ? out.scatter[2] : (s1 ? out.scatter[1] : out.scatter[0]);
+  __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(base) + (scatter ? row.scat : (long long)row.m) * ld + col0;
+  if (n0 + NC <= Nout && (reinterpret_cast<uintptr_t>(dst) & 31) == 0) {
+#pragma unroll
+    for (int v = 0; v < NC / 16; ++v) st_global_v8(dst + v * 16, &packed[v * 8]);
+  } else {
+#pragma unroll
+    for (int v = 0; v < NC / 8; ++v)
+      if (n0 + v * 8 < Nout)
+        *reinterpret_cast<uint4*>(dst + v * 8) = make_uint4(packed[4 * v], packed[4 * v + 1], packed[4 * v + 2], packed[4 * v + 3]);
+  }
+}
+
+// A warp puts NC bias values from column n_base on into its own piece of shared memory, in fp32 (values past the end
+// of the row are not read by anybody).
+template <int NC>
+__device__ __forceinline__ void stage_bias(float* s_bias, const __nv_bfloat16* bias, int n_base, int Nout, int lane) {
+  for (int v = lane; v < NC / 8; v += 32)
+    if (n_base + v * 8 < Nout) {
+      const uint4 raw = __ldg(reinterpret_cast<const uint4*>(bias + n_base + v * 8));
+      const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+        *reinterpret_cast<float4*>(s_bias + v * 8 + 4 * q) =
+            make_float4(__uint_as_float(w[2 * q] << 16), __uint_as_float(w[2 * q] & 0xFFFF0000u),
+                        __uint_as_float(w[2 * q + 1] << 16), __uint_as_float(w[2 * q + 1] & 0xFFFF0000u));
+    }
+  __syncwarp();
+}
+
+// ---------------------------------------------------------------------------------------------------------------
+// Problems that fill the chip.  Persistent clusters of two CTAs, one per pair of SMs, on tiles of 256 x BN: each
+// CTA fetches its own 128 rows of A and half of the tile's rows of W, so a K step of 64 costs an SM 32 KB from L2
+// (BN = 256) for the 4.2 MFLOP it computes, two thirds of what a 128 x 256 tile per CTA costs, and the tensor core
+// reads each operand half from its own SM's shared memory once.
+//   warp 0      TMA producer (both CTAs, each its own operand rows; all bytes reported to the even CTA's barrier)
+//   warp 1      MMA issuer (even CTA only): 4 x tcgen05.mma M256 N=BN K16 per stage; the commit frees both CTAs' stage
+//   warps 2..9  epilogue (both CTAs, each its own 128 rows; two warps share 32 rows, half of the columns each)
+// Two accumulators in TMEM let the epilogue of tile i overlap the MMAs of tile i + 1.
+// Bound: at BN = 256 the tensor core (512 clocks a K step) and what an SM can fetch from L2 (64 bytes a clock, 512
+// clocks for 32 KB) meet; at large sizes the 1 kW cap lowers the clock of both.  Measured, 8774 x 9216 x 3072: 325 us,
+// 1530 TFLOP/s (one CTA per 128 x 256 tile, 48 KB a step: 352 us, bound by the fetch); 8774 x 3072 x 12288: 443 us
+// (481); 3510 x 3072 x 12288: 188 us on 256 x 224 (the narrower tile leaves the last of three rounds fuller: 200 on
+// 256 x 256).
+// ---------------------------------------------------------------------------------------------------------------
+template <int BN>
+struct PairCfg {
+  static constexpr int kBBytes = BN / 2 * kBK * 2;
+  static constexpr int kStageBytes = kABytes + kBBytes;
+  static constexpr int kStages = 196608 / kStageBytes;         // 192 KB: 6 (BN = 256) to 8 (BN = 128)
+  static constexpr int kTmemCols = 2 * BN > 256 ? 512 : 256;   // (a power of two)
+  static constexpr size_t kBiasBytes = kEpiWarps * 2 * (BN / 2) * 4;   // a warp's columns of two tiles
+  static constexpr size_t kSmem = kAlignSlack + (size_t)kStages * kStageBytes + kBiasBytes + kBarrierBytes;
+};
+
+// Tile order of the persistent pairs.  Consecutive tile numbers run down kGroupM row tiles (of 256) before moving to
+// the next column tile, and only then to the next band of rows: the 74 tiles in flight at any time then cover about
+// 12 x 6 tiles, whose operands stay in L2 and are shared by the pairs working on them, instead of every pair
+// streaming its own panel of A from DRAM.
+constexpr int kGroupM = 12;
 __device__ __forceinline__ void tile_coords(int tile, int m_tiles, int n_tiles, int& mt, int& nt) {
   const int per_group = kGroupM * n_tiles;
   const int group = tile / per_group;
@@ -107,35 +214,44 @@ __device__ __forceinline__ void tile_coords(int tile, int m_tiles, int n_tiles, 
   nt = r / rows;
 }
 
+template <int BN>
 __global__ void __launch_bounds__(kGemmThreads, 1)
-tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
-               const __nv_bfloat16* __restrict__ bias, const GemmOut out, int M, int Nout, int K,
-               int* __restrict__ status) {
+tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
+                    const __nv_bfloat16* __restrict__ bias, const GemmOut out, int M, int Nout, int K,
+                    int* __restrict__ status) {
+  using Cfg = PairCfg<BN>;
+  constexpr int kStages = Cfg::kStages;
   extern __shared__ uint8_t smem_raw[];
+  // The dynamic shared memory starts at the same offset in both CTAs, and so does everything carved from it: a
+  // descriptor or a barrier offset means the same place in either.
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)kStages * kStageBytes);
-  uint64_t* full = bars;                    // [kStages] TMA -> MMA
-  uint64_t* empty = bars + kStages;         // [kStages] MMA -> TMA
-  uint64_t* acc_full = bars + 2 * kStages;  // [2] MMA -> epilogue
-  uint64_t* acc_empty = acc_full + 2;       // [2] epilogue -> MMA
+  float* s_bias_all = reinterpret_cast<float*>(smem + (size_t)kStages * Cfg::kStageBytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(s_bias_all) + Cfg::kBiasBytes);
+  uint64_t* full = bars;                    // [kStages] both CTAs' TMA -> MMA (the even CTA's is the one in use)
+  uint64_t* empty = bars + kStages;         // [kStages] MMA -> TMA (each CTA its own)
+  uint64_t* acc_full = bars + 2 * kStages;  // [2] MMA -> epilogue (each CTA its own)
+  uint64_t* acc_empty = acc_full + 2;       // [2] both CTAs' epilogues -> MMA (the even CTA's)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m_tiles = (M + kBM - 1) / kBM, n_tiles = (Nout + kBN - 1) / kBN;
+  const uint32_t rank = cluster_rank();
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const int m_tiles = (M + 2 * kBM - 1) / (2 * kBM), n_tiles = (Nout + BN - 1) / BN;
   const int n_tiles_total = m_tiles * n_tiles;
   const int k_blocks = (K + kBK - 1) / kBK;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 4); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&acc_full[i], 1); mbar_init(&acc_empty[i], 2 * kEpiWarps); }
     *abort_flag = 0;
     mbar_fence_init();
   }
   if (warp == 0 && lane == 0) { tma_prefetch_desc(&tm_a); tma_prefetch_desc(&tm_w); }
-  if (warp == 1) { tmem_alloc(tmem_slot, kTmemCols); tmem_relinquish(); }
+  if (warp == 1) tmem_alloc_pair(tmem_slot, Cfg::kTmemCols);
   tc_fence_before();
-  __syncthreads();
+  __syncwarp();
+  cluster_sync();                           // both CTAs' barriers exist before anybody signals across
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
@@ -144,19 +260,23 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     if (lane == 0) {
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < n_tiles_total && ok; tile += gridDim.x) {
+      for (int tile = pair; tile < n_tiles_total && ok; tile += n_pairs) {
         int mt, nt;
         tile_coords(tile, m_tiles, n_tiles, mt, nt);
+        const int row_a = (2 * mt + (int)rank) * kBM, row_w = nt * BN + (int)rank * (BN / 2);
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!(ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag))) break;
-          uint8_t* sa = smem + (size_t)stage * kStageBytes;
-          mbar_expect_tx(&full[stage], kStageBytes);
-          tma_load_2d(sa, &tm_a, &full[stage], kb * kBK, mt * kBM);
-          tma_load_2d(sa + kABytes, &tm_w, &full[stage], kb * kBK, nt * kBN);
+          const uint32_t sa = smem_u32(smem + (size_t)stage * Cfg::kStageBytes);
+          // The even CTA's barrier counts the bytes of both CTAs.  The odd CTA's may land before it is armed: its
+          // phase cannot complete before the arrival that arms it.
+          if (rank == 0) mbar_expect_tx(&full[stage], 2 * Cfg::kStageBytes);
+          const uint32_t bar = cluster_map(smem_u32(&full[stage]), 0);
+          tma_load_2d_pair(sa, &tm_a, bar, kb * kBK, row_a);
+          tma_load_2d_pair(sa + kABytes, &tm_w, bar, kb * kBK, row_w);
           if (++stage == kStages) { stage = 0; phase ^= 1; }
         }
       }
-      // On the way out make sure every stage that was armed has landed (bounded): the CTA must
+      // On the way out make sure every stage that was armed has been consumed (bounded): the CTA must
       // not retire with bulk copies still writing its shared memory.
       for (int i = 0; i < kStages; ++i) {
         if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag)) break;
@@ -164,94 +284,240 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
+    // ------------------------------------------------------------ MMA issuer (even CTA)
     // All 32 lanes run the loop and one elected lane issues: tile counters, stage addresses and descriptors
     // then stay warp-uniform values instead of one diverged lane's private registers, which is what the
     // tensor-core instructions are fed from.
-    {
+    if (rank == 0) {
       const bool leader = elect_one();
-      constexpr uint32_t idesc = idesc_bf16(kBM, kBN, 0);
+      constexpr uint32_t idesc = idesc_bf16(2 * kBM, BN, 0);
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
       int t = 0;
-      for (int tile = blockIdx.x; tile < n_tiles_total && ok; tile += gridDim.x, ++t) {
+      for (int tile = pair; tile < n_tiles_total && ok; tile += n_pairs, ++t) {
         const int acc = t & 1;
         if (!(ok = mbar_wait_warp(&acc_empty[acc], ((t >> 1) & 1) ^ 1, abort_flag))) break;
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)acc * kBN;
+        const uint32_t d_tmem = tmem_base + (uint32_t)acc * BN;
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!(ok = mbar_wait_warp(&full[stage], phase, abort_flag))) break;
           tc_fence_after();
-          const uint32_t sa = smem_u32(smem + (size_t)stage * kStageBytes);
+          const uint32_t sa = smem_u32(smem + (size_t)stage * Cfg::kStageBytes);
           const uint64_t da = smem_desc_sw128(sa, 1024), db = smem_desc_sw128(sa + kABytes, 1024);
           if (leader) {
 #pragma unroll
             for (int k = 0; k < kBK / 16; ++k)   // +32 bytes (encoded >>4) per K step of 16 inside the swizzle atom
-              mma_ss(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
-            mma_commit(&empty[stage]);
+              mma_ss_pair(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
+            mma_commit_pair(&empty[stage]);
           }
           if (++stage == kStages) { stage = 0; phase ^= 1; }
         }
-        if (ok && leader) mma_commit(&acc_full[acc]);
+        if (ok && leader) mma_commit_pair(&acc_full[acc]);
       }
     }
   } else {
-    // ------------------------------------------------------------ epilogue (warps 2..5)
+    // ------------------------------------------------------------ epilogue (warps 2..9)
     const int quad = warp & 3;                 // TMEM lane quadrant this warp may read
+    const int half = (warp - 2) >> 2;          // which half of the tile's columns it finishes
+    float* s_bias_warp = s_bias_all + (size_t)(warp - 2) * BN;
     bool ok = true;
     int t = 0;
-    for (int tile = blockIdx.x; tile < n_tiles_total && ok; tile += gridDim.x, ++t) {
+    for (int tile = pair; tile < n_tiles_total && ok; tile += n_pairs, ++t) {
       int mt, nt;
       tile_coords(tile, m_tiles, n_tiles, mt, nt);
       const int acc = t & 1;
-      ok = mbar_wait(&acc_full[acc], (t >> 1) & 1, abort_flag);
-      ok = __all_sync(0xFFFFFFFFu, ok);
+      const int n_first = nt * BN + half * (BN / 2);
+      // bias and destination of this tile are fetched while its MMAs still run
+      const float* s_bias = s_bias_warp + acc * (BN / 2);
+      stage_bias<BN / 2>(s_bias_warp + acc * (BN / 2), bias, n_first, Nout, lane);
+      const RowOut row = row_out(out, (2 * mt + (int)rank) * kBM + quad * 32 + lane, M);
+      ok = mbar_wait_warp(&acc_full[acc], (t >> 1) & 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
-      const int m = mt * kBM + quad * 32 + lane;
-      const bool row_ok = m < M;
-      int b = 0, li = 0;
-      if (row_ok) { b = m / out.n_sel; li = m - b * out.n_sel; }
-      long long scat_row = 0;
-      if (row_ok) scat_row = (long long)b * out.n_rows + (out.idx ? out.idx[li] : li);
-      const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)acc * kBN;
-#pragma unroll 1
-      for (int c = 0; c < kBN / 32; ++c) {
-        const int n0 = nt * kBN + c * 32;
-        if (n0 >= Nout) break;                 // warp-uniform
-        uint32_t r[32];
-        tmem_ld32(t_row + c * 32, r);
+      const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN + half * (BN / 2));
+      constexpr int kCh = BN % 64 == 0 ? 32 : 16;      // columns per TMEM read: a divisor of the half tile, and of
+      constexpr int kChunks = BN / 2 / kCh;            // its offset, so that no read straddles two segments
+      uint32_t r[2][kCh];
+      tmem_ld(t_row, r[0]);
+#pragma unroll
+      for (int c = 0; c < kChunks; ++c) {
+        const int n0 = n_first + c * kCh;
         tmem_ld_wait();
-        if (row_ok) {
-          const int seg = n0 / out.seg_cols, col0 = n0 - seg * out.seg_cols;
-          const long long drow = out.scatter[seg] ? scat_row : (long long)m;
-          __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(out.ptr[seg]) + drow * out.ld[seg] + col0;
-          const float* gate = out.gate ? out.gate + (long long)b * out.gate_ld + col0 : nullptr;
-          const float seg_scale = (seg == 0 && out.seg0_scale != 0.f) ? out.seg0_scale : 1.0f;   // warp-uniform
-#pragma unroll
-          for (int v = 0; v < 4; ++v) {        // 8 columns = one 16-byte store
-            if (n0 + v * 8 < Nout) {
-              const uint4 braw = __ldg(reinterpret_cast<const uint4*>(bias + n0 + v * 8));
-              const uint32_t bw[4] = {braw.x, braw.y, braw.z, braw.w};
-              uint32_t packed[4];
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                float f0 = __uint_as_float(r[v * 8 + 2 * q]) + __uint_as_float(bw[q] << 16);
-                float f1 = __uint_as_float(r[v * 8 + 2 * q + 1]) + __uint_as_float(bw[q] & 0xFFFF0000u);
-                if (out.act == 1) { f0 = gelu_tanh_f(f0); f1 = gelu_tanh_f(f1); }
-                if (seg_scale != 1.0f) { f0 *= seg_scale; f1 *= seg_scale; }
-                if (gate) { f0 *= gate[v * 8 + 2 * q]; f1 *= gate[v * 8 + 2 * q + 1]; }
-                const __nv_bfloat162 p = __floats2bfloat162_rn(f0, f1);
-                packed[q] = *reinterpret_cast<const uint32_t*>(&p);
-              }
-              *reinterpret_cast<uint4*>(dst + v * 8) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-            }
-          }
-        }
+        if (c + 1 < kChunks) tmem_ld(t_row + (c + 1) * kCh, r[(c + 1) & 1]);
+        if (n0 < Nout) emit<kCh>(r[c & 1], s_bias + c * kCh, n0, Nout, out, row);      // warp-uniform
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[acc]);
+      if (lane == 0) mbar_arrive_cluster(cluster_map(smem_u32(&acc_empty[acc]), 0));
+    }
+  }
+
+  // ---------------------------------------------------------------- teardown
+  tc_fence_before();
+  __syncwarp();
+  cluster_sync();                            // neither CTA leaves while the other may still reach into it
+  if (threadIdx.x == 0 && *abort_flag) atomicExch(status, 1);
+  if (warp == 1) { tc_fence_after(); tmem_dealloc_pair(tmem_base, Cfg::kTmemCols); }
+}
+
+// ---------------------------------------------------------------------------------------------------------------
+// Problems that do not: one tile of 128 x BN per CTA, one launch wave, everything about latency.  A cluster of
+// `split` CTAs shares a tile, each taking a run of its K steps; they then trade partial sums through distributed
+// shared memory, each finishing BN / split of the tile's columns (the partial sums of the other CTAs are added in
+// rank order, so a result does not depend on timing).  Warp roles as above; the epilogue warps fetch bias and
+// destination rows while the MMAs run.  Bound by latency: of 4.7 us at 148 x 768 x 256 (14.0 with one CTA per 128 x 256
+// tile and the bias fetched between accumulator reads) 0.8 us are the K loop, the rest is launch, first fetch and
+// epilogue.  614 x 256 x 768 over two CTAs a tile: 6.1 us (15.6), 371 x 768 x 3072 over four: 9.6 (16.7 over one).
+// ---------------------------------------------------------------------------------------------------------------
+template <int BN>
+struct SplitCfg {
+  static constexpr int kBBytes = BN * kBK * 2;
+  static constexpr int kStageBytes = kABytes + kBBytes;
+  static constexpr int kStages = BN == 128 ? 4 : 6;
+  static constexpr size_t kBiasBytes = kEpiWarps * (BN / 2) * 4;
+  static constexpr int kMaxSplit = BN / 32;                    // a warp finishes at least 16 columns
+  static constexpr size_t part_bytes(int split) { return (size_t)(split - 1) * (BN / split) * kBM * 4; }
+  static constexpr size_t smem(int split) {
+    return kAlignSlack + (size_t)kStages * kStageBytes + part_bytes(split) + kBiasBytes + kBarrierBytes;
+  }
+};
+
+template <int BN>
+__global__ void __launch_bounds__(kGemmThreads)
+tc_gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
+                     const __nv_bfloat16* __restrict__ bias, const GemmOut out, int M, int Nout, int K, int split,
+                     int* __restrict__ status) {
+  using Cfg = SplitCfg<BN>;
+  constexpr int kStages = Cfg::kStages;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  float* s_bias_all = reinterpret_cast<float*>(smem + (size_t)kStages * Cfg::kStageBytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(s_bias_all) + Cfg::kBiasBytes);
+  uint64_t* full = bars;                    // [kStages] TMA -> MMA
+  uint64_t* empty = bars + kStages;         // [kStages] MMA -> TMA
+  uint64_t* acc_full = bars + 2 * kStages;  // MMA -> epilogue
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  float4* s_part = reinterpret_cast<float4*>(reinterpret_cast<uint8_t*>(bars) + kBarrierBytes);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = split > 1 ? (int)cluster_rank() : 0;
+  const int tile = blockIdx.x / split;
+  const int m_tiles = (M + kBM - 1) / kBM;
+  const int mt = tile % m_tiles, nt = tile / m_tiles;
+  const int k_blocks = (K + kBK - 1) / kBK;
+  const int kb0 = k_blocks * rank / split, kb1 = k_blocks * (rank + 1) / split;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    mbar_init(acc_full, 1);
+    *abort_flag = 0;
+    mbar_fence_init();
+  }
+  if (warp == 0 && lane == 0) { tma_prefetch_desc(&tm_a); tma_prefetch_desc(&tm_w); }
+  if (warp == 1) { tmem_alloc(tmem_slot, BN); tmem_relinquish(); }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (split > 1) cluster_arrive();           // waited for before anything is sent to another CTA
+  const uint32_t tmem_base = *tmem_slot;
+
+  if (warp == 0) {
+    // ------------------------------------------------------------ TMA producer
+    if (lane == 0) {
+      int stage = 0; uint32_t phase = 0;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag)) break;
+        uint8_t* sa = smem + (size_t)stage * Cfg::kStageBytes;
+        mbar_expect_tx(&full[stage], Cfg::kStageBytes);
+        tma_load_2d(sa, &tm_a, &full[stage], kb * kBK, mt * kBM);
+        tma_load_2d(sa + kABytes, &tm_w, &full[stage], kb * kBK, nt * BN);
+        if (++stage == kStages) { stage = 0; phase ^= 1; }
+      }
+      for (int i = 0; i < kStages; ++i) {      // all armed stages consumed before the CTA retires
+        if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag)) break;
+        if (++stage == kStages) { stage = 0; phase ^= 1; }
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------ MMA issuer
+    const bool leader = elect_one();
+    constexpr uint32_t idesc = idesc_bf16(kBM, BN, 0);
+    int stage = 0; uint32_t phase = 0;
+    bool ok = true;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      if (!(ok = mbar_wait_warp(&full[stage], phase, abort_flag))) break;
+      tc_fence_after();
+      const uint32_t sa = smem_u32(smem + (size_t)stage * Cfg::kStageBytes);
+      const uint64_t da = smem_desc_sw128(sa, 1024), db = smem_desc_sw128(sa + kABytes, 1024);
+      if (leader) {
+#pragma unroll
+        for (int k = 0; k < kBK / 16; ++k) mma_ss(tmem_base, da + 2 * k, db + 2 * k, idesc, (kb > kb0) || k != 0);
+        mma_commit(&empty[stage]);
+      }
+      if (++stage == kStages) { stage = 0; phase ^= 1; }
+    }
+    if (ok && leader) mma_commit(acc_full);
+  }
+
+  // ------------------------------------------------------------ epilogue (warps 2..9)
+  const int quad = warp & 3;                 // TMEM lane quadrant this warp may read
+  const int half = (warp - 2) >> 2;
+  const int tile_row = quad * 32 + lane;
+  const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16);
+  const int width = BN / split;              // columns this CTA finishes: [rank * width, (rank + 1) * width)
+  const int c_first = rank * width + half * (width / 2);       // ... and this warp: width / 2 of them
+  float* s_bias = s_bias_all + (size_t)(warp - 2) * (BN / 2);
+  RowOut row = {};
+  bool ok = true;
+  if (warp >= 2) {
+    stage_bias<BN / 2>(s_bias, bias, nt * BN + c_first, Nout, lane);
+    row = row_out(out, mt * kBM + tile_row, M);
+    ok = mbar_wait_warp(acc_full, 0, abort_flag);
+    if (ok) tc_fence_after();
+  }
+  if (split > 1) {
+    __syncwarp();
+    cluster_wait();                          // the other CTAs have started (long since)
+    if (warp >= 2 && ok) {
+      // everybody else's columns go to them: slot of the sender, four columns per 16-byte word, row by row
+      for (int c = half * 16; c < BN; c += 32) {
+        const int owner = c / width;
+        if (owner == rank) continue;         // warp-uniform
+        uint32_t r[16];
+        tmem_ld16(t_row + c, r);
+        tmem_ld_wait();
+        const int slot = rank < owner ? rank : rank - 1;
+        const uint32_t base =
+            cluster_map(smem_u32(s_part + ((size_t)slot * (width / 4) + (c - owner * width) / 4) * kBM + tile_row), (uint32_t)owner);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          st_cluster_v4(base + q * kBM * 16, __uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
+                        __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
+      }
+    }
+    __syncwarp();
+    cluster_sync();                          // every wait above is bounded, so everybody gets here
+  }
+  if (warp >= 2 && ok) {
+    for (int c = c_first; c < c_first + width / 2; c += 16) {
+      const int n0 = nt * BN + c;
+      if (n0 >= Nout) break;                 // warp-uniform
+      uint32_t r[16];
+      tmem_ld16(t_row + c, r);
+      tmem_ld_wait();
+      for (int s = 0; s < split - 1; ++s) {
+        const float4* part = s_part + ((size_t)s * (width / 4) + (c - rank * width) / 4) * kBM + tile_row;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float4 v = part[q * kBM];
+          r[4 * q] = __float_as_uint(__uint_as_float(r[4 * q]) + v.x);
+          r[4 * q + 1] = __float_as_uint(__uint_as_float(r[4 * q + 1]) + v.y);
+          r[4 * q + 2] = __float_as_uint(__uint_as_float(r[4 * q + 2]) + v.z);
+          r[4 * q + 3] = __float_as_uint(__uint_as_float(r[4 * q + 3]) + v.w);
+        }
+      }
+      emit<16>(r, s_bias + (c - c_first), n0, Nout, out, row);
     }
   }
 
@@ -259,7 +525,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *abort_flag) atomicExch(status, 1);
-  if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, kTmemCols); }
+  if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, BN); }
 }
 
 // Self-test of the bounded wait: the barrier below is initialised for one arrival that never comes.
@@ -281,6 +547,100 @@ int launch_wait_timeout_selftest(int* d_status, int budget_us, cudaStream_t s) {
   return HERO_OK;
 }
 
+// ---------------------------------------------------------------------------------------------------------------
+// Which kernel, which tile, how many CTAs per tile.  The estimate is in SM clocks: rounds of tiles times K steps times
+// the clocks of a step, plus what a launch costs outside its K loop.  A K step is bound by what an SM can fetch from L2
+// (about 64 bytes per clock): 24 / 32 KB for a tile of 128 x 64 / 128 x 128 in a CTA, 24 / 32 KB per CTA of a pair on
+// 256 x 128 / 256 x 256 (where the tensor core needs 512 clocks as well).  Measured (us) where the choice is close:
+//   M x N x K            pair 256  pair 224  pair 192  pair 128  CTA 128  CTA 64
+//   3510 x 3072 x 3072      51.8      49.5      54.3      64.7     86.3   131.4
+//   5254 x 1152 x 1152      17.6      16.5      15.6      19.0     27.9    42.1
+//   1394 x 3072 x 1024      12.2      15.3      14.5      13.3     17.4
+//   1394 x 1024 x 1024      11.5                           9.3      8.9    13.7
+//   371 x 3072 x 768         9.9                           8.0      7.6     6.7
+// ---------------------------------------------------------------------------------------------------------------
+namespace {
+
+struct GemmPlan { int bn; int split; };        // split 0: the pair kernel
+
+GemmPlan plan_gemm(int M, int Nout, int K) {
+  const int sms = num_sms();
+  const long long kb = (K + kBK - 1) / kBK;
+  auto ceil_div = [](long long a, long long b) { return (a + b - 1) / b; };
+  GemmPlan best = {256, 0};
+  long long best_t = -1;
+  auto consider = [&](int bn, int split, long long t) {
+    if (best_t < 0 || t < best_t) { best_t = t; best = {bn, split}; }
+  };
+  for (int bn : {256, 224, 192, 128}) {
+    const long long tiles = ceil_div(M, 2 * kBM) * ceil_div(Nout, bn);
+    consider(bn, 0, ceil_div(tiles, sms / 2) * kb * (256 + bn * 9 / 8) + 9000 + bn * 8);
+  }
+  for (int bn : {128, 64}) {
+    const long long tiles = ceil_div(M, kBM) * ceil_div(Nout, bn);
+    const int max_split = bn == 128 ? SplitCfg<128>::kMaxSplit : SplitCfg<64>::kMaxSplit;
+    for (int split = 1; split <= max_split; split *= 2) {
+      if (split > kb) break;
+      if (tiles * split > 0x7FFFFFFFll) continue;
+      const long long waves = ceil_div(tiles * split, sms);
+      consider(bn, split, waves * (ceil_div(kb, split) * (bn == 128 ? 520 : 390) + (bn == 128 ? 7000 : 6500)) +
+                              1500 + (split > 1 ? 500 * split : 0));
+    }
+  }
+  return best;
+}
+
+template <int BN>
+int launch_pair(const CUtensorMap& tm_a, const CUtensorMap& tm_w, const void* bias, const GemmOut& out, int M, int Nout,
+                int K, int* d_status, cudaStream_t s) {
+  static PerDeviceOnce attr_once;            // the opt-in is a property of the kernel ON a device
+  HERO_TRY(per_device_once(attr_once, [](int) {
+    HERO_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_pair_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)PairCfg<BN>::kSmem));
+    return HERO_OK;
+  }));
+  const int tiles = ((M + 2 * kBM - 1) / (2 * kBM)) * ((Nout + BN - 1) / BN);
+  const int pairs = tiles < num_sms() / 2 ? tiles : num_sms() / 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(2 * pairs));
+  cfg.blockDim = dim3(kGemmThreads);
+  cfg.dynamicSmemBytes = PairCfg<BN>::kSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  HERO_CUDA_TRY(cudaLaunchKernelEx(&cfg, tc_gemm_pair_kernel<BN>, tm_a, tm_w, (const __nv_bfloat16*)bias, out, M, Nout, K,
+                                   d_status));
+  return HERO_OK;
+}
+
+template <int BN>
+int launch_split(const CUtensorMap& tm_a, const CUtensorMap& tm_w, const void* bias, const GemmOut& out, int M, int Nout,
+                 int K, int split, int* d_status, cudaStream_t s) {
+  static PerDeviceOnce attr_once;
+  HERO_TRY(per_device_once(attr_once, [](int) {
+    HERO_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_split_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)SplitCfg<BN>::smem(SplitCfg<BN>::kMaxSplit)));
+    return HERO_OK;
+  }));
+  const int tiles = ((M + kBM - 1) / kBM) * ((Nout + BN - 1) / BN);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(tiles * split));
+  cfg.blockDim = dim3(kGemmThreads);
+  cfg.dynamicSmemBytes = SplitCfg<BN>::smem(split);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)split; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = split > 1 ? 1 : 0;
+  HERO_CUDA_TRY(cudaLaunchKernelEx(&cfg, tc_gemm_split_kernel<BN>, tm_a, tm_w, (const __nv_bfloat16*)bias, out, M, Nout, K,
+                                   split, d_status));
+  return HERO_OK;
+}
+
+}  // namespace
+
 int launch_tc_gemm(const void* a, const void* w, const void* bias, int M, int Nout, int K, const GemmOut& out,
                    int* d_status, cudaStream_t s) {
   if (M <= 0) return HERO_OK;
@@ -288,6 +648,7 @@ int launch_tc_gemm(const void* a, const void* w, const void* bias, int M, int No
   if (!aligned16(a) || !aligned16(w) || !aligned16(bias)) return HERO_ERR_ALIGN;
   for (int i = 0; i < 3; ++i)
     if (out.ptr[i] && (!aligned16(out.ptr[i]) || out.ld[i] % 8)) return HERO_ERR_ALIGN;
+  const GemmPlan plan = plan_gemm(M, Nout, K);
   CUtensorMap tm_a, tm_w;
   {
     const uint64_t dims[2] = {(uint64_t)K, (uint64_t)M};
@@ -298,20 +659,19 @@ int launch_tc_gemm(const void* a, const void* w, const void* bias, int M, int No
   {
     const uint64_t dims[2] = {(uint64_t)K, (uint64_t)Nout};
     const uint64_t str[1] = {(uint64_t)K * 2};
-    const uint32_t box[2] = {(uint32_t)kBK, (uint32_t)kBN};
+    const uint32_t box[2] = {(uint32_t)kBK, (uint32_t)(plan.split == 0 ? plan.bn / 2 : plan.bn)};
     HERO_TRY(make_tmap_bf16(&tm_w, w, 2, dims, str, box));
   }
-  static PerDeviceOnce attr_once;            // the opt-in is a property of the kernel ON a device
-  HERO_TRY(per_device_once(attr_once, [](int) {
-    HERO_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem));
-    return HERO_OK;
-  }));
-  const int tiles = ((M + kBM - 1) / kBM) * ((Nout + kBN - 1) / kBN);
-  const int grid = tiles < num_sms() ? tiles : num_sms();
-  tc_gemm_kernel<<<grid, kGemmThreads, kGemmSmem, s>>>(tm_a, tm_w, (const __nv_bfloat16*)bias, out, M, Nout, K,
-                                                       d_status);
-  HERO_CUDA_TRY(cudaGetLastError());
-  return HERO_OK;
+  if (plan.split == 0) {
+    switch (plan.bn) {
+      case 256: return launch_pair<256>(tm_a, tm_w, bias, out, M, Nout, K, d_status, s);
+      case 224: return launch_pair<224>(tm_a, tm_w, bias, out, M, Nout, K, d_status, s);
+      case 192: return launch_pair<192>(tm_a, tm_w, bias, out, M, Nout, K, d_status, s);
+      default: return launch_pair<128>(tm_a, tm_w, bias, out, M, Nout, K, d_status, s);
+    }
+  }
+  return plan.bn == 128 ? launch_split<128>(tm_a, tm_w, bias, out, M, Nout, K, plan.split, d_status, s)
+                        : launch_split<64>(tm_a, tm_w, bias, out, M, Nout, K, plan.split, d_status, s);
 }
 
 }  // namespace hero
