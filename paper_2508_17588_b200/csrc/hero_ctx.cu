@@ -164,7 +164,7 @@ bool is_full(const hero_config& g, int step) {
 int run_gemm(hero_ctx* c, const void* a, const void* w, const void* bias, int M, int Nout, int K, const GemmOut& out) {
   LaunchScope scope(c, HERO_PROF_GEMM);
   if (c->cfg.dtype == HERO_DTYPE_BF16) return launch_tc_gemm(a, w, bias, M, Nout, K, out, c->d_status, c->stream);
-  return launch_simt_gemm(a, w, bias, M, Nout, K, out, c->cfg.dtype, c->stream);
+  return launch_simt_gemm((const float*)a, (const float*)w, (const float*)bias, M, Nout, K, out, c->stream);
 }
 
 int run_attention(hero_ctx* c, const void* q, const void* k, const void* v, void* o, int n_q) {
@@ -172,7 +172,8 @@ int run_attention(hero_ctx* c, const void* q, const void* k, const void* v, void
   LaunchScope scope(c, HERO_PROF_ATTENTION);
   if (g.dtype == HERO_DTYPE_BF16)
     return launch_tc_attention(q, k, v, o, g.batch, n_q, c->N, g.n_heads, true, c->d_status, c->status_ctas, c->stream);
-  return launch_simt_attention(q, k, v, o, g.batch, n_q, c->N, g.n_heads, g.head_dim, g.dtype, c->stream);
+  return launch_simt_attention((const float*)q, (const float*)k, (const float*)v, (float*)o, g.batch, n_q, c->N, g.n_heads,
+                               g.head_dim, c->stream);
 }
 
 // adaLN vectors of blocks [l0, l1) into their slots of c->mod, at most kMaxModBatch blocks per launch
@@ -283,8 +284,8 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
       HERO_TRY(launch_tc_attention(c->ws_q, c->kv_cmp[0], c->kv_cmp[1], c->ws_o, B, n_sel, n_att, g.n_heads, true,
                                    c->d_status, c->status_ctas, c->stream));
     else
-      HERO_TRY(launch_simt_attention(c->ws_q, c->kv_cmp[0], c->kv_cmp[1], c->ws_o, B, n_sel, n_att, g.n_heads, g.head_dim,
-                                     g.dtype, c->stream));
+      HERO_TRY(launch_simt_attention((const float*)c->ws_q, (const float*)c->kv_cmp[0], (const float*)c->kv_cmp[1],
+                                     (float*)c->ws_o, B, n_sel, n_att, g.n_heads, g.head_dim, c->stream));
   } else {
     HERO_TRY(run_attention(c, c->ws_q, kdst, vdst, c->ws_o, n_sel));
   }

@@ -158,11 +158,11 @@ int launch_gather_ln_modulate(const void* x, const void* add, const int* idx, co
                               const float* scale, int mod_ld, void* a, int B, int N, int n_sel, int D,
                               float eps, int dtype, cudaStream_t s);
 
-// fp32 / generic CUDA-core path (config 1 runs in fp32, where tensor cores would break parity)
-int launch_simt_gemm(const void* a, const void* w, const void* bias, int M, int Nout, int K,
-                     const GemmOut& out, int dtype, cudaStream_t s);
-int launch_simt_attention(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N,
-                          int heads, int head_dim, int dtype, cudaStream_t s);
+// fp32 CUDA-core path (config 1 runs in fp32, where tensor cores would break parity)
+int launch_simt_gemm(const float* a, const float* w, const float* bias, int M, int Nout, int K, const GemmOut& out,
+                     cudaStream_t s);
+int launch_simt_attention(const float* q, const float* k, const float* v, float* o, int B, int n_q, int N, int heads,
+                          int head_dim, cudaStream_t s);
 
 // bf16 tensor-core path (tcgen05 + TMEM + TMA)
 int tc_init_driver_api();   // resolves cuTensorMapEncodeTiled once

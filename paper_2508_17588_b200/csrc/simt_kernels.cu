@@ -1,183 +1,404 @@
-// CUDA-core GEMM and attention for the fp32 run mode (config "tiny": fp32 parity at ~1e-5
-// against the float64 oracle rules out tensor-core input rounding).  Same epilogue contract
-// as the tensor-core path: bias, optional GELU-tanh / gate, and the merge of Eq. 3 done by
-// writing rows straight into their cache slots.
+// CUDA-core GEMM and attention for the fp32 run mode (fp32 parity at ~1e-5 against the float64 oracle rules out
+// tensor-core input rounding).  Same epilogue contract as the tensor-core path: bias, optional GELU-tanh / gate, and
+// the merge of Eq. 3 done by writing rows straight into their cache slots.
+//
+// Both kernels form dot products of K-contiguous rows from shared memory: operands are copied row by row with
+// cp.async (no transposition), rows are padded to 4 floats more than a multiple of 32 so that eight neighbouring rows
+// read 16 bytes each without a bank conflict, and the products are accumulated in packed pairs of even and odd k
+// (fma.rn.f32x2: the same roundings as two FMAs, half the issue slots).
 #include "hero_internal.h"
+#include "tc_common.cuh"
 
 namespace hero {
 namespace {
-
-template <typename T>
-__device__ __forceinline__ float ldf(const T* p);
-template <>
-__device__ __forceinline__ float ldf<float>(const float* p) { return __ldg(p); }
-template <>
-__device__ __forceinline__ float ldf<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-template <typename T>
-__device__ __forceinline__ void stf(T* p, float v);
-template <>
-__device__ __forceinline__ void stf<float>(float* p, float v) { *p = v; }
-template <>
-__device__ __forceinline__ void stf<__nv_bfloat16>(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
 
 __device__ __forceinline__ float gelu_tanh(float t) {
   const float kAlpha = 0.7978845608028654f;   // sqrt(2/pi)
   return 0.5f * t * (1.0f + tanhf(kAlpha * (t + 0.044715f * t * t * t)));
 }
 
-// C tile 64x64, K step 16, 256 threads, 4x4 outputs per thread, fp32 FMA accumulation.
-constexpr int BM = 64, BN = 64, BK = 16;
-template <typename T>
-__global__ void __launch_bounds__(256) simt_gemm_kernel(const T* __restrict__ A, const T* __restrict__ W,
-                                                        const T* __restrict__ bias, int M, int Nout, int K,
+// 16 bytes from global to shared memory; zeros when the source does not exist.
+__device__ __forceinline__ void cp_async16(float* dst, const float* src, bool exists) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(dst)), "l"(src), "r"(exists ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+__device__ __forceinline__ void dot4(float2& acc, const float4& a, const float4& b) {
+  acc = __ffma2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y), acc);
+  acc = __ffma2_rn(make_float2(a.z, a.w), make_float2(b.z, b.w), acc);
+}
+
+// ---------------------------------------------------------------------------------------------------------------
+// C[M, Nout] = A[M, K] W[Nout, K]^T + bias.  Tile BM x BN per CTA of 256 threads in KG groups: group g multiplies the
+// g-th 32 of every KG * 32 k (so that a problem of few tiles still keeps all four schedulers of an SM busy), each
+// thread TM x TN outputs, rows ty + i * (BM / TM) and columns tx + j * (BN / TN).  The groups' sums are added in group
+// order.  Three chunks of k in the ring.
+// ---------------------------------------------------------------------------------------------------------------
+constexpr int kGemmPitch = 36;           // floats per staged row of 32
+template <int BM, int BN, int TM, int TN>
+struct SimtCfg {
+  static constexpr int kGroupThreads = (BM / TM) * (BN / TN);
+  static constexpr int kGroups = 256 / kGroupThreads;
+  static constexpr int kStages = 3;
+  static constexpr int kStageFloats = kGroups * (BM + BN) * kGemmPitch;
+  static constexpr size_t kSmem = (size_t)kStages * kStageFloats * sizeof(float);
+  static_assert((size_t)(kGroups - 1) * BM * BN <= (size_t)kStages * kStageFloats, "the sums of the groups fit in the ring");
+};
+
+template <int BM, int BN, int TM, int TN>
+__global__ void __launch_bounds__(256) simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ W,
+                                                        const float* __restrict__ bias, int M, int Nout, int K,
                                                         const GemmOut out) {
-  __shared__ float sA[BK][BM + 1];
-  __shared__ float sW[BK][BN + 1];
+  using Cfg = SimtCfg<BM, BN, TM, TN>;
+  constexpr int TX = BN / TN, TY = BM / TM, KG = Cfg::kGroups, kChunk = KG * 32;
+  extern __shared__ __align__(16) float ring[];
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += BK) {
-    for (int e = threadIdx.x; e < BM * BK; e += 256) {
-      const int r = e / BK, c = e - r * BK;
-      const int gm = m0 + r, gk = k0 + c;
-      sA[c][r] = (gm < M && gk < K) ? ldf(A + (long long)gm * K + gk) : 0.f;
-      const int gn = n0 + r;
-      sW[c][r] = (gn < Nout && gk < K) ? ldf(W + (long long)gn * K + gk) : 0.f;
+  const int group = threadIdx.x / Cfg::kGroupThreads, lt = threadIdx.x % Cfg::kGroupThreads;
+  const int tx = lt % TX, ty = lt / TX;
+  const int chunks = (K + kChunk - 1) / kChunk;
+
+  auto load = [&](int chunk) {
+    float* st = ring + (chunk % Cfg::kStages) * Cfg::kStageFloats;
+    // 16-byte packets: (row of A or W, group, packet of 8)
+    for (int e = threadIdx.x; e < (BM + BN) * KG * 8; e += 256) {
+      const int p = e & 7, g = (e >> 3) % KG, r = (e >> 3) / KG;
+      const int k = chunk * kChunk + g * 32 + p * 4;
+      const bool is_a = r < BM;
+      const int row = is_a ? m0 + r : n0 + r - BM;
+      const bool exists = k < K && row < (is_a ? M : Nout);
+      const float* src = (is_a ? A : W) + (exists ? (long long)row * K + k : 0);
+      cp_async16(st + (g * (BM + BN) + r) * kGemmPitch + p * 4, src, exists);
     }
-    __syncthreads();
+  };
+  float2 acc[TM][TN];
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float a[4], w[4];
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) { a[i] = sA[kk][ty * 4 + i]; w[i] = sW[kk][tx * 4 + i]; }
+    for (int j = 0; j < TN; ++j) acc[i][j] = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], w[j], acc[i][j]);
-    }
-    __syncthreads();
+  for (int c = 0; c < Cfg::kStages - 1; ++c) {
+    if (c < chunks) load(c);
+    cp_async_commit();
   }
+  for (int c = 0; c < chunks; ++c) {
+    cp_async_wait<Cfg::kStages - 2>();
+    __syncthreads();                       // chunk c is there for everybody, and nobody reads chunk c - 1 any more
+    if (c + Cfg::kStages - 1 < chunks) load(c + Cfg::kStages - 1);
+    cp_async_commit();
+    const float* sa = ring + (c % Cfg::kStages) * Cfg::kStageFloats + group * (BM + BN) * kGemmPitch;
+    const float* sw = sa + BM * kGemmPitch;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
+    for (int k = 0; k < 32; k += 4) {
+      float4 a[TM], w[TN];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) a[i] = *reinterpret_cast<const float4*>(sa + (ty + i * TY) * kGemmPitch + k);
+#pragma unroll
+      for (int j = 0; j < TN; ++j) w[j] = *reinterpret_cast<const float4*>(sw + (tx + j * TX) * kGemmPitch + k);
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) dot4(acc[i][j], a[i], w[j]);
+    }
+  }
+  cp_async_wait<0>();
+  __syncthreads();                         // the ring is free: the other groups hand their sums to group 0
+  if (KG > 1 && group > 0) {
+    float* dst = ring + (group - 1) * BM * BN + lt;
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) dst[(i * TN + j) * Cfg::kGroupThreads] = acc[i][j].x + acc[i][j].y;
+  }
+  if (KG > 1) __syncthreads();
+  if (group > 0) return;
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    const int m = m0 + ty + i * TY;
     if (m >= M) continue;
     const int b = m / out.n_sel, li = m - b * out.n_sel;
+    const long long scat = (long long)b * out.n_rows + (out.idx ? __ldg(out.idx + li) : li);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
+    for (int j = 0; j < TN; ++j) {
+      const int n = n0 + tx + j * TX;
       if (n >= Nout) continue;
-      const int seg = n / out.seg_cols, col = n - seg * out.seg_cols;
-      float v = acc[i][j] + ldf(bias + n);
+      float v = acc[i][j].x + acc[i][j].y;
+#pragma unroll
+      for (int g = 1; g < KG; ++g) v += ring[(g - 1) * BM * BN + (i * TN + j) * Cfg::kGroupThreads + lt];
+      const bool s1 = n >= out.seg_cols, s2 = n >= 2 * out.seg_cols;
+      const int col = n - (s2 ? 2 * out.seg_cols : (s1 ? out.seg_cols : 0));
+      v += __ldg(bias + n);
       if (out.act == 1) v = gelu_tanh(v);
       if (out.gate) v *= out.gate[(long long)b * out.gate_ld + col];
-      const long long row = out.scatter[seg] ? (long long)b * out.n_rows + (out.idx ? out.idx[li] : li) : (long long)m;
-      stf(reinterpret_cast<T*>(out.ptr[seg]) + row * out.ld[seg] + col, v);
+      void* const base = s2 ? out.ptr[2] : (s1 ? out.ptr[1] : out.ptr[0]);
+      const long long ld = s2 ? out.ld[2] : (s1 ? out.ld[1] : out.ld[0]);
+      const int scatter = s2 ? out.scatter[2] : (s1 ? out.scatter[1] : out.scatter[0]);
+      static_cast<float*>(base)[(scatter ? scat : (long long)m) * ld + col] = v;
     }
   }
 }
 
-// One warp per (query row, head).  Keys are taken 32 at a time: each lane scores one key
-// (full dot product over head_dim), the warp agrees on the running maximum, and the
-// probability-weighted V rows are accumulated with the lanes owning head_dim/32 columns each.
-// Online softmax: no score matrix is stored.
-template <typename T, int HD>
-__global__ void __launch_bounds__(128) simt_attention_kernel(const T* __restrict__ Q, const T* __restrict__ Kc,
-                                                             const T* __restrict__ Vc, T* __restrict__ O, int B,
-                                                             int n_q, int N, int heads) {
-  constexpr int PER = HD / 32;
-  __shared__ float s_q[4][HD];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long w = (long long)blockIdx.x * 4 + warp;
-  const long long total = (long long)B * n_q * heads;
-  const bool active = w < total;
-  const long long wq = active ? w : 0;
-  const int h = (int)(wq % heads);
-  const long long mrow = wq / heads;           // b * n_q + i
-  const int b = (int)(mrow / n_q);
+// ---------------------------------------------------------------------------------------------------------------
+// Flash attention in fp32.  A CTA of 128 threads takes 32 queries of one (batch, head) over a run of keys, 64 at a
+// time (two tiles in flight); a thread owns four query rows (8 row groups) and, of a score tile, the keys tx + 16 j, of
+// the output, HD / 16 features.  Online softmax with a running maximum: no score matrix is stored, P of a warp's own
+// rows passes through shared memory.  Where the grid would leave SMs idle the keys are split over a cluster of
+// `split` CTAs, which then merge their (maximum, sum, output) rows through distributed shared memory, in rank order.
+// ---------------------------------------------------------------------------------------------------------------
+constexpr int kAttQ = 32, kAttK = 64, kAttRows = 4;
+template <int HD>
+struct SimtAttCfg {
+  static constexpr int kPitch = HD + 4, kPPitch = kAttK + 4;
+  static constexpr int kTileFloats = kAttK * kPitch;
+  static constexpr int kFloats = kAttQ * kPitch + kAttQ * kPPitch + 4 * kTileFloats + 2 * kAttQ;
+  static constexpr size_t kSmem = (size_t)kFloats * sizeof(float);
+};
+
+__device__ __forceinline__ float ld_cluster(uint32_t cluster_addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
+  return v;
+}
+
+template <int HD>
+__global__ void __launch_bounds__(128) simt_attention_kernel(const float* __restrict__ Q, const float* __restrict__ Kc,
+                                                             const float* __restrict__ Vc, float* __restrict__ O,
+                                                             int n_q, int N, int heads, int split) {
+  using Cfg = SimtAttCfg<HD>;
+  constexpr int kPitch = Cfg::kPitch, CPT = HD / 16;       // output features per thread
+  extern __shared__ __align__(16) float smem[];
+  float* s_q = smem;
+  float* s_p = s_q + kAttQ * kPitch;
+  float* s_kv = s_p + kAttQ * Cfg::kPPitch;                // [2][K tile, V tile]
+  float* s_ml = s_kv + 4 * Cfg::kTileFloats;               // [kAttQ] maxima, [kAttQ] sums
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int rank = blockIdx.x % split;
+  const int q_tiles = (n_q + kAttQ - 1) / kAttQ;
+  int rest = blockIdx.x / split;
+  const int q0 = (rest % q_tiles) * kAttQ;
+  rest /= q_tiles;
+  const int h = rest % heads, b = rest / heads;
   const int D = heads * HD;
-  const T* q = Q + mrow * D + h * HD;
-  for (int c = lane; c < HD; c += 32) s_q[warp][c] = ldf(q + c);
-  __syncwarp();
+  const float* qb = Q + (long long)b * n_q * D + h * HD;
+  const float* kb = Kc + (long long)b * N * D + h * HD;
+  const float* vb = Vc + (long long)b * N * D + h * HD;
+  const int tiles = (N + kAttK - 1) / kAttK;
+  const int t0 = tiles * rank / split, t1 = tiles * (rank + 1) / split;
+
+  auto load_rows = [&](float* dst, const float* src, int first, int rows, int limit) {
+    for (int e = threadIdx.x; e < rows * (HD / 4); e += 128) {
+      const int r = e / (HD / 4), p = e % (HD / 4);
+      const bool exists = first + r < limit;
+      cp_async16(dst + r * kPitch + p * 4, src + (exists ? (long long)(first + r) * D + p * 4 : 0), exists);
+    }
+  };
+  load_rows(s_q, qb, q0, kAttQ, n_q);
+  if (t0 < t1) {
+    load_rows(s_kv, kb, t0 * kAttK, kAttK, N);
+    load_rows(s_kv + Cfg::kTileFloats, vb, t0 * kAttK, kAttK, N);
+  }
+  cp_async_commit();
+
   const float scale = rsqrtf((float)HD);
-  float m_run = -INFINITY, l_run = 0.f, acc[PER];
+  float m_run[kAttRows], l_run[kAttRows], o[kAttRows][CPT];
 #pragma unroll
-  for (int p = 0; p < PER; ++p) acc[p] = 0.f;
-  const T* kb = Kc + (long long)b * N * D + h * HD;
-  const T* vb = Vc + (long long)b * N * D + h * HD;
-  for (int j0 = 0; j0 < N; j0 += 32) {
-    const int j = j0 + lane;
-    float s = -INFINITY;
-    if (j < N) {
-      const T* kr = kb + (long long)j * D;
-      float dot = 0.f;
-#pragma unroll 8
-      for (int c = 0; c < HD; ++c) dot = fmaf(s_q[warp][c], ldf(kr + c), dot);
-      s = dot * scale;
-    }
-    float m_tile = s;
+  for (int i = 0; i < kAttRows; ++i) {
+    m_run[i] = -INFINITY; l_run[i] = 0.f;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m_tile = fmaxf(m_tile, __shfl_xor_sync(0xFFFFFFFFu, m_tile, o));
-    const float m_new = fmaxf(m_run, m_tile);
-    const float alpha = expf(m_run - m_new);          // exp(-inf) = 0 on the first tile
-    const float p = (j < N) ? expf(s - m_new) : 0.f;
-    float psum = p;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) psum += __shfl_xor_sync(0xFFFFFFFFu, psum, o);
-    l_run = l_run * alpha + psum;
-#pragma unroll
-    for (int pp = 0; pp < PER; ++pp) acc[pp] *= alpha;
-    const int cnt = min(32, N - j0);
-    for (int t = 0; t < cnt; ++t) {
-      const float pt = __shfl_sync(0xFFFFFFFFu, p, t);
-      const T* vr = vb + (long long)(j0 + t) * D;
-#pragma unroll
-      for (int pp = 0; pp < PER; ++pp) acc[pp] = fmaf(pt, ldf(vr + lane + 32 * pp), acc[pp]);
-    }
-    m_run = m_new;
+    for (int c = 0; c < CPT; ++c) o[i][c] = 0.f;
   }
-  if (active) {
-    T* o = O + mrow * D + h * HD;
+  for (int t = t0; t < t1; ++t) {
+    const int buf = (t - t0) & 1;
+    float* s_k = s_kv + buf * 2 * Cfg::kTileFloats;
+    const float* s_v = s_k + Cfg::kTileFloats;
+    cp_async_wait<0>();
+    __syncthreads();                       // tile t is there, and nobody reads the other buffer any more
+    if (t + 1 < t1) {
+      float* nk = s_kv + (buf ^ 1) * 2 * Cfg::kTileFloats;
+      load_rows(nk, kb, (t + 1) * kAttK, kAttK, N);
+      load_rows(nk + Cfg::kTileFloats, vb, (t + 1) * kAttK, kAttK, N);
+      cp_async_commit();
+    }
+    float2 s2[kAttRows][4];
 #pragma unroll
-    for (int pp = 0; pp < PER; ++pp) stf(o + lane + 32 * pp, acc[pp] / l_run);
+    for (int i = 0; i < kAttRows; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s2[i][j] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int c = 0; c < HD; c += 4) {
+      float4 q[kAttRows], k[4];
+#pragma unroll
+      for (int i = 0; i < kAttRows; ++i) q[i] = *reinterpret_cast<const float4*>(s_q + (ty * kAttRows + i) * kPitch + c);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) k[j] = *reinterpret_cast<const float4*>(s_k + (tx + 16 * j) * kPitch + c);
+#pragma unroll
+      for (int i = 0; i < kAttRows; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dot4(s2[i][j], q[i], k[j]);
+    }
+#pragma unroll
+    for (int i = 0; i < kAttRows; ++i) {
+      float s[4], m = m_run[i];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        s[j] = t * kAttK + tx + 16 * j < N ? (s2[i][j].x + s2[i][j].y) * scale : -INFINITY;
+        m = fmaxf(m, s[j]);
+      }
+#pragma unroll
+      for (int d = 1; d < 16; d <<= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, d));
+      const float alpha = expf(m_run[i] - m);          // (m is finite: a tile has at least one key)
+      m_run[i] = m;
+      l_run[i] *= alpha;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float p = expf(s[j] - m);
+        l_run[i] += p;
+        s_p[(ty * kAttRows + i) * Cfg::kPPitch + tx + 16 * j] = p;
+      }
+#pragma unroll
+      for (int c = 0; c < CPT; ++c) o[i][c] *= alpha;
+    }
+    __syncwarp();                          // a warp reads the P rows that its own lanes wrote
+#pragma unroll 4
+    for (int k = 0; k < kAttK; k += 4) {
+      float4 p[kAttRows];
+#pragma unroll
+      for (int i = 0; i < kAttRows; ++i)
+        p[i] = *reinterpret_cast<const float4*>(s_p + (ty * kAttRows + i) * Cfg::kPPitch + k);
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        float v[CPT];
+#pragma unroll
+        for (int c = 0; c < CPT; c += (CPT < 4 ? 2 : 4)) {
+          const float* src = s_v + (k + kk) * kPitch + (CPT < 4 ? tx * 2 : tx * 4 + 16 * c);
+          if constexpr (CPT < 4) {
+            const float2 w = *reinterpret_cast<const float2*>(src);
+            v[0] = w.x; v[1] = w.y;
+          } else {
+            const float4 w = *reinterpret_cast<const float4*>(src);
+            v[c] = w.x; v[c + 1] = w.y; v[c + 2] = w.z; v[c + 3] = w.w;
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < kAttRows; ++i) {
+          const float pk = kk == 0 ? p[i].x : (kk == 1 ? p[i].y : (kk == 2 ? p[i].z : p[i].w));
+#pragma unroll
+          for (int c = 0; c < CPT; ++c) o[i][c] = fmaf(pk, v[c], o[i][c]);
+        }
+      }
+    }
+    __syncwarp();
   }
+#pragma unroll
+  for (int i = 0; i < kAttRows; ++i)
+#pragma unroll
+    for (int d = 1; d < 16; d <<= 1) l_run[i] += __shfl_xor_sync(0xFFFFFFFFu, l_run[i], d);
+  auto feature = [&](int c) { return CPT < 4 ? tx * 2 + c : tx * 4 + (c & 3) + 16 * (c & ~3); };
+
+  if (split == 1) {
+#pragma unroll
+    for (int i = 0; i < kAttRows; ++i) {
+      const int row = q0 + ty * kAttRows + i;
+      if (row >= n_q) continue;
+      float* dst = O + ((long long)b * n_q + row) * D + h * HD;
+#pragma unroll
+      for (int c = 0; c < CPT; ++c) dst[feature(c)] = o[i][c] / l_run[i];
+    }
+    return;
+  }
+  // Merge: every CTA lays its rows out over its (now idle) key and value tiles, then finishes kAttQ / split rows of all.
+  cp_async_wait<0>();
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kAttRows; ++i) {
+    const int row = ty * kAttRows + i;
+#pragma unroll
+    for (int c = 0; c < CPT; ++c) s_kv[row * HD + feature(c)] = o[i][c];
+    if (tx == 0) { s_ml[row] = m_run[i]; s_ml[kAttQ + row] = l_run[i]; }
+  }
+  tc::cluster_sync();
+  for (int e = threadIdx.x; e < kAttQ / split * HD; e += 128) {
+    const int row = rank * (kAttQ / split) + e / HD, col = e % HD;
+    float m = -INFINITY;
+    for (int r = 0; r < split; ++r) m = fmaxf(m, ld_cluster(tc::cluster_map(tc::smem_u32(s_ml + row), r)));
+    float l = 0.f, acc = 0.f;
+    for (int r = 0; r < split; ++r) {
+      const float w = expf(ld_cluster(tc::cluster_map(tc::smem_u32(s_ml + row), r)) - m);
+      l = fmaf(w, ld_cluster(tc::cluster_map(tc::smem_u32(s_ml + kAttQ + row), r)), l);
+      acc = fmaf(w, ld_cluster(tc::cluster_map(tc::smem_u32(s_kv + row * HD + col), r)), acc);
+    }
+    if (q0 + row < n_q) O[((long long)b * n_q + q0 + row) * D + h * HD + col] = acc / l;
+  }
+  tc::cluster_sync();                      // nobody leaves while its rows are being read
+}
+
+template <int BM, int BN, int TM, int TN>
+int gemm_launch(const float* a, const float* w, const float* bias, int M, int Nout, int K, const GemmOut& out,
+                cudaStream_t s) {
+  using Cfg = SimtCfg<BM, BN, TM, TN>;
+  static PerDeviceOnce once;
+  HERO_TRY(per_device_once(once, [](int) {
+    HERO_CUDA_TRY(cudaFuncSetAttribute(simt_gemm_kernel<BM, BN, TM, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)Cfg::kSmem));
+    return HERO_OK;
+  }));
+  const dim3 grid((Nout + BN - 1) / BN, (M + BM - 1) / BM);
+  simt_gemm_kernel<BM, BN, TM, TN><<<grid, 256, Cfg::kSmem, s>>>(a, w, bias, M, Nout, K, out);
+  HERO_CUDA_TRY(cudaGetLastError());
+  return HERO_OK;
+}
+
+template <int HD>
+int attention_launch(const float* q, const float* k, const float* v, float* o, int B, int n_q, int N, int heads,
+                     cudaStream_t s) {
+  using Cfg = SimtAttCfg<HD>;
+  static PerDeviceOnce once;
+  HERO_TRY(per_device_once(once, [](int) {
+    HERO_CUDA_TRY(cudaFuncSetAttribute(simt_attention_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmem));
+    return HERO_OK;
+  }));
+  const long long groups = (long long)B * heads * ((n_q + kAttQ - 1) / kAttQ);
+  const int tiles = (N + kAttK - 1) / kAttK;
+  // keys over a cluster while that still leaves every CTA a tile and the grid within one CTA per SM
+  int split = 1;
+  while (split < 8 && split * 2 <= tiles && groups * split * 2 <= num_sms()) split *= 2;
+  if (groups * split > 0x7FFFFFFFll) return HERO_ERR_ARG;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(groups * split));
+  cfg.blockDim = dim3(128);
+  cfg.dynamicSmemBytes = Cfg::kSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)split; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = split > 1 ? 1 : 0;
+  HERO_CUDA_TRY(cudaLaunchKernelEx(&cfg, simt_attention_kernel<HD>, q, k, v, o, n_q, N, heads, split));
+  return HERO_OK;
 }
 
 }  // namespace
 
-int launch_simt_gemm(const void* a, const void* w, const void* bias, int M, int Nout, int K, const GemmOut& out,
-                     int dtype, cudaStream_t s) {
+int launch_simt_gemm(const float* a, const float* w, const float* bias, int M, int Nout, int K, const GemmOut& out,
+                     cudaStream_t s) {
   if (M <= 0) return HERO_OK;
-  dim3 grid((Nout + BN - 1) / BN, (M + BM - 1) / BM);
-  if (dtype == HERO_DTYPE_BF16)
-    simt_gemm_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>((const __nv_bfloat16*)a, (const __nv_bfloat16*)w,
-                                                         (const __nv_bfloat16*)bias, M, Nout, K, out);
-  else
-    simt_gemm_kernel<float><<<grid, 256, 0, s>>>((const float*)a, (const float*)w, (const float*)bias, M, Nout, K, out);
-  HERO_CUDA_TRY(cudaGetLastError());
-  return HERO_OK;
+  // 64 x 64 tiles (8 x 4 outputs a thread, two groups) where they give every SM work of its own, else 32 x 32 (4 x 4
+  // outputs, four groups)
+  const long long tiles = (long long)((M + 63) / 64) * ((Nout + 63) / 64);
+  if (tiles >= num_sms()) return gemm_launch<64, 64, 8, 4>(a, w, bias, M, Nout, K, out, s);
+  return gemm_launch<32, 32, 4, 4>(a, w, bias, M, Nout, K, out, s);
 }
 
-int launch_simt_attention(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N, int heads,
-                          int head_dim, int dtype, cudaStream_t s) {
-  const long long total = (long long)B * n_q * heads;
-  if (total == 0) return HERO_OK;
-  const unsigned blocks = (unsigned)((total + 3) / 4);
-#define HERO_ATT(T, HD)                                                                                       \
-  simt_attention_kernel<T, HD><<<blocks, 128, 0, s>>>((const T*)q, (const T*)k, (const T*)v, (T*)o, B, n_q, N, heads)
-  if (dtype == HERO_DTYPE_BF16) {
-    if (head_dim == 64) HERO_ATT(__nv_bfloat16, 64);
-    else if (head_dim == 32) HERO_ATT(__nv_bfloat16, 32);
-    else if (head_dim == 128) HERO_ATT(__nv_bfloat16, 128);
-    else return HERO_ERR_ARG;
-  } else {
-    if (head_dim == 64) HERO_ATT(float, 64);
-    else if (head_dim == 32) HERO_ATT(float, 32);
-    else if (head_dim == 128) HERO_ATT(float, 128);
-    else return HERO_ERR_ARG;
+int launch_simt_attention(const float* q, const float* k, const float* v, float* o, int B, int n_q, int N, int heads,
+                          int head_dim, cudaStream_t s) {
+  if (B <= 0 || n_q <= 0) return HERO_OK;
+  switch (head_dim) {
+    case 32: return attention_launch<32>(q, k, v, o, B, n_q, N, heads, s);
+    case 64: return attention_launch<64>(q, k, v, o, B, n_q, N, heads, s);
+    case 128: return attention_launch<128>(q, k, v, o, B, n_q, N, heads, s);
+    default: return HERO_ERR_ARG;
   }
-#undef HERO_ATT
-  HERO_CUDA_TRY(cudaGetLastError());
-  return HERO_OK;
 }
 
 }  // namespace hero

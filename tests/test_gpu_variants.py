@@ -5,7 +5,7 @@ import pytest
 import torch
 
 from workloads import synthetic as S
-from tests.util import rel_l2, to_dev, to_host
+from tests.util import make_pair, rel_l2, to_dev, to_host
 
 pytestmark = pytest.mark.gpu
 
@@ -38,3 +38,31 @@ def test_gemm_tile_variants(M, N, K):
     want = a.astype(np.float64) @ w.astype(np.float64).T + bias.astype(np.float64)
     assert rel_l2(to_host(guard[:M]), want) <= GEMM_TOL
     assert bool((guard[M] == 7.0).all())
+
+
+# fp32 dot products of up to K = 1540 terms and 1045 keys, summed in fp32: the error of such a sum grows with the root
+# of its length, sqrt(1540) * 2^-24 = 2.3e-6, and a block chains a handful of them.
+FP32_TOL = 2e-5
+
+
+@pytest.mark.parametrize("over", [
+    # attention: head dimensions, one query tile and less, keys whole or split over clusters of 2, 4 and 8
+    dict(hidden=128, head_dim=32, n_heads=4, grid_h=5, grid_w=6, n_text=1, batch=1),       # 31 rows: half a key tile
+    dict(hidden=128, head_dim=64, n_heads=2, grid_h=8, grid_w=8, n_text=1, batch=2),       # 65 keys: one in tile two
+    dict(hidden=128, head_dim=128, n_heads=1, grid_h=19, grid_w=23, n_text=5, batch=1),    # 442 keys over four
+    dict(hidden=64, head_dim=64, n_heads=1, grid_h=33, grid_w=31, n_text=22, batch=1),     # 1045 keys over eight
+    # GEMM: 64 x 64 tiles in the full pass, 32 x 32 in the refresh, widths that are no multiple of either
+    dict(hidden=384, head_dim=32, n_heads=12, ffn_dim=1540, grid_h=19, grid_w=23, n_text=5, batch=2, has_gate=1),
+    dict(hidden=192, head_dim=64, n_heads=3, ffn_dim=52, grid_h=31, grid_w=33, n_text=0, batch=2),
+], ids=["half_tile", "65_keys", "hd128_split4", "split8", "wide", "narrow_ffn"])
+def test_fp32_block_variants(over):
+    cfgd = dict(S.CONFIGS["tiny"], n_blocks=1, n_shallow=1, frames=1, seed=41, **over)
+    orc, hero, _ = make_pair(cfgd)
+    x_host = S.tokens(cfgd)
+    for s in range(4):                                     # two full passes, two refreshes
+        temb = S.temb(cfgd, s)
+        want = orc.step(s, x_host, temb)
+        x = to_dev(x_host, "fp32")
+        hero.hero_step(s, x, to_dev(temb, "fp32"))
+        assert rel_l2(to_host(x) - x_host, want - x_host) <= FP32_TOL, s
+    hero.close()
