@@ -518,32 +518,45 @@ gather_ln_modulate_kernel(const T* __restrict__ x, const T* __restrict__ add, co
   }
 }
 
-// bf16 rows of 256 * VPL elements: one WARP per refreshed row, the row held in registers (VPL
-// 16-byte packets per lane), statistics by warp shuffles alone - no block barrier per row, 8 independent
-// rows in flight per CTA.  The CTAs are persistent and each serves ONE batch item: it first puts that
-// item's (1 + scale) and shift vectors into shared memory in fp32 (24 KB at D = 3072, once per CTA), so a
-// row costs its own 6 KB in and 6 KB out of HBM plus shared-memory reads - not 24 KB of L1/L2 traffic for
-// the vectors again.  Layout of the vectors: four planes of float4, [low/high half of a packet's (1 + scale),
-// low/high half of its shift][packet], so that the lanes of a warp read consecutive 16-byte words.
-template <int VPL>
-__global__ void __launch_bounds__(256, (VPL > 12) ? 1 : 2)
-gather_ln_modulate_warp_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ add,
-                               const int* __restrict__ idx, const float* __restrict__ shift,
-                               const float* __restrict__ scale, int mod_ld, __nv_bfloat16* __restrict__ a, int N,
-                               int n_sel, int B, float eps) {
-  using V = Vec<__nv_bfloat16>;
-  constexpr int D = VPL * 256, kPackets = VPL * 32;
-  extern __shared__ float4 s_mod[];                 // [4][kPackets]
+// Rows of up to 32 * VPL packets of 16 bytes: one WARP per refreshed row, the row held in registers (VPL packets per
+// lane, the last of them predicated), statistics by warp shuffles alone - no block barrier per row, 8 independent rows
+// in flight per CTA.  Each CTA serves ONE batch item.
+// The CTAs are persistent and first put their item's (1 + scale) and shift vectors into shared memory in fp32 (24 KB at
+// D = 3072, once per CTA), so a row costs its own 6 KB in and 6 KB out of HBM plus shared-memory reads - not 24 KB of
+// L1/L2 traffic for the vectors again (reading them straight into registers was slower even with one row per warp: 4.6
+// against 4.1 us for 1394 rows of 1024).  Layout: planes of float4, [quarter q of a packet's (1 + scale), of its
+// shift][packet], so that the lanes of a warp read consecutive words.
+// Measured (bf16), against one CTA per row through shared memory: 5254 rows of 1152 26.0 -> 8.0 us, 371 of 768
+// 3.8 -> 3.4, 614 of 256 3.2 -> 2.8; 3510 rows of 3072 12.8 us (3.4 TB/s, mostly ramp), 35552 rows 94 us (4.6 TB/s).
+//
+// An instantiation serves every row width up to its own that the next smaller one does not: the chunks beyond that
+// one's are predicated.
+__host__ __device__ constexpr int ln_full_chunks(int vpl) {
+  return vpl <= 6 ? vpl - 1 : (vpl == 8 ? 6 : (vpl == 10 ? 8 : (vpl == 12 ? 10 : 12)));
+}
+__host__ __device__ constexpr int ln_ctas_per_sm(int vpl) {      // what the registers of a row allow
+  return vpl <= 2 ? 6 : (vpl <= 4 ? 4 : (vpl <= 6 ? 3 : (vpl <= 12 ? 2 : 1)));
+}
+// (EXACT: the row has exactly 32 * VPL packets, nothing is predicated; the wide rows have no registers to spare for it.)
+template <typename T, int VPL, bool EXACT>
+__global__ void __launch_bounds__(256, ln_ctas_per_sm(VPL))
+gather_ln_modulate_warp_kernel(const T* __restrict__ x, const T* __restrict__ add, const int* __restrict__ idx,
+                               const float* __restrict__ shift, const float* __restrict__ scale, int mod_ld,
+                               T* __restrict__ a, int N, int n_sel, int B, int D, float eps) {
+  using V = Vec<T>;
+  constexpr int Q = V::N / 4;                       // float4s of modulation per packet and vector
+  constexpr int kFull = EXACT ? VPL : ln_full_chunks(VPL);    // chunks of 32 packets that every row it serves has
+  const int packets = EXACT ? VPL * 32 : D / V::N;
+  if (EXACT) D = VPL * 32 * V::N;
+  extern __shared__ float4 s_mod[];                 // [2 * Q][packets]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = blockIdx.x % B, slot = blockIdx.x / B, slots = gridDim.x / B;
-  {
-    const float4* sc = reinterpret_cast<const float4*>(scale + (long long)b * mod_ld);
-    const float4* sh = reinterpret_cast<const float4*>(shift + (long long)b * mod_ld);
-    for (int i = threadIdx.x; i < 2 * kPackets; i += 256) {        // float4 i covers columns [4i, 4i + 4)
-      const float4 s4 = __ldg(sc + i), h4 = __ldg(sh + i);
-      s_mod[(i & 1) * kPackets + (i >> 1)] = make_float4(1.0f + s4.x, 1.0f + s4.y, 1.0f + s4.z, 1.0f + s4.w);
-      s_mod[(2 + (i & 1)) * kPackets + (i >> 1)] = h4;
-    }
+  const float4* sc = reinterpret_cast<const float4*>(scale + (long long)b * mod_ld);
+  const float4* sh = reinterpret_cast<const float4*>(shift + (long long)b * mod_ld);
+  for (int i = threadIdx.x; i < Q * packets; i += 256) {         // float4 i covers columns [4i, 4i + 4)
+    const float4 s4 = __ldg(sc + i), h4 = __ldg(sh + i);
+    s_mod[(i % Q) * packets + i / Q] = make_float4(1.0f + s4.x, 1.0f + s4.y, 1.0f + s4.z, 1.0f + s4.w);
+    s_mod[(Q + i % Q) * packets + i / Q] = h4;
   }
   __syncthreads();
   for (int i = slot * 8 + warp; i < n_sel; i += slots * 8) {
@@ -551,69 +564,102 @@ gather_ln_modulate_warp_kernel(const __nv_bfloat16* __restrict__ x, const __nv_b
     const V* xr = reinterpret_cast<const V*>(x + row * D);
     V raw[VPL];
 #pragma unroll
-    for (int c = 0; c < VPL; ++c) raw[c].raw = __ldcs(&xr[c * 32 + lane].raw);
-    float f[VPL][8];
+    for (int c = 0; c < VPL; ++c)
+      if (c < kFull || c * 32 + lane < packets) raw[c].raw = __ldcs(&xr[c * 32 + lane].raw);
+    float f[VPL][V::N];
 #pragma unroll
-    for (int c = 0; c < VPL; ++c) raw[c].unpack(f[c]);
+    for (int c = 0; c < VPL; ++c) {
+      if (c < kFull || c * 32 + lane < packets) {
+        raw[c].unpack(f[c]);
+      } else {
+#pragma unroll
+        for (int q = 0; q < V::N; ++q) f[c][q] = 0.f;
+      }
+    }
     if (add) {
       const V* ar = reinterpret_cast<const V*>(add + row * D);
 #pragma unroll
-      for (int c = 0; c < VPL; ++c) raw[c].raw = __ldcs(&ar[c * 32 + lane].raw);
+      for (int c = 0; c < VPL; ++c)
+        if (c < kFull || c * 32 + lane < packets) raw[c].raw = __ldcs(&ar[c * 32 + lane].raw);
 #pragma unroll
       for (int c = 0; c < VPL; ++c) {
-        float g[8];
-        raw[c].unpack(g);
+        if (c < kFull || c * 32 + lane < packets) {
+          float g[V::N];
+          raw[c].unpack(g);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) f[c][q] += g[q];
+          for (int q = 0; q < V::N; ++q) f[c][q] += g[q];
+        }
       }
     }
     float sum = 0.f;
 #pragma unroll
     for (int c = 0; c < VPL; ++c)
 #pragma unroll
-      for (int q = 0; q < 8; ++q) sum += f[c][q];
+      for (int q = 0; q < V::N; ++q) sum += f[c][q];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
     const float mean = sum / (float)D;
     float sq = 0.f;
 #pragma unroll
     for (int c = 0; c < VPL; ++c)
+      if (c < kFull || c * 32 + lane < packets) {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) { const float d = f[c][q] - mean; sq = fmaf(d, d, sq); }
+        for (int q = 0; q < V::N; ++q) { const float d = f[c][q] - mean; sq = fmaf(d, d, sq); }
+      }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, o);
     const float rstd = 1.0f / sqrtf(sq / (float)D + eps);
     V* out = reinterpret_cast<V*>(a + ((long long)b * n_sel + i) * D);
 #pragma unroll
     for (int c = 0; c < VPL; ++c) {
-      const int v = c * 32 + lane;       // packet index: columns [8v, 8v + 8)
-      const float4 s0 = s_mod[v], s1 = s_mod[kPackets + v], h0 = s_mod[2 * kPackets + v], h1 = s_mod[3 * kPackets + v];
-      const float scl[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-      const float sft[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
-      float r[8];
+      const int v = c * 32 + lane;       // packet index: columns [V::N * v, V::N * (v + 1))
+      if (c < kFull || v < packets) {
+        float r[V::N];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) r[q] = fmaf((f[c][q] - mean) * rstd, scl[q], sft[q]);
-      V o; o.pack(r);
-      __stcs(&out[v].raw, o.raw);
+        for (int q = 0; q < Q; ++q) {
+          const float4 s4 = s_mod[q * packets + v], h4 = s_mod[(Q + q) * packets + v];
+          r[4 * q] = fmaf((f[c][4 * q] - mean) * rstd, s4.x, h4.x);
+          r[4 * q + 1] = fmaf((f[c][4 * q + 1] - mean) * rstd, s4.y, h4.y);
+          r[4 * q + 2] = fmaf((f[c][4 * q + 2] - mean) * rstd, s4.z, h4.z);
+          r[4 * q + 3] = fmaf((f[c][4 * q + 3] - mean) * rstd, s4.w, h4.w);
+        }
+        V o; o.pack(r);
+        __stcs(&out[v].raw, o.raw);
+      }
     }
   }
 }
 
-template <int VPL>
+template <typename T, int VPL>
 int gather_ln_warp(const void* x, const void* add, const int* idx, const float* shift, const float* scale, int mod_ld,
-                   void* a, int N, int n_sel, int B, float eps, cudaStream_t s) {
-  using T = __nv_bfloat16;
-  // persistent CTAs, the same number for every batch item; two per SM (one for the widest rows) is all that fits
-  const int per_sm = VPL > 12 ? 1 : 2;
-  int slots = (num_sms() * per_sm + B - 1) / B;
+                   void* a, int N, int n_sel, int B, int D, float eps, cudaStream_t s) {
+  // the same number of CTAs for every batch item, at most as many as stay resident
+  const int resident = (num_sms() * ln_ctas_per_sm(VPL) + B - 1) / B;
   const int need = (n_sel + 7) / 8;
-  if (slots > need) slots = need;
-  if (slots < 1) slots = 1;
-  const size_t smem = (size_t)4 * VPL * 32 * sizeof(float4);
-  gather_ln_modulate_warp_kernel<VPL><<<(unsigned)(slots * B), 256, smem, s>>>(
-      (const T*)x, (const T*)add, idx, shift, scale, mod_ld, (T*)a, N, n_sel, B, eps);
+  const unsigned grid = (unsigned)((need < resident ? need : resident) * B);
+  const size_t smem = (size_t)2 * D * sizeof(float);
+  bool exact = false;
+  if constexpr (VPL >= 8) exact = D == VPL * 32 * Vec<T>::N;
+  if (exact)
+    gather_ln_modulate_warp_kernel<T, VPL, VPL >= 8><<<grid, 256, smem, s>>>(
+        (const T*)x, (const T*)add, idx, shift, scale, mod_ld, (T*)a, N, n_sel, B, D, eps);
+  else
+    gather_ln_modulate_warp_kernel<T, VPL, false><<<grid, 256, smem, s>>>(
+        (const T*)x, (const T*)add, idx, shift, scale, mod_ld, (T*)a, N, n_sel, B, D, eps);
   HERO_CUDA_TRY(cudaGetLastError());
   return HERO_OK;
+}
+
+// Rows of at most 16 packets a lane; wider ones go through shared memory (gather_ln_modulate_kernel).
+constexpr int kLnMaxPackets = 16;
+template <typename T>
+int gather_ln_dispatch(const void* x, const void* add, const int* idx, const float* shift, const float* scale, int mod_ld,
+                       void* a, int N, int n_sel, int B, int D, float eps, cudaStream_t s) {
+  const int vpl = (D / Vec<T>::N + 31) / 32;
+#define HERO_LN(V) if (vpl <= V) return gather_ln_warp<T, V>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s)
+  HERO_LN(1); HERO_LN(2); HERO_LN(3); HERO_LN(4); HERO_LN(5); HERO_LN(6); HERO_LN(8); HERO_LN(10); HERO_LN(12); HERO_LN(16);
+#undef HERO_LN
+  return HERO_ERR_ARG;
 }
 
 template <typename T>
@@ -816,23 +862,21 @@ int launch_gather_ln_modulate(const void* x, const void* add, const int* idx, co
                               int dtype, cudaStream_t s) {
   const long long rows = (long long)B * n_sel;
   if (rows == 0) return HERO_OK;
+  const bool bf16 = dtype == HERO_DTYPE_BF16;
+  const int per = bf16 ? 8 : 4;
+  if (D % per) return HERO_ERR_ALIGN;
+  // the warp kernel reads the adaLN vectors as float4: every item's slice starts 16-byte aligned when mod_ld % 4 == 0
+  const bool vec_ok = mod_ld % 4 == 0 && ((reinterpret_cast<uintptr_t>(shift) | reinterpret_cast<uintptr_t>(scale)) & 15) == 0;
+  if (vec_ok && D / per <= 32 * kLnMaxPackets)
+    return bf16 ? gather_ln_dispatch<__nv_bfloat16>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s)
+                : gather_ln_dispatch<float>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s);
   const size_t smem = (size_t)D * sizeof(float);
-  if (dtype == HERO_DTYPE_BF16) {
-    using T = __nv_bfloat16;
-    if (D % 8) return HERO_ERR_ALIGN;
-    // the adaLN vectors are read as float4: every block's slice starts 16-byte aligned when mod_ld % 4 == 0
-    const bool vec_ok = mod_ld % 4 == 0 && ((reinterpret_cast<uintptr_t>(shift) | reinterpret_cast<uintptr_t>(scale)) & 15) == 0;
-    if (vec_ok && D == 1024) return gather_ln_warp<4>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, eps, s);
-    if (vec_ok && D == 2048) return gather_ln_warp<8>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, eps, s);
-    if (vec_ok && D == 3072) return gather_ln_warp<12>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, eps, s);
-    if (vec_ok && D == 4096) return gather_ln_warp<16>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, eps, s);
-    gather_ln_modulate_kernel<T><<<(unsigned)rows, kLnThreads, smem, s>>>((const T*)x, (const T*)add, idx, shift,
-                                                                           scale, mod_ld, (T*)a, N, n_sel, D, eps);
-  } else {
-    if (D % 4) return HERO_ERR_ALIGN;
+  if (bf16)
+    gather_ln_modulate_kernel<__nv_bfloat16><<<(unsigned)rows, kLnThreads, smem, s>>>(
+        (const __nv_bfloat16*)x, (const __nv_bfloat16*)add, idx, shift, scale, mod_ld, (__nv_bfloat16*)a, N, n_sel, D, eps);
+  else
     gather_ln_modulate_kernel<float><<<(unsigned)rows, kLnThreads, smem, s>>>(
         (const float*)x, (const float*)add, idx, shift, scale, mod_ld, (float*)a, N, n_sel, D, eps);
-  }
   HERO_CUDA_TRY(cudaGetLastError());
   return HERO_OK;
 }

@@ -40,6 +40,31 @@ def test_gemm_tile_variants(M, N, K):
     assert bool((guard[M] == 7.0).all())
 
 
+@pytest.mark.parametrize("dtype,B,N,D,n_sel,with_add", [
+    # 1 .. 16 packets a lane with the last ones partly or not at all there, few rows and several per warp; wider rows
+    # than the warp kernel takes
+    ("bf16", 2, 40, 8, 40, True), ("bf16", 1, 9, 264, 9, False), ("bf16", 2, 2700, 1152, 2650, True),
+    ("bf16", 3, 2000, 2056, 1900, False), ("bf16", 2, 40, 2816, 17, True), ("bf16", 1, 5000, 4088, 4900, False),
+    ("bf16", 1, 20, 4104, 20, True), ("fp32", 2, 3000, 132, 2900, True), ("fp32", 1, 50, 2048, 33, False),
+    ("fp32", 1, 5000, 1540, 5000, True), ("fp32", 1, 20, 2052, 20, False)])
+def test_gather_ln_variants(dtype, B, N, D, n_sel, with_add):
+    g = torch.Generator(device="cuda").manual_seed(D + n_sel)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    x = (torch.randn(B, N, D, device="cuda", generator=g) * 2 + 0.5).to(dt)
+    add = (torch.randn(B, N, D, device="cuda", generator=g) * 0.3).to(dt) if with_add else None
+    idx = torch.randperm(N, device="cuda", generator=g)[:n_sel].sort().values
+    mod = torch.randn(B, 4 * D, device="cuda", generator=g) * 0.5
+    out = torch.full((B, n_sel, D), float("nan"), device="cuda", dtype=dt)
+    H().hero_gather_ln_modulate(x, add, idx.int(), mod[:, :D], mod[:, D:2 * D], out)
+    rows = x[:, idx].double() + (0 if add is None else add[:, idx].double())
+    mean = rows.mean(-1, keepdim=True)
+    var = (rows - mean).square().mean(-1, keepdim=True)
+    want = (rows - mean) / (var + 1e-5).sqrt() * (1 + mod[:, None, D:2 * D].double()) + mod[:, None, :D].double()
+    # one rounding to the output type (2^-8 relative at most in bf16) over fp32 statistics of D terms (sqrt(4104) 2^-24)
+    tol = 2.0 ** -8 if dtype == "bf16" else 2e-5
+    assert float((out.double() - want).abs().max()) <= tol * float(want.abs().max())
+
+
 # fp32 dot products of up to K = 1540 terms and 1045 keys, summed in fp32: the error of such a sum grows with the root
 # of its length, sqrt(1540) * 2^-24 = 2.3e-6, and a block chains a handful of them.
 FP32_TOL = 2e-5
