@@ -44,6 +44,7 @@ template <typename T, int MODE>
 __global__ void __launch_bounds__(kThreads) moments_kernel(const T* __restrict__ a, const T* __restrict__ b,
                                                           const T* __restrict__ c, long long n, float coef,
                                                           double* __restrict__ out) {
+  stream_order();
   constexpr int V = Pack<T>::N;
   const long long n_vec = n / V;
   const long long stride = (long long)gridDim.x * kThreads;
@@ -99,14 +100,13 @@ int launch(const void* a, const void* b, const void* c, long long n, float coef,
   long long blocks = (n / per + kThreads - 1) / kThreads;
   blocks = blocks < 1 ? 1 : (blocks > (long long)sms * 8 ? (long long)sms * 8 : blocks);
   if (dtype == HERO_DTYPE_BF16)
-    moments_kernel<__nv_bfloat16, MODE><<<(int)blocks, kThreads, 0, s>>>(
-        static_cast<const __nv_bfloat16*>(a), static_cast<const __nv_bfloat16*>(b),
-        static_cast<const __nv_bfloat16*>(c), n, coef, out);
+    HERO_TRY(launch_streaming(moments_kernel<__nv_bfloat16, MODE>, blocks, kThreads, s,
+                           static_cast<const __nv_bfloat16*>(a), static_cast<const __nv_bfloat16*>(b),
+                           static_cast<const __nv_bfloat16*>(c), n, coef, out));
   else
-    moments_kernel<float, MODE><<<(int)blocks, kThreads, 0, s>>>(static_cast<const float*>(a),
-                                                                static_cast<const float*>(b),
-                                                                static_cast<const float*>(c), n, coef, out);
-  HERO_CUDA_TRY(cudaGetLastError());
+    HERO_TRY(launch_streaming(moments_kernel<float, MODE>, blocks, kThreads, s,
+                           static_cast<const float*>(a), static_cast<const float*>(b), static_cast<const float*>(c),
+                           n, coef, out));
   return HERO_OK;
 }
 

@@ -55,6 +55,61 @@ int per_device_once(PerDeviceOnce& once, F&& fn) {
   }
   return HERO_OK;
 }
+
+// ---------------------------------------------------------------------------
+// Launches.  Kernels are launched with programmatic stream serialisation: their blocks may be placed while the kernel
+// before them on the stream still runs, so that launch latency, block start and set-up (barriers, TMEM, tensor-map
+// prefetch) are over when that kernel ends.  In return every block of every kernel calls stream_order() before it
+// touches anything another kernel writes or reads:
+//   * the wait returns when all earlier work on the stream is complete and visible (the kernel before has itself waited
+//     for its own predecessor, so completion carries over), and
+//   * only then may the next kernel's blocks be placed.  A block that uses tensor memory has to have its columns by
+//     then: a block of the next kernel on the same SM could otherwise take them and hold them until this kernel ends.
+//     (stream_order_wait is the first half alone; the second then happens when the block ends.)
+// Measured, all kernels against none (which is the launch order the kernels had before): mini42 schedule (307 rows, 42
+// blocks) 5.36 -> 3.54 ms, width 768 cached step 0.391 -> 0.294, width 1024 cached step 1.156 -> 1.021, fp32 model of width
+// 128 0.141 -> 0.108; the 3072-wide 42-block cached step 59.74 -> 59.39.  Kernels that stream large tensors through more
+// blocks than fit the chip are the exception (launch_streaming): placed early, the residual and extrapolation passes of
+// that step made it 60.5 ms.
+// ---------------------------------------------------------------------------
+#ifdef __CUDACC__
+__device__ __forceinline__ void stream_order_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void stream_order() {
+  stream_order_wait();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+template <class... Params, class... Args>
+int launch_kernel_as(bool early, void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
+                     unsigned cluster, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  HERO_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...));
+  return HERO_OK;
+}
+template <class... Params, class... Args>
+int launch_kernel(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, unsigned cluster,
+                  Args&&... args) {
+  return launch_kernel_as(true, kernel, grid, threads, smem, s, cluster, static_cast<Args&&>(args)...);
+}
+// A kernel that streams large tensors through many small blocks (256 threads, eight resident per SM): placed early only
+// where all its blocks are resident at once.
+int num_sms();
+template <class... Params, class... Args>
+int launch_streaming(void (*kernel)(Params...), long long blocks, unsigned threads, cudaStream_t s, Args&&... args) {
+  return launch_kernel_as(blocks <= 8ll * num_sms(), kernel, (unsigned)blocks, threads, 0, s, 1,
+                          static_cast<Args&&>(args)...);
+}
 static inline size_t dtype_size(int dtype) { return dtype == HERO_DTYPE_BF16 ? 2 : 4; }
 
 // ---------------------------------------------------------------------------
@@ -180,7 +235,5 @@ long long tc_attention_grid(int B, int n_q, int heads);   // CTAs of one attenti
 
 // one thread block, no TMA, no TMEM: a bounded wait on a barrier nobody arms; raises *d_status and returns
 int launch_wait_timeout_selftest(int* d_status, int budget_us, cudaStream_t s);
-
-int num_sms();
 
 }  // namespace hero

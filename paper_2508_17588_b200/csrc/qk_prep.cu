@@ -43,6 +43,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 template <typename T>
 __global__ void __launch_bounds__(256) qk_prep_kernel(QkPrepArgs a) {
+  stream_order();
   const int lane = threadIdx.x & 31;
   const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
   const long long n_items = (long long)a.B * a.n_sel * a.n_heads * 2;
@@ -116,6 +117,7 @@ __global__ void __launch_bounds__(256) qk_prep_kernel(QkPrepArgs a) {
 // position in the 8-lane group that covers the head) and two such chunks half the problem apart, so
 // that 32 bytes per thread are in flight; the LayerNorm sums run over the 8-lane group.
 __global__ void __launch_bounds__(256) qk_prep_hd64_kernel(QkPrepArgs a, int n_chunks_half) {
+  stream_order();
   const int c0 = blockIdx.x * blockDim.x + threadIdx.x;
   const int per_row = a.D >> 3;
   const int n_chunks = (int)((long long)a.B * a.n_sel * 2 * per_row);
@@ -201,8 +203,7 @@ int launch_qk_prep(const QkPrepArgs& a, int dtype, cudaStream_t s) {
   const long long n_chunks = (long long)a.B * a.n_sel * 2 * (a.D / 8);
   if (dtype == HERO_DTYPE_BF16 && a.head_dim == 64 && a.D == a.n_heads * 64 && n_chunks < (1ll << 30)) {
     const int half = (int)((n_chunks + 1) / 2);
-    qk_prep_hd64_kernel<<<(half + 255) / 256, 256, 0, s>>>(a, half);
-    HERO_CUDA_TRY(cudaGetLastError());
+    HERO_TRY(launch_streaming(qk_prep_hd64_kernel, (half + 255) / 256, 256, s, a, half));
     return HERO_OK;
   }
   int dev = 0, sms = 0;
@@ -210,9 +211,8 @@ int launch_qk_prep(const QkPrepArgs& a, int dtype, cudaStream_t s) {
   HERO_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const long long want = (n_items + 7) / 8;                       // 8 warps per block
   const int grid = (int)(want < (long long)sms * 8 ? want : (long long)sms * 8);
-  if (dtype == HERO_DTYPE_BF16) qk_prep_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(a);
-  else qk_prep_kernel<float><<<grid, 256, 0, s>>>(a);
-  HERO_CUDA_TRY(cudaGetLastError());
+  if (dtype == HERO_DTYPE_BF16) HERO_TRY(launch_streaming(qk_prep_kernel<__nv_bfloat16>, grid, 256, s, a));
+  else HERO_TRY(launch_streaming(qk_prep_kernel<float>, grid, 256, s, a));
   return HERO_OK;
 }
 

@@ -6,8 +6,8 @@
 // band sum to a closed form, so a warp knows where its part of the list starts without asking anybody; inside the band
 // each lane rebuilds the keys of its token's patch mates from the old ages, ranks the token, and the warp compacts the
 // winners in ascending row order with ballots.  Ages are double-buffered (read old, write new) because a patch spans
-// several grid rows.  Bound by latency (integer work, a few hundred bytes per warp): 17550 tokens in 14 blocks take
-// SELECT_NOW us; one thread block per selected block, walking the tokens 1024 at a time, took 70.
+// several grid rows.  Bound by latency (integer work, a few hundred bytes per warp): 2790 tokens in 8 blocks take 5.8 us
+// with a cold cache; one thread block per selected block, walking the tokens 1024 at a time, took 59 us for 17550.
 #include "hero_internal.h"
 
 namespace hero {
@@ -42,6 +42,7 @@ __device__ __forceinline__ int band_total_rounded(const SelectGeom& g, int rows)
 }
 
 __global__ void __launch_bounds__(kSelWarps * 32) select_kernel(const SelectGeom g, const SelectBatch batch) {
+  stream_order();
   const int e = blockIdx.y;
   const int lane = threadIdx.x & 31;
   const int H = g.grid_h, W = g.grid_w, ph = g.patch_h, pw = g.patch_w;
@@ -112,8 +113,8 @@ __global__ void __launch_bounds__(kSelWarps * 32) select_kernel(const SelectGeom
 int launch_select(const SelectGeom& g, const SelectBatch& batch, cudaStream_t s) {
   if (batch.n <= 0) return HERO_OK;
   const int bands = g.frames * ((g.grid_h + g.patch_h - 1) / g.patch_h);
-  select_kernel<<<dim3((unsigned)((bands + kSelWarps - 1) / kSelWarps), (unsigned)batch.n), kSelWarps * 32, 0, s>>>(g, batch);
-  HERO_CUDA_TRY(cudaGetLastError());
+  HERO_TRY(launch_kernel(select_kernel, dim3((unsigned)((bands + kSelWarps - 1) / kSelWarps), (unsigned)batch.n),
+                         kSelWarps * 32, 0, s, 1, g, batch));
   return HERO_OK;
 }
 

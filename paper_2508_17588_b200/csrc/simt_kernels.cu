@@ -52,6 +52,7 @@ template <int BM, int BN, int TM, int TN>
 __global__ void __launch_bounds__(256) simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ W,
                                                         const float* __restrict__ bias, int M, int Nout, int K,
                                                         const GemmOut out) {
+  stream_order();
   using Cfg = SimtCfg<BM, BN, TM, TN>;
   constexpr int TX = BN / TN, TY = BM / TM, KG = Cfg::kGroups, kChunk = KG * 32;
   extern __shared__ __align__(16) float ring[];
@@ -166,6 +167,7 @@ template <int HD>
 __global__ void __launch_bounds__(128) simt_attention_kernel(const float* __restrict__ Q, const float* __restrict__ Kc,
                                                              const float* __restrict__ Vc, float* __restrict__ O,
                                                              int n_q, int N, int heads, int split) {
+  stream_order();
   using Cfg = SimtAttCfg<HD>;
   constexpr int kPitch = Cfg::kPitch, CPT = HD / 16;       // output features per thread
   extern __shared__ __align__(16) float smem[];
@@ -345,8 +347,7 @@ int gemm_launch(const float* a, const float* w, const float* bias, int M, int No
     return HERO_OK;
   }));
   const dim3 grid((Nout + BN - 1) / BN, (M + BM - 1) / BM);
-  simt_gemm_kernel<BM, BN, TM, TN><<<grid, 256, Cfg::kSmem, s>>>(a, w, bias, M, Nout, K, out);
-  HERO_CUDA_TRY(cudaGetLastError());
+  HERO_TRY(launch_kernel(simt_gemm_kernel<BM, BN, TM, TN>, grid, 256, Cfg::kSmem, s, 1, a, w, bias, M, Nout, K, out));
   return HERO_OK;
 }
 
@@ -365,17 +366,8 @@ int attention_launch(const float* q, const float* k, const float* v, float* o, i
   int split = 1;
   while (split < 8 && split * 2 <= tiles && groups * split * 2 <= num_sms()) split *= 2;
   if (groups * split > 0x7FFFFFFFll) return HERO_ERR_ARG;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(groups * split));
-  cfg.blockDim = dim3(128);
-  cfg.dynamicSmemBytes = Cfg::kSmem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)split; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = split > 1 ? 1 : 0;
-  HERO_CUDA_TRY(cudaLaunchKernelEx(&cfg, simt_attention_kernel<HD>, q, k, v, o, n_q, N, heads, split));
-  return HERO_OK;
+  return launch_kernel(simt_attention_kernel<HD>, (unsigned)(groups * split), 128, Cfg::kSmem, s, (unsigned)split, q, k,
+                       v, o, n_q, N, heads, split);
 }
 
 }  // namespace

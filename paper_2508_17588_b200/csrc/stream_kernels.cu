@@ -99,6 +99,7 @@ template <typename T>
 __global__ void __launch_bounds__(kStreamThreads) extrapolate_kernel(const T* __restrict__ g_prev,
                                                                      const T* __restrict__ g_last,
                                                                      T* __restrict__ out, long long n, float c) {
+  stream_order();
   using V = Vec<T>;
   const long long n_vec = n / V::N;
   const V* p = reinterpret_cast<const V*>(g_prev);
@@ -139,6 +140,7 @@ template <typename T>
 __global__ void __launch_bounds__(kStreamThreads)
 extrapolate_residual_kernel(T* __restrict__ x, const T* __restrict__ ga_prev, const T* __restrict__ ga_last,
                             const T* __restrict__ gf_prev, const T* __restrict__ gf_last, long long n, float c) {
+  stream_order();
   using V = Vec<T>;
   const long long n_vec = n / V::N;
   V* xv = reinterpret_cast<V*>(x);
@@ -176,6 +178,7 @@ extrapolate_residual_kernel(T* __restrict__ x, const T* __restrict__ ga_prev, co
 template <typename T>
 __global__ void __launch_bounds__(kStreamThreads) extrapolate_group_kernel(T* __restrict__ x, const DeepGroup grp,
                                                                            long long first, long long n, float c) {
+  stream_order();
   using V = Vec<T>;
   const long long n_vec = n / V::N;
   V* xv = reinterpret_cast<V*>(x + first);
@@ -211,6 +214,7 @@ __global__ void __launch_bounds__(kStreamThreads) extrapolate_group_kernel(T* __
 template <typename T>
 __global__ void __launch_bounds__(kStreamThreads) residual2_kernel(T* __restrict__ x, const T* __restrict__ ga,
                                                                    const T* __restrict__ gf, long long n) {
+  stream_order();
   using V = Vec<T>;
   const long long n_vec = n / V::N;
   V* xv = reinterpret_cast<V*>(x);
@@ -276,6 +280,7 @@ template <typename T>
 __global__ void __launch_bounds__(kStreamThreads) residual2_acc_kernel(T* __restrict__ x, const T* __restrict__ ga,
                                                                        const T* __restrict__ gf,
                                                                        float* __restrict__ acc, long long n) {
+  stream_order();
   using V = Vec<T>;
   const long long n_vec = n / V::N;
   V* xv = reinterpret_cast<V*>(x);
@@ -308,6 +313,7 @@ __global__ void __launch_bounds__(kStreamThreads) extrapolate_stack_kernel(T* __
                                                                            const float* __restrict__ s_prev,
                                                                            const float* __restrict__ s_last,
                                                                            long long n, float c) {
+  stream_order();
   using V = Vec<T>;
   const long long n_vec = n / V::N;
   V* xv = reinterpret_cast<V*>(x);
@@ -339,6 +345,7 @@ template <bool GATHER>
 __global__ void __launch_bounds__(256) move_rows_kernel(const uint4* __restrict__ src, const int* __restrict__ idx,
                                                         uint4* __restrict__ dst, int B, int N, int n_sel,
                                                         int row_vec) {
+  stream_order();
   const long long warp_global = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long n_warps = ((long long)gridDim.x * blockDim.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -436,6 +443,7 @@ template <typename T, int MAXB>
 __global__ void __launch_bounds__(256, 2) modulation_kernel(const T* __restrict__ temb, const T* __restrict__ w_mod,
                                                          const T* __restrict__ b_mod, float* __restrict__ mod,
                                                          int B, int n_out, int E) {
+  stream_order();
   extern __shared__ float s_act[];
   modulation_stage_activations<T>(temb, s_act, B, E);
   modulation_rows<T, MAXB>(s_act, w_mod, b_mod, mod, B, n_out, E);
@@ -445,6 +453,7 @@ __global__ void __launch_bounds__(256, 2) modulation_kernel(const T* __restrict_
 template <typename T, int MAXB>
 __global__ void __launch_bounds__(256, 2) modulation_batch_kernel(const T* __restrict__ temb, const ModBatch batch, int B,
                                                                int n_out, int E) {
+  stream_order();
   extern __shared__ float s_act[];
   modulation_stage_activations<T>(temb, s_act, B, E);
   modulation_rows<T, MAXB>(s_act, static_cast<const T*>(batch.w_mod[blockIdx.y]), static_cast<const T*>(batch.b_mod[blockIdx.y]),
@@ -474,6 +483,7 @@ __global__ void __launch_bounds__(kLnThreads)
 gather_ln_modulate_kernel(const T* __restrict__ x, const T* __restrict__ add, const int* __restrict__ idx,
                           const float* __restrict__ shift, const float* __restrict__ scale, int mod_ld,
                           T* __restrict__ a, int N, int n_sel, int D, float eps) {
+  stream_order();
   extern __shared__ float s_row[];   // [D]
   __shared__ float red[kLnThreads / 32];
   using V = Vec<T>;
@@ -543,6 +553,7 @@ __global__ void __launch_bounds__(256, ln_ctas_per_sm(VPL))
 gather_ln_modulate_warp_kernel(const T* __restrict__ x, const T* __restrict__ add, const int* __restrict__ idx,
                                const float* __restrict__ shift, const float* __restrict__ scale, int mod_ld,
                                T* __restrict__ a, int N, int n_sel, int B, int D, float eps) {
+  stream_order();
   using V = Vec<T>;
   constexpr int Q = V::N / 4;                       // float4s of modulation per packet and vector
   constexpr int kFull = EXACT ? VPL : ln_full_chunks(VPL);    // chunks of 32 packets that every row it serves has
@@ -641,12 +652,11 @@ int gather_ln_warp(const void* x, const void* add, const int* idx, const float* 
   bool exact = false;
   if constexpr (VPL >= 8) exact = D == VPL * 32 * Vec<T>::N;
   if (exact)
-    gather_ln_modulate_warp_kernel<T, VPL, VPL >= 8><<<grid, 256, smem, s>>>(
-        (const T*)x, (const T*)add, idx, shift, scale, mod_ld, (T*)a, N, n_sel, B, D, eps);
+    HERO_TRY(launch_kernel(gather_ln_modulate_warp_kernel<T, VPL, VPL >= 8>, grid, 256, smem, s, 1, (const T*)x,
+                           (const T*)add, idx, shift, scale, mod_ld, (T*)a, N, n_sel, B, D, eps));
   else
-    gather_ln_modulate_warp_kernel<T, VPL, false><<<grid, 256, smem, s>>>(
-        (const T*)x, (const T*)add, idx, shift, scale, mod_ld, (T*)a, N, n_sel, B, D, eps);
-  HERO_CUDA_TRY(cudaGetLastError());
+    HERO_TRY(launch_kernel(gather_ln_modulate_warp_kernel<T, VPL, false>, grid, 256, smem, s, 1, (const T*)x,
+                           (const T*)add, idx, shift, scale, mod_ld, (T*)a, N, n_sel, B, D, eps));
   return HERO_OK;
 }
 
@@ -664,8 +674,8 @@ int gather_ln_dispatch(const void* x, const void* add, const int* idx, const flo
 
 template <typename T>
 int extrapolate_t(const void* p, const void* l, void* o, long long n, float c, cudaStream_t s) {
-  extrapolate_kernel<T><<<stream_grid(n / Vec<T>::N), kStreamThreads, 0, s>>>((const T*)p, (const T*)l, (T*)o, n, c);
-  HERO_CUDA_TRY(cudaGetLastError());
+  HERO_TRY(launch_streaming(extrapolate_kernel<T>, stream_grid(n / Vec<T>::N), kStreamThreads, s, (const T*)p,
+                         (const T*)l, (T*)o, n, c));
   return HERO_OK;
 }
 
@@ -686,17 +696,16 @@ int launch_extrapolate_residual(void* x, const void* ga_prev, const void* ga_las
     const long long n_vec = n / Vec<T>::N;
     long long blocks = (n_vec + kStreamThreads - 1) / kStreamThreads;
     blocks = blocks < 1 ? 1 : (blocks > (long long)num_sms() * 32 ? (long long)num_sms() * 32 : blocks);
-    extrapolate_residual_kernel<T><<<(int)blocks, kStreamThreads, 0, s>>>(
-        (T*)x, (const T*)ga_prev, (const T*)ga_last, (const T*)gf_prev, (const T*)gf_last, n, c);
+    HERO_TRY(launch_streaming(extrapolate_residual_kernel<T>, blocks, kStreamThreads, s, (T*)x,
+                           (const T*)ga_prev, (const T*)ga_last, (const T*)gf_prev, (const T*)gf_last, n, c));
   } else {
     using T = float;
     const long long n_vec = n / Vec<T>::N;
     long long blocks = (n_vec + kStreamThreads - 1) / kStreamThreads;
     blocks = blocks < 1 ? 1 : (blocks > (long long)num_sms() * 32 ? (long long)num_sms() * 32 : blocks);
-    extrapolate_residual_kernel<T><<<(int)blocks, kStreamThreads, 0, s>>>(
-        (T*)x, (const T*)ga_prev, (const T*)ga_last, (const T*)gf_prev, (const T*)gf_last, n, c);
+    HERO_TRY(launch_streaming(extrapolate_residual_kernel<T>, blocks, kStreamThreads, s, (T*)x,
+                           (const T*)ga_prev, (const T*)ga_last, (const T*)gf_prev, (const T*)gf_last, n, c));
   }
-  HERO_CUDA_TRY(cudaGetLastError());
   return HERO_OK;
 }
 
@@ -709,22 +718,23 @@ int launch_extrapolate_group(void* x, const DeepGroup& grp, long long first, lon
   long long blocks = (n / per + kStreamThreads - 1) / kStreamThreads;
   blocks = blocks < 1 ? 1 : (blocks > (long long)num_sms() * 16 ? (long long)num_sms() * 16 : blocks);
   if (dtype == HERO_DTYPE_BF16)
-    extrapolate_group_kernel<__nv_bfloat16><<<(int)blocks, kStreamThreads, 0, s>>>((__nv_bfloat16*)x, grp, first, n, c);
+    HERO_TRY(launch_streaming(extrapolate_group_kernel<__nv_bfloat16>, blocks, kStreamThreads, s,
+                           (__nv_bfloat16*)x, grp, first, n, c));
   else
-    extrapolate_group_kernel<float><<<(int)blocks, kStreamThreads, 0, s>>>((float*)x, grp, first, n, c);
-  HERO_CUDA_TRY(cudaGetLastError());
+    HERO_TRY(launch_streaming(extrapolate_group_kernel<float>, blocks, kStreamThreads, s, (float*)x, grp,
+                           first, n, c));
   return HERO_OK;
 }
 
 int launch_residual2(void* x, const void* ga, const void* gf, long long n, int dtype, cudaStream_t s) {
   if (dtype == HERO_DTYPE_BF16) {
     using T = __nv_bfloat16;
-    residual2_kernel<T><<<stream_grid(n / Vec<T>::N), kStreamThreads, 0, s>>>((T*)x, (const T*)ga, (const T*)gf, n);
+    HERO_TRY(launch_streaming(residual2_kernel<T>, stream_grid(n / Vec<T>::N), kStreamThreads, s, (T*)x,
+                           (const T*)ga, (const T*)gf, n));
   } else {
-    residual2_kernel<float><<<stream_grid(n / 4), kStreamThreads, 0, s>>>((float*)x, (const float*)ga,
-                                                                           (const float*)gf, n);
+    HERO_TRY(launch_streaming(residual2_kernel<float>, stream_grid(n / 4), kStreamThreads, s, (float*)x,
+                           (const float*)ga, (const float*)gf, n));
   }
-  HERO_CUDA_TRY(cudaGetLastError());
   return HERO_OK;
 }
 
@@ -737,12 +747,12 @@ static int wide_grid(long long n_vec) {
 int launch_residual2_acc(void* x, const void* ga, const void* gf, float* acc, long long n, int dtype, cudaStream_t s) {
   if (dtype == HERO_DTYPE_BF16) {
     using T = __nv_bfloat16;
-    residual2_acc_kernel<T><<<wide_grid(n / Vec<T>::N), kStreamThreads, 0, s>>>((T*)x, (const T*)ga, (const T*)gf, acc, n);
+    HERO_TRY(launch_streaming(residual2_acc_kernel<T>, wide_grid(n / Vec<T>::N), kStreamThreads, s, (T*)x,
+                           (const T*)ga, (const T*)gf, acc, n));
   } else {
-    residual2_acc_kernel<float><<<wide_grid(n / 4), kStreamThreads, 0, s>>>((float*)x, (const float*)ga,
-                                                                          (const float*)gf, acc, n);
+    HERO_TRY(launch_streaming(residual2_acc_kernel<float>, wide_grid(n / 4), kStreamThreads, s, (float*)x,
+                           (const float*)ga, (const float*)gf, acc, n));
   }
-  HERO_CUDA_TRY(cudaGetLastError());
   return HERO_OK;
 }
 
@@ -751,15 +761,17 @@ int launch_extrapolate_stack(void* x, const float* s_prev, const float* s_last, 
   const float c = (float)k / (float)d;
   if (dtype == HERO_DTYPE_BF16) {
     using T = __nv_bfloat16;
-    extrapolate_stack_kernel<T><<<wide_grid(n / Vec<T>::N), kStreamThreads, 0, s>>>((T*)x, s_prev, s_last, n, c);
+    HERO_TRY(launch_streaming(extrapolate_stack_kernel<T>, wide_grid(n / Vec<T>::N), kStreamThreads, s, (T*)x,
+                           s_prev, s_last, n, c));
   } else {
-    extrapolate_stack_kernel<float><<<wide_grid(n / 4), kStreamThreads, 0, s>>>((float*)x, s_prev, s_last, n, c);
+    HERO_TRY(launch_streaming(extrapolate_stack_kernel<float>, wide_grid(n / 4), kStreamThreads, s, (float*)x,
+                           s_prev, s_last, n, c));
   }
-  HERO_CUDA_TRY(cudaGetLastError());
   return HERO_OK;
 }
 
 static __global__ void attend_list_kernel(const int* __restrict__ idx, int n_sel, int n_text, int* __restrict__ list) {
+  stream_order();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n_text) list[i] = i;
   else if (i < n_text + n_sel) list[i] = idx[i - n_text];
@@ -767,8 +779,7 @@ static __global__ void attend_list_kernel(const int* __restrict__ idx, int n_sel
 int launch_attend_list(const int* idx, int n_sel, int n_text, int* list, cudaStream_t s) {
   const int n = n_text + n_sel;
   if (n <= 0) return HERO_OK;
-  attend_list_kernel<<<(n + 255) / 256, 256, 0, s>>>(idx, n_sel, n_text, list);
-  HERO_CUDA_TRY(cudaGetLastError());
+  HERO_TRY(launch_kernel(attend_list_kernel, (n + 255) / 256, 256, 0, s, 1, idx, n_sel, n_text, list));
   return HERO_OK;
 }
 static int move_rows(bool gather, const void* src, const int* idx, void* dst, int B, int N, int n_sel, int D,
@@ -781,12 +792,11 @@ static int move_rows(bool gather, const void* src, const int* idx, void* dst, in
   const long long cap = (long long)num_sms() * 16;
   if (blocks > cap) blocks = cap;
   if (gather)
-    move_rows_kernel<true><<<(int)blocks, 256, 0, s>>>((const uint4*)src, idx, (uint4*)dst, B, N, n_sel,
-                                                       (int)(row_bytes / 16));
+    HERO_TRY(launch_streaming(move_rows_kernel<true>, blocks, 256, s, (const uint4*)src, idx,
+                           (uint4*)dst, B, N, n_sel, (int)(row_bytes / 16)));
   else
-    move_rows_kernel<false><<<(int)blocks, 256, 0, s>>>((const uint4*)src, idx, (uint4*)dst, B, N, n_sel,
-                                                        (int)(row_bytes / 16));
-  HERO_CUDA_TRY(cudaGetLastError());
+    HERO_TRY(launch_streaming(move_rows_kernel<false>, blocks, 256, s, (const uint4*)src, idx,
+                           (uint4*)dst, B, N, n_sel, (int)(row_bytes / 16)));
   return HERO_OK;
 }
 
@@ -801,21 +811,22 @@ int launch_scatter_rows(const void* src, const int* idx, void* dst, int B, int N
 
 // The kernels are instantiated for 1, 2, 4 and 8 batch items so that a warp's accumulators are as many as it needs.
 template <typename T, int MAXB>
-static void modulation_batch_launch(const void* temb, const ModBatch& batch, int B, int n_out, int E, dim3 grid,
+static int modulation_batch_launch(const void* temb, const ModBatch& batch, int B, int n_out, int E, dim3 grid,
                                     size_t smem, cudaStream_t s) {
-  modulation_batch_kernel<T, MAXB><<<grid, 256, smem, s>>>((const T*)temb, batch, B, n_out, E);
+  return launch_kernel(modulation_batch_kernel<T, MAXB>, grid, 256, smem, s, 1, (const T*)temb, batch, B, n_out, E);
 }
 template <typename T, int MAXB>
-static void modulation_launch(const void* temb, const void* w_mod, const void* b_mod, float* mod, int B, int n_out,
+static int modulation_launch(const void* temb, const void* w_mod, const void* b_mod, float* mod, int B, int n_out,
                               int E, int blocks, size_t smem, cudaStream_t s) {
-  modulation_kernel<T, MAXB><<<blocks, 256, smem, s>>>((const T*)temb, (const T*)w_mod, (const T*)b_mod, mod, B, n_out, E);
+  return launch_kernel(modulation_kernel<T, MAXB>, (unsigned)blocks, 256, smem, s, 1, (const T*)temb, (const T*)w_mod,
+                       (const T*)b_mod, mod, B, n_out, E);
 }
 #define HERO_MOD_DISPATCH(FN, T, ...)                      \
   do {                                                     \
-    if (B <= 1) FN<T, 1>(__VA_ARGS__);                     \
-    else if (B <= 2) FN<T, 2>(__VA_ARGS__);                \
-    else if (B <= 4) FN<T, 4>(__VA_ARGS__);                \
-    else FN<T, kModMaxB>(__VA_ARGS__);                     \
+    if (B <= 1) return FN<T, 1>(__VA_ARGS__);              \
+    if (B <= 2) return FN<T, 2>(__VA_ARGS__);              \
+    if (B <= 4) return FN<T, 4>(__VA_ARGS__);              \
+    return FN<T, kModMaxB>(__VA_ARGS__);                   \
   } while (0)
 
 int launch_modulation_batch(const void* temb, const ModBatch& batch, int B, int n_out, int E, int dtype,
@@ -834,8 +845,6 @@ int launch_modulation_batch(const void* temb, const ModBatch& batch, int B, int 
     if (E % 4) return HERO_ERR_ALIGN;
     HERO_MOD_DISPATCH(modulation_batch_launch, float, temb, batch, B, n_out, E, grid, smem, s);
   }
-  HERO_CUDA_TRY(cudaGetLastError());
-  return HERO_OK;
 }
 
 int launch_modulation(const void* temb, const void* w_mod, const void* b_mod, float* mod, int B, int n_out, int E,
@@ -852,8 +861,6 @@ int launch_modulation(const void* temb, const void* w_mod, const void* b_mod, fl
     if (E % 4) return HERO_ERR_ALIGN;
     HERO_MOD_DISPATCH(modulation_launch, float, temb, w_mod, b_mod, mod, B, n_out, E, blocks, smem, s);
   }
-  HERO_CUDA_TRY(cudaGetLastError());
-  return HERO_OK;
 }
 #undef HERO_MOD_DISPATCH
 
@@ -872,12 +879,12 @@ int launch_gather_ln_modulate(const void* x, const void* add, const int* idx, co
                 : gather_ln_dispatch<float>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s);
   const size_t smem = (size_t)D * sizeof(float);
   if (bf16)
-    gather_ln_modulate_kernel<__nv_bfloat16><<<(unsigned)rows, kLnThreads, smem, s>>>(
-        (const __nv_bfloat16*)x, (const __nv_bfloat16*)add, idx, shift, scale, mod_ld, (__nv_bfloat16*)a, N, n_sel, D, eps);
+    HERO_TRY(launch_kernel(gather_ln_modulate_kernel<__nv_bfloat16>, (unsigned)rows, kLnThreads, smem, s, 1,
+                           (const __nv_bfloat16*)x, (const __nv_bfloat16*)add, idx, shift, scale, mod_ld,
+                           (__nv_bfloat16*)a, N, n_sel, D, eps));
   else
-    gather_ln_modulate_kernel<float><<<(unsigned)rows, kLnThreads, smem, s>>>(
-        (const float*)x, (const float*)add, idx, shift, scale, mod_ld, (float*)a, N, n_sel, D, eps);
-  HERO_CUDA_TRY(cudaGetLastError());
+    HERO_TRY(launch_kernel(gather_ln_modulate_kernel<float>, (unsigned)rows, kLnThreads, smem, s, 1, (const float*)x,
+                           (const float*)add, idx, shift, scale, mod_ld, (float*)a, N, n_sel, D, eps));
   return HERO_OK;
 }
 

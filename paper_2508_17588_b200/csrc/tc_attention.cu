@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(kAttThreads, 1)
 tc_attention_safe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                          const __grid_constant__ CUtensorMap tm_v, __nv_bfloat16* __restrict__ O, int n_q, int N,
                          int heads, const float c, int* __restrict__ status, int* __restrict__ cta_words) {
+  stream_order_wait();                                                 // (TMEM is taken further down, if at all)
   if (cta_words != nullptr && cta_words[blockIdx.x] != 1) return;      // block-uniform
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -512,6 +513,7 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  stream_order();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -761,15 +763,15 @@ int launch_tc_attention(const void* q, const void* k, const void* v, void* o, in
   int* cta_words = grid <= status_ctas ? d_status + 1 : nullptr;
   if (cta_words) {
     if (q_prescaled)
-      tc_attention_fast_kernel<true><<<(unsigned)grid, kFastThreads, kFastSmem, s>>>(
-          tm_q, tm_k, tm_v, (__nv_bfloat16*)o, n_q, N, heads, d_status, cta_words);
+      HERO_TRY(launch_kernel(tc_attention_fast_kernel<true>, (unsigned)grid, kFastThreads, kFastSmem, s, 1, tm_q,
+                             tm_k, tm_v, (__nv_bfloat16*)o, n_q, N, heads, d_status, cta_words));
     else
-      tc_attention_fast_kernel<false><<<(unsigned)grid, kFastThreads, kFastSmem, s>>>(
-          tm_q, tm_k, tm_v, (__nv_bfloat16*)o, n_q, N, heads, d_status, cta_words);
+      HERO_TRY(launch_kernel(tc_attention_fast_kernel<false>, (unsigned)grid, kFastThreads, kFastSmem, s, 1, tm_q,
+                             tm_k, tm_v, (__nv_bfloat16*)o, n_q, N, heads, d_status, cta_words));
   }
-  tc_attention_safe_kernel<<<(unsigned)grid, kAttThreads, kAttSmem, s>>>(
-      tm_q, tm_k, tm_v, (__nv_bfloat16*)o, n_q, N, heads, q_prescaled ? 1.0f : kScoreScaleLog2, d_status, cta_words);
-  HERO_CUDA_TRY(cudaGetLastError());
+  HERO_TRY(launch_kernel(tc_attention_safe_kernel, (unsigned)grid, kAttThreads, kAttSmem, s, 1, tm_q, tm_k, tm_v,
+                         (__nv_bfloat16*)o, n_q, N, heads, q_prescaled ? 1.0f : kScoreScaleLog2, d_status,
+                         cta_words));
   return HERO_OK;
 }
 

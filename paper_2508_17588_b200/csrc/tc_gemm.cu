@@ -254,6 +254,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
   cluster_sync();                           // both CTAs' barriers exist before anybody signals across
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  stream_order();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -421,6 +422,7 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
   tc_fence_after();
   if (split > 1) cluster_arrive();           // waited for before anything is sent to another CTA
   const uint32_t tmem_base = *tmem_slot;
+  stream_order();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -601,18 +603,8 @@ int launch_pair(const CUtensorMap& tm_a, const CUtensorMap& tm_w, const void* bi
   }));
   const int tiles = ((M + 2 * kBM - 1) / (2 * kBM)) * ((Nout + BN - 1) / BN);
   const int pairs = tiles < num_sms() / 2 ? tiles : num_sms() / 2;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(2 * pairs));
-  cfg.blockDim = dim3(kGemmThreads);
-  cfg.dynamicSmemBytes = PairCfg<BN>::kSmem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = 1;
-  HERO_CUDA_TRY(cudaLaunchKernelEx(&cfg, tc_gemm_pair_kernel<BN>, tm_a, tm_w, (const __nv_bfloat16*)bias, out, M, Nout, K,
-                                   d_status));
-  return HERO_OK;
+  return launch_kernel(tc_gemm_pair_kernel<BN>, (unsigned)(2 * pairs), kGemmThreads, PairCfg<BN>::kSmem, s,
+                       2, tm_a, tm_w, (const __nv_bfloat16*)bias, out, M, Nout, K, d_status);
 }
 
 template <int BN>
@@ -625,18 +617,8 @@ int launch_split(const CUtensorMap& tm_a, const CUtensorMap& tm_w, const void* b
     return HERO_OK;
   }));
   const int tiles = ((M + kBM - 1) / kBM) * ((Nout + BN - 1) / BN);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(tiles * split));
-  cfg.blockDim = dim3(kGemmThreads);
-  cfg.dynamicSmemBytes = SplitCfg<BN>::smem(split);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)split; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = split > 1 ? 1 : 0;
-  HERO_CUDA_TRY(cudaLaunchKernelEx(&cfg, tc_gemm_split_kernel<BN>, tm_a, tm_w, (const __nv_bfloat16*)bias, out, M, Nout, K,
-                                   split, d_status));
-  return HERO_OK;
+  return launch_kernel(tc_gemm_split_kernel<BN>, (unsigned)(tiles * split), kGemmThreads, SplitCfg<BN>::smem(split), s,
+                       (unsigned)split, tm_a, tm_w, (const __nv_bfloat16*)bias, out, M, Nout, K, split, d_status);
 }
 
 }  // namespace
