@@ -236,25 +236,24 @@ int hero_gemm_bf16(const void *d_a, const void *d_w, const void *d_bias, void *d
                    int M, int N, int K, int act, void *stream);
 /* O[b,i,h,:] = softmax_j(Q[b,i,h,:] . K[b,j,h,:] / sqrt(head_dim)) V[b,j,h,:], j over all N
  * rows; Q,O are [B,n_q,heads*64] bf16, K,V are [B,N,heads*64] bf16.  No score matrix is stored
- * (Sec. 4.3: the refresh stays compatible with FlashAttention-style kernels).  Two launches: a fast
- * kernel that scales every row by the maximum of its first 96 scores for good, and a second one that
- * recomputes, with a running maximum, the thread blocks in which some later score exceeded that maximum
- * by more than 2^100 (no such block on ordinary inputs: it then returns at once). */
+ * (Sec. 4.3: the refresh stays compatible with FlashAttention-style kernels).  One launch: every row is
+ * scaled by the maximum of its first 96 scores for good, and a thread block in which some later score exceeded that
+ * maximum by more than 2^100 recomputes its rows with a running maximum before it ends (none does on ordinary inputs). */
 int hero_attention_bf16(const void *d_q, const void *d_k, const void *d_v, void *d_o,
                         int B, int n_q, int N, int heads, void *stream);
-/* The same result from the second kernel alone (running maximum, accumulator rescaled in place when a
- * tile exceeds it by 2^8): what hero_attention_bf16 falls back to, exposed for tests and for inputs
- * known to have an extreme dynamic range. */
+/* The same result with the running maximum throughout (accumulator rescaled in place when a tile exceeds it
+ * by 2^8): what a thread block of hero_attention_bf16 falls back to, exposed for tests and for inputs known to
+ * have an extreme dynamic range. */
 int hero_attention_bf16_safe(const void *d_q, const void *d_k, const void *d_v, void *d_o,
                              int B, int n_q, int N, int heads, void *stream);
 
 /* hero_attention_bf16 for a caller that has folded the softmax scale into its queries: d_q holds
  * Q * log2(e) / sqrt(head_dim) (= Q * 0.18033688 at head_dim 64), so a score is the base-2 exponent of its
  * weight and O = sum_j 2^(Q'.K_j) V_j / sum_j 2^(Q'.K_j), the same softmax (Sec. 4.3).  This is the form
- * hero_step and hero_refresh_block use (their QKV projection writes q that way): the fast kernel then takes
+ * hero_step and hero_refresh_block use (their QKV projection writes q that way): the kernel then takes
  * 2^score as it stands, with no row maximum at all.  Exact while every row's largest score lies within
- * about +-100 (bf16 and fp32 share the exponent range); a row sum outside [2^-100, 2^100) hands its thread
- * block to the second kernel, as above.  Shapes, layouts and errors as hero_attention_bf16. */
+ * about +-100 (bf16 and fp32 share the exponent range); a row sum outside [2^-100, 2^100) makes its thread
+ * block recompute, as above.  Shapes, layouts and errors as hero_attention_bf16. */
 int hero_attention_bf16_q_scaled(const void *d_q, const void *d_k, const void *d_v, void *d_o,
                                  int B, int n_q, int N, int heads, void *stream);
 

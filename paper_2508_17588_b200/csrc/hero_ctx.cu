@@ -70,8 +70,9 @@ struct hero_ctx {
   void *ws_a = nullptr, *ws_q = nullptr, *ws_o = nullptr, *ws_u = nullptr;
   float* mod = nullptr;                  // [n_blocks, B, n_mod*D] adaLN vectors, one slot per block
   int* idx_ws = nullptr;                 // [n_shallow, idx_cap] selection lists of the current step
-  int* d_status = nullptr;                // word 0: kernels that gave up on a wait; then one word per attention CTA
-  int status_ctas = 0;
+  float* att_parts = nullptr;             // bf16: partial results of the attention's cut query groups
+  size_t status_bytes = 0;
+  int* d_status = nullptr;                // word 0: thread blocks that gave up on a wait; from word 4: counters of att_parts
   void *x_stage = nullptr, *temb_stage = nullptr;
   int n_full = 0, s_prev = 0, s_last = 0;
   int mode1_n_sel = 0;
@@ -171,7 +172,8 @@ int run_attention(hero_ctx* c, const void* q, const void* k, const void* v, void
   const hero_config& g = c->cfg;
   LaunchScope scope(c, HERO_PROF_ATTENTION);
   if (g.dtype == HERO_DTYPE_BF16)
-    return launch_tc_attention(q, k, v, o, g.batch, n_q, c->N, g.n_heads, true, c->d_status, c->status_ctas, c->stream);
+    return launch_tc_attention(q, k, v, o, g.batch, n_q, c->N, g.n_heads, true, c->att_parts, c->d_status + 4,
+                               c->d_status, nullptr, c->stream);
   return launch_simt_attention((const float*)q, (const float*)k, (const float*)v, (float*)o, g.batch, n_q, c->N, g.n_heads,
                                g.head_dim, c->stream);
 }
@@ -282,7 +284,7 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
     LaunchScope scope(c, HERO_PROF_ATTENTION);
     if (g.dtype == HERO_DTYPE_BF16)
       HERO_TRY(launch_tc_attention(c->ws_q, c->kv_cmp[0], c->kv_cmp[1], c->ws_o, B, n_sel, n_att, g.n_heads, true,
-                                   c->d_status, c->status_ctas, c->stream));
+                                   c->att_parts, c->d_status + 4, c->d_status, nullptr, c->stream));
     else
       HERO_TRY(launch_simt_attention((const float*)c->ws_q, (const float*)c->kv_cmp[0], (const float*)c->kv_cmp[1],
                                      (float*)c->ws_o, B, n_sel, n_att, g.n_heads, g.head_dim, c->stream));
@@ -515,9 +517,9 @@ int hero_init(hero_ctx** out, const hero_config* cfg, const hero_block_weights* 
   A(&c->ws_u, (size_t)cfg->batch * c->N * cfg->ffn_dim * c->esz);
   A((void**)&c->mod, (size_t)cfg->n_blocks * cfg->batch * c->n_mod * cfg->hidden * sizeof(float));
   A((void**)&c->idx_ws, (size_t)(cfg->n_shallow > 0 ? cfg->n_shallow : 1) * c->idx_cap * sizeof(int));
-  // the largest attention launch of this context is the full pass (n_q = N)
-  c->status_ctas = cfg->dtype == HERO_DTYPE_BF16 ? (int)tc_attention_grid(cfg->batch, c->N, cfg->n_heads) : 0;
-  A((void**)&c->d_status, (size_t)(4 + c->status_ctas) * sizeof(int));
+  if (cfg->dtype == HERO_DTYPE_BF16) A((void**)&c->att_parts, tc_attention_part_bytes());
+  c->status_bytes = (4 + (cfg->dtype == HERO_DTYPE_BF16 ? tc_attention_part_counters() : 0)) * sizeof(int);
+  A((void**)&c->d_status, c->status_bytes);
   A(&c->x_stage, tensor);
   A(&c->temb_stage, (size_t)cfg->batch * cfg->temb_dim * c->esz);
   if (rc != HERO_OK) { hero_destroy(c); return rc; }
@@ -525,7 +527,7 @@ int hero_init(hero_ctx** out, const hero_config* cfg, const hero_block_weights* 
     cudaError_t er = cudaMemcpy(c->rope_tab, rope_host.data(), rope_host.size() * sizeof(float2), cudaMemcpyHostToDevice);
     if (er != cudaSuccess) { set_cuda_error(er, "cudaMemcpy(rope table)"); hero_destroy(c); return HERO_ERR_CUDA; }
   }
-  cudaError_t e = cudaMemsetAsync(c->d_status, 0, (size_t)(4 + c->status_ctas) * sizeof(int), c->stream);
+  cudaError_t e = cudaMemsetAsync(c->d_status, 0, c->status_bytes, c->stream);
   if (e != cudaSuccess) { set_cuda_error(e, "cudaMemsetAsync"); hero_destroy(c); return HERO_ERR_CUDA; }
   rc = hero_reset(c);
   if (rc != HERO_OK) { hero_destroy(c); return rc; }
@@ -585,7 +587,7 @@ int hero_check_status(hero_ctx* c) {
   HERO_CUDA_TRY(cudaMemcpyAsync(&st, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   HERO_CUDA_TRY(cudaStreamSynchronize(c->stream));
   if (st != 0) {
-    cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
+    cudaMemsetAsync(c->d_status, 0, c->status_bytes, c->stream);     // (a block that gave up has not counted its parts in)
     return HERO_ERR_TIMEOUT;
   }
   return HERO_OK;
@@ -837,8 +839,7 @@ int hero_gather_ln_modulate(const void* d_x, const void* d_add, const int* d_idx
 
 // The isolated tensor-core calls own a status word each; a timeout is reported on the next call.
 // The words live in the memory of the device that is current at the call (one set per device, kept until exit):
-// word 0 for give-ups, then one word per attention CTA (larger grids run the safe attention kernel alone).
-constexpr int kIsolatedStatusCtas = 65536;
+// word 0 counts give-ups.
 static int* isolated_status() {
   static PerDeviceOnce once;
   static int* word[kMaxDevices];
@@ -846,7 +847,7 @@ static int* isolated_status() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
   const int rc = per_device_once(once, [](int d) {
     int* p = nullptr;
-    const size_t bytes = (size_t)(4 + kIsolatedStatusCtas) * sizeof(int);
+    const size_t bytes = 4 * sizeof(int);
     if (cudaMalloc((void**)&p, bytes) != cudaSuccess) { cudaGetLastError(); return HERO_ERR_NOMEM; }
     if (cudaMemset(p, 0, bytes) != cudaSuccess) { cudaFree(p); return HERO_ERR_CUDA; }
     word[d] = p;
@@ -884,7 +885,7 @@ int hero_attention_bf16(const void* q, const void* k, const void* v, void* o, in
   if (!q || !k || !v || !o) return HERO_ERR_ARG;
   int* st = isolated_status();
   if (!st) return HERO_ERR_NOMEM;
-  return launch_tc_attention(q, k, v, o, B, n_q, N, heads, false, st, kIsolatedStatusCtas, (cudaStream_t)stream);
+  return launch_tc_attention(q, k, v, o, B, n_q, N, heads, false, nullptr, nullptr, st, nullptr, (cudaStream_t)stream);
 }
 
 int hero_attention_bf16_q_scaled(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N,
@@ -894,7 +895,7 @@ int hero_attention_bf16_q_scaled(const void* q, const void* k, const void* v, vo
   if (!q || !k || !v || !o) return HERO_ERR_ARG;
   int* st = isolated_status();
   if (!st) return HERO_ERR_NOMEM;
-  return launch_tc_attention(q, k, v, o, B, n_q, N, heads, true, st, kIsolatedStatusCtas, (cudaStream_t)stream);
+  return launch_tc_attention(q, k, v, o, B, n_q, N, heads, true, nullptr, nullptr, st, nullptr, (cudaStream_t)stream);
 }
 
 int hero_attention_bf16_safe(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N, int heads,

@@ -223,12 +223,14 @@ int launch_simt_attention(const float* q, const float* k, const float* v, float*
 int tc_init_driver_api();   // resolves cuTensorMapEncodeTiled once
 int launch_tc_gemm(const void* a, const void* w, const void* bias, int M, int Nout, int K,
                    const GemmOut& out, int* d_status, cudaStream_t s);
-// d_status: word 0 (give-up counter) followed by status_ctas per-CTA words
 // The tensor-core attention serves head_dim 64: a score s enters the softmax as 2^(s * kScoreScaleLog2).
 constexpr float kScoreScaleLog2 = 0.125f * 1.4426950408889634f;   // 1/sqrt(64) * log2(e)
 // q_prescaled: Q holds q * kScoreScaleLog2 (the softmax scale folded into the projection)
 int launch_tc_attention(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N,
-                        int heads, bool q_prescaled, int* d_status, int status_ctas, cudaStream_t s);
+                        int heads, bool q_prescaled, float* parts, int* part_count, int* d_status, int* cta_words,
+                        cudaStream_t s);
+size_t tc_attention_part_bytes();       // workspace of an attention launch that may cut query groups
+size_t tc_attention_part_counters();    // and its counters (ints, zero between launches)
 int launch_tc_attention_safe(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N,
                              int heads, bool q_prescaled, int* d_status, cudaStream_t s);
 long long tc_attention_grid(int B, int n_q, int heads);   // CTAs of one attention launch

@@ -30,10 +30,22 @@
 //    the exponent of its weight: that instantiation (PRESCALED) takes p = 2^s as it stands - no maximum,
 //    no first-tile exchange, no multiply-add per pair of scores - and is exact while a row's largest score
 //    stays within about +-100; its row sum must then lie in [2^-100, 2^100), else the CTA is marked.
-//  * tc_attention_safe_kernel recomputes exactly those CTAs (same grid, every other CTA returns at
-//    once) with a running maximum that moves whenever a tile exceeds it by 2^8, rescaling the
-//    accumulator in TMEM; it is also the whole computation when no per-CTA status words are available.
-//    12 warps, one thread per row, one-pass tiles with a two-pass redo when the maximum has to move.
+//  * The safe path (safe_roles) keeps a running maximum that moves whenever a tile exceeds it by 2^8, rescaling the
+//    accumulator in TMEM: 12 warps, one thread per row.  A thread block of the fast kernel whose row sums say that the
+//    range assumption failed recomputes its queries with it before it ends (a second launch for the failed blocks, as it
+//    used to be, cost every attention 2-4 us at small sizes and 14 us at 1728 blocks for finding nothing to do);
+//    tc_attention_safe_kernel is the same path as a kernel of its own.
+//
+// The fast kernel comes in three modes (attention_plan says which runs when).  With the scale folded into Q there is no
+// maximum, so the partial results of a query group over disjoint runs of keys simply add; that is what the last two use:
+//  * kWhole: one thread block per query group (256 queries of one batch item and head), all keys;
+//  * kCluster, for grids that leave SMs idle: a cluster of blocks per group, each with a run of the key tiles; they trade
+//    16-column pieces of their accumulators through distributed shared memory, each finishing its own;
+//  * kCut, for grids of several rounds over long key sequences: persistent blocks, one per SM, work through whole groups a
+//    grid apart (so that the blocks in flight stay on few heads and share their K and V in L2), and what is left for the
+//    last, partly filled round is cut into runs of key tiles over ALL blocks.  Every warp lays its rows of a part out in a
+//    workspace and counts itself in; the one that completes the count adds all parts and writes the rows.
+// Parts are added in a fixed order, so that no result depends on timing, and nobody ever waits for another block of kCut.
 //
 #include <cuda.h>
 
@@ -172,53 +184,88 @@ __device__ __forceinline__ void fused_tile(uint32_t t_buf, float c, float neg_mc
   m_tile = fmaxf(mx[0], mx[1]);
 }
 
-// Status words: status[0] counts the CTAs that gave up on a bounded wait; cta_words (may be null) holds one
-// word per CTA: 0 = done, 1 = the fast kernel's range assumption failed here (to be recomputed), 2 = gave up.
-// With cta_words given, this kernel only works on the CTAs marked 1.
-__global__ void __launch_bounds__(kAttThreads, 1)
-tc_attention_safe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                         const __grid_constant__ CUtensorMap tm_v, __nv_bfloat16* __restrict__ O, int n_q, int N,
-                         int heads, const float c, int* __restrict__ status, int* __restrict__ cta_words) {
-  stream_order_wait();                                                 // (TMEM is taken further down, if at all)
-  if (cta_words != nullptr && cta_words[blockIdx.x] != 1) return;      // block-uniform
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint8_t* s_q = smem;
-  uint8_t* s_kv = smem + kQTiles * kQBytes;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(s_kv + (size_t)kKvStages * kKvStageBytes);
-  uint64_t* q_full = bars;
-  uint64_t* kv_full = bars + 1;                    // [kKvStages]           TMA -> both issuers
+// The two passes of softmax_tile in reads of 16 columns, for a caller that has no registers for a whole row.
+__device__ __forceinline__ float softmax_tile_lean(uint32_t t_buf, int valid, float c, float& m_used, float& alpha,
+                                                   bool& grow) {
+  float m_tile = -INFINITY;
+#pragma unroll 1
+  for (int ch = 0; ch < kKT / 16; ++ch) {
+    uint32_t s[16];
+    tmem_ld16(t_buf + ch * 16, s);
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (ch * 16 + i < valid) m_tile = fmaxf(m_tile, __uint_as_float(s[i]));
+  }
+  grow = (m_tile - m_used) * c > kRescaleLog2;
+  const float m_new = grow ? m_tile : m_used;
+  alpha = grow ? ex2((m_used - m_new) * c) : 1.0f;
+  m_used = m_new;
+  const float neg_mc = -m_new * c;
+  float sum = 0.f;
+#pragma unroll 1
+  for (int ch = 0; ch < kKT / 16; ++ch) {              // P of chunk ch goes over columns that were read before
+    uint32_t s[16], packed[8];
+    tmem_ld16(t_buf + ch * 16, s);
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int col = ch * 16 + 2 * i;
+      const float p0 = col < valid ? ex2(fmaf(__uint_as_float(s[2 * i]), c, neg_mc)) : 0.f;
+      const float p1 = col + 1 < valid ? ex2(fmaf(__uint_as_float(s[2 * i + 1]), c, neg_mc)) : 0.f;
+      sum += p0 + p1;
+      const __nv_bfloat162 b = __floats2bfloat162_rn(p0, p1);
+      packed[i] = *reinterpret_cast<const uint32_t*>(&b);
+    }
+    tmem_st8(t_buf + ch * 8, packed);
+  }
+  return sum;
+}
+
+// One thread block's work on the safe path.
+struct SafeWork {
+  const CUtensorMap *tm_q, *tm_k, *tm_v;
+  __nv_bfloat16* O;
+  int n_q, N, heads, qg, h, b;
+  float c;                       // factor that turns a score into the exponent of its weight
+  uint32_t row_mask;             // which 32-row slices (query tile * 4 + quadrant) of the group are written
+  uint8_t *s_q, *s_kv;
+  uint64_t* bars;                // kSafeBars barriers, set up by safe_init_barriers, never used before
+  volatile int* abort_flag;
+  uint32_t tmem_base;
+};
+constexpr int kSafeBars = 1 + 2 * kKvStages + 4 + 4 + 2 * kQTiles;
+// The last query group of a (batch, head) may reach into its second tile by no row at all: that tile's
+// issuer and softmax warps then have nothing to do and the K/V stages are released by one issuer alone.
+__device__ __forceinline__ int live_tiles(int qg, int n_q) { return (qg * kQTiles + 1) * kQT < n_q ? kQTiles : 1; }
+__device__ __forceinline__ void safe_init_barriers(uint64_t* bars, int n_tiles) {
+  mbar_init(bars, 1);
+  for (int i = 0; i < kKvStages; ++i) { mbar_init(bars + 1 + i, 1); mbar_init(bars + 1 + kKvStages + i, n_tiles); }
+  for (int i = 0; i < 4; ++i) { mbar_init(bars + 1 + 2 * kKvStages + i, 1); mbar_init(bars + 5 + 2 * kKvStages + i, 4); }
+  for (int i = 0; i < 2 * kQTiles; ++i) mbar_init(bars + 9 + 2 * kKvStages + i, 1);
+}
+
+// Warp 0: TMA producer, warps 1 and 2: MMA issuers, warps 4 .. 11: softmax (any others: nothing).
+template <bool LEAN>
+__device__ __forceinline__ void safe_roles(const SafeWork& w) {
+  const CUtensorMap &tm_q = *w.tm_q, &tm_k = *w.tm_k, &tm_v = *w.tm_v;
+  const int n_q = w.n_q, N = w.N, heads = w.heads, qg = w.qg, h = w.h, b = w.b;
+  const float c = w.c;
+  const uint32_t row_mask = w.row_mask;
+  uint8_t *const s_q = w.s_q, *const s_kv = w.s_kv;
+  volatile int* const abort_flag = w.abort_flag;
+  const uint32_t tmem_base = w.tmem_base;
+  __nv_bfloat16* const O = w.O;
+  uint64_t* q_full = w.bars;
+  uint64_t* kv_full = q_full + 1;                  // [kKvStages]           TMA -> both issuers
   uint64_t* kv_empty = kv_full + kKvStages;        // [kKvStages], count 2  both issuers -> TMA
   uint64_t* s_full = kv_empty + kKvStages;         // [qt][parity]  issuer -> softmax: S is ready
   uint64_t* p_full = s_full + 4;                   // [qt][parity]  softmax -> issuer: P is in TMEM
   uint64_t* pv_full = p_full + 4;                  // [qt]          issuer -> softmax: P V of tile j done (phase j)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pv_full + 2);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
+  uint64_t* pv_last = pv_full + kQTiles;           // [qt]          issuer -> softmax: all P V done
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int q_groups = (n_q + kQT * kQTiles - 1) / (kQT * kQTiles);
-  const int qg = blockIdx.x % q_groups;
-  const int h = (blockIdx.x / q_groups) % heads;
-  const int b = blockIdx.x / (q_groups * heads);
   const int n_kv = (N + kKT - 1) / kKT;
-  // the last query group of a (batch, head) may reach into its second tile by no row at all: that tile's
-  // issuer and softmax warps then have nothing to do and the K/V stages are released by one issuer alone
-  const int n_tiles = (qg * kQTiles + 1) * kQT < n_q ? kQTiles : 1;
-
-  if (threadIdx.x == 0) {
-    mbar_init(q_full, 1);
-    for (int i = 0; i < kKvStages; ++i) { mbar_init(&kv_full[i], 1); mbar_init(&kv_empty[i], n_tiles); }
-    for (int i = 0; i < 4; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_full[i], 4); }
-    for (int i = 0; i < kQTiles; ++i) mbar_init(&pv_full[i], 1);
-    *abort_flag = 0;
-    mbar_fence_init();
-  }
-  if (warp == 0 && lane == 0) { tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v); }
-  if (warp == 1) { tmem_alloc(tmem_slot, kAttTmemCols); tmem_relinquish(); }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const int n_tiles = live_tiles(qg, n_q);
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -270,6 +317,7 @@ tc_attention_safe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
 #pragma unroll
         for (int k = 0; k < kKT / 16; ++k) mma_ts(t_tile + kColO, buf + 8 * k, dv + 128 * k, idesc_pv, (j | k) != 0);
         mma_commit(&pv_full[t]);
+        if (j == n_kv - 1) mma_commit(&pv_last[t]);
         mma_commit(&kv_empty[st]);               // second arrival comes from the other tile's issuer
         if (j + 2 < n_kv) {
           // S of tile j+2 overwrites the buffer whose P the product above reads: safe because the
@@ -297,15 +345,20 @@ tc_attention_safe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       float alpha = 1.0f, sum;
       bool grow = true;                                // first and ragged tiles take the two-pass path
       uint32_t packed[kKT / 2];
-      if (j > 0 && !ragged) {
+      if (!LEAN && j > 0 && !ragged) {
         float m_tile;
         fused_tile(t_buf, c, -m_used * c, packed, sum, m_tile);
         grow = __any_sync(0xFFFFFFFFu, (m_tile - m_used) * c > kRescaleLog2);
       }
       if (grow) {                                      // warp-uniform
         bool moved;
-        sum = ragged ? softmax_tile<true>(t_buf, valid, c, m_used, alpha, moved)
-                     : softmax_tile<false>(t_buf, valid, c, m_used, alpha, moved);
+        if (LEAN) {
+          sum = softmax_tile_lean(t_buf, valid, c, m_used, alpha, moved);
+          grow = __any_sync(0xFFFFFFFFu, moved);
+        } else {
+          sum = ragged ? softmax_tile<true>(t_buf, valid, c, m_used, alpha, moved)
+                       : softmax_tile<false>(t_buf, valid, c, m_used, alpha, moved);
+        }
       } else {
 #pragma unroll
         for (int ch = 0; ch < kKT / 32; ++ch)
@@ -314,8 +367,8 @@ tc_attention_safe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       l_run = fmaf(l_run, alpha, sum);
       if (j > 0 && grow) {
         // Rare (warp-uniform): the maximum moved, so the accumulator is scaled down before this tile's
-        // product is added to it - once P V of tile j-1 has completed.  pv_full is only looked at here and
-        // at the very end, yet the parity wait is unambiguous: S of tile j was issued after P V of tile j-2
+        // product is added to it - once P V of tile j-1 has completed.  pv_full is only looked at here, yet the
+        // parity wait is unambiguous: S of tile j was issued after P V of tile j-2
         // (so that one is complete) and P V of tile j cannot start before this warp's arrival below, hence
         // the barrier has completed either j-1 or j phases and "phase j-1 complete" is exactly the question.
         ok = mbar_wait_warp(&pv_full[t], (j - 1) & 1, abort_flag);
@@ -340,7 +393,8 @@ tc_attention_safe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       __syncwarp();
       if (lane == 0) mbar_arrive(&p_full[t * 2 + (j & 1)]);
     }
-    if (ok) ok = mbar_wait_warp(&pv_full[t], (n_kv - 1) & 1, abort_flag);
+    // (Not pv_full: the other warps may still be two tiles behind this one, and its parity cannot tell that.)
+    if (ok) ok = mbar_wait_warp(&pv_last[t], 0, abort_flag);
     if (ok) {
       tc_fence_after();
       const int qi = (qg * kQTiles + t) * kQT + quad * 32 + lane;
@@ -351,7 +405,7 @@ tc_attention_safe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         uint32_t r[16];
         tmem_ld16(lane_base + kColO + ch * 16, r);     // warp-collective: every lane loads
         tmem_ld_wait();
-        if (qi < n_q) {
+        if (qi < n_q && (row_mask >> (t * 4 + quad) & 1)) {
           uint32_t w[8];
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
@@ -365,15 +419,45 @@ tc_attention_safe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       }
     }
   }
+}
 
-  // ---------------------------------------------------------------- teardown
+// status[0] counts the thread blocks that gave up on a bounded wait.
+__global__ void __launch_bounds__(kAttThreads, 1)
+tc_attention_safe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+                         const __grid_constant__ CUtensorMap tm_v, __nv_bfloat16* __restrict__ O, int n_q, int N,
+                         int heads, const float c, int* __restrict__ status) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  SafeWork w = {&tm_q, &tm_k, &tm_v, O, n_q, N, heads};
+  w.s_q = smem;
+  w.s_kv = smem + kQTiles * kQBytes;
+  w.bars = reinterpret_cast<uint64_t*>(w.s_kv + (size_t)kKvStages * kKvStageBytes);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(w.bars + kSafeBars);
+  w.abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  w.c = c;
+  w.row_mask = ~0u;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int q_groups = (n_q + kQT * kQTiles - 1) / (kQT * kQTiles);
+  w.qg = blockIdx.x % q_groups;
+  w.h = (blockIdx.x / q_groups) % heads;
+  w.b = blockIdx.x / (q_groups * heads);
+  if (threadIdx.x == 0) {
+    safe_init_barriers(w.bars, live_tiles(w.qg, n_q));
+    *w.abort_flag = 0;
+    mbar_fence_init();
+  }
+  if (warp == 0 && lane == 0) { tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v); }
+  if (warp == 1) { tmem_alloc(tmem_slot, kAttTmemCols); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    if (*abort_flag) atomicAdd(status, 1);
-    if (cta_words != nullptr) cta_words[blockIdx.x] = *abort_flag ? 2 : 0;
-  }
-  if (warp == 1) { __syncwarp(); tc_fence_after(); tmem_dealloc(tmem_base, kAttTmemCols); }
+  tc_fence_after();
+  w.tmem_base = *tmem_slot;
+  stream_order();
+  safe_roles<false>(w);
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && *w.abort_flag) atomicAdd(status, 1);
+  if (warp == 1) { __syncwarp(); tc_fence_after(); tmem_dealloc(w.tmem_base, kAttTmemCols); }
 }
 
 // =============================================================================================
@@ -383,7 +467,10 @@ constexpr int kFastSoftmaxWarps = 16;            // 2 query tiles x 4 TMEM lane 
 constexpr int kFastThreads = 32 * (kFirstSoftmaxWarp + kFastSoftmaxWarps);   // 20 warps
 constexpr int kHalf = kKT / 2;                   // score columns of a key tile that one thread owns
 constexpr int kXchgFloats = kQTiles * kQT * 2;   // one slot per (query row, column half)
-constexpr size_t kFastSmem = kAttSmem + 2 * kXchgFloats * sizeof(float) + 64;
+constexpr int kMaxBad = 64;                      // out-of-range row slices a block keeps a list of
+constexpr size_t kFastBarBytes = 512;
+constexpr size_t kFastSmem = 1024 + 2 * kQTiles * kQBytes + (size_t)kKvStages * kKvStageBytes + kFastBarBytes +
+                             2 * kXchgFloats * sizeof(float) + (kMaxBad + 2) * sizeof(int);
 constexpr float kRowSumLimit = 1.2676506e30f;    // 2^100: a row sum at or beyond it voids the fixed-maximum assumption
 constexpr float kRowSumFloor = 7.8886091e-31f;   // 2^-100: below it a row without a maximum has lost its small terms
 static_assert(kHalf % 16 == 0 && (kHalf / 16) % 2 == 1, "three 16-column reads per half: the ping-pong below ends on ra");
@@ -464,47 +551,122 @@ __device__ __forceinline__ float half_tile(uint32_t t_s, int valid, const float2
   return (a01.x + a01.y) + (a23.x + a23.y);
 }
 
-template <bool PRESCALED>
+// (its registers are its own business: a call keeps the fast path's allocation out of it)
+static __device__ __noinline__ void safe_recompute(const SafeWork& w) { safe_roles<true>(w); }
+
+// 16 output features of one row: accumulator times 1 / row sum, bf16.
+__device__ __forceinline__ void emit16(const uint32_t (&r)[16], float inv, __nv_bfloat16* dst) {
+  uint32_t w[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const __nv_bfloat162 pk = __floats2bfloat162_rn(__uint_as_float(r[2 * q]) * inv, __uint_as_float(r[2 * q + 1]) * inv);
+    w[q] = *reinterpret_cast<const uint32_t*>(&pk);
+  }
+  *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+  *reinterpret_cast<uint4*>(dst + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+}
+
+// How one launch's query groups are dealt out.  Block c takes the groups c, c + blocks, ... (`rounds` of them at most), then
+// one share of the key tiles of the remaining `tail` groups, laid end to end and numbered from 0.  These fall into spans of
+// equal length (one group each, or all of them together), every span into `per_span` shares whose lengths differ by one
+// tile at most: share_base, the first share_rest of them one more.
+struct AttentionPlan {
+  int groups, blocks, rounds, tiles;             // tiles: key tiles of a group
+  int tail, span, per_span, share_base, share_rest;
+  __device__ __forceinline__ int share_start(int c) const {
+    const int s = c / per_span, i = c - s * per_span;
+    return min(s * span + i * share_base + min(i, share_rest), tail * tiles);
+  }
+  __device__ __forceinline__ int share_of(int unit) const {      // the block whose share holds this tile
+    const int s = unit / span, v = unit - s * span, border = share_rest * (share_base + 1);
+    return s * per_span + (v < border ? v / (share_base + 1) : share_rest + (v - border) / share_base);
+  }
+};
+// A run of key tiles of one group; a block's runs in the order it works on them.
+struct Run {
+  int group, first, n;                           // key tiles [first, first + n) of the group
+};
+enum AttentionMode { kWhole, kCluster, kCut };
+template <AttentionMode MODE>
+struct RunIter {
+  const AttentionPlan& plan;
+  int block, k = 0, u = 0, end = 0;
+  __device__ __forceinline__ RunIter(const AttentionPlan& p, int c) : plan(p), block(c) {}
+  __device__ __forceinline__ bool next(Run& r) {
+    if (MODE != kCut) {                          // one run only
+      if (k++) return false;
+      r.group = MODE == kWhole ? block : block / plan.per_span;
+      r.first = MODE == kWhole ? 0 : plan.share_start(block) - r.group * plan.tiles;
+      r.n = MODE == kWhole ? plan.tiles : plan.share_start(block + 1) - r.group * plan.tiles - r.first;
+      return true;
+    }
+    if (k < plan.rounds) {
+      r.group = block + k * plan.blocks; r.first = 0; r.n = plan.tiles;
+      ++k;
+      return r.group < plan.groups;
+    }
+    if (plan.tail == 0) return false;
+    if (k == plan.rounds) { u = plan.share_start(block); end = plan.share_start(block + 1); ++k; }
+    if (u >= end) return false;
+    const int g = u / plan.tiles;
+    r.group = plan.groups - plan.tail + g;
+    r.first = u - g * plan.tiles;
+    r.n = min(end - u, plan.tiles - r.first);
+    u += r.n;
+    return true;
+  }
+};
+// Workspace of a launch that cuts groups: per block two slots (its first and its last run), per slot and softmax warp
+// 32 rows x 32 accumulator columns (eight float4 planes) and the 32 row sums; one counter per block and warp.
+constexpr int kPartFloats = 8 * 32 * 4 + 32;
+constexpr size_t kSlotFloats = (size_t)kFastSoftmaxWarps * kPartFloats;
+
+// cta_words (may be null): one word per query group, set to 2 where a block gave up on a bounded wait.
+template <bool PRESCALED, AttentionMode MODE>
 __global__ void __launch_bounds__(kFastThreads, 1)
 tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                          const __grid_constant__ CUtensorMap tm_v, __nv_bfloat16* __restrict__ O, int n_q, int N,
-                         int heads, int* __restrict__ status, int* __restrict__ cta_words) {
+                         int heads, const __grid_constant__ AttentionPlan plan, float* __restrict__ parts,
+                         int* __restrict__ part_count, int* __restrict__ status, int* __restrict__ cta_words) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint8_t* s_q = smem;
-  uint8_t* s_kv = smem + kQTiles * kQBytes;
+  uint8_t* s_q = smem;                             // [2] query groups: the next one is fetched while this one is worked on
+  uint8_t* s_kv = smem + 2 * kQTiles * kQBytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(s_kv + (size_t)kKvStages * kKvStageBytes);
-  uint64_t* q_full = bars;
-  uint64_t* kv_full = bars + 1;                    // [kKvStages]           TMA -> both issuers
+  uint64_t* q_full = bars;                         // [2]           TMA -> both issuers
+  uint64_t* q_empty = q_full + 2;                  // [2], count 2  both issuers -> TMA
+  uint64_t* kv_full = q_empty + 2;                 // [kKvStages]           TMA -> both issuers
   uint64_t* kv_empty = kv_full + kKvStages;        // [kKvStages], count 2  both issuers -> TMA
   uint64_t* s_full = kv_empty + kKvStages;         // [qt][parity]  issuer -> softmax: S is ready
   uint64_t* p_full = s_full + 4;                   // [qt][parity]  softmax -> issuer: P is in TMEM (8 warps)
-  uint64_t* pv_full = p_full + 4;                  // [qt]          issuer -> softmax: the last P V is done
+  uint64_t* pv_full = p_full + 4;                  // [qt]          issuer -> softmax: the last P V of a run is done
   uint64_t* pair_bar = pv_full + 2;                // [qt][quadrant] the two warps that share 32 query rows
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pair_bar + 8);
+  uint64_t* safe_bars = pair_bar + 8;              // for the safe path, should this block need it
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(safe_bars + kSafeBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  int* cta_bad = const_cast<int*>(abort_flag) + 1;
-  float* xchg_m = reinterpret_cast<float*>(smem + kAttSmem - 1024);   // behind the barrier block (512 bytes are plenty)
-  float* xchg_l = xchg_m + kXchgFloats;
+  static_assert((4 + 2 * kKvStages + 4 + 4 + 2 + 8 + kSafeBars) * 8 + 8 <= (int)kFastBarBytes, "barrier block");
+  float* xchg = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kFastBarBytes);   // [2][kXchgFloats]
+  int* n_bad = reinterpret_cast<int*>(xchg + 2 * kXchgFloats);
+  int* bad = n_bad + 1;                            // [kMaxBad] group * 8 + query tile * 4 + quadrant
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q_groups = (n_q + kQT * kQTiles - 1) / (kQT * kQTiles);
-  const int qg = blockIdx.x % q_groups;
-  const int h = (blockIdx.x / q_groups) % heads;
-  const int b = blockIdx.x / (q_groups * heads);
-  const int n_kv = (N + kKT - 1) / kKT;
-  // the last query group of a (batch, head) may reach into its second tile by no row at all: that tile's
-  // issuer and softmax warps then have nothing to do and the K/V stages are released by one issuer alone
-  const int n_tiles = (qg * kQTiles + 1) * kQT < n_q ? kQTiles : 1;
+  const int block = blockIdx.x;
+  const int sid = warp - kFirstSoftmaxWarp;
+  const int t_own = (sid >> 2) & 1;                    // a softmax warp's query tile
+  const int hh = sid >> 3;                             // ... which 48 of a tile's 96 score columns
+  const int quad = warp & 3;                           // ... the TMEM lane quadrant it may touch
+  const int row = quad * 32 + lane;                    // ... query row within the tile
+  static_assert(PRESCALED || MODE == kWhole, "parts of a group add up only where there is no maximum");
 
   if (threadIdx.x == 0) {
-    mbar_init(q_full, 1);
-    for (int i = 0; i < kKvStages; ++i) { mbar_init(&kv_full[i], 1); mbar_init(&kv_empty[i], n_tiles); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&q_full[i], 1); mbar_init(&q_empty[i], 2); }
+    for (int i = 0; i < kKvStages; ++i) { mbar_init(&kv_full[i], 1); mbar_init(&kv_empty[i], 2); }
     for (int i = 0; i < 4; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_full[i], 8); }
     for (int i = 0; i < kQTiles; ++i) mbar_init(&pv_full[i], 1);
     for (int i = 0; i < 8; ++i) mbar_init(&pair_bar[i], 2);
     *abort_flag = 0;
-    *cta_bad = 0;
+    *n_bad = 0;
     mbar_fence_init();
   }
   if (warp == 0 && lane == 0) { tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v); }
@@ -514,21 +676,45 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   stream_order();
+  // The row sum tells whether the fixed scaling was good enough (Inf and NaN are caught too; without a maximum the sum must
+  // not be vanishingly small either).  If not, the warp's rows are left to the safe path below; of the warps that come to
+  // the same verdict on them, the first half's in the first block records them.
+  auto in_range = [&](float l_row, int qi, int group) -> bool {
+    const bool bad_row = qi < n_q && !(l_row < kRowSumLimit && (!PRESCALED || l_row > kRowSumFloor));
+    if (!__any_sync(0xFFFFFFFFu, bad_row)) return true;
+    if (lane == 0 && hh == 0 && (MODE != kCluster || block % plan.per_span == 0)) {
+      const int at = atomicAdd(n_bad, 1);
+      if (at < kMaxBad) bad[at] = group * 8 + t_own * 4 + quad;
+    }
+    return false;
+  };
+  bool finished = false;                               // kCluster: this warp's rows are complete in TMEM, their sum is
+  float l_cluster = 0.f;
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      mbar_expect_tx(q_full, n_tiles * kQBytes);
-      for (int t = 0; t < n_tiles; ++t)
-        tma_load_2d(s_q + t * kQBytes, &tm_q, q_full, h * kHD, b * n_q + (qg * kQTiles + t) * kQT);
-      int stage = 0; uint32_t phase = 0;
-      for (int j = 0; j < n_kv; ++j) {
-        if (!mbar_wait(&kv_empty[stage], phase ^ 1, abort_flag)) break;
-        uint8_t* sk = s_kv + (size_t)stage * kKvStageBytes;
-        mbar_expect_tx(&kv_full[stage], kKvStageBytes);
-        tma_load_3d(sk, &tm_k, &kv_full[stage], h * kHD, j * kKT, b);
-        tma_load_3d(sk + kKBytes, &tm_v, &kv_full[stage], h * kHD, j * kKT, b);
-        if (++stage == kKvStages) { stage = 0; phase ^= 1; }
+      RunIter<MODE> it(plan, block);
+      Run run;
+      int stage = 0, qb = 0; uint32_t phase = 0, q_phase = 0;
+      bool ok = true;
+      while (ok && it.next(run)) {
+        const int qg = run.group % q_groups, bh = run.group / q_groups, h = bh % heads, b = bh / heads;
+        const int n_tiles = live_tiles(qg, n_q);
+        if (!(ok = mbar_wait(&q_empty[qb], q_phase ^ 1, abort_flag))) break;
+        mbar_expect_tx(&q_full[qb], n_tiles * kQBytes);
+        for (int t = 0; t < n_tiles; ++t)
+          tma_load_2d(s_q + (qb * kQTiles + t) * kQBytes, &tm_q, &q_full[qb], h * kHD, b * n_q + (qg * kQTiles + t) * kQT);
+        for (int j = run.first; j < run.first + run.n; ++j) {
+          if (!(ok = mbar_wait(&kv_empty[stage], phase ^ 1, abort_flag))) break;
+          uint8_t* sk = s_kv + (size_t)stage * kKvStageBytes;
+          mbar_expect_tx(&kv_full[stage], kKvStageBytes);
+          tma_load_3d(sk, &tm_k, &kv_full[stage], h * kHD, j * kKT, b);
+          tma_load_3d(sk + kKBytes, &tm_v, &kv_full[stage], h * kHD, j * kKT, b);
+          if (++stage == kKvStages) { stage = 0; phase ^= 1; }
+        }
+        qb ^= 1;
+        if (qb == 0) q_phase ^= 1;
       }
       for (int i = 0; i < kKvStages; ++i) {      // all armed stages consumed before the CTA retires
         if (!mbar_wait(&kv_empty[stage], phase ^ 1, abort_flag)) break;
@@ -537,59 +723,84 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     }
   } else if (warp == 1 || warp == 2) {
     // ------------------------------------------------------------ MMA issuer warp of query tile t
-    if (warp - 1 < n_tiles) {
-      const bool leader = elect_one();
-      const int t = warp - 1;
-      constexpr uint32_t idesc_s = idesc_bf16(kQT, kKT, 0);    // S = Q K^T : both operands K-contiguous
-      constexpr uint32_t idesc_pv = idesc_bf16(kQT, kHD, 1);   // O += P V  : V is N(head_dim)-contiguous
-      const uint64_t dq = smem_desc_sw128(smem_u32(s_q + t * kQBytes), 1024);
-      const uint32_t t_tile = tmem_base + (uint32_t)t * kTileCols;
-      auto issue_s = [&](int j) {
-        const int st = j % kKvStages;
-        const uint64_t dk = smem_desc_sw128(smem_u32(s_kv + (size_t)st * kKvStageBytes), 1024);
-        const uint32_t d = t_tile + (uint32_t)(j & 1) * kKT;
+    // Scores run two key tiles ahead of P V, across the border between two runs as well (the next run's queries are
+    // there by then).  The K/V ring counts every tile of the block; the score buffers count this query tile's.
+    const bool leader = elect_one();
+    const int t = warp - 1;
+    constexpr uint32_t idesc_s = idesc_bf16(kQT, kKT, 0);    // S = Q K^T : both operands K-contiguous
+    constexpr uint32_t idesc_pv = idesc_bf16(kQT, kHD, 1);   // O += P V  : V is N(head_dim)-contiguous
+    const uint32_t t_tile = tmem_base + (uint32_t)t * kTileCols;
+    RunIter<MODE> ahead(plan, block), it(plan, block);
+    Run run;
+    int a_left = 0, a_qb = 1, a_stage = 0, s_cnt = 0;
+    uint32_t a_phase = 0, aq_phase = 1;
+    bool a_live = false;
+    // The next score tile, if there is one.  (A run whose second query tile has no row: that tile's issuer follows the
+    // ring without issuing anything.)
+    auto issue_s = [&]() -> bool {
+      if (a_left == 0) {
+        Run next;
+        if (!ahead.next(next)) return true;
+        a_left = next.n;
+        a_live = t < live_tiles(next.group % q_groups, n_q);
+        a_qb ^= 1;
+        if (a_qb == 0) aq_phase ^= 1;
+        if (!mbar_wait_warp(&q_full[a_qb], aq_phase, abort_flag)) return false;
+      }
+      if (!mbar_wait_warp(&kv_full[a_stage], a_phase, abort_flag)) return false;
+      tc_fence_after();
+      --a_left;
+      if (a_live) {
+        const uint64_t dq = smem_desc_sw128(smem_u32(s_q + (a_qb * kQTiles + t) * kQBytes), 1024);
+        const uint64_t dk = smem_desc_sw128(smem_u32(s_kv + (size_t)a_stage * kKvStageBytes), 1024);
+        const uint32_t d = t_tile + (uint32_t)(s_cnt & 1) * kKT;
         if (leader) {
 #pragma unroll
           for (int k = 0; k < kHD / 16; ++k) mma_ss(d, dq + 2 * k, dk + 2 * k, idesc_s, k != 0);
-          mma_commit(&s_full[t * 2 + (j & 1)]);
+          mma_commit(&s_full[t * 2 + (s_cnt & 1)]);
+          if (a_left == 0) mma_commit(&q_empty[a_qb]);       // these queries are done with
         }
-      };
-      bool ok = mbar_wait_warp(q_full, 0, abort_flag);
-      for (int j = 0; j < 2 && j < n_kv && ok; ++j) {           // two score tiles ahead of the softmax
-        if ((ok = mbar_wait_warp(&kv_full[j], 0, abort_flag))) { tc_fence_after(); issue_s(j); }
+        ++s_cnt;
+      } else if (leader && a_left == 0) {
+        mbar_arrive(&q_empty[a_qb]);
       }
-      for (int j = 0; j < n_kv && ok; ++j) {
-        const int st = j % kKvStages;
-        // V tile: rows = keys (128 bytes each), 8-key groups 1024 bytes apart; 16 keys per MMA = 2048 bytes
-        const uint64_t dv = smem_desc_sw128(smem_u32(s_kv + (size_t)st * kKvStageBytes + kKBytes), 1024);
-        if (!(ok = mbar_wait_warp(&p_full[t * 2 + (j & 1)], (j >> 1) & 1, abort_flag))) break;
-        tc_fence_after();
-        const uint32_t buf = t_tile + (uint32_t)(j & 1) * kKT;
-        if (leader) {
-          // P of keys [16k, 16k+16) sits in 8 columns: the first 48 keys in columns [0, 24) of the buffer,
-          // the last 48 in columns [48, 72) (each half of the softmax writes inside its own score columns)
-#pragma unroll
-          for (int k = 0; k < kKT / 16; ++k)
-            mma_ts(t_tile + kColO, buf + (k / 3) * kHalf + (k % 3) * 8, dv + 128 * k, idesc_pv, (j | k) != 0);
-          if (j == n_kv - 1) mma_commit(&pv_full[t]);
-          mma_commit(&kv_empty[st]);             // second arrival comes from the other tile's issuer
-        }
-        if (j + 2 < n_kv) {
-          // S of tile j+2 overwrites the buffer whose P the product above reads: safe because the
-          // tensor core executes this thread's MMAs in issue order
-          if (!(ok = mbar_wait_warp(&kv_full[(j + 2) % kKvStages], ((j + 2) / kKvStages) & 1, abort_flag))) break;
+      if (++a_stage == kKvStages) { a_stage = 0; a_phase ^= 1; }
+      return true;
+    };
+    bool ok = issue_s() && issue_s();              // two score tiles ahead of the softmax
+    int stage = 0, cnt = 0;
+    while (ok && it.next(run)) {
+      const bool live = t < live_tiles(run.group % q_groups, n_q);
+      for (int j = 0; j < run.n; ++j) {
+        if (live) {
+          // V tile: rows = keys (128 bytes each), 8-key groups 1024 bytes apart; 16 keys per MMA = 2048 bytes
+          const uint64_t dv = smem_desc_sw128(smem_u32(s_kv + (size_t)stage * kKvStageBytes + kKBytes), 1024);
+          if (!(ok = mbar_wait_warp(&p_full[t * 2 + (cnt & 1)], (cnt >> 1) & 1, abort_flag))) break;
           tc_fence_after();
-          issue_s(j + 2);
+          const uint32_t buf = t_tile + (uint32_t)(cnt & 1) * kKT;
+          if (leader) {
+            // P of keys [16k, 16k+16) sits in 8 columns: the first 48 keys in columns [0, 24) of the buffer,
+            // the last 48 in columns [48, 72) (each half of the softmax writes inside its own score columns).
+            // (The first product of a run overwrites the accumulator: its P came after the run before was read out.)
+#pragma unroll
+            for (int k = 0; k < kKT / 16; ++k)
+              mma_ts(t_tile + kColO, buf + (k / 3) * kHalf + (k % 3) * 8, dv + 128 * k, idesc_pv, (j | k) != 0);
+            if (j == run.n - 1) mma_commit(&pv_full[t]);
+            mma_commit(&kv_empty[stage]);          // second arrival comes from the other tile's issuer
+          }
+          ++cnt;
+        } else if (leader) {
+          mbar_arrive(&kv_empty[stage]);
         }
+        if (++stage == kKvStages) stage = 0;
+        // the scores two tiles on overwrite the buffer whose P the product above reads: safe because the
+        // tensor core executes this thread's MMAs in issue order
+        if (!(ok = issue_s())) break;
       }
     }
-  } else if (warp >= kFirstSoftmaxWarp && (((warp - kFirstSoftmaxWarp) >> 2) & 1) < n_tiles) {
+  } else if (warp >= kFirstSoftmaxWarp) {
     // ------------------------------------------------------------ softmax
-    const int sid = warp - kFirstSoftmaxWarp;
-    const int t = (sid >> 2) & 1;                      // query tile
-    const int hh = sid >> 3;                           // which 48 of a tile's 96 score columns
-    const int quad = warp & 3;                         // TMEM lane quadrant this warp may touch
-    const int row = quad * 32 + lane;                  // query row within the tile
+    const int t = t_own;
     const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)t * kTileCols;
     uint64_t* my_pair = &pair_bar[t * 4 + quad];
     const float c = PRESCALED ? 1.0f : kScoreScaleLog2;
@@ -597,110 +808,284 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     float2 nm2 = make_float2(0.f, 0.f);
     const float cs = c / kPolySpan;
     float bs = 0.5f;
-    float l_half = 0.f;
-    uint32_t pair_phase = 0;
+    uint32_t pair_phase = 0, pv_phase = 0;
+    int cnt = 0;                                       // key tiles of this query tile so far
     bool ok = true;
-    for (int j = 0; j < n_kv; ++j) {
-      ok = mbar_wait_warp(&s_full[t * 2 + (j & 1)], (j >> 1) & 1, abort_flag);
-      if (!ok) break;
-      tc_fence_after();
-      const uint32_t t_s = lane_base + (uint32_t)(j & 1) * kKT + (uint32_t)hh * kHalf;
-      int valid = N - j * kKT - hh * kHalf;            // columns of this half that are keys
-      valid = valid < 0 ? 0 : (valid > kHalf ? kHalf : valid);
-      if (!PRESCALED && j == 0) {
-        // First tile: the maximum over its (existing) keys becomes the row's scaling maximum for good.
-        // Both halves read their columns, trade their maxima through shared memory, and then form P
-        // from the scores they still hold in registers.
-        uint32_t s[kHalf];
+    RunIter<MODE> it(plan, block);
+    Run run;
+    while (ok && it.next(run)) {
+      const int qg = run.group % q_groups;
+      if (t >= live_tiles(qg, n_q)) continue;
+      float l_half = 0.f;
+      const int n_left = N - run.first * kKT - hh * kHalf;
+      for (int j = 0; j < run.n; ++j, ++cnt) {
+        ok = mbar_wait_warp(&s_full[t * 2 + (cnt & 1)], (cnt >> 1) & 1, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t t_s = lane_base + (uint32_t)(cnt & 1) * kKT + (uint32_t)hh * kHalf;
+        int valid = n_left - j * kKT;                  // columns of this half that are keys
+        valid = valid < 0 ? 0 : (valid > kHalf ? kHalf : valid);
+        if (!PRESCALED && j == 0) {
+          // First tile: the maximum over its (existing) keys becomes the row's scaling maximum for good.
+          // Both halves read their columns, trade their maxima through shared memory, and then form P
+          // from the scores they still hold in registers.
+          uint32_t s[kHalf];
 #pragma unroll
-        for (int ch = 0; ch < kHalf / 16; ++ch) tmem_ld16(t_s + ch * 16, *reinterpret_cast<uint32_t(*)[16]>(&s[ch * 16]));
-        tmem_ld_wait();
-        float m = -INFINITY;
+          for (int ch = 0; ch < kHalf / 16; ++ch) tmem_ld16(t_s + ch * 16, *reinterpret_cast<uint32_t(*)[16]>(&s[ch * 16]));
+          tmem_ld_wait();
+          float m = -INFINITY;
 #pragma unroll
-        for (int i = 0; i < kHalf; ++i)
-          if (i < valid) m = fmaxf(m, __uint_as_float(s[i]));
-        xchg_m[(t * kQT + row) * 2 + hh] = m;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(my_pair);
-        if (!(ok = mbar_wait_warp(my_pair, pair_phase, abort_flag))) break;
-        pair_phase ^= 1;
-        m = fmaxf(xchg_m[(t * kQT + row) * 2], xchg_m[(t * kQT + row) * 2 + 1]);   // finite: column 0 always exists
-        nm2 = make_float2(-m * c, -m * c);
-        bs = fmaf(-m, cs, 0.5f);
-        float2 acc = make_float2(0.f, 0.f);
+          for (int i = 0; i < kHalf; ++i)
+            if (i < valid) m = fmaxf(m, __uint_as_float(s[i]));
+          xchg[(t * kQT + row) * 2 + hh] = m;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(my_pair);
+          if (!(ok = mbar_wait_warp(my_pair, pair_phase, abort_flag))) break;
+          pair_phase ^= 1;
+          m = fmaxf(xchg[(t * kQT + row) * 2], xchg[(t * kQT + row) * 2 + 1]);   // finite: column 0 always exists
+          nm2 = make_float2(-m * c, -m * c);
+          bs = fmaf(-m, cs, 0.5f);
+          float2 acc = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int ch = 0; ch < kHalf / 16; ++ch) {
-          uint32_t pk[8];
+          for (int ch = 0; ch < kHalf / 16; ++ch) {
+            uint32_t pk[8];
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int col = ch * 16 + 2 * i;
-            const float2 x = __ffma2_rn(f2(s[col], s[col + 1]), c2, nm2);
-            float2 p = make_float2(ex2(x.x), ex2(x.y));
-            if (col >= valid) p.x = 0.f;
-            if (col + 1 >= valid) p.y = 0.f;
-            acc = __fadd2_rn(acc, p);
-            const __nv_bfloat162 bb = __floats2bfloat162_rn(p.x, p.y);
-            pk[i] = *reinterpret_cast<const uint32_t*>(&bb);
+            for (int i = 0; i < 8; ++i) {
+              const int col = ch * 16 + 2 * i;
+              const float2 x = __ffma2_rn(f2(s[col], s[col + 1]), c2, nm2);
+              float2 p = make_float2(ex2(x.x), ex2(x.y));
+              if (col >= valid) p.x = 0.f;
+              if (col + 1 >= valid) p.y = 0.f;
+              acc = __fadd2_rn(acc, p);
+              const __nv_bfloat162 bb = __floats2bfloat162_rn(p.x, p.y);
+              pk[i] = *reinterpret_cast<const uint32_t*>(&bb);
+            }
+            tmem_st8(t_s + ch * 8, pk);
           }
-          tmem_st8(t_s + ch * 8, pk);
+          l_half = acc.x + acc.y;
+        } else if (valid == kHalf) {
+          l_half += half_tile<false, PRESCALED>(t_s, valid, c2, nm2, cs, bs);
+        } else {
+          l_half += half_tile<true, PRESCALED>(t_s, valid, c2, nm2, cs, bs);
         }
-        l_half = acc.x + acc.y;
-      } else if (valid == kHalf) {
-        l_half += half_tile<false, PRESCALED>(t_s, valid, c2, nm2, cs, bs);
-      } else {
-        l_half += half_tile<true, PRESCALED>(t_s, valid, c2, nm2, cs, bs);
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&p_full[t * 2 + (cnt & 1)]);
       }
-      tmem_st_wait();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&p_full[t * 2 + (j & 1)]);
-    }
-    // The row sum is the sum of the halves'; it also tells whether the fixed maximum was good enough.
-    if (ok) {
-      xchg_l[(t * kQT + row) * 2 + hh] = l_half;
+      if (!ok) break;
+      // The row sum is the sum of the halves'.  (Two exchange buffers in turn: a warp may be a run ahead of its partner
+      // but not two.  Without a maximum to trade, PRESCALED has both; otherwise the exchange of the maxima lies between.)
+      float* const xl = xchg + (PRESCALED ? (int)(pair_phase & 1) : 1) * kXchgFloats;
+      xl[(t * kQT + row) * 2 + hh] = l_half;
       __syncwarp();
       if (lane == 0) mbar_arrive(my_pair);
-      ok = mbar_wait_warp(my_pair, pair_phase, abort_flag);
-    }
-    if (ok) {
-      const float l_row = xchg_l[(t * kQT + row) * 2] + xchg_l[(t * kQT + row) * 2 + 1];
+      if (!(ok = mbar_wait_warp(my_pair, pair_phase, abort_flag))) break;
+      pair_phase ^= 1;
+      float l_row = xl[(t * kQT + row) * 2] + xl[(t * kQT + row) * 2 + 1];
+      if (!(ok = mbar_wait_warp(&pv_full[t], pv_phase, abort_flag))) break;
+      pv_phase ^= 1;
+      tc_fence_after();
+
+      if (MODE == kCluster) {
+        finished = true;
+        l_cluster = l_row;
+        break;
+      }
+
+      // Each half finishes 32 of the row's 64 output features.
+      const uint32_t t_out = lane_base + kColO + hh * 32;
       const int qi = (qg * kQTiles + t) * kQT + row;
-      // (also catches Inf and NaN; without a maximum the sum must not be vanishingly small either)
-      const bool bad = qi < n_q && !(l_row < kRowSumLimit && (!PRESCALED || l_row > kRowSumFloor));
-      if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(cta_bad, 1);
-      ok = mbar_wait_warp(&pv_full[t], 0, abort_flag);
-      if (ok) {
-        tc_fence_after();
-        const float inv = 1.0f / l_row;
-        // each half writes 32 of the row's 64 output features
-        __nv_bfloat16* dst = O + ((long long)b * n_q + qi) * ((long long)heads * kHD) + h * kHD + hh * 32;
+      const int bh = run.group / q_groups, h = bh % heads, b = bh / heads;
+      __nv_bfloat16* const dst = O + ((long long)b * n_q + qi) * ((long long)heads * kHD) + h * kHD + hh * 32;
+      if (MODE == kWhole || run.n == plan.tiles) {
+        if (in_range(l_row, qi, run.group)) {
+          const float inv = 1.0f / l_row;
 #pragma unroll
+          for (int ch = 0; ch < 2; ++ch) {
+            uint32_t r[16];
+            tmem_ld16(t_out + ch * 16, r);             // warp-collective: every lane loads
+            tmem_ld_wait();
+            if (qi < n_q) emit16(r, inv, dst + ch * 16);
+          }
+        }
+        continue;
+      }
+      // A part of the keys only.  The first of a group's parts may be the second run of its block, the others are the
+      // first runs of theirs.
+      const int u0 = (run.group - plan.groups + plan.tail) * plan.tiles;
+      const int c_first = plan.share_of(u0), c_last = plan.share_of(u0 + plan.tiles - 1);
+      const int first_slot = 2 * c_first + (plan.share_start(c_first) >= u0 ? 0 : 1);
+      {
+        float* const part = parts + (size_t)(block == c_first ? first_slot : 2 * block) * kSlotFloats + sid * kPartFloats;
+#pragma unroll 1
         for (int ch = 0; ch < 2; ++ch) {
           uint32_t r[16];
-          tmem_ld16(lane_base + kColO + hh * 32 + ch * 16, r);     // warp-collective: every lane loads
+          tmem_ld16(t_out + ch * 16, r);
           tmem_ld_wait();
-          if (qi < n_q) {
-            uint32_t w[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              const __nv_bfloat162 pk = __floats2bfloat162_rn(__uint_as_float(r[2 * q]) * inv,
-                                                              __uint_as_float(r[2 * q + 1]) * inv);
-              w[q] = *reinterpret_cast<const uint32_t*>(&pk);
+          for (int q = 0; q < 4; ++q)
+            __stcg(reinterpret_cast<float4*>(part) + (ch * 4 + q) * 32 + lane,
+                   make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]), __uint_as_float(r[4 * q + 2]),
+                               __uint_as_float(r[4 * q + 3])));
+        }
+        __stcg(part + 8 * 32 * 4 + lane, l_row);
+      }
+      __threadfence();
+      __syncwarp();
+      int before = 0;
+      if (lane == 0) before = atomicAdd(part_count + c_first * kFastSoftmaxWarps + sid, 1);
+      before = __shfl_sync(0xFFFFFFFFu, before, 0);
+      if (before < c_last - c_first) continue;         // the others are not all there yet
+      __threadfence();
+      if (lane == 0) part_count[c_first * kFastSoftmaxWarps + sid] = 0;          // for the next launch
+      l_row = 0.f;
+      for (int k = c_first; k <= c_last; ++k)
+        l_row += __ldcg(parts + (size_t)(k == c_first ? first_slot : 2 * k) * kSlotFloats + sid * kPartFloats + 8 * 32 * 4 + lane);
+      if (!in_range(l_row, qi, run.group)) continue;
+#pragma unroll 1
+      for (int ch = 0; ch < 2; ++ch) {
+        float4 sum[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sum[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+        for (int k = c_first; k <= c_last; ++k) {
+          const float4* part = reinterpret_cast<const float4*>(
+              parts + (size_t)(k == c_first ? first_slot : 2 * k) * kSlotFloats + sid * kPartFloats);
+          float4 v[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) v[q] = __ldcg(part + (ch * 4 + q) * 32 + lane);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) { sum[q].x += v[q].x; sum[q].y += v[q].y; sum[q].z += v[q].z; sum[q].w += v[q].w; }
+        }
+        uint32_t r[16];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          r[4 * q] = __float_as_uint(sum[q].x); r[4 * q + 1] = __float_as_uint(sum[q].y);
+          r[4 * q + 2] = __float_as_uint(sum[q].z); r[4 * q + 3] = __float_as_uint(sum[q].w);
+        }
+        if (qi < n_q) emit16(r, 1.0f / l_row, dst + ch * 16);
+      }
+    }
+  }
+
+  if (MODE == kCluster) {
+    // ---------------------------------------------------------------- the cluster's parts
+    // Piece p (16 columns) of the accumulators is finished by rank p % split; it receives the others' sums in its (idle)
+    // key and value ring: [piece / split][sender][four columns][row of 256] words of 16 bytes, behind them the row sums.
+    const int split = plan.per_span;
+    const int rank = block % split, group = block / split;
+    constexpr int kRows = kQTiles * kQT;
+    float4* const pieces = reinterpret_cast<float4*>(s_kv);
+    float* const sums = reinterpret_cast<float*>(pieces + 2 * 3 * 4 * kRows);    // (two pieces from three senders at most)
+    auto piece_at = [&](int p, int sender, int q) {
+      return pieces + (((p / split) * split + sender) * 4 + q) * kRows + t_own * kQT + row;
+    };
+    const uint32_t t_out = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)t_own * kTileCols + kColO;
+    __syncwarp();
+    cluster_sync();                                    // every block's ring is idle
+    if (finished) {
+      for (int to = 0; to < split; ++to) {
+        if (to == rank) continue;
+        if (hh == 0) st_cluster_f32(cluster_map(smem_u32(sums + rank * kRows + t_own * kQT + row), (uint32_t)to), l_cluster);
+#pragma unroll 1
+        for (int p = to; p < 4; p += split) {
+          if ((p >> 1) != hh) continue;                // each half sends the columns of its own
+          uint32_t r[16];
+          tmem_ld16(t_out + p * 16, r);
+          tmem_ld_wait();
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            st_cluster_v4(cluster_map(smem_u32(piece_at(p, rank, q)), (uint32_t)to), __uint_as_float(r[4 * q]),
+                          __uint_as_float(r[4 * q + 1]), __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
+        }
+      }
+    }
+    __syncwarp();
+    cluster_sync();
+    if (finished) {
+      const int qg = group % q_groups, bh = group / q_groups, h = bh % heads, b = bh / heads;
+      const int qi = (qg * kQTiles + t_own) * kQT + row;
+      __nv_bfloat16* const dst = O + ((long long)b * n_q + qi) * ((long long)heads * kHD) + h * kHD;
+      float l_row = 0.f;
+      for (int k = 0; k < split; ++k) l_row += k == rank ? l_cluster : sums[k * kRows + t_own * kQT + row];
+      if (in_range(l_row, qi, group)) {                // (all ranks come to the same verdict; the first records it)
+        const float inv = 1.0f / l_row;
+#pragma unroll 1
+        for (int p = rank; p < 4; p += split) {
+          if ((split == 4 ? 0 : p >> 1) != hh) continue;
+          uint32_t r[16];
+          tmem_ld16(t_out + p * 16, r);
+          tmem_ld_wait();
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int k = 0; k < split; ++k) {
+              const float4 o = k == rank ? make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
+                                                       __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]))
+                                         : *piece_at(p, k, q);
+              v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
             }
-            *reinterpret_cast<uint4*>(dst + ch * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-            *reinterpret_cast<uint4*>(dst + ch * 16 + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+            r[4 * q] = __float_as_uint(v.x); r[4 * q + 1] = __float_as_uint(v.y);
+            r[4 * q + 2] = __float_as_uint(v.z); r[4 * q + 3] = __float_as_uint(v.w);
           }
+          if (qi < n_q) emit16(r, inv, dst + p * 16);
         }
       }
     }
   }
 
-  // ---------------------------------------------------------------- teardown
+  // ---------------------------------------------------------------- rows out of range: once more, on the safe path
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    if (*abort_flag) atomicAdd(status, 1);
-    cta_words[blockIdx.x] = *abort_flag ? 2 : (*cta_bad ? 1 : 0);
+  const int n_marked = *n_bad;
+  if (n_marked > 0 && !*abort_flag) {                  // block-uniform
+    // One group at a time: the listed ones, or, where the list was too short, every group this block had a run of.
+    const bool listed = n_marked <= kMaxBad;
+    RunIter<MODE> it(plan, block);
+    Run run;
+    bool used = false;
+    for (int i = 0; listed ? i < n_marked : it.next(run); ++i) {
+      uint32_t mask = ~0u;
+      int group;
+      if (listed) {
+        group = bad[i] >> 3;
+        mask = 0;
+        bool seen = false;
+        for (int k = 0; k < n_marked; ++k)
+          if (bad[k] >> 3 == group) { mask |= 1u << (bad[k] & 7); seen |= k < i; }
+        if (seen) continue;
+      } else {
+        group = run.group;
+      }
+      const int qg = group % q_groups, bh = group / q_groups;
+      if (threadIdx.x == 0) {
+        if (used)
+          for (int k = 0; k < kSafeBars; ++k) mbar_inval(&safe_bars[k]);
+        safe_init_barriers(safe_bars, live_tiles(qg, n_q));
+        mbar_fence_init();
+      }
+      used = true;
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // (kCluster has used the ring through plain stores)
+      __syncthreads();
+      tc_fence_after();
+      const SafeWork w = {&tm_q, &tm_k, &tm_v, O,    n_q, N,    heads,     qg,         bh % heads, bh / heads,
+                          PRESCALED ? 1.0f : kScoreScaleLog2, mask, s_q, s_kv, safe_bars, abort_flag, tmem_base};
+      safe_recompute(w);
+      tc_fence_before();
+      __syncthreads();
+      if (*abort_flag) break;
+    }
+  }
+
+  // ---------------------------------------------------------------- teardown
+  if (threadIdx.x == 0 && *abort_flag) {
+    atomicAdd(status, 1);
+    if (cta_words != nullptr) {
+      RunIter<MODE> it(plan, block);
+      Run run;
+      while (it.next(run)) cta_words[run.group] = 2;
+    }
   }
   if (warp == 1) { __syncwarp(); tc_fence_after(); tmem_dealloc(tmem_base, kAttTmemCols); }
 }
@@ -727,15 +1112,30 @@ static int make_attention_maps(const void* q, const void* k, const void* v, int 
   return HERO_OK;
 }
 
+constexpr int kMaxSplit = 4;
+static int g_resident_clusters[kMaxDevices][kMaxSplit + 1];      // clusters of this many blocks that a device holds at once
+
 static int attention_kernel_attributes() {
   static PerDeviceOnce attr_once;            // the opt-in is a property of the kernel ON a device
-  return per_device_once(attr_once, [](int) {
+  return per_device_once(attr_once, [](int dev) {
     HERO_CUDA_TRY(cudaFuncSetAttribute(tc_attention_safe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kAttSmem));
-    HERO_CUDA_TRY(cudaFuncSetAttribute(tc_attention_fast_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kFastSmem));
-    HERO_CUDA_TRY(cudaFuncSetAttribute(tc_attention_fast_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kFastSmem));
+    for (auto kernel : {tc_attention_fast_kernel<false, kWhole>, tc_attention_fast_kernel<true, kWhole>,
+                        tc_attention_fast_kernel<true, kCluster>, tc_attention_fast_kernel<true, kCut>})
+      HERO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFastSmem));
+    for (int split = 2; split <= kMaxSplit; ++split) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)(split * 64));
+      cfg.blockDim = dim3(kFastThreads);
+      cfg.dynamicSmemBytes = kFastSmem;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = (unsigned)split; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      HERO_CUDA_TRY(cudaOccupancyMaxActiveClusters(&g_resident_clusters[dev][split],
+                                                   tc_attention_fast_kernel<true, kCluster>, &cfg));
+    }
     return HERO_OK;
   });
 }
@@ -745,40 +1145,79 @@ long long tc_attention_grid(int B, int n_q, int heads) {
   return q_groups * heads * B;
 }
 
-// d_status[0] counts CTAs that gave up; d_status[1 .. 1 + status_ctas) are the per-CTA words.  When the grid
-// fits in them the fast kernel runs, followed by the safe kernel on the CTAs the fast one marked; otherwise the
-// safe kernel does everything.  q_prescaled: the caller has multiplied Q by log2(e) / sqrt(head_dim) already, so
-// a score IS the exponent of its weight; the fast kernel then takes 2^s as it stands, with no maximum at all
-// (exact while a row's largest score stays within about +-100, the row sum telling when it did not).
+// Which mode, and how the groups are dealt out.  Measured (us; queries x keys x heads x batch):
+//   * a cluster wherever all clusters are on the chip at once (what does not fit waits for a whole cluster's worth of free
+//     SMs): 371 x 1562 x 12, 24 groups, whole 18.9, over four 12.8; 620 x 1319 x 8 x 2, 48 groups, whole 15.8, over two 15.4,
+//     over three (which do not all fit) 24.1.  Under six key tiles there is nothing to win.
+//   * cutting the last round pays from about 64 key tiles on (a part costs some 5 us of fences, counting and adding up):
+//     1755 x 17776 x 48 x 2, 672 groups, 860 -> 851, 4388 x 17776 x 48 x 2, 1728 groups, 2087 -> 2069, the whole 3072-wide
+//     cached step 59.6 -> 58.7 ms; but 2970 x 3196 x 48 x 2 (34 tiles) 295 -> 299 and 2627 x 2627 x 18 x 2 84 -> 90.
+struct PlannedAttention { AttentionMode mode; AttentionPlan plan; };
+static PlannedAttention attention_plan(long long groups, int N, bool may_cluster, bool may_cut) {
+  const long long tiles = (N + kKT - 1) / kKT, sms = num_sms(), tail = groups % sms;
+  AttentionPlan plan = {(int)groups, (int)groups, 1, (int)tiles, 0, 1, 1, 1, 0};
+  auto spans = [&](long long n_spans, long long span, long long shares) {
+    plan.span = (int)span; plan.per_span = (int)shares;
+    plan.share_base = (int)(span / shares); plan.share_rest = (int)(span % shares);
+    plan.tail = (int)(n_spans * span / tiles);
+  };
+  int dev = 0;
+  if (may_cluster && tiles >= 6 && cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices)
+    for (int split = kMaxSplit; split >= 2; --split)
+      if (groups <= g_resident_clusters[dev][split]) {
+        spans(groups, tiles, split);
+        plan.blocks = (int)(groups * split);
+        return {kCluster, plan};
+      }
+  if (may_cut && groups > sms && tail > 0 && tiles >= 64 && tail * tiles <= 0x3FFFFFFF) {
+    plan.blocks = (int)sms;
+    plan.rounds = (int)(groups / sms);
+    spans(1, tail * tiles, sms);
+    return {kCut, plan};
+  }
+  return {kWhole, plan};
+}
+
+size_t tc_attention_part_bytes() { return (size_t)2 * num_sms() * kSlotFloats * sizeof(float); }
+size_t tc_attention_part_counters() { return (size_t)num_sms() * kFastSoftmaxWarps; }
+
+// d_status[0] counts thread blocks that gave up on a wait; cta_words may be null.  q_prescaled: the caller has multiplied Q
+// by log2(e) / sqrt(head_dim) already, so a score IS the exponent of its weight; the kernel then takes 2^s as it stands,
+// with no maximum at all (exact while a row's largest score stays within about +-100, the row sum telling when it did not).
+// parts, part_count (tc_attention_part_bytes, tc_attention_part_counters zeroed ints; both null: groups stay whole) are the
+// caller's for one launch at a time.
 int launch_tc_attention(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N, int heads,
-                        bool q_prescaled, int* d_status, int status_ctas, cudaStream_t s) {
+                        bool q_prescaled, float* parts, int* part_count, int* d_status, int* cta_words, cudaStream_t s) {
   if (B <= 0 || n_q <= 0) return HERO_OK;
   if (N <= 0 || heads <= 0) return HERO_ERR_ARG;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o)) return HERO_ERR_ALIGN;
   CUtensorMap tm_q, tm_k, tm_v;
   HERO_TRY(make_attention_maps(q, k, v, B, n_q, N, heads, &tm_q, &tm_k, &tm_v));
   HERO_TRY(attention_kernel_attributes());
-  const long long grid = tc_attention_grid(B, n_q, heads);
-  if (grid > 0x7FFFFFFFll) return HERO_ERR_ARG;
-  int* cta_words = grid <= status_ctas ? d_status + 1 : nullptr;
-  if (cta_words) {
-    if (q_prescaled)
-      HERO_TRY(launch_kernel(tc_attention_fast_kernel<true>, (unsigned)grid, kFastThreads, kFastSmem, s, 1, tm_q,
-                             tm_k, tm_v, (__nv_bfloat16*)o, n_q, N, heads, d_status, cta_words));
-    else
-      HERO_TRY(launch_kernel(tc_attention_fast_kernel<false>, (unsigned)grid, kFastThreads, kFastSmem, s, 1, tm_q,
-                             tm_k, tm_v, (__nv_bfloat16*)o, n_q, N, heads, d_status, cta_words));
-  }
-  HERO_TRY(launch_kernel(tc_attention_safe_kernel, (unsigned)grid, kAttThreads, kAttSmem, s, 1, tm_q, tm_k, tm_v,
-                         (__nv_bfloat16*)o, n_q, N, heads, q_prescaled ? 1.0f : kScoreScaleLog2, d_status,
-                         cta_words));
-  return HERO_OK;
+  const long long groups = tc_attention_grid(B, n_q, heads);
+  if (groups > 0x7FFFFFFFll / 8) return HERO_ERR_ARG;
+  const PlannedAttention p = attention_plan(groups, N, q_prescaled, q_prescaled && parts != nullptr);
+  return launch_kernel(!q_prescaled ? tc_attention_fast_kernel<false, kWhole>
+                       : p.mode == kWhole ? tc_attention_fast_kernel<true, kWhole>
+                       : p.mode == kCluster ? tc_attention_fast_kernel<true, kCluster> : tc_attention_fast_kernel<true, kCut>,
+                       (unsigned)p.plan.blocks, kFastThreads, kFastSmem, s,
+                       p.mode == kCluster ? (unsigned)p.plan.per_span : 1u, tm_q, tm_k, tm_v, (__nv_bfloat16*)o, n_q, N,
+                       heads, p.plan, parts, part_count, d_status, cta_words);
 }
 
-// Test hook: the safe kernel alone on every CTA (what runs when there are no per-CTA words).
+// The safe path alone, as a kernel of its own.
 int launch_tc_attention_safe(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N, int heads,
                              bool q_prescaled, int* d_status, cudaStream_t s) {
-  return launch_tc_attention(q, k, v, o, B, n_q, N, heads, q_prescaled, d_status, 0, s);
+  if (B <= 0 || n_q <= 0) return HERO_OK;
+  if (N <= 0 || heads <= 0) return HERO_ERR_ARG;
+  if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o)) return HERO_ERR_ALIGN;
+  CUtensorMap tm_q, tm_k, tm_v;
+  HERO_TRY(make_attention_maps(q, k, v, B, n_q, N, heads, &tm_q, &tm_k, &tm_v));
+  HERO_TRY(attention_kernel_attributes());
+  const long long groups = tc_attention_grid(B, n_q, heads);
+  if (groups > 0x7FFFFFFFll) return HERO_ERR_ARG;
+  return launch_kernel(tc_attention_safe_kernel, (unsigned)groups, kAttThreads, kAttSmem, s, 1, tm_q, tm_k, tm_v,
+                       (__nv_bfloat16*)o, n_q, N, heads, q_prescaled ? 1.0f : kScoreScaleLog2, d_status);
 }
 
 }  // namespace hero
@@ -795,7 +1234,7 @@ int launch_tc_attention_safe(const void* q, const void* k, const void* v, void* 
 // exits (kStaticScratchInts * 4 bytes = 64.25 KiB per GPU).
 //
 // Layout: word 0 counts the CTAs of the latest call that gave up on a bounded wait, word 1 + i
-// is CTA i's word (0 = done, 1 = left to the safe kernel, which then clears it, 2 = gave up).  The
+// is CTA i's word (0 = done, 2 = gave up).  The
 // array is shared by every call and keeps the previous call's contents, so each call clears the
 // words it is going to use on its stream before the kernels run; two calls that overlap on the
 // GPU (different streams, no dependency) race on it.
@@ -853,7 +1292,7 @@ extern "C" int hero_attention_bf16_static(const void* d_q, const void* d_k, cons
   HERO_TRY(static_setup(&scratch));
   // the array still holds the previous call's records: clear the words this grid will use
   HERO_CUDA_TRY(cudaMemsetAsync(scratch, 0, (size_t)(1 + grid) * sizeof(int), s));
-  HERO_TRY(launch_tc_attention(d_q, d_k, d_v, d_o, B, n_q, N, heads, false, scratch, kStaticMaxCtas, s));
+  HERO_TRY(launch_tc_attention(d_q, d_k, d_v, d_o, B, n_q, N, heads, false, nullptr, nullptr, scratch, scratch + 1, s));
   if (h_gave_up) {
     HERO_CUDA_TRY(cudaMemcpyAsync(h_gave_up, scratch, sizeof(int), cudaMemcpyDeviceToHost, s));
     HERO_CUDA_TRY(cudaStreamSynchronize(s));

@@ -91,3 +91,57 @@ def test_fp32_block_variants(over):
         hero.hero_step(s, x, to_dev(temb, "fp32"))
         assert rel_l2(to_host(x) - x_host, want - x_host) <= FP32_TOL, s
     hero.close()
+
+
+@pytest.mark.parametrize("B,frames,grid_h,grid_w,n_text,heads,ratio_den,key_offset", [
+    # one block per query group; one query row; one and two query tiles in the last group
+    (2, 1, 9, 11, 2, 1, 4, 0), (3, 1, 16, 24, 1, 2, 384, 0), (2, 5, 18, 31, 120, 16, 4, 0),
+    # clusters of two, three and four, runs of unequal length, one key in the last tile
+    (1, 1, 33, 45, 77, 12, 4, 0), (1, 10, 20, 25, 0, 1, 10, 100), (2, 1, 31, 43, 12, 9, 3, 0), (2, 1, 20, 25, 76, 12, 2, 100),
+    # groups cut over all blocks: one whole round and 27 groups, two whole rounds and four groups (37 parts each, one row in
+    # the last), with and without rows that the fixed scaling cannot hold (a constant added to all scores of a row)
+    (1, 8, 25, 31, 0, 7, 8, 0), (1, 8, 25, 31, 0, 7, 8, 100), (1, 8, 24, 32, 1, 12, 16, 100)])
+def test_attention_modes(B, frames, grid_h, grid_w, n_text, heads, ratio_den, key_offset):
+    """One block whose attention branch is the attention itself (identity projection, no modulation)."""
+    D, N = heads * 64, frames * grid_h * grid_w + n_text
+    cfg = dict(n_blocks=1, n_shallow=1, hidden=D, n_heads=heads, head_dim=64, ffn_dim=32, temb_dim=8, batch=B, frames=frames,
+               grid_h=grid_h, grid_w=grid_w, n_text=n_text, patch_h=2, patch_w=2, ratio_num=1, ratio_den=ratio_den,
+               quota_mode=0, warmup_full_steps=1, full_interval=0, dtype="bf16", has_gate=0, seed=5)
+    g = torch.Generator(device="cuda").manual_seed(N + heads)
+    mk = lambda *s, std=1.0: (torch.randn(*s, device="cuda", generator=g) * std).bfloat16()
+    zero = lambda *s: torch.zeros(*s, device="cuda", dtype=torch.bfloat16)
+    w = dict(w_mod=zero(4 * D, 8), b_mod=zero(4 * D), w_qkv=mk(3 * D, D, std=1.5 / D ** 0.5), b_qkv=mk(3 * D, std=0.1),
+             w_o=torch.eye(D, device="cuda", dtype=torch.bfloat16), b_o=zero(D), w_1=zero(32, D), b_1=zero(32),
+             w_2=zero(D, 32), b_2=zero(D))
+    u = torch.randn(heads, 64, device="cuda", generator=g)
+    w["b_qkv"][D:2 * D] += (key_offset * u / u.norm(dim=1, keepdim=True)).view(-1).bfloat16()
+    hero = H().Hero(cfg, [w])
+    temb, idx = mk(B, 8), torch.empty(N, dtype=torch.int32, device="cuda")
+    scale = 0.125 * 1.4426950408889634
+    for cached in (False, True, True):
+        x = mk(B, N, D)
+        rows = torch.arange(N, device="cuda")
+        xd = x.double()
+        if cached:
+            n = hero.hero_select_tokens(0, idx)
+            rows = idx[:n].long()
+            hero.hero_refresh_block(0, x, temb, idx, n)
+        else:
+            hero.hero_refresh_block(0, x, temb)
+        hero.hero_check_status()
+        k, v, got = (hero.hero_state_get(0, name).cuda().view(B, N, D) for name in ("k", "v", "g_attn"))
+        r = xd[:, rows]
+        a = ((r - r.mean(-1, keepdim=True)) / (r.var(-1, unbiased=False, keepdim=True) + 1e-5).sqrt()).bfloat16().double()
+        q = ((a @ w["w_qkv"][:D].double().T + w["b_qkv"][:D].double()) * scale).bfloat16()
+        want = torch.empty(B, len(rows), D, device="cuda", dtype=torch.double)
+        for b in range(B):
+            for h in range(heads):
+                c = slice(h * 64, h * 64 + 64)
+                p = torch.softmax(q[b, :, c].double() @ k[b, :, c].double().T * 0.6931471805599453, -1)
+                want[b, :, c] = p @ v[b, :, c].double()
+        err = (got[:, rows].double() - want).norm(dim=-1) / want.norm(dim=-1)
+        # per row: output rounding 2^-9, weights rounded to 2^-9 each, q 2^-9 (scores of a few units, so the weights move
+        # by a few times that); the sum of three bounds with a factor of two for the scores
+        assert float(err.max()) <= 2.0 ** -6, (cached, int(err.argmax()))
+        assert float((got[:, rows].double() - want).norm() / want.norm()) <= 2.0 ** -7
+    hero.close()
