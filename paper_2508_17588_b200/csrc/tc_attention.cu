@@ -50,6 +50,7 @@
 #include <cuda.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "hero_internal.h"
 #include "tc_common.cuh"
@@ -630,9 +631,13 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                          int* __restrict__ part_count, int* __restrict__ status, int* __restrict__ cta_words) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint8_t* s_q = smem;                             // [2] query groups: the next one is fetched while this one is worked on
-  uint8_t* s_kv = smem + 2 * kQTiles * kQBytes;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(s_kv + (size_t)kKvStages * kKvStageBytes);
+  // Two query groups (the next one is fetched while this one is worked on) and the ring; in kCluster, one query group, a
+  // shorter ring, and behind it the place for the other blocks' pieces.
+  constexpr int kStages = MODE == kCluster ? 4 : kKvStages;
+  constexpr int kQBufs = MODE == kCluster ? 1 : 2;
+  uint8_t* s_q = smem;
+  uint8_t* s_kv = smem + kQBufs * kQTiles * kQBytes;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 2 * kQTiles * kQBytes + (size_t)kKvStages * kKvStageBytes);
   uint64_t* q_full = bars;                         // [2]           TMA -> both issuers
   uint64_t* q_empty = q_full + 2;                  // [2], count 2  both issuers -> TMA
   uint64_t* kv_full = q_empty + 2;                 // [kKvStages]           TMA -> both issuers
@@ -661,7 +666,7 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) { mbar_init(&q_full[i], 1); mbar_init(&q_empty[i], 2); }
-    for (int i = 0; i < kKvStages; ++i) { mbar_init(&kv_full[i], 1); mbar_init(&kv_empty[i], 2); }
+    for (int i = 0; i < kStages; ++i) { mbar_init(&kv_full[i], 1); mbar_init(&kv_empty[i], 2); }
     for (int i = 0; i < 4; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_full[i], 8); }
     for (int i = 0; i < kQTiles; ++i) mbar_init(&pv_full[i], 1);
     for (int i = 0; i < 8; ++i) mbar_init(&pair_bar[i], 2);
@@ -675,7 +680,7 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  stream_order();
+  if (MODE == kCluster) cluster_arrive();              // waited for before anything is sent to another block
   // The row sum tells whether the fixed scaling was good enough (Inf and NaN are caught too; without a maximum the sum must
   // not be vanishingly small either).  If not, the warp's rows are left to the safe path below; of the warps that come to
   // the same verdict on them, the first half's in the first block records them.
@@ -688,6 +693,15 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     }
     return false;
   };
+  // First output feature of a row's half (a block of one run knows it from the start).
+  auto row_of = [&](int group) { return (group % q_groups * kQTiles + t_own) * kQT + row; };
+  auto output_of = [&](int group, int qi) {
+    const int bh = group / q_groups, h = bh % heads, b = bh / heads;
+    return O + ((long long)b * n_q + qi) * ((long long)heads * kHD) + h * kHD;
+  };
+  const int only_group = MODE == kCluster ? block / plan.per_span : block;
+  int qi = row_of(only_group);
+  __nv_bfloat16* dst = output_of(only_group, qi);
   bool finished = false;                               // kCluster: this warp's rows are complete in TMEM, their sum is
   float l_cluster = 0.f;
 
@@ -697,10 +711,12 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       RunIter<MODE> it(plan, block);
       Run run;
       int stage = 0, qb = 0; uint32_t phase = 0, q_phase = 0;
-      bool ok = true;
+      bool ok = true, first = true;
       while (ok && it.next(run)) {
         const int qg = run.group % q_groups, bh = run.group / q_groups, h = bh % heads, b = bh / heads;
         const int n_tiles = live_tiles(qg, n_q);
+        if (first) stream_order();                     // (where to begin is known by then)
+        first = false;
         if (!(ok = mbar_wait(&q_empty[qb], q_phase ^ 1, abort_flag))) break;
         mbar_expect_tx(&q_full[qb], n_tiles * kQBytes);
         for (int t = 0; t < n_tiles; ++t)
@@ -711,20 +727,23 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
           mbar_expect_tx(&kv_full[stage], kKvStageBytes);
           tma_load_3d(sk, &tm_k, &kv_full[stage], h * kHD, j * kKT, b);
           tma_load_3d(sk + kKBytes, &tm_v, &kv_full[stage], h * kHD, j * kKT, b);
-          if (++stage == kKvStages) { stage = 0; phase ^= 1; }
+          if (++stage == kStages) { stage = 0; phase ^= 1; }
         }
         qb ^= 1;
         if (qb == 0) q_phase ^= 1;
       }
-      for (int i = 0; i < kKvStages; ++i) {      // all armed stages consumed before the CTA retires
+      for (int i = 0; i < kStages; ++i) {      // all armed stages consumed before the CTA retires
         if (!mbar_wait(&kv_empty[stage], phase ^ 1, abort_flag)) break;
-        if (++stage == kKvStages) { stage = 0; phase ^= 1; }
+        if (++stage == kStages) { stage = 0; phase ^= 1; }
       }
+    } else {
+      stream_order();
     }
   } else if (warp == 1 || warp == 2) {
     // ------------------------------------------------------------ MMA issuer warp of query tile t
     // Scores run two key tiles ahead of P V, across the border between two runs as well (the next run's queries are
     // there by then).  The K/V ring counts every tile of the block; the score buffers count this query tile's.
+    stream_order();
     const bool leader = elect_one();
     const int t = warp - 1;
     constexpr uint32_t idesc_s = idesc_bf16(kQT, kKT, 0);    // S = Q K^T : both operands K-contiguous
@@ -764,7 +783,7 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       } else if (leader && a_left == 0) {
         mbar_arrive(&q_empty[a_qb]);
       }
-      if (++a_stage == kKvStages) { a_stage = 0; a_phase ^= 1; }
+      if (++a_stage == kStages) { a_stage = 0; a_phase ^= 1; }
       return true;
     };
     bool ok = issue_s() && issue_s();              // two score tiles ahead of the softmax
@@ -792,7 +811,7 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         } else if (leader) {
           mbar_arrive(&kv_empty[stage]);
         }
-        if (++stage == kKvStages) stage = 0;
+        if (++stage == kStages) stage = 0;
         // the scores two tiles on overwrite the buffer whose P the product above reads: safe because the
         // tensor core executes this thread's MMAs in issue order
         if (!(ok = issue_s())) break;
@@ -800,6 +819,7 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     }
   } else if (warp >= kFirstSoftmaxWarp) {
     // ------------------------------------------------------------ softmax
+    stream_order();
     const int t = t_own;
     const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)t * kTileCols;
     uint64_t* my_pair = &pair_bar[t * 4 + quad];
@@ -895,9 +915,10 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
 
       // Each half finishes 32 of the row's 64 output features.
       const uint32_t t_out = lane_base + kColO + hh * 32;
-      const int qi = (qg * kQTiles + t) * kQT + row;
-      const int bh = run.group / q_groups, h = bh % heads, b = bh / heads;
-      __nv_bfloat16* const dst = O + ((long long)b * n_q + qi) * ((long long)heads * kHD) + h * kHD + hh * 32;
+      if (MODE == kCut) {
+        qi = row_of(run.group);
+        dst = output_of(run.group, qi);
+      }
       if (MODE == kWhole || run.n == plan.tiles) {
         if (in_range(l_row, qi, run.group)) {
           const float inv = 1.0f / l_row;
@@ -906,7 +927,7 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
             uint32_t r[16];
             tmem_ld16(t_out + ch * 16, r);             // warp-collective: every lane loads
             tmem_ld_wait();
-            if (qi < n_q) emit16(r, inv, dst + ch * 16);
+            if (qi < n_q) emit16(r, inv, dst + hh * 32 + ch * 16);
           }
         }
         continue;
@@ -964,75 +985,85 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
           r[4 * q] = __float_as_uint(sum[q].x); r[4 * q + 1] = __float_as_uint(sum[q].y);
           r[4 * q + 2] = __float_as_uint(sum[q].z); r[4 * q + 3] = __float_as_uint(sum[q].w);
         }
-        if (qi < n_q) emit16(r, 1.0f / l_row, dst + ch * 16);
+        if (qi < n_q) emit16(r, 1.0f / l_row, dst + hh * 32 + ch * 16);
       }
     }
   }
 
+  if (warp == 3) stream_order();
   if (MODE == kCluster) {
     // ---------------------------------------------------------------- the cluster's parts
-    // Piece p (16 columns) of the accumulators is finished by rank p % split; it receives the others' sums in its (idle)
-    // key and value ring: [piece / split][sender][four columns][row of 256] words of 16 bytes, behind them the row sums.
-    const int split = plan.per_span;
-    const int rank = block % split, group = block / split;
+    // Piece p (16 columns) of the accumulators is finished by rank p % split, which receives the others' in turn:
+    // [piece / split][sender][four columns][row of 256] words of 16 bytes, behind them the row sums.
+    const int rank = block % plan.per_span;
     constexpr int kRows = kQTiles * kQT;
-    float4* const pieces = reinterpret_cast<float4*>(s_kv);
-    float* const sums = reinterpret_cast<float*>(pieces + 2 * 3 * 4 * kRows);    // (two pieces from three senders at most)
-    auto piece_at = [&](int p, int sender, int q) {
-      return pieces + (((p / split) * split + sender) * 4 + q) * kRows + t_own * kQT + row;
-    };
+    float4* const pieces = reinterpret_cast<float4*>(s_kv + (size_t)kStages * kKvStageBytes);
+    float* const sums = reinterpret_cast<float*>(pieces + 4 * 4 * kRows);        // (behind four pieces, the most there are)
+    static_assert(kQTiles * kQBytes + 4 * kKvStageBytes + (4 * 4 * 16 + 3 * 4) * kRows <=
+                  2 * kQTiles * kQBytes + kKvStages * kKvStageBytes, "ring and pieces fit");
+    const int my_row = t_own * kQT + row;
     const uint32_t t_out = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)t_own * kTileCols + kColO;
-    __syncwarp();
-    cluster_sync();                                    // every block's ring is idle
-    if (finished) {
-      for (int to = 0; to < split; ++to) {
-        if (to == rank) continue;
-        if (hh == 0) st_cluster_f32(cluster_map(smem_u32(sums + rank * kRows + t_own * kQT + row), (uint32_t)to), l_cluster);
-#pragma unroll 1
-        for (int p = to; p < 4; p += split) {
-          if ((p >> 1) != hh) continue;                // each half sends the columns of its own
+    auto merge = [&](auto split_c) {
+      constexpr int S = decltype(split_c)::value;
+      __syncwarp();
+      cluster_wait();                                  // the other blocks have started (long since)
+      if (finished) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {                  // each half sends two pieces, or keeps them
+          const int p = hh * 2 + i, to = p % S;
+          if (to == rank) continue;                    // warp-uniform
           uint32_t r[16];
           tmem_ld16(t_out + p * 16, r);
           tmem_ld_wait();
+          const int slot = (p / S) * (S - 1) + (rank < to ? rank : rank - 1);
+          const uint32_t at = cluster_map(smem_u32(pieces + slot * 4 * kRows + my_row), (uint32_t)to);
 #pragma unroll
           for (int q = 0; q < 4; ++q)
-            st_cluster_v4(cluster_map(smem_u32(piece_at(p, rank, q)), (uint32_t)to), __uint_as_float(r[4 * q]),
-                          __uint_as_float(r[4 * q + 1]), __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
+            st_cluster_v4(at + q * kRows * 16, __uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
+                          __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
         }
-      }
-    }
-    __syncwarp();
-    cluster_sync();
-    if (finished) {
-      const int qg = group % q_groups, bh = group / q_groups, h = bh % heads, b = bh / heads;
-      const int qi = (qg * kQTiles + t_own) * kQT + row;
-      __nv_bfloat16* const dst = O + ((long long)b * n_q + qi) * ((long long)heads * kHD) + h * kHD;
-      float l_row = 0.f;
-      for (int k = 0; k < split; ++k) l_row += k == rank ? l_cluster : sums[k * kRows + t_own * kQT + row];
-      if (in_range(l_row, qi, group)) {                // (all ranks come to the same verdict; the first records it)
-        const float inv = 1.0f / l_row;
-#pragma unroll 1
-        for (int p = rank; p < 4; p += split) {
-          if ((split == 4 ? 0 : p >> 1) != hh) continue;
-          uint32_t r[16];
-          tmem_ld16(t_out + p * 16, r);
-          tmem_ld_wait();
+        if (hh == 0) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int k = 0; k < split; ++k) {
-              const float4 o = k == rank ? make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
-                                                       __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]))
-                                         : *piece_at(p, k, q);
-              v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
-            }
-            r[4 * q] = __float_as_uint(v.x); r[4 * q + 1] = __float_as_uint(v.y);
-            r[4 * q + 2] = __float_as_uint(v.z); r[4 * q + 3] = __float_as_uint(v.w);
-          }
-          if (qi < n_q) emit16(r, inv, dst + p * 16);
+          for (int to = 0; to < S; ++to)
+            if (to != rank)
+              st_cluster_f32(cluster_map(smem_u32(sums + (rank < to ? rank : rank - 1) * kRows + my_row), (uint32_t)to), l_cluster);
         }
       }
-    }
+      __syncwarp();
+      cluster_sync();
+      if (!finished) return;
+      float l_row = 0.f;                               // (added in rank order, as everything here)
+#pragma unroll
+      for (int k = 0; k < S; ++k) l_row += k == rank ? l_cluster : sums[(k < rank ? k : k - 1) * kRows + my_row];
+      if (!in_range(l_row, qi, only_group)) return;    // (all ranks come to the same verdict; the first records it)
+      const float inv = 1.0f / l_row;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int p = S == 4 ? rank : hh * 2 + i;      // of four ranks each has one piece: its first half finishes it
+        if (p % S != rank || (S == 4 && (hh != 0 || i != 0))) continue;          // warp-uniform
+        uint32_t r[16];
+        tmem_ld16(t_out + p * 16, r);
+        tmem_ld_wait();
+        const float4* at = pieces + (p / S) * (S - 1) * 4 * kRows + my_row;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int k = 0; k < S; ++k) {
+            const float4 o = k == rank ? make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
+                                                     __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]))
+                                       : at[((k < rank ? k : k - 1) * 4 + q) * kRows];
+            v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+          }
+          r[4 * q] = __float_as_uint(v.x); r[4 * q + 1] = __float_as_uint(v.y);
+          r[4 * q + 2] = __float_as_uint(v.z); r[4 * q + 3] = __float_as_uint(v.w);
+        }
+        if (qi < n_q) emit16(r, inv, dst + p * 16);
+      }
+    };
+    if (plan.per_span == 2) merge(std::integral_constant<int, 2>{});
+    else if (plan.per_span == 3) merge(std::integral_constant<int, 3>{});
+    else merge(std::integral_constant<int, 4>{});
   }
 
   // ---------------------------------------------------------------- rows out of range: once more, on the safe path
