@@ -164,7 +164,9 @@ bool is_full(const hero_config& g, int step) {
 
 int run_gemm(hero_ctx* c, const void* a, const void* w, const void* bias, int M, int Nout, int K, const GemmOut& out) {
   LaunchScope scope(c, HERO_PROF_GEMM);
-  if (c->cfg.dtype == HERO_DTYPE_BF16) return launch_tc_gemm(a, w, bias, M, Nout, K, out, c->d_status, c->stream);
+  GemmOut o = out;
+  o.weights_settled = 1;               // (behind a kernel of this context, which waited for whatever wrote the weights)
+  if (c->cfg.dtype == HERO_DTYPE_BF16) return launch_tc_gemm(a, w, bias, M, Nout, K, o, c->d_status, c->stream);
   return launch_simt_gemm((const float*)a, (const float*)w, (const float*)bias, M, Nout, K, out, c->stream);
 }
 

@@ -254,26 +254,44 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
   cluster_sync();                           // both CTAs' barriers exist before anybody signals across
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  stream_order();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
       int stage = 0; uint32_t phase = 0;
       bool ok = true;
+      auto load = [&](int kb, int row, bool weights) {
+        const uint32_t sa = smem_u32(smem + (size_t)stage * Cfg::kStageBytes), bar = cluster_map(smem_u32(&full[stage]), 0);
+        if (weights) tma_load_2d_pair(sa + kABytes, &tm_w, bar, kb * kBK, row);
+        else tma_load_2d_pair(sa, &tm_a, bar, kb * kBK, row);
+      };
+      // The even CTA's barrier counts the bytes of both CTAs.  The odd CTA's may land before it is armed: its
+      // phase cannot complete before the arrival that arms it.
+      int ahead = 0;                         // stages whose weights were fetched before the wait for the kernel before
       for (int tile = pair; tile < n_tiles_total && ok; tile += n_pairs) {
         int mt, nt;
         tile_coords(tile, m_tiles, n_tiles, mt, nt);
         const int row_a = (2 * mt + (int)rank) * kBM, row_w = nt * BN + (int)rank * (BN / 2);
+        if (tile == pair) {
+          if (out.weights_settled) {
+            for (; ahead < kStages && ahead < k_blocks; ++ahead) {
+              stage = ahead;
+              if (rank == 0) mbar_expect_tx(&full[stage], 2 * Cfg::kStageBytes);
+              load(ahead, row_w, true);
+            }
+            stage = 0;
+          }
+          stream_order();
+        }
         for (int kb = 0; kb < k_blocks; ++kb) {
-          if (!(ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag))) break;
-          const uint32_t sa = smem_u32(smem + (size_t)stage * Cfg::kStageBytes);
-          // The even CTA's barrier counts the bytes of both CTAs.  The odd CTA's may land before it is armed: its
-          // phase cannot complete before the arrival that arms it.
-          if (rank == 0) mbar_expect_tx(&full[stage], 2 * Cfg::kStageBytes);
-          const uint32_t bar = cluster_map(smem_u32(&full[stage]), 0);
-          tma_load_2d_pair(sa, &tm_a, bar, kb * kBK, row_a);
-          tma_load_2d_pair(sa + kABytes, &tm_w, bar, kb * kBK, row_w);
+          if (ahead > 0) {
+            --ahead;
+          } else {
+            if (!(ok = mbar_wait(&empty[stage], phase ^ 1, abort_flag))) break;
+            if (rank == 0) mbar_expect_tx(&full[stage], 2 * Cfg::kStageBytes);
+            load(kb, row_w, true);
+          }
+          load(kb, row_a, false);
           if (++stage == kStages) { stage = 0; phase ^= 1; }
         }
       }
@@ -283,12 +301,15 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
         if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag)) break;
         if (++stage == kStages) { stage = 0; phase ^= 1; }
       }
+    } else {
+      stream_order();
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (even CTA)
     // All 32 lanes run the loop and one elected lane issues: tile counters, stage addresses and descriptors
     // then stay warp-uniform values instead of one diverged lane's private registers, which is what the
     // tensor-core instructions are fed from.
+    stream_order();
     if (rank == 0) {
       const bool leader = elect_one();
       constexpr uint32_t idesc = idesc_bf16(2 * kBM, BN, 0);
@@ -318,6 +339,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
     }
   } else {
     // ------------------------------------------------------------ epilogue (warps 2..9)
+    stream_order();
     const int quad = warp & 3;                 // TMEM lane quadrant this warp may read
     const int half = (warp - 2) >> 2;          // which half of the tile's columns it finishes
     float* s_bias_warp = s_bias_all + (size_t)(warp - 2) * BN;
@@ -366,9 +388,10 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
 // `split` CTAs shares a tile, each taking a run of its K steps; they then trade partial sums through distributed
 // shared memory, each finishing BN / split of the tile's columns (the partial sums of the other CTAs are added in
 // rank order, so a result does not depend on timing).  Warp roles as above; the epilogue warps fetch bias and
-// destination rows while the MMAs run.  Bound by latency: of 4.7 us at 148 x 768 x 256 (14.0 with one CTA per 128 x 256
-// tile and the bias fetched between accumulator reads) 0.8 us are the K loop, the rest is launch, first fetch and
-// epilogue.  614 x 256 x 768 over two CTAs a tile: 6.1 us (15.6), 371 x 768 x 3072 over four: 9.6 (16.7 over one).
+// destination rows while the MMAs run, and the producer fetches the first weights while the kernel before still runs.
+// Bound by latency: of 3.4 us at 148 x 768 x 256 (4.0 without the early weights, 14.0 with one CTA per 128 x 256 tile and
+// the bias fetched between accumulator reads) 1.1 us are the K loop, the rest is launch, first fetch and epilogue.
+// 614 x 256 x 768 over two CTAs a tile: 4.2 us (4.6 over one), 371 x 768 x 3072 over four: 8.1 (13.2 over one).
 // ---------------------------------------------------------------------------------------------------------------
 template <int BN>
 struct SplitCfg {
@@ -422,27 +445,39 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
   tc_fence_after();
   if (split > 1) cluster_arrive();           // waited for before anything is sent to another CTA
   const uint32_t tmem_base = *tmem_slot;
-  stream_order();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
       int stage = 0; uint32_t phase = 0;
+      int ahead = kb0;                         // K steps whose weights were fetched before the wait for the kernel before
+      if (out.weights_settled) {
+        for (; ahead < kb1 && ahead < kb0 + kStages; ++ahead) {
+          mbar_expect_tx(&full[ahead - kb0], Cfg::kStageBytes);
+          tma_load_2d(smem + (size_t)(ahead - kb0) * Cfg::kStageBytes + kABytes, &tm_w, &full[ahead - kb0], ahead * kBK, nt * BN);
+        }
+      }
+      stream_order();
       for (int kb = kb0; kb < kb1; ++kb) {
-        if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag)) break;
         uint8_t* sa = smem + (size_t)stage * Cfg::kStageBytes;
-        mbar_expect_tx(&full[stage], Cfg::kStageBytes);
+        if (kb >= ahead) {
+          if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag)) break;
+          mbar_expect_tx(&full[stage], Cfg::kStageBytes);
+          tma_load_2d(sa + kABytes, &tm_w, &full[stage], kb * kBK, nt * BN);
+        }
         tma_load_2d(sa, &tm_a, &full[stage], kb * kBK, mt * kBM);
-        tma_load_2d(sa + kABytes, &tm_w, &full[stage], kb * kBK, nt * BN);
         if (++stage == kStages) { stage = 0; phase ^= 1; }
       }
       for (int i = 0; i < kStages; ++i) {      // all armed stages consumed before the CTA retires
         if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag)) break;
         if (++stage == kStages) { stage = 0; phase ^= 1; }
       }
+    } else {
+      stream_order();
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
+    stream_order();
     const bool leader = elect_one();
     constexpr uint32_t idesc = idesc_bf16(kBM, BN, 0);
     int stage = 0; uint32_t phase = 0;
@@ -473,6 +508,7 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
   RowOut row = {};
   bool ok = true;
   if (warp >= 2) {
+    stream_order();
     stage_bias<BN / 2>(s_bias, bias, nt * BN + c_first, Nout, lane);
     row = row_out(out, mt * kBM + tile_row, M);
     ok = mbar_wait_warp(acc_full, 0, abort_flag);
@@ -551,15 +587,20 @@ int launch_wait_timeout_selftest(int* d_status, int budget_us, cudaStream_t s) {
 
 // ---------------------------------------------------------------------------------------------------------------
 // Which kernel, which tile, how many CTAs per tile.  The estimate is in SM clocks: rounds of tiles times K steps times
-// the clocks of a step, plus what a launch costs outside its K loop.  A K step is bound by what an SM can fetch from L2
-// (about 64 bytes per clock): 24 / 32 KB for a tile of 128 x 64 / 128 x 128 in a CTA, 24 / 32 KB per CTA of a pair on
-// 256 x 128 / 256 x 256 (where the tensor core needs 512 clocks as well).  Measured (us) where the choice is close:
-//   M x N x K            pair 256  pair 224  pair 192  pair 128  CTA 128  CTA 64
-//   3510 x 3072 x 3072      51.8      49.5      54.3      64.7     86.3   131.4
-//   5254 x 1152 x 1152      17.6      16.5      15.6      19.0     27.9    42.1
-//   1394 x 3072 x 1024      12.2      15.3      14.5      13.3     17.4
-//   1394 x 1024 x 1024      11.5                           9.3      8.9    13.7
-//   371 x 3072 x 768         9.9                           8.0      7.6     6.7
+// the clocks of a step (bound by what an SM can fetch from L2, about 64 bytes per clock at best: 24 / 32 KB for a tile of
+// 128 x 64 / 128 x 128 in a CTA, 24 to 32 KB per CTA of a pair), plus what a launch costs outside its K loop, which is as
+// much again for a small problem: start, epilogue, and for a split tile the exchange.  Fitted to launches in a row (us):
+//   M x N x K            pair 256  pair 224  pair 192  pair 128  CTA 128  over 2  over 4   CTA 64  over 2
+//   148 x 768 x 256                                        4.9      4.2     4.7     5.0      3.4     3.7
+//   148 x 256 x 768                                        5.5      5.4     5.2     5.1      4.6     4.2
+//   371 x 3072 x 768                                       7.2      6.2     6.7    18.4      5.8    11.0
+//   371 x 768 x 3072                                      13.6     13.2     9.5     8.1     12.1     8.1
+//   1394 x 1024 x 1024      9.9       9.2       8.3       7.4      7.2    12.7              11.6
+//   1394 x 3072 x 1024     11.4      13.2      12.3      12.2     14.4    27.1              23.8
+//   1394 x 1024 x 4096     23.4      21.2      19.6      19.0     20.4    25.4              32.5
+//   5254 x 1152 x 1152     15.9      15.1      14.2      17.0     21.9    40.8              37.4
+//   5254 x 3456 x 1152     32.2      33.7      35.2      41.7     62.5
+//   3510 x 3072 x 3072     51.8      49.5      54.3      64.7     86.3
 // ---------------------------------------------------------------------------------------------------------------
 namespace {
 
@@ -574,19 +615,22 @@ GemmPlan plan_gemm(int M, int Nout, int K) {
   auto consider = [&](int bn, int split, long long t) {
     if (best_t < 0 || t < best_t) { best_t = t; best = {bn, split}; }
   };
-  for (int bn : {256, 224, 192, 128}) {
-    const long long tiles = ceil_div(M, 2 * kBM) * ceil_div(Nout, bn);
-    consider(bn, 0, ceil_div(tiles, sms / 2) * kb * (256 + bn * 9 / 8) + 9000 + bn * 8);
+  struct { int bn, step, fixed; } const pair[] = {{256, 560, 11500}, {224, 510, 10100}, {192, 500, 8000}, {128, 460, 7400}};
+  for (const auto& p : pair) {
+    const long long tiles = ceil_div(M, 2 * kBM) * ceil_div(Nout, p.bn);
+    consider(p.bn, 0, ceil_div(tiles, sms / 2) * kb * p.step + p.fixed);
   }
   for (int bn : {128, 64}) {
     const long long tiles = ceil_div(M, kBM) * ceil_div(Nout, bn);
     const int max_split = bn == 128 ? SplitCfg<128>::kMaxSplit : SplitCfg<64>::kMaxSplit;
-    for (int split = 1; split <= max_split; split *= 2) {
-      if (split > kb) break;
-      if (tiles * split > 0x7FFFFFFFll) continue;
-      const long long waves = ceil_div(tiles * split, sms);
-      consider(bn, split, waves * (ceil_div(kb, split) * (bn == 128 ? 520 : 390) + (bn == 128 ? 7000 : 6500)) +
-                              1500 + (split > 1 ? 500 * split : 0));
+    for (int split = 1; split <= max_split && split <= kb; split *= 2) {
+      const long long ctas = tiles * split;
+      if (ctas > 0x7FFFFFFFll) continue;
+      // (clusters of four do not fill the chip: they need four free SMs of one processing cluster)
+      const long long waves = ceil_div(ctas, split == 4 ? sms * 7 / 8 : sms);
+      const long long step = bn == 64 ? 390 : 400 + (ctas < 100 ? ctas : 100);
+      const long long exchange = split == 1 ? 0 : (bn == 64 ? 1700 : (split == 2 ? 2000 : 3500));
+      consider(bn, split, waves * (ceil_div(kb, split) * step + (bn == 64 ? 4500 : 6300) + exchange));
     }
   }
   return best;

@@ -26,7 +26,7 @@ GEMM_TOL = 2.0 ** -9
     (681, 3536, 8), (1394, 1024, 1024), (1281, 1160, 1544),
     # one tile per CTA: 128 and 64 columns, K whole or over clusters of two and four CTAs (uneven K runs among them)
     (544, 1968, 8), (640, 3080, 136), (7, 1464, 8), (1, 8, 72), (33, 8, 592), (129, 1096, 520), (257, 520, 1544),
-    (136, 2904, 760), (23, 16, 1768), (129, 200, 4104), (300, 776, 3080)])
+    (136, 2904, 760), (23, 16, 1768), (129, 200, 4104), (300, 776, 3080), (371, 768, 3072), (100, 40, 2056)])
 def test_gemm_tile_variants(M, N, K):
     rng = np.random.default_rng(M + 7 * N + 13 * K)
     a = S.round_bf16(rng.standard_normal((M, K)).astype(np.float32))
