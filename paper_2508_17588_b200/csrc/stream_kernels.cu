@@ -175,7 +175,10 @@ extrapolate_residual_kernel(T* __restrict__ x, const T* __restrict__ ga_prev, co
 // the residual stream, so x can stay in registers while the blocks' four history tensors stream by.  Per
 // element and block that is 8 bytes read instead of 12 moved (x is read and written once per launch, not
 // once per block), and the sum is rounded to the storage type once.  The adds keep the order of the blocks.
-template <typename T>
+// E entries of the group are in flight per thread: four keep a large pass at the memory's rate (25 GB: 6.6 TB/s); where the
+// elements give every SM less than two blocks the pass is a chain of loads, and sixteen make it shorter (56 entries of
+// 157k elements: 36 -> 14 us).
+template <typename T, int E>
 __global__ void __launch_bounds__(kStreamThreads) extrapolate_group_kernel(T* __restrict__ x, const DeepGroup grp,
                                                                            long long first, long long n, float c) {
   stream_order();
@@ -186,14 +189,22 @@ __global__ void __launch_bounds__(kStreamThreads) extrapolate_group_kernel(T* __
   for (long long i = (long long)blockIdx.x * kStreamThreads + threadIdx.x; i < n_vec; i += stride) {
     float fx[V::N];
     ld_stream(xv + i).unpack(fx);
-#pragma unroll 4
-    for (int e = 0; e < grp.n_entries; ++e) {
-      const V vp = ld_stream(reinterpret_cast<const V*>(static_cast<const T*>(grp.prev[e]) + first) + i);
-      const V vl = ld_stream(reinterpret_cast<const V*>(static_cast<const T*>(grp.last[e]) + first) + i);
-      float fp_[V::N], fl_[V::N];
-      vp.unpack(fp_); vl.unpack(fl_);
+    for (int e0 = 0; e0 < grp.n_entries; e0 += E) {
+      V vp[E], vl[E];
 #pragma unroll
-      for (int j = 0; j < V::N; ++j) fx[j] += fmaf(fl_[j] - fp_[j], c, fl_[j]);
+      for (int u = 0; u < E; ++u)
+        if (e0 + u < grp.n_entries) {
+          vp[u] = ld_stream(reinterpret_cast<const V*>(static_cast<const T*>(grp.prev[e0 + u]) + first) + i);
+          vl[u] = ld_stream(reinterpret_cast<const V*>(static_cast<const T*>(grp.last[e0 + u]) + first) + i);
+        }
+#pragma unroll
+      for (int u = 0; u < E; ++u)
+        if (e0 + u < grp.n_entries) {
+          float fp_[V::N], fl_[V::N];
+          vp[u].unpack(fp_); vl[u].unpack(fl_);
+#pragma unroll
+          for (int j = 0; j < V::N; ++j) fx[j] += fmaf(fl_[j] - fp_[j], c, fl_[j]);
+        }
     }
     V r; r.pack(fx);
     st_stream(xv + i, r);
@@ -717,12 +728,15 @@ int launch_extrapolate_group(void* x, const DeepGroup& grp, long long first, lon
   if (first % per != 0) return HERO_ERR_ALIGN;            // keeps every 16-byte access aligned
   long long blocks = (n / per + kStreamThreads - 1) / kStreamThreads;
   blocks = blocks < 1 ? 1 : (blocks > (long long)num_sms() * 16 ? (long long)num_sms() * 16 : blocks);
-  if (dtype == HERO_DTYPE_BF16)
-    HERO_TRY(launch_streaming(extrapolate_group_kernel<__nv_bfloat16>, blocks, kStreamThreads, s,
-                           (__nv_bfloat16*)x, grp, first, n, c));
-  else
-    HERO_TRY(launch_streaming(extrapolate_group_kernel<float>, blocks, kStreamThreads, s, (float*)x, grp,
-                           first, n, c));
+  const bool few = blocks < 2ll * num_sms();
+  if (dtype == HERO_DTYPE_BF16) {
+    using T = __nv_bfloat16;
+    HERO_TRY(launch_streaming(few ? extrapolate_group_kernel<T, 16> : extrapolate_group_kernel<T, 4>, blocks, kStreamThreads,
+                              s, (T*)x, grp, first, n, c));
+  } else {
+    HERO_TRY(launch_streaming(few ? extrapolate_group_kernel<float, 16> : extrapolate_group_kernel<float, 4>, blocks,
+                              kStreamThreads, s, (float*)x, grp, first, n, c));
+  }
   return HERO_OK;
 }
 
