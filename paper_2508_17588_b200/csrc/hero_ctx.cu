@@ -181,7 +181,7 @@ int run_attention(hero_ctx* c, const void* q, const void* k, const void* v, void
 }
 
 // adaLN vectors of blocks [l0, l1) into their slots of c->mod, at most kMaxModBatch blocks per launch
-int modulation_for_blocks(hero_ctx* c, int l0, int l1, const void* d_temb) {
+int modulation_for_blocks(hero_ctx* c, int l0, int l1, const void* d_temb, bool after_select) {
   const hero_config& g = c->cfg;
   const int mod_ld = c->n_mod * g.hidden;
   for (int l = l0; l < l1; l += kMaxModBatch) {
@@ -192,7 +192,8 @@ int modulation_for_blocks(hero_ctx* c, int l0, int l1, const void* d_temb) {
       mb.mod[mb.n] = c->mod + (size_t)b * g.batch * mod_ld;
     }
     HERO_LAUNCH(c, HERO_PROF_MODULATION,
-                launch_modulation_batch(d_temb, mb, g.batch, mod_ld, g.temb_dim, g.dtype, c->stream));
+                launch_modulation_batch(d_temb, mb, g.batch, mod_ld, g.temb_dim, after_select && l == l0, g.dtype,
+                                        c->stream));
   }
   return HERO_OK;
 }
@@ -681,7 +682,7 @@ static int step_impl(hero_ctx* c, int step, void* d_x, const void* d_temb, void*
       c->stack_new = c->stack_n == 0 ? 0 : (c->stack_last ^ 1);
       HERO_CUDA_TRY(cudaMemsetAsync(c->stack_hist[c->stack_new], 0, (size_t)c->elems * sizeof(float), c->stream));
     }
-    HERO_TRY(modulation_for_blocks(c, 0, g.n_blocks, d_temb));
+    HERO_TRY(modulation_for_blocks(c, 0, g.n_blocks, d_temb, false));
     for (int l = 0; l < g.n_blocks; ++l) HERO_TRY(refresh_block(c, l, d_x, d_temb, nullptr, c->N, true));
     if (collapse) { c->stack_last = c->stack_new; if (c->stack_n < 2) c->stack_n++; }
     c->s_prev = c->s_last; c->s_last = step; c->n_full++;
@@ -709,7 +710,7 @@ static int step_impl(hero_ctx* c, int step, void* d_x, const void* d_temb, void*
     for (int l = 0; l < n_draws; ++l) { c->blk[l].ages_cur ^= 1; c->blk[l].calls++; }
     for (int l = n_draws; l < g.n_shallow; ++l) n_sel[l] = n_sel[0];
   }
-  HERO_TRY(modulation_for_blocks(c, 0, g.n_shallow, d_temb));
+  HERO_TRY(modulation_for_blocks(c, 0, g.n_shallow, d_temb, true));
   for (int l = 0; l < g.n_blocks; ++l) {
     if (l < g.n_shallow) {
       if (n_sel[l] > 0) {

@@ -206,7 +206,9 @@ struct ModBatch {
   const void* b_mod[kMaxModBatch];
   float* mod[kMaxModBatch];
 };
-int launch_modulation_batch(const void* temb, const ModBatch& batch, int B, int n_out, int E, int dtype, cudaStream_t s);
+// (beside: the kernel in front on the stream is this step's launch_select)
+int launch_modulation_batch(const void* temb, const ModBatch& batch, int B, int n_out, int E, bool beside, int dtype,
+                            cudaStream_t s);
 int launch_modulation(const void* temb, const void* w_mod, const void* b_mod, float* mod, int B,
                       int n_out, int E, int dtype, cudaStream_t s);
 // a[m,:] = LN(x[row(m),:] (+ add[row(m),:])) * (1 + scale[b,:]) + shift[b,:]

@@ -460,15 +460,18 @@ __global__ void __launch_bounds__(256, 2) modulation_kernel(const T* __restrict_
   modulation_rows<T, MAXB>(s_act, w_mod, b_mod, mod, B, n_out, E);
 }
 
-// The same for several blocks at once: blockIdx.y picks the block's weights and output.
+// The same for several blocks at once: blockIdx.y picks the block's weights and output.  `beside`: the kernel in front is
+// the token selection of the same step, which has nothing to do with this one (and which has itself waited for everything
+// that came before): the two run side by side, and the wait that makes this kernel's end stand for both comes last.
 template <typename T, int MAXB>
 __global__ void __launch_bounds__(256, 2) modulation_batch_kernel(const T* __restrict__ temb, const ModBatch batch, int B,
-                                                               int n_out, int E) {
-  stream_order();
+                                                               int n_out, int E, bool beside) {
+  if (!beside) stream_order();
   extern __shared__ float s_act[];
   modulation_stage_activations<T>(temb, s_act, B, E);
   modulation_rows<T, MAXB>(s_act, static_cast<const T*>(batch.w_mod[blockIdx.y]), static_cast<const T*>(batch.b_mod[blockIdx.y]),
                      batch.mod[blockIdx.y], B, n_out, E);
+  if (beside) stream_order();
 }
 
 // ------------------------------------------------------------------ gather + LayerNorm + modulate (Eq. 2 prologue)
@@ -825,9 +828,9 @@ int launch_scatter_rows(const void* src, const int* idx, void* dst, int B, int N
 
 // The kernels are instantiated for 1, 2, 4 and 8 batch items so that a warp's accumulators are as many as it needs.
 template <typename T, int MAXB>
-static int modulation_batch_launch(const void* temb, const ModBatch& batch, int B, int n_out, int E, dim3 grid,
+static int modulation_batch_launch(const void* temb, const ModBatch& batch, int B, int n_out, int E, bool beside, dim3 grid,
                                     size_t smem, cudaStream_t s) {
-  return launch_kernel(modulation_batch_kernel<T, MAXB>, grid, 256, smem, s, 1, (const T*)temb, batch, B, n_out, E);
+  return launch_kernel(modulation_batch_kernel<T, MAXB>, grid, 256, smem, s, 1, (const T*)temb, batch, B, n_out, E, beside);
 }
 template <typename T, int MAXB>
 static int modulation_launch(const void* temb, const void* w_mod, const void* b_mod, float* mod, int B, int n_out,
@@ -843,7 +846,7 @@ static int modulation_launch(const void* temb, const void* w_mod, const void* b_
     return FN<T, kModMaxB>(__VA_ARGS__);                   \
   } while (0)
 
-int launch_modulation_batch(const void* temb, const ModBatch& batch, int B, int n_out, int E, int dtype,
+int launch_modulation_batch(const void* temb, const ModBatch& batch, int B, int n_out, int E, bool beside, int dtype,
                             cudaStream_t s) {
   if (B > kModMaxB || batch.n < 0 || batch.n > kMaxModBatch) return HERO_ERR_ARG;
   if (batch.n == 0) return HERO_OK;
@@ -854,10 +857,10 @@ int launch_modulation_batch(const void* temb, const ModBatch& batch, int B, int 
   const dim3 grid(bx, batch.n);
   if (dtype == HERO_DTYPE_BF16) {
     if (E % 8) return HERO_ERR_ALIGN;
-    HERO_MOD_DISPATCH(modulation_batch_launch, __nv_bfloat16, temb, batch, B, n_out, E, grid, smem, s);
+    HERO_MOD_DISPATCH(modulation_batch_launch, __nv_bfloat16, temb, batch, B, n_out, E, beside, grid, smem, s);
   } else {
     if (E % 4) return HERO_ERR_ALIGN;
-    HERO_MOD_DISPATCH(modulation_batch_launch, float, temb, batch, B, n_out, E, grid, smem, s);
+    HERO_MOD_DISPATCH(modulation_batch_launch, float, temb, batch, B, n_out, E, beside, grid, smem, s);
   }
 }
 
