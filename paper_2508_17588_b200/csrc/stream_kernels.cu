@@ -435,18 +435,37 @@ __device__ __forceinline__ void modulation_rows(const float* s_act, const T* __r
         }
       }
     }
+    // Sums over the warp, all of them together: as long as a lane holds more than one value, the two halves of a pair of
+    // lanes share them out (a quarter of the shuffles of one butterfly per value).
+    constexpr int kSums = kModRows * MAXB;
+    float v[kSums];
 #pragma unroll
-    for (int r = 0; r < kModRows; ++r) {
+    for (int r = 0; r < kModRows; ++r)
 #pragma unroll
-      for (int b = 0; b < MAXB; ++b) {
-        if (b < B) {
-          float v = acc[r][b];
+      for (int b = 0; b < MAXB; ++b) v[r * MAXB + b] = acc[r][b];
+    int which = 0;                                     // which value ends up in this lane
+    int n = kSums;
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-          if (lane == 0 && j0 + r < n_out) mod[(long long)b * n_out + j0 + r] = v + to_f(b_mod[j0 + r]);
+    for (int o = 16; o > 0; o >>= 1) {
+      if (n > 1) {
+        n >>= 1;
+        const bool upper = lane & o;
+#pragma unroll
+        for (int i = 0; i < kSums / 2; ++i) {
+          if (i < n) {
+            const float give = upper ? v[i] : v[i + n], keep = upper ? v[i + n] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
+          }
         }
+        which += upper ? n : 0;
+      } else {
+        v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], o);
       }
     }
+    static_assert(kSums <= 32, "a lane per value");
+    const int r = which / MAXB, b = which - r * MAXB;
+    if ((lane & (32 / kSums - 1)) == 0 && b < B && j0 + r < n_out)
+      mod[(long long)b * n_out + j0 + r] = v[0] + to_f(b_mod[j0 + r]);
   }
 }
 
