@@ -69,6 +69,7 @@ struct hero_ctx {
   int rope_pairs[3] = {0, 0, 0};
   void *ws_a = nullptr, *ws_q = nullptr, *ws_o = nullptr, *ws_u = nullptr;
   float* mod = nullptr;                  // [n_blocks, B, n_mod*D] adaLN vectors, one slot per block
+  int* pos_ws = nullptr;                 // [n_shallow, idx_cap] every video token's place in those lists, or -1
   int* idx_ws = nullptr;                 // [n_shallow, idx_cap] selection lists of the current step
   float* att_parts = nullptr;             // bf16: partial results of the attention's cut query groups
   size_t status_bytes = 0;
@@ -198,10 +199,17 @@ int modulation_for_blocks(hero_ctx* c, int l0, int l1, const void* d_temb, bool 
   return HERO_OK;
 }
 
-// Eq. 2 on the listed rows + Eq. 3's merge + the residual adds of Algorithm 1.  mod_ready: the block's adaLN
-// vectors are in its slot already (hero_step computes them for all blocks of the step in one launch).
-int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const int* d_idx, int n_sel,
-                  bool mod_ready = false) {
+// What hero_step knows about the block after the one being refreshed: that it is refreshed too, and on which rows.
+struct NextRefresh {
+  int n_sel = 0;               // 0: not refreshed, or not to be prepared here
+  const int* pos = nullptr;    // as SelectBatch::pos; null: all rows
+};
+
+// Eq. 2 on the listed rows + Eq. 3's merge + the residual adds of Algorithm 1.  In a step (`in_step`) the adaLN vectors of
+// all its blocks are in their slots already, the residual pass may prepare the next block's input on the way (`next`), and
+// the block before may have done so for this one (`prepared`).
+int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const int* d_idx, int n_sel, bool in_step = false,
+                  bool prepared = false, const NextRefresh& next = {}) {
   const hero_config& g = c->cfg;
   const int B = g.batch, N = c->N, D = g.hidden, F = g.ffn_dim;
   const bool full = d_idx == nullptr;
@@ -226,7 +234,7 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
   }
 
   float* mod = c->mod + (size_t)block * B * mod_ld;       // this block's slot; hero_step fills all slots up front
-  if (!mod_ready)
+  if (!in_step)
     HERO_LAUNCH(c, HERO_PROF_MODULATION,
                 launch_modulation(d_temb, w.w_mod, w.b_mod, mod, B, mod_ld, g.temb_dim, g.dtype, c->stream));
   const float* shift1 = mod;
@@ -239,7 +247,9 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
   // attention branch
   const void* host_rows = c->first_rows_src;
   c->first_rows_src = nullptr;
-  if (host_rows && d_idx) {
+  if (prepared) {
+    // (the rows are in ws_a)
+  } else if (host_rows && d_idx) {
     // x is still on its way to the device (hero_step_host): fetch the listed rows from the caller's pinned
     // buffer, once, normalise them from that compact copy, and plant them in the device copy of x, where the
     // FFN branch below will look for them.  The upload under way writes the same values over them.
@@ -319,14 +329,19 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
     c->wait_x_upload = false;
     HERO_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->x_uploaded, 0));
   }
-  if (collapse) {
+  if (next.n_sel > 0) {
+    const float* mod_next = c->mod + (size_t)(block + 1) * B * mod_ld;
+    HERO_LAUNCH(c, HERO_PROF_RESIDUAL,
+                launch_residual_ln(d_x, ga, gf, next.pos, g.n_text, mod_next,
+                                   mod_next + D, mod_ld, c->ws_a, B, N, next.n_sel, D, 1e-5f, g.dtype, c->stream));
+  } else if (collapse) {
     HERO_LAUNCH(c, HERO_PROF_RESIDUAL,
                 launch_residual2_acc(d_x, ga, gf, c->stack_hist[c->stack_new], c->elems, g.dtype, c->stream));
-    return HERO_OK;
+  } else {
+    HERO_LAUNCH(c, HERO_PROF_RESIDUAL, launch_residual2(d_x, ga, gf, c->elems, g.dtype, c->stream));
   }
-  HERO_LAUNCH(c, HERO_PROF_RESIDUAL, launch_residual2(d_x, ga, gf, c->elems, g.dtype, c->stream));
 
-  if (full) {
+  if (full && !collapse) {
     if (deep) {
       bm.last_slot = new_slot;
       if (bm.n_hist < 2) bm.n_hist++;
@@ -520,6 +535,7 @@ int hero_init(hero_ctx** out, const hero_config* cfg, const hero_block_weights* 
   A(&c->ws_u, (size_t)cfg->batch * c->N * cfg->ffn_dim * c->esz);
   A((void**)&c->mod, (size_t)cfg->n_blocks * cfg->batch * c->n_mod * cfg->hidden * sizeof(float));
   A((void**)&c->idx_ws, (size_t)(cfg->n_shallow > 0 ? cfg->n_shallow : 1) * c->idx_cap * sizeof(int));
+  A((void**)&c->pos_ws, (size_t)(cfg->n_shallow > 0 ? cfg->n_shallow : 1) * c->idx_cap * sizeof(int));
   if (cfg->dtype == HERO_DTYPE_BF16) A((void**)&c->att_parts, tc_attention_part_bytes());
   c->status_bytes = (4 + (cfg->dtype == HERO_DTYPE_BF16 ? tc_attention_part_counters() : 0)) * sizeof(int);
   A((void**)&c->d_status, c->status_bytes);
@@ -612,6 +628,7 @@ int hero_select_tokens(hero_ctx* c, int block, int* d_idx, int cap, int* n_sel) 
   batch.block[0] = block; batch.call[0] = bm.calls;
   batch.ages_in[0] = bm.ages[bm.ages_cur]; batch.ages_out[0] = bm.ages[bm.ages_cur ^ 1];
   batch.idx[0] = d_idx;
+  batch.pos[0] = nullptr;
   HERO_LAUNCH(c, HERO_PROF_SELECT, launch_select(geom_of(c->cfg), batch, c->stream));
   bm.ages_cur ^= 1;
   bm.calls++;
@@ -677,13 +694,21 @@ static int step_impl(hero_ctx* c, int step, void* d_x, const void* d_temb, void*
   if (!aligned16(d_x) || !aligned16(d_temb)) return HERO_ERR_ALIGN;
   const hero_config& g = c->cfg;
   const bool collapse = g.deep_collapse && g.n_shallow < g.n_blocks;
+  // one pass from block to block instead of two where that is faster (see residual_ln_kernel)
+  const bool fuse = residual_ln_serves(g.hidden, g.dtype);
   if (is_full(g, step)) {
     if (collapse) {                          // the deep stack's branch outputs are summed into a fresh slot
       c->stack_new = c->stack_n == 0 ? 0 : (c->stack_last ^ 1);
       HERO_CUDA_TRY(cudaMemsetAsync(c->stack_hist[c->stack_new], 0, (size_t)c->elems * sizeof(float), c->stream));
     }
     HERO_TRY(modulation_for_blocks(c, 0, g.n_blocks, d_temb, false));
-    for (int l = 0; l < g.n_blocks; ++l) HERO_TRY(refresh_block(c, l, d_x, d_temb, nullptr, c->N, true));
+    bool prepared = false;
+    for (int l = 0; l < g.n_blocks; ++l) {
+      NextRefresh next;
+      if (fuse && l + 1 < g.n_blocks && !(collapse && l >= g.n_shallow)) next.n_sel = c->N;
+      HERO_TRY(refresh_block(c, l, d_x, d_temb, nullptr, c->N, true, prepared, next));
+      prepared = next.n_sel > 0;
+    }
     if (collapse) { c->stack_last = c->stack_new; if (c->stack_n < 2) c->stack_n++; }
     c->s_prev = c->s_last; c->s_last = step; c->n_full++;
     return HERO_OK;
@@ -705,17 +730,23 @@ static int step_impl(hero_ctx* c, int step, void* d_x, const void* d_temb, void*
       batch.block[l] = l; batch.call[l] = bm.calls;
       batch.ages_in[l] = bm.ages[bm.ages_cur]; batch.ages_out[l] = bm.ages[bm.ages_cur ^ 1];
       batch.idx[l] = c->idx_ws + (size_t)l * c->idx_cap;
+      batch.pos[l] = c->pos_ws + (size_t)l * c->idx_cap;
     }
     HERO_LAUNCH(c, HERO_PROF_SELECT, launch_select(geom_of(g), batch, c->stream));
     for (int l = 0; l < n_draws; ++l) { c->blk[l].ages_cur ^= 1; c->blk[l].calls++; }
     for (int l = n_draws; l < g.n_shallow; ++l) n_sel[l] = n_sel[0];
   }
   HERO_TRY(modulation_for_blocks(c, 0, g.n_shallow, d_temb, true));
+  bool prepared = false;                     // the next refreshed block's rows are in ws_a
   for (int l = 0; l < g.n_blocks; ++l) {
     if (l < g.n_shallow) {
       if (n_sel[l] > 0) {
+        NextRefresh next;
+        if (fuse && l + 1 < g.n_shallow && n_sel[l + 1] > 0)
+          next = {n_sel[l + 1], c->pos_ws + (size_t)(g.share_selection ? 0 : l + 1) * c->idx_cap};
         HERO_TRY(refresh_block(c, l, d_x, d_temb, c->idx_ws + (size_t)(g.share_selection ? 0 : l) * c->idx_cap, n_sel[l],
-                               true));
+                               true, prepared, next));
+        prepared = next.n_sel > 0;
       } else {
         HERO_LAUNCH(c, HERO_PROF_RESIDUAL,
                     launch_residual2(d_x, c->blk[l].g[0], c->blk[l].g[1], c->elems, g.dtype, c->stream));

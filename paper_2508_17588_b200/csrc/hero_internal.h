@@ -149,6 +149,7 @@ struct SelectBatch {
   const uint16_t* ages_in[kMaxSelectBatch];
   uint16_t* ages_out[kMaxSelectBatch];
   int* idx[kMaxSelectBatch];
+  int* pos[kMaxSelectBatch];              // place of every video token in its list, -1 where it is not in it
 };
 
 // ---------------------------------------------------------------------------
@@ -215,6 +216,13 @@ int launch_modulation(const void* temb, const void* w_mod, const void* b_mod, fl
 int launch_gather_ln_modulate(const void* x, const void* add, const int* idx, const float* shift,
                               const float* scale, int mod_ld, void* a, int B, int N, int n_sel, int D,
                               float eps, int dtype, cudaStream_t s);
+
+// x = (x + ga) + gf for all rows and the LayerNorm + modulate of the rows that the next
+// block refreshes (pos: as SelectBatch::pos; null: all rows) into a [B, n_sel, D].  Rows as wide as residual_ln_serves.
+bool residual_ln_serves(int D, int dtype);
+int launch_residual_ln(void* x, const void* ga, const void* gf, const int* pos, int n_text, const float* shift,
+                       const float* scale, int mod_ld, void* a, int B, int N, int n_sel, int D, float eps, int dtype,
+                       cudaStream_t s);
 
 // fp32 CUDA-core path (config 1 runs in fp32, where tensor cores would break parity)
 int launch_simt_gemm(const float* a, const float* w, const float* bias, int M, int Nout, int K, const GemmOut& out,

@@ -52,6 +52,7 @@ __global__ void __launch_bounds__(kSelWarps * 32) select_kernel(const SelectGeom
   const uint16_t* __restrict__ ages_in = batch.ages_in[e];
   uint16_t* __restrict__ ages_out = batch.ages_out[e];
   int* __restrict__ idx = batch.idx[e];
+  int* __restrict__ pos = batch.pos[e];
   const int call = batch.call[e];
   const uint32_t h_block = mix32(mix32(g.seed_lo ^ (uint32_t)batch.block[e]) + (uint32_t)call);
   const long long off = (long long)call * ph * pw, ra = g.ratio_num, rb = g.ratio_den;
@@ -101,7 +102,9 @@ __global__ void __launch_bounds__(kSelWarps * 32) select_kernel(const SelectGeom
     }
     const unsigned ballot = __ballot_sync(0xFFFFFFFFu, pick);
     if (i < n_band) {
-      if (pick) idx[start + __popc(ballot & ((1u << lane) - 1u))] = g.n_text + v;
+      const int place = start + __popc(ballot & ((1u << lane) - 1u));
+      if (pick) idx[place] = g.n_text + v;
+      if (pos) pos[v] = pick ? place : -1;
       ages_out[v] = pick ? (uint16_t)0 : (uint16_t)min(age_v + 1u, 65535u);
     }
     start += __popc(ballot);

@@ -580,6 +580,64 @@ __host__ __device__ constexpr int ln_full_chunks(int vpl) {
 __host__ __device__ constexpr int ln_ctas_per_sm(int vpl) {      // what the registers of a row allow
   return vpl <= 2 ? 6 : (vpl <= 4 ? 4 : (vpl <= 6 ? 3 : (vpl <= 12 ? 2 : 1)));
 }
+// One batch item's (1 + scale) and shift into shared memory: [2 * Q][packets] float4.
+template <typename T>
+__device__ __forceinline__ void ln_stage_modulation(float4* s_mod, const float* __restrict__ scale, const float* __restrict__ shift,
+                                                    int packets) {
+  constexpr int Q = Vec<T>::N / 4;                  // float4s of modulation per packet and vector
+  const float4* sc = reinterpret_cast<const float4*>(scale);
+  const float4* sh = reinterpret_cast<const float4*>(shift);
+  for (int i = threadIdx.x; i < Q * packets; i += 256) {         // float4 i covers columns [4i, 4i + 4)
+    const float4 s4 = __ldg(sc + i), h4 = __ldg(sh + i);
+    s_mod[(i % Q) * packets + i / Q] = make_float4(1.0f + s4.x, 1.0f + s4.y, 1.0f + s4.z, 1.0f + s4.w);
+    s_mod[(Q + i % Q) * packets + i / Q] = h4;
+  }
+  __syncthreads();
+}
+// Statistics of a row held by a warp (absent packets are zeros), normalised, modulated and written to `out`.
+template <typename T, int VPL, int FULL>
+__device__ __forceinline__ void ln_finish_row(const float (&f)[VPL][Vec<T>::N], const float4* s_mod, int packets, int D, float eps,
+                                              int lane, T* out_row) {
+  using V = Vec<T>;
+  constexpr int Q = V::N / 4;
+  float sum = 0.f;
+#pragma unroll
+  for (int c = 0; c < VPL; ++c)
+#pragma unroll
+    for (int q = 0; q < V::N; ++q) sum += f[c][q];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+  const float mean = sum / (float)D;
+  float sq = 0.f;
+#pragma unroll
+  for (int c = 0; c < VPL; ++c)
+    if (c < FULL || c * 32 + lane < packets) {
+#pragma unroll
+      for (int q = 0; q < V::N; ++q) { const float d = f[c][q] - mean; sq = fmaf(d, d, sq); }
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, o);
+  const float rstd = 1.0f / sqrtf(sq / (float)D + eps);
+  V* out = reinterpret_cast<V*>(out_row);
+#pragma unroll
+  for (int c = 0; c < VPL; ++c) {
+    const int v = c * 32 + lane;         // packet index: columns [V::N * v, V::N * (v + 1))
+    if (c < FULL || v < packets) {
+      float r[V::N];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const float4 s4 = s_mod[q * packets + v], h4 = s_mod[(Q + q) * packets + v];
+        r[4 * q] = fmaf((f[c][4 * q] - mean) * rstd, s4.x, h4.x);
+        r[4 * q + 1] = fmaf((f[c][4 * q + 1] - mean) * rstd, s4.y, h4.y);
+        r[4 * q + 2] = fmaf((f[c][4 * q + 2] - mean) * rstd, s4.z, h4.z);
+        r[4 * q + 3] = fmaf((f[c][4 * q + 3] - mean) * rstd, s4.w, h4.w);
+      }
+      V o; o.pack(r);
+      __stcs(&out[v].raw, o.raw);
+    }
+  }
+}
+
 // (EXACT: the row has exactly 32 * VPL packets, nothing is predicated; the wide rows have no registers to spare for it.)
 template <typename T, int VPL, bool EXACT>
 __global__ void __launch_bounds__(256, ln_ctas_per_sm(VPL))
@@ -588,21 +646,13 @@ gather_ln_modulate_warp_kernel(const T* __restrict__ x, const T* __restrict__ ad
                                T* __restrict__ a, int N, int n_sel, int B, int D, float eps) {
   stream_order();
   using V = Vec<T>;
-  constexpr int Q = V::N / 4;                       // float4s of modulation per packet and vector
   constexpr int kFull = EXACT ? VPL : ln_full_chunks(VPL);    // chunks of 32 packets that every row it serves has
   const int packets = EXACT ? VPL * 32 : D / V::N;
   if (EXACT) D = VPL * 32 * V::N;
-  extern __shared__ float4 s_mod[];                 // [2 * Q][packets]
+  extern __shared__ float4 s_mod[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = blockIdx.x % B, slot = blockIdx.x / B, slots = gridDim.x / B;
-  const float4* sc = reinterpret_cast<const float4*>(scale + (long long)b * mod_ld);
-  const float4* sh = reinterpret_cast<const float4*>(shift + (long long)b * mod_ld);
-  for (int i = threadIdx.x; i < Q * packets; i += 256) {         // float4 i covers columns [4i, 4i + 4)
-    const float4 s4 = __ldg(sc + i), h4 = __ldg(sh + i);
-    s_mod[(i % Q) * packets + i / Q] = make_float4(1.0f + s4.x, 1.0f + s4.y, 1.0f + s4.z, 1.0f + s4.w);
-    s_mod[(Q + i % Q) * packets + i / Q] = h4;
-  }
-  __syncthreads();
+  ln_stage_modulation<T>(s_mod, scale + (long long)b * mod_ld, shift + (long long)b * mod_ld, packets);
   for (int i = slot * 8 + warp; i < n_sel; i += slots * 8) {
     const long long row = (long long)b * N + (idx ? __ldg(idx + i) : i);
     const V* xr = reinterpret_cast<const V*>(x + row * D);
@@ -635,43 +685,80 @@ gather_ln_modulate_warp_kernel(const T* __restrict__ x, const T* __restrict__ ad
         }
       }
     }
-    float sum = 0.f;
-#pragma unroll
-    for (int c = 0; c < VPL; ++c)
-#pragma unroll
-      for (int q = 0; q < V::N; ++q) sum += f[c][q];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-    const float mean = sum / (float)D;
-    float sq = 0.f;
+    ln_finish_row<T, VPL, kFull>(f, s_mod, packets, D, eps, lane, a + ((long long)b * n_sel + i) * D);
+  }
+}
+
+// The end of one refreshed block and the start of the next in one pass: x = (x + ga) + gf for every row, and the rows that
+// the next block refreshes, as stored, normalised and modulated into their places in its compact input.  pos gives a video
+// row's place (-1: not refreshed; null: every row of x, in order).  Against the two passes one after the other it saves a
+// launch and the second reading of x: in a whole step of 42 blocks of 614 rows x 256 1.3 us a block (2.92 -> 2.80 ms), of
+// 8 blocks of 5820 x 1024 0.8, of 4 blocks of 1562 x 768 1.1.  A collapsed deep stack's blocks, which add a fp32 sum to the
+// streams of a row, keep the two passes (16 blocks of 5254 x 1152: 4.46 ms apart, 4.47 in one).
+constexpr int rln_ctas_per_sm(int vpl) { return vpl <= 3 ? 3 : 2; }      // what the registers of three rows allow
+template <typename T, int VPL>
+__global__ void __launch_bounds__(256, rln_ctas_per_sm(VPL))
+residual_ln_kernel(T* __restrict__ x, const T* __restrict__ ga, const T* __restrict__ gf,
+                   const int* __restrict__ pos, int n_text, const float* __restrict__ shift, const float* __restrict__ scale,
+                   int mod_ld, T* __restrict__ a, int N, int n_sel, int B, int D, float eps) {
+  stream_order();
+  using V = Vec<T>;
+  constexpr int kFull = ln_full_chunks(VPL);
+  const int packets = D / V::N;
+  extern __shared__ float4 s_mod[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b = blockIdx.x % B, slot = blockIdx.x / B, slots = gridDim.x / B;
+  ln_stage_modulation<T>(s_mod, scale + (long long)b * mod_ld, shift + (long long)b * mod_ld, packets);
+  for (int i = slot * 8 + warp; i < N; i += slots * 8) {
+    const int place = pos == nullptr ? i : (i < n_text ? -1 : __ldg(pos + i - n_text));
+    const long long first = ((long long)b * N + i) * D;
+    V* xr = reinterpret_cast<V*>(x + first);
+    const V* ar = reinterpret_cast<const V*>(ga + first);
+    const V* fr = reinterpret_cast<const V*>(gf + first);
+    V vx[VPL], va[VPL], vf[VPL];
 #pragma unroll
     for (int c = 0; c < VPL; ++c)
       if (c < kFull || c * 32 + lane < packets) {
-#pragma unroll
-        for (int q = 0; q < V::N; ++q) { const float d = f[c][q] - mean; sq = fmaf(d, d, sq); }
+        vx[c] = ld_stream(xr + c * 32 + lane); va[c] = ld_stream(ar + c * 32 + lane); vf[c] = ld_stream(fr + c * 32 + lane);
       }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, o);
-    const float rstd = 1.0f / sqrtf(sq / (float)D + eps);
-    V* out = reinterpret_cast<V*>(a + ((long long)b * n_sel + i) * D);
+    float f[VPL][V::N];
 #pragma unroll
     for (int c = 0; c < VPL; ++c) {
-      const int v = c * 32 + lane;       // packet index: columns [V::N * v, V::N * (v + 1))
-      if (c < kFull || v < packets) {
-        float r[V::N];
+      if (c < kFull || c * 32 + lane < packets) {
+        float fa[V::N], ff[V::N];
+        vx[c].unpack(f[c]); va[c].unpack(fa); vf[c].unpack(ff);
 #pragma unroll
-        for (int q = 0; q < Q; ++q) {
-          const float4 s4 = s_mod[q * packets + v], h4 = s_mod[(Q + q) * packets + v];
-          r[4 * q] = fmaf((f[c][4 * q] - mean) * rstd, s4.x, h4.x);
-          r[4 * q + 1] = fmaf((f[c][4 * q + 1] - mean) * rstd, s4.y, h4.y);
-          r[4 * q + 2] = fmaf((f[c][4 * q + 2] - mean) * rstd, s4.z, h4.z);
-          r[4 * q + 3] = fmaf((f[c][4 * q + 3] - mean) * rstd, s4.w, h4.w);
-        }
-        V o; o.pack(r);
-        __stcs(&out[v].raw, o.raw);
+        for (int q = 0; q < V::N; ++q) f[c][q] = (f[c][q] + fa[q]) + ff[q];
+        V r; r.pack(f[c]);
+        st_stream(xr + c * 32 + lane, r);
+        r.unpack(f[c]);                    // (the next block sees x as it is stored)
+      } else {
+#pragma unroll
+        for (int q = 0; q < V::N; ++q) f[c][q] = 0.f;
       }
     }
+    if (place >= 0) ln_finish_row<T, VPL, kFull>(f, s_mod, packets, D, eps, lane, a + ((long long)b * n_sel + place) * D);
   }
+}
+
+template <typename T, int VPL>
+int residual_ln_launch(void* x, const void* ga, const void* gf, const int* pos, int n_text, const float* shift,
+                       const float* scale, int mod_ld, void* a, int N, int n_sel, int B, int D, float eps, cudaStream_t s) {
+  const int resident = (num_sms() * rln_ctas_per_sm(VPL) + B - 1) / B, need = (N + 7) / 8;
+  return launch_kernel(residual_ln_kernel<T, VPL>, (unsigned)((need < resident ? need : resident) * B), 256,
+                       (size_t)2 * D * sizeof(float), s, 1, (T*)x, (const T*)ga, (const T*)gf, pos, n_text, shift, scale,
+                       mod_ld, (T*)a, N, n_sel, B, D, eps);
+}
+constexpr int kResidualLnPackets = 6;        // a lane's packets of three tensors stay in registers up to here
+template <typename T>
+int residual_ln_dispatch(void* x, const void* ga, const void* gf, const int* pos, int n_text, const float* shift,
+                         const float* scale, int mod_ld, void* a, int N, int n_sel, int B, int D, float eps, cudaStream_t s) {
+  const int vpl = (D / Vec<T>::N + 31) / 32;
+#define HERO_RLN(V) \
+  if (vpl <= V) return residual_ln_launch<T, V>(x, ga, gf, pos, n_text, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s)
+  HERO_RLN(1); HERO_RLN(2); HERO_RLN(3); HERO_RLN(4); HERO_RLN(5); HERO_RLN(6);
+#undef HERO_RLN
+  return HERO_ERR_ARG;
 }
 
 template <typename T, int VPL>
@@ -899,6 +986,16 @@ int launch_modulation(const void* temb, const void* w_mod, const void* b_mod, fl
   }
 }
 #undef HERO_MOD_DISPATCH
+
+bool residual_ln_serves(int D, int dtype) { return D / (dtype == HERO_DTYPE_BF16 ? 8 : 4) <= 32 * kResidualLnPackets; }
+
+int launch_residual_ln(void* x, const void* ga, const void* gf, const int* pos, int n_text, const float* shift,
+                       const float* scale, int mod_ld, void* a, int B, int N, int n_sel, int D, float eps, int dtype,
+                       cudaStream_t s) {
+  return dtype == HERO_DTYPE_BF16
+             ? residual_ln_dispatch<__nv_bfloat16>(x, ga, gf, pos, n_text, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s)
+             : residual_ln_dispatch<float>(x, ga, gf, pos, n_text, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s);
+}
 
 int launch_gather_ln_modulate(const void* x, const void* add, const int* idx, const float* shift,
                               const float* scale, int mod_ld, void* a, int B, int N, int n_sel, int D, float eps,

@@ -145,3 +145,32 @@ def test_attention_modes(B, frames, grid_h, grid_w, n_text, heads, ratio_den, ke
         assert float(err.max()) <= 2.0 ** -6, (cached, int(err.argmax()))
         assert float((got[:, rows].double() - want).norm() / want.norm()) <= 2.0 ** -7
     hero.close()
+
+
+@pytest.mark.parametrize("dtype,over", [
+    # the pass from block to block: one packet a lane and less, several with the last one partly there, the widest it serves
+    # and one beyond; lists of different length from block to block, one list for all, empty lists, a collapsed deep stack
+    ("fp32", dict(hidden=64, head_dim=32, n_heads=2, ffn_dim=64, batch=3, n_text=3)),
+    ("fp32", dict(hidden=768, head_dim=64, n_heads=12, ffn_dim=64, ratio_num=1, ratio_den=3, share_selection=1)),
+    ("fp32", dict(hidden=832, head_dim=64, n_heads=13, ffn_dim=64)),
+    ("bf16", dict(hidden=64, head_dim=64, n_heads=1, ffn_dim=64, n_text=0, ratio_num=1, ratio_den=90)),
+    ("bf16", dict(hidden=448, head_dim=64, n_heads=7, ffn_dim=64, deep_collapse=1)),
+    ("bf16", dict(hidden=1536, head_dim=64, n_heads=24, ffn_dim=64, batch=1)),
+    ("bf16", dict(hidden=1600, head_dim=64, n_heads=25, ffn_dim=64, batch=1))],
+    ids=["fp32_64", "fp32_768_shared", "fp32_832", "bf16_64_sparse", "bf16_448_collapse", "bf16_1536", "bf16_1600"])
+def test_pass_from_block_to_block(dtype, over):
+    cfgd = dict(S.CONFIGS["tiny"], n_blocks=5, n_shallow=3, frames=1, grid_h=9, grid_w=7, seed=43, temb_dim=64, dtype=dtype,
+                full_interval=3, **{**dict(batch=2), **over})
+    orc, hero, _ = make_pair(cfgd)
+    x_host = S.tokens(cfgd)
+    for s in range(7):                                     # full, full, two cached, full, two cached
+        temb = S.temb(cfgd, s)
+        want = orc.step(s, x_host, temb)
+        x = to_dev(x_host, dtype)
+        hero.hero_step(s, x, to_dev(temb, dtype))
+        # fp32 as above; bf16: x is rounded once per block (independent errors of 2^-9 of x at most, whatever the size of the
+        # update), on top of the blocks' own tolerance of 2e-2 of the update
+        update = np.linalg.norm(want - x_host)
+        bound = FP32_TOL * update if dtype == "fp32" else 5 ** 0.5 * 2.0 ** -9 * np.linalg.norm(want) + 2e-2 * update
+        assert np.linalg.norm(to_host(x) - want) <= bound, s
+    hero.close()
