@@ -48,6 +48,7 @@ struct hero_ctx {
   long long elems = 0;                   // B*N*D
   std::vector<hero_block_weights> w;
   std::vector<BlockMem> blk;
+  uint16_t* ages[2] = {nullptr, nullptr};   // [n_shallow, n_video] each, see BlockMem::ages
   void* kv_tmp[2] = {nullptr, nullptr};  // K/V of deep blocks during full passes (never cached)
   // deep-stack collapse: branch outputs of a deep block are transient, their fp32 sum over the stack is kept
   void* deep_g[2] = {nullptr, nullptr};
@@ -347,7 +348,8 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
       if (bm.n_hist < 2) bm.n_hist++;
     } else {
       bm.filled = kAllCaches;
-      HERO_CUDA_TRY(cudaMemsetAsync(bm.ages[bm.ages_cur], 0, (size_t)c->n_video * sizeof(uint16_t), c->stream));
+      if (!in_step)                            // (hero_step has cleared all blocks' counters)
+        HERO_CUDA_TRY(cudaMemsetAsync(bm.ages[bm.ages_cur], 0, (size_t)c->n_video * sizeof(uint16_t), c->stream));
     }
   }
   return HERO_OK;
@@ -501,10 +503,14 @@ int hero_init(hero_ctx** out, const hero_config* cfg, const hero_block_weights* 
     BlockMem& bm = c->blk[l];
     if (l < cfg->n_shallow) {
       A(&bm.k, tensor); A(&bm.v, tensor); A(&bm.g[0], tensor); A(&bm.g[1], tensor);
-      A((void**)&bm.ages[0], (size_t)c->n_video * 2); A((void**)&bm.ages[1], (size_t)c->n_video * 2);
     } else if (!cfg->deep_collapse) {
       for (int br = 0; br < 2; ++br) for (int s = 0; s < 2; ++s) A(&bm.hist[br][s], tensor);
     }
+  }
+  // the age counters of all blocks lie side by side, so that a full step clears them in one go
+  for (int k = 0; k < 2 && cfg->n_shallow > 0; ++k) {
+    A((void**)&c->ages[k], (size_t)cfg->n_shallow * c->n_video * sizeof(uint16_t));
+    for (int l = 0; l < cfg->n_shallow; ++l) c->blk[l].ages[k] = c->ages[k] + (size_t)l * c->n_video;
   }
   if (cfg->deep_collapse && cfg->n_shallow < cfg->n_blocks) {
     A(&c->deep_g[0], tensor); A(&c->deep_g[1], tensor);
@@ -700,6 +706,10 @@ static int step_impl(hero_ctx* c, int step, void* d_x, const void* d_temb, void*
     if (collapse) {                          // the deep stack's branch outputs are summed into a fresh slot
       c->stack_new = c->stack_n == 0 ? 0 : (c->stack_last ^ 1);
       HERO_CUDA_TRY(cudaMemsetAsync(c->stack_hist[c->stack_new], 0, (size_t)c->elems * sizeof(float), c->stream));
+    }
+    if (g.n_shallow > 0) {
+      HERO_CUDA_TRY(cudaMemsetAsync(c->ages[0], 0, (size_t)g.n_shallow * c->n_video * sizeof(uint16_t), c->stream));
+      for (int l = 0; l < g.n_shallow; ++l) c->blk[l].ages_cur = 0;
     }
     HERO_TRY(modulation_for_blocks(c, 0, g.n_blocks, d_temb, false));
     bool prepared = false;
