@@ -164,11 +164,12 @@ bool is_full(const hero_config& g, int step) {
   return g.full_interval > 0 && (step - (g.warmup_full_steps - 1)) % g.full_interval == 0;
 }
 
-int run_gemm(hero_ctx* c, const void* a, const void* w, const void* bias, int M, int Nout, int K, const GemmOut& out) {
+int run_gemm(hero_ctx* c, const void* a, const void* w, const void* bias, int M, int Nout, int K, const GemmOut& out,
+             const QkEpilogue* qk = nullptr) {
   LaunchScope scope(c, HERO_PROF_GEMM);
   GemmOut o = out;
   o.weights_settled = 1;               // (behind a kernel of this context, which waited for whatever wrote the weights)
-  if (c->cfg.dtype == HERO_DTYPE_BF16) return launch_tc_gemm(a, w, bias, M, Nout, K, o, c->d_status, c->stream);
+  if (c->cfg.dtype == HERO_DTYPE_BF16) return launch_tc_gemm(a, w, bias, M, Nout, K, o, qk, c->d_status, c->stream);
   return launch_simt_gemm((const float*)a, (const float*)w, (const float*)bias, M, Nout, K, out, c->stream);
 }
 
@@ -269,23 +270,26 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
   o_qkv.ptr[1] = kdst;    o_qkv.ld[1] = D; o_qkv.scatter[1] = 1;
   o_qkv.ptr[2] = vdst;    o_qkv.ld[2] = D; o_qkv.scatter[2] = 1;
   o_qkv.seg_cols = D; o_qkv.idx = d_idx; o_qkv.n_sel = n_sel; o_qkv.n_rows = N;
-  // The tensor-core attention takes q with the softmax scale folded in (a score is then the exponent of its
-  // weight): by the projection's epilogue, or by the q/k treatment below when that runs and has the last word on q.
-  const bool fold_scale = g.dtype == HERO_DTYPE_BF16;
-  const bool qk_treated = g.qk_norm || g.rope;
-  if (fold_scale && !qk_treated) o_qkv.seg0_scale = kScoreScaleLog2;
-  HERO_TRY(run_gemm(c, c->ws_a, w.w_qkv, w.b_qkv, M, 3 * D, D, o_qkv));
-  if (qk_treated) {
+  // The tensor-core attention takes q with the softmax scale folded in (a score is then the exponent of its weight), by the
+  // projection's epilogue, which in bf16 is also where q and k get their LayerNorm and turn.
+  const bool bf16 = g.dtype == HERO_DTYPE_BF16, qk_treated = g.qk_norm || g.rope;
+  if (bf16 && !qk_treated) o_qkv.seg0_scale = kScoreScaleLog2;
+  QkEpilogue qk = {};
+  if (g.qk_norm) { qk.qn_w = w.qn_w; qk.qn_b = w.qn_b; qk.kn_w = w.kn_w; qk.kn_b = w.kn_b; }
+  qk.rope = g.rope ? c->rope_tab : nullptr;
+  qk.n_text = g.n_text; qk.frames = g.frames; qk.grid_h = g.grid_h; qk.grid_w = g.grid_w;
+  qk.eps = 1e-6f; qk.q_scale = kScoreScaleLog2;
+  HERO_TRY(run_gemm(c, c->ws_a, w.w_qkv, w.b_qkv, M, 3 * D, D, o_qkv, bf16 && qk_treated ? &qk : nullptr));
+  if (!bf16 && qk_treated) {
     QkPrepArgs qa = {};
-    if (fold_scale) qa.q_scale = kScoreScaleLog2;
     qa.q = c->ws_q; qa.k = kdst; qa.idx = d_idx;
-    if (g.qk_norm) { qa.qn_w = w.qn_w; qa.qn_b = w.qn_b; qa.kn_w = w.kn_w; qa.kn_b = w.kn_b; }
-    qa.rope = g.rope ? c->rope_tab : nullptr;
+    qa.qn_w = qk.qn_w; qa.qn_b = qk.qn_b; qa.kn_w = qk.kn_w; qa.kn_b = qk.kn_b;
+    qa.rope = qk.rope;
     qa.B = B; qa.N = N; qa.n_sel = n_sel; qa.D = D; qa.n_heads = g.n_heads; qa.head_dim = g.head_dim;
     qa.n_text = g.n_text; qa.frames = g.frames; qa.grid_h = g.grid_h; qa.grid_w = g.grid_w;
     qa.p_t = c->rope_pairs[0]; qa.p_h = c->rope_pairs[1]; qa.p_w = c->rope_pairs[2];
-    qa.eps = 1e-6f;
-    HERO_LAUNCH(c, HERO_PROF_GATHER_LN, launch_qk_prep(qa, g.dtype, c->stream));
+    qa.eps = qk.eps;
+    HERO_LAUNCH(c, HERO_PROF_GATHER_LN, launch_qk_prep(qa, c->stream));
   }
   if (g.attend_mode == 1 && !full) {
     // Eq. 3 read literally: the refreshed queries see the refreshed rows (just written) and the text rows
@@ -919,7 +923,7 @@ int hero_gemm_bf16(const void* a, const void* w, const void* bias, void* cmat, i
   GemmOut o = {};
   o.ptr[0] = cmat; o.ld[0] = N; o.scatter[0] = 0;
   o.seg_cols = (N + 31) / 32 * 32; o.n_sel = M; o.n_rows = M; o.act = act;
-  return launch_tc_gemm(a, w, bias, M, N, K, o, st, (cudaStream_t)stream);
+  return launch_tc_gemm(a, w, bias, M, N, K, o, nullptr, st, (cudaStream_t)stream);
 }
 
 int hero_attention_bf16(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N, int heads,

@@ -178,20 +178,27 @@ int launch_residual2(void* x, const void* ga, const void* gf, long long n, int d
 int launch_residual2_acc(void* x, const void* ga, const void* gf, float* acc, long long n, int dtype, cudaStream_t s);
 int launch_extrapolate_stack(void* x, const float* s_prev, const float* s_last, long long n, int k, int d, int dtype,
                              cudaStream_t s);
-// Per-head LayerNorm and rotary embedding of fresh q (compact) and k (in the cache) rows.
+// Per-head LayerNorm and rotary embedding of bf16 q and k rows (head_dim 64), by the QKV projection's epilogue, before the
+// rows are rounded and stored.
+struct QkEpilogue {
+  const void *qn_w, *qn_b, *kn_w, *kn_b;   // [64] bf16, or all null
+  const float2* rope;                      // (cos, sin) per (axis position, pair) or null
+  int n_text, frames, grid_h, grid_w;
+  float eps, q_scale;
+};
+// The same for fp32 rows, as a pass of its own over fresh q (compact) and k (in the cache) rows.
 struct QkPrepArgs {
   void* q;                 // [B, n_sel, D]
   void* k;                 // [B, N, D], rows idx[i] (or i when idx is null)
   const int* idx;
-  const void *qn_w, *qn_b, *kn_w, *kn_b;   // [head_dim] in the run dtype, or all null
+  const void *qn_w, *qn_b, *kn_w, *kn_b;   // [head_dim], or all null
   const float2* rope;      // (cos, sin) per (axis position, pair) or null
   int B, N, n_sel, D, n_heads, head_dim;
   int n_text, frames, grid_h, grid_w;
   int p_t, p_h, p_w;       // rotary pairs per axis
   float eps;
-  float q_scale;           // when not 0: factor on the finished q rows (the softmax scale, folded in here)
 };
-int launch_qk_prep(const QkPrepArgs& a, int dtype, cudaStream_t s);
+int launch_qk_prep(const QkPrepArgs& a, cudaStream_t s);
 // list[i] = i for i < n_text, list[n_text + i] = idx[i] for i < n_sel (rows a literal Eq. 3 attends to)
 int launch_attend_list(const int* idx, int n_sel, int n_text, int* list, cudaStream_t s);
 int launch_gather_rows(const void* src, const int* idx, void* dst, int B, int N, int n_sel, int D,
@@ -233,7 +240,7 @@ int launch_simt_attention(const float* q, const float* k, const float* v, float*
 // bf16 tensor-core path (tcgen05 + TMEM + TMA)
 int tc_init_driver_api();   // resolves cuTensorMapEncodeTiled once
 int launch_tc_gemm(const void* a, const void* w, const void* bias, int M, int Nout, int K,
-                   const GemmOut& out, int* d_status, cudaStream_t s);
+                   const GemmOut& out, const QkEpilogue* qk, int* d_status, cudaStream_t s);
 // The tensor-core attention serves head_dim 64: a score s enters the softmax as 2^(s * kScoreScaleLog2).
 constexpr float kScoreScaleLog2 = 0.125f * 1.4426950408889634f;   // 1/sqrt(64) * log2(e)
 // q_prescaled: Q holds q * kScoreScaleLog2 (the softmax scale folded into the projection)

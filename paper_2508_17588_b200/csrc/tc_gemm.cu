@@ -157,6 +157,104 @@ __device__ __forceinline__ void emit(const uint32_t (&acc)[NC], const float* s_b
   }
 }
 
+// (a kernel without this treatment has no use for the parameter)
+template <bool QK> struct QkParam {};
+template <> struct QkParam<true> : QkEpilogue {};
+
+// What the q and k columns of a row go through besides (QkEpilogue): where its angles stand in the table, worked out
+// while the MMAs run.  Pairs 0..7 of a head turn with the frame, 8..19 with the grid row, 20..31 with the grid column.
+struct RowAngles { int t, h, w; };           // entry of the axis' first pair; t < 0: the row is not turned
+constexpr int kPairsT = 8, kPairsH = 12;
+__device__ __forceinline__ RowAngles row_angles(const QkEpilogue& qk, const RowOut& row, int n_rows) {
+  RowAngles a = {-1, 0, 0};
+  const int token = (int)(row.scat - (long long)row.b * n_rows) - qk.n_text;
+  if (row.ok && qk.rope != nullptr && token >= 0) {
+    const int per_frame = qk.grid_h * qk.grid_w;
+    const int ft = token / per_frame, in_frame = token - ft * per_frame;
+    const int gh = in_frame / qk.grid_w, gw = in_frame - gh * qk.grid_w;
+    a.t = ft * kPairsT;
+    a.h = qk.frames * kPairsT + gh * kPairsH;
+    a.w = qk.frames * kPairsT + qk.grid_h * kPairsH + gw * kPairsH;
+  }
+  return a;
+}
+// Finish one head (64 columns from n0 on) of one row of the QKV projection: bias, for q and k the LayerNorm over the
+// head's features and the turn by the row's position, for q the softmax scale; bf16; stored as in emit.  The row never
+// leaves the thread's registers between the projection and its final form: a pass of its own over q and the fresh rows of
+// the K cache read and wrote them once more (77 us in a block of 5940 rows x 3072: that cached step of 6 blocks 10.08 ->
+// 9.84 ms; of 4 blocks of 371 x 768 228 -> 222 us).
+__device__ __forceinline__ void emit_head(const uint32_t (&acc)[2][32], const float* s_bias, int n0, const GemmOut& out,
+                                          const RowOut& row, const QkEpilogue& qk, const RowAngles& ang) {
+  float2 f[32];
+#pragma unroll
+  for (int v = 0; v < 16; ++v) {
+    const float4 b4 = *reinterpret_cast<const float4*>(s_bias + v * 4);
+    const uint32_t* a = &acc[v / 8][(v % 8) * 4];
+    f[2 * v] = __fadd2_rn(make_float2(__uint_as_float(a[0]), __uint_as_float(a[1])), make_float2(b4.x, b4.y));
+    f[2 * v + 1] = __fadd2_rn(make_float2(__uint_as_float(a[2]), __uint_as_float(a[3])), make_float2(b4.z, b4.w));
+  }
+  const int seg = n0 >= 2 * out.seg_cols ? 2 : (n0 >= out.seg_cols ? 1 : 0);            // warp-uniform
+  if (seg < 2 && qk.qn_w != nullptr) {
+    float2 s2 = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) s2 = __fadd2_rn(s2, f[i]);
+    const float mu = (s2.x + s2.y) * (1.0f / 64.0f);
+    float2 q2 = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+      f[i] = __fadd2_rn(f[i], make_float2(-mu, -mu));
+      q2 = __ffma2_rn(f[i], f[i], q2);
+    }
+    const float rstd = rsqrtf((q2.x + q2.y) * (1.0f / 64.0f) + qk.eps);
+    const uint4* gw = static_cast<const uint4*>(seg ? qk.kn_w : qk.qn_w);
+    const uint4* gb = static_cast<const uint4*>(seg ? qk.kn_b : qk.qn_b);
+#pragma unroll
+    for (int v = 0; v < 8; ++v) {
+      const uint4 w4 = __ldg(gw + v), b4 = __ldg(gb + v);
+      const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        f[4 * v + q] = __ffma2_rn(__fmul2_rn(f[4 * v + q], make_float2(rstd, rstd)),
+                                  make_float2(__uint_as_float(w[q] << 16), __uint_as_float(w[q] & 0xFFFF0000u)),
+                                  make_float2(__uint_as_float(b[q] << 16), __uint_as_float(b[q] & 0xFFFF0000u)));
+    }
+  }
+  if (seg < 2 && ang.t >= 0) {
+#pragma unroll
+    for (int i = 0; i < 32; i += 2) {
+      const int entry = i < kPairsT ? ang.t + i : (i < kPairsT + kPairsH ? ang.h + i - kPairsT : ang.w + i - kPairsT - kPairsH);
+      const float4 cs = __ldg(reinterpret_cast<const float4*>(qk.rope + entry));         // two (cos, sin)
+      const float2 x = f[i], y = f[i + 1];
+      f[i] = make_float2(x.x * cs.x - x.y * cs.y, x.x * cs.y + x.y * cs.x);
+      f[i + 1] = make_float2(y.x * cs.z - y.y * cs.w, y.x * cs.w + y.y * cs.z);
+    }
+  }
+  if (seg == 0) {
+#pragma unroll
+    for (int i = 0; i < 32; ++i) f[i] = __fmul2_rn(f[i], make_float2(qk.q_scale, qk.q_scale));
+  }
+  if (!row.ok) return;
+  void* const base = seg == 2 ? out.ptr[2] : (seg == 1 ? out.ptr[1] : out.ptr[0]);
+  const long long ld = seg == 2 ? out.ld[2] : (seg == 1 ? out.ld[1] : out.ld[0]);
+  const int scatter = seg == 2 ? out.scatter[2] : (seg == 1 ? out.scatter[1] : out.scatter[0]);
+  __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(base) + (scatter ? row.scat : (long long)row.m) * ld + n0 - seg * out.seg_cols;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    uint32_t packed[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const __nv_bfloat162 p = __floats2bfloat162_rn(f[8 * v + i].x, f[8 * v + i].y);
+      packed[i] = *reinterpret_cast<const uint32_t*>(&p);
+    }
+    if ((reinterpret_cast<uintptr_t>(dst) & 31) == 0) {
+      st_global_v8(dst + v * 16, packed);
+    } else {
+      *reinterpret_cast<uint4*>(dst + v * 16) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+      *reinterpret_cast<uint4*>(dst + v * 16 + 8) = make_uint4(packed[4], packed[5], packed[6], packed[7]);
+    }
+  }
+}
+
 // A warp puts NC bias values from column n_base on into its own piece of shared memory, in fp32 (values past the end
 // of the row are not read by anybody).
 template <int NC>
@@ -214,11 +312,12 @@ __device__ __forceinline__ void tile_coords(int tile, int m_tiles, int n_tiles, 
   nt = r / rows;
 }
 
-template <int BN>
+template <int BN, bool QK>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
-                    const __nv_bfloat16* __restrict__ bias, const GemmOut out, int M, int Nout, int K,
+                    const __nv_bfloat16* __restrict__ bias, const GemmOut out, const QkParam<QK> qk, int M, int Nout, int K,
                     int* __restrict__ status) {
+  static_assert(!QK || BN % 128 == 0, "an epilogue warp's columns are whole heads");
   using Cfg = PairCfg<BN>;
   constexpr int kStages = Cfg::kStages;
   extern __shared__ uint8_t smem_raw[];
@@ -354,20 +453,33 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
       const float* s_bias = s_bias_warp + acc * (BN / 2);
       stage_bias<BN / 2>(s_bias_warp + acc * (BN / 2), bias, n_first, Nout, lane);
       const RowOut row = row_out(out, (2 * mt + (int)rank) * kBM + quad * 32 + lane, M);
+      RowAngles ang = {};
+      if constexpr (QK) ang = row_angles(qk, row, out.n_rows);
       ok = mbar_wait_warp(&acc_full[acc], (t >> 1) & 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
       const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN + half * (BN / 2));
-      constexpr int kCh = BN % 64 == 0 ? 32 : 16;      // columns per TMEM read: a divisor of the half tile, and of
-      constexpr int kChunks = BN / 2 / kCh;            // its offset, so that no read straddles two segments
-      uint32_t r[2][kCh];
-      tmem_ld(t_row, r[0]);
+      if constexpr (QK) {
+#pragma unroll 1
+        for (int c = 0; c < BN / 2; c += 64) {
+          uint32_t r[2][32];
+          tmem_ld32(t_row + c, r[0]);
+          tmem_ld32(t_row + c + 32, r[1]);
+          tmem_ld_wait();
+          if (n_first + c < Nout) emit_head(r, s_bias + c, n_first + c, out, row, qk, ang);          // warp-uniform
+        }
+      } else {
+        constexpr int kCh = BN % 64 == 0 ? 32 : 16;      // columns per TMEM read: a divisor of the half tile, and of
+        constexpr int kChunks = BN / 2 / kCh;            // its offset, so that no read straddles two segments
+        uint32_t r[2][kCh];
+        tmem_ld(t_row, r[0]);
 #pragma unroll
-      for (int c = 0; c < kChunks; ++c) {
-        const int n0 = n_first + c * kCh;
-        tmem_ld_wait();
-        if (c + 1 < kChunks) tmem_ld(t_row + (c + 1) * kCh, r[(c + 1) & 1]);
-        if (n0 < Nout) emit<kCh>(r[c & 1], s_bias + c * kCh, n0, Nout, out, row);      // warp-uniform
+        for (int c = 0; c < kChunks; ++c) {
+          const int n0 = n_first + c * kCh;
+          tmem_ld_wait();
+          if (c + 1 < kChunks) tmem_ld(t_row + (c + 1) * kCh, r[(c + 1) & 1]);
+          if (n0 < Nout) emit<kCh>(r[c & 1], s_bias + c * kCh, n0, Nout, out, row);      // warp-uniform
+        }
       }
       tc_fence_before();
       __syncwarp();
@@ -406,11 +518,12 @@ struct SplitCfg {
   }
 };
 
-template <int BN>
+template <int BN, bool QK>
 __global__ void __launch_bounds__(kGemmThreads)
 tc_gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
-                     const __nv_bfloat16* __restrict__ bias, const GemmOut out, int M, int Nout, int K, int split,
-                     int* __restrict__ status) {
+                     const __nv_bfloat16* __restrict__ bias, const GemmOut out, const QkParam<QK> qk, int M, int Nout, int K,
+                     int split, int* __restrict__ status) {
+  static_assert(!QK || BN == 128, "an epilogue warp's columns are a whole head");
   using Cfg = SplitCfg<BN>;
   constexpr int kStages = Cfg::kStages;
   extern __shared__ uint8_t smem_raw[];
@@ -537,7 +650,15 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     __syncwarp();
     cluster_sync();                          // every wait above is bounded, so everybody gets here
   }
-  if (warp >= 2 && ok) {
+  if constexpr (QK) {                        // (split is 1: the warp's 64 columns are one head)
+    if (warp >= 2 && ok && nt * BN + c_first < Nout) {
+      uint32_t r[2][32];
+      tmem_ld32(t_row + c_first, r[0]);
+      tmem_ld32(t_row + c_first + 32, r[1]);
+      tmem_ld_wait();
+      emit_head(r, s_bias, nt * BN + c_first, out, row, qk, row_angles(qk, row, out.n_rows));
+    }
+  } else if (warp >= 2 && ok) {
     for (int c = c_first; c < c_first + width / 2; c += 16) {
       const int n0 = nt * BN + c;
       if (n0 >= Nout) break;                 // warp-uniform
@@ -606,7 +727,8 @@ namespace {
 
 struct GemmPlan { int bn; int split; };        // split 0: the pair kernel
 
-GemmPlan plan_gemm(int M, int Nout, int K) {
+// (qk: only what gives an epilogue warp whole heads)
+GemmPlan plan_gemm(int M, int Nout, int K, bool qk) {
   const int sms = num_sms();
   const long long kb = (K + kBK - 1) / kBK;
   auto ceil_div = [](long long a, long long b) { return (a + b - 1) / b; };
@@ -617,12 +739,14 @@ GemmPlan plan_gemm(int M, int Nout, int K) {
   };
   struct { int bn, step, fixed; } const pair[] = {{256, 560, 11500}, {224, 510, 10100}, {192, 500, 8000}, {128, 460, 7400}};
   for (const auto& p : pair) {
+    if (qk && p.bn % 128 != 0) continue;
     const long long tiles = ceil_div(M, 2 * kBM) * ceil_div(Nout, p.bn);
     consider(p.bn, 0, ceil_div(tiles, sms / 2) * kb * p.step + p.fixed);
   }
   for (int bn : {128, 64}) {
+    if (qk && bn != 128) continue;
     const long long tiles = ceil_div(M, kBM) * ceil_div(Nout, bn);
-    const int max_split = bn == 128 ? SplitCfg<128>::kMaxSplit : SplitCfg<64>::kMaxSplit;
+    const int max_split = qk ? 1 : bn == 128 ? SplitCfg<128>::kMaxSplit : SplitCfg<64>::kMaxSplit;
     for (int split = 1; split <= max_split && split <= kb; split *= 2) {
       const long long ctas = tiles * split;
       if (ctas > 0x7FFFFFFFll) continue;
@@ -636,45 +760,49 @@ GemmPlan plan_gemm(int M, int Nout, int K) {
   return best;
 }
 
-template <int BN>
-int launch_pair(const CUtensorMap& tm_a, const CUtensorMap& tm_w, const void* bias, const GemmOut& out, int M, int Nout,
-                int K, int* d_status, cudaStream_t s) {
+template <int BN, bool QK = false>
+int launch_pair(const CUtensorMap& tm_a, const CUtensorMap& tm_w, const void* bias, const GemmOut& out, const QkEpilogue& qk,
+                int M, int Nout, int K, int* d_status, cudaStream_t s) {
   static PerDeviceOnce attr_once;            // the opt-in is a property of the kernel ON a device
   HERO_TRY(per_device_once(attr_once, [](int) {
-    HERO_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_pair_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    HERO_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_pair_kernel<BN, QK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)PairCfg<BN>::kSmem));
     return HERO_OK;
   }));
   const int tiles = ((M + 2 * kBM - 1) / (2 * kBM)) * ((Nout + BN - 1) / BN);
   const int pairs = tiles < num_sms() / 2 ? tiles : num_sms() / 2;
-  return launch_kernel(tc_gemm_pair_kernel<BN>, (unsigned)(2 * pairs), kGemmThreads, PairCfg<BN>::kSmem, s,
-                       2, tm_a, tm_w, (const __nv_bfloat16*)bias, out, M, Nout, K, d_status);
+  QkParam<QK> param;
+  if constexpr (QK) static_cast<QkEpilogue&>(param) = qk;
+  return launch_kernel(tc_gemm_pair_kernel<BN, QK>, (unsigned)(2 * pairs), kGemmThreads, PairCfg<BN>::kSmem, s,
+                       2, tm_a, tm_w, (const __nv_bfloat16*)bias, out, param, M, Nout, K, d_status);
 }
 
-template <int BN>
-int launch_split(const CUtensorMap& tm_a, const CUtensorMap& tm_w, const void* bias, const GemmOut& out, int M, int Nout,
-                 int K, int split, int* d_status, cudaStream_t s) {
+template <int BN, bool QK = false>
+int launch_split(const CUtensorMap& tm_a, const CUtensorMap& tm_w, const void* bias, const GemmOut& out, const QkEpilogue& qk,
+                 int M, int Nout, int K, int split, int* d_status, cudaStream_t s) {
   static PerDeviceOnce attr_once;
   HERO_TRY(per_device_once(attr_once, [](int) {
-    HERO_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_split_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    HERO_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_split_kernel<BN, QK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)SplitCfg<BN>::smem(SplitCfg<BN>::kMaxSplit)));
     return HERO_OK;
   }));
   const int tiles = ((M + kBM - 1) / kBM) * ((Nout + BN - 1) / BN);
-  return launch_kernel(tc_gemm_split_kernel<BN>, (unsigned)(tiles * split), kGemmThreads, SplitCfg<BN>::smem(split), s,
-                       (unsigned)split, tm_a, tm_w, (const __nv_bfloat16*)bias, out, M, Nout, K, split, d_status);
+  QkParam<QK> param;
+  if constexpr (QK) static_cast<QkEpilogue&>(param) = qk;
+  return launch_kernel(tc_gemm_split_kernel<BN, QK>, (unsigned)(tiles * split), kGemmThreads, SplitCfg<BN>::smem(split), s,
+                       (unsigned)split, tm_a, tm_w, (const __nv_bfloat16*)bias, out, param, M, Nout, K, split, d_status);
 }
 
 }  // namespace
 
 int launch_tc_gemm(const void* a, const void* w, const void* bias, int M, int Nout, int K, const GemmOut& out,
-                   int* d_status, cudaStream_t s) {
+                   const QkEpilogue* qk, int* d_status, cudaStream_t s) {
   if (M <= 0) return HERO_OK;
   if (K % 8 || Nout % 8 || out.seg_cols % 32) return HERO_ERR_ALIGN;
   if (!aligned16(a) || !aligned16(w) || !aligned16(bias)) return HERO_ERR_ALIGN;
   for (int i = 0; i < 3; ++i)
     if (out.ptr[i] && (!aligned16(out.ptr[i]) || out.ld[i] % 8)) return HERO_ERR_ALIGN;
-  const GemmPlan plan = plan_gemm(M, Nout, K);
+  const GemmPlan plan = plan_gemm(M, Nout, K, qk != nullptr);
   CUtensorMap tm_a, tm_w;
   {
     const uint64_t dims[2] = {(uint64_t)K, (uint64_t)M};
@@ -688,16 +816,23 @@ int launch_tc_gemm(const void* a, const void* w, const void* bias, int M, int No
     const uint32_t box[2] = {(uint32_t)kBK, (uint32_t)(plan.split == 0 ? plan.bn / 2 : plan.bn)};
     HERO_TRY(make_tmap_bf16(&tm_w, w, 2, dims, str, box));
   }
+  if (qk) {
+    if (out.seg_cols % 64 || Nout != 3 * out.seg_cols || out.act || out.gate || out.seg0_scale != 0.f) return HERO_ERR_ARG;
+    if (plan.split) return launch_split<128, true>(tm_a, tm_w, bias, out, *qk, M, Nout, K, 1, d_status, s);
+    return plan.bn == 256 ? launch_pair<256, true>(tm_a, tm_w, bias, out, *qk, M, Nout, K, d_status, s)
+                          : launch_pair<128, true>(tm_a, tm_w, bias, out, *qk, M, Nout, K, d_status, s);
+  }
+  const QkEpilogue none = {};
   if (plan.split == 0) {
     switch (plan.bn) {
-      case 256: return launch_pair<256>(tm_a, tm_w, bias, out, M, Nout, K, d_status, s);
-      case 224: return launch_pair<224>(tm_a, tm_w, bias, out, M, Nout, K, d_status, s);
-      case 192: return launch_pair<192>(tm_a, tm_w, bias, out, M, Nout, K, d_status, s);
-      default: return launch_pair<128>(tm_a, tm_w, bias, out, M, Nout, K, d_status, s);
+      case 256: return launch_pair<256>(tm_a, tm_w, bias, out, none, M, Nout, K, d_status, s);
+      case 224: return launch_pair<224>(tm_a, tm_w, bias, out, none, M, Nout, K, d_status, s);
+      case 192: return launch_pair<192>(tm_a, tm_w, bias, out, none, M, Nout, K, d_status, s);
+      default: return launch_pair<128>(tm_a, tm_w, bias, out, none, M, Nout, K, d_status, s);
     }
   }
-  return plan.bn == 128 ? launch_split<128>(tm_a, tm_w, bias, out, M, Nout, K, plan.split, d_status, s)
-                        : launch_split<64>(tm_a, tm_w, bias, out, M, Nout, K, plan.split, d_status, s);
+  return plan.bn == 128 ? launch_split<128>(tm_a, tm_w, bias, out, none, M, Nout, K, plan.split, d_status, s)
+                        : launch_split<64>(tm_a, tm_w, bias, out, none, M, Nout, K, plan.split, d_status, s);
 }
 
 }  // namespace hero
