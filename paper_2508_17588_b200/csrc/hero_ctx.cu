@@ -205,6 +205,7 @@ int modulation_for_blocks(hero_ctx* c, int l0, int l1, const void* d_temb, bool 
 struct NextRefresh {
   int n_sel = 0;               // 0: not refreshed, or not to be prepared here
   const int* pos = nullptr;    // as SelectBatch::pos; null: all rows
+  bool adds_branches = false;  // not refreshed but extrapolated, by a pass over x that adds this block's branches too
 };
 
 // Eq. 2 on the listed rows + Eq. 3's merge + the residual adds of Algorithm 1.  In a step (`in_step`) the adaLN vectors of
@@ -334,7 +335,9 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
     c->wait_x_upload = false;
     HERO_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->x_uploaded, 0));
   }
-  if (next.n_sel > 0) {
+  if (next.adds_branches) {
+    // (nothing to do here)
+  } else if (next.n_sel > 0) {
     const float* mod_next = c->mod + (size_t)(block + 1) * B * mod_ld;
     HERO_LAUNCH(c, HERO_PROF_RESIDUAL,
                 launch_residual_ln(d_x, ga, gf, next.pos, g.n_text, mod_next,
@@ -379,13 +382,25 @@ int extrapolate_block(hero_ctx* c, int block, void* d_x, int k, int d) {
 }
 
 // Blocks [l0, l1) (all extrapolated) over elements [first, first + n) of the residual stream, at most
-// kMaxDeepGroup blocks per launch.
-int extrapolate_blocks(hero_ctx* c, int l0, int l1, void* d_x, long long first, long long n, int k, int d) {
-  for (int l = l0; l < l1; l += kMaxDeepGroup) {
+// kMaxDeepGroup blocks per launch; before them, if given, the branches of the refreshed block in front (its place among
+// the launch's entries is that of a block).
+int extrapolate_blocks(hero_ctx* c, int l0, int l1, void* d_x, long long first, long long n, int k, int d,
+                       const BlockMem* in_front = nullptr) {
+  for (int l = l0; l < l1;) {
     DeepGroup grp;
-    grp.n_entries = 0;
-    for (int b = l; b < l1 && b < l + kMaxDeepGroup; ++b) {
-      const BlockMem& bm = c->blk[b];
+    grp.n_plain = grp.n_entries = 0;
+    int room = kMaxDeepGroup;
+    if (in_front && l == l0) {
+      for (int br = 0; br < 2; ++br) {
+        grp.prev[grp.n_entries] = nullptr;
+        grp.last[grp.n_entries] = in_front->g[br];
+        grp.n_entries++;
+      }
+      grp.n_plain = 2;
+      --room;
+    }
+    for (; l < l1 && room > 0; ++l, --room) {
+      const BlockMem& bm = c->blk[l];
       if (bm.n_hist == 0) return HERO_ERR_STATE;
       const int last = bm.last_slot, prev = bm.n_hist >= 2 ? (last ^ 1) : last;   // one slot only: Delta = 0
       for (int br = 0; br < 2; ++br) {
@@ -752,15 +767,18 @@ static int step_impl(hero_ctx* c, int step, void* d_x, const void* d_temb, void*
   }
   HERO_TRY(modulation_for_blocks(c, 0, g.n_shallow, d_temb, true));
   bool prepared = false;                     // the next refreshed block's rows are in ws_a
+  const BlockMem* in_front = nullptr;        // the last refreshed block, if its branches are not in x yet
   for (int l = 0; l < g.n_blocks; ++l) {
     if (l < g.n_shallow) {
       if (n_sel[l] > 0) {
         NextRefresh next;
         if (fuse && l + 1 < g.n_shallow && n_sel[l + 1] > 0)
           next = {n_sel[l + 1], c->pos_ws + (size_t)(g.share_selection ? 0 : l + 1) * c->idx_cap};
+        next.adds_branches = l + 1 == g.n_shallow && l + 1 < g.n_blocks && !collapse;
         HERO_TRY(refresh_block(c, l, d_x, d_temb, c->idx_ws + (size_t)(g.share_selection ? 0 : l) * c->idx_cap, n_sel[l],
                                true, prepared, next));
         prepared = next.n_sel > 0;
+        if (next.adds_branches) in_front = &c->blk[l];
       } else {
         HERO_LAUNCH(c, HERO_PROF_RESIDUAL,
                     launch_residual2(d_x, c->blk[l].g[0], c->blk[l].g[1], c->elems, g.dtype, c->stream));
@@ -776,7 +794,7 @@ static int step_impl(hero_ctx* c, int step, void* d_x, const void* d_temb, void*
         const long long first = (long long)p * per;
         const long long n = first >= c->elems ? 0 : (c->elems - first < per ? c->elems - first : per);
         if (n <= 0) break;
-        HERO_TRY(extrapolate_blocks(c, l, g.n_blocks, d_x, first, n, k, d));
+        HERO_TRY(extrapolate_blocks(c, l, g.n_blocks, d_x, first, n, k, d, in_front));
         HERO_CUDA_TRY(cudaEventRecord(c->piece_done[p], c->stream));
         HERO_CUDA_TRY(cudaStreamWaitEvent(c->copy_stream, c->piece_done[p], 0));
         HERO_CUDA_TRY(cudaMemcpyAsync(static_cast<char*>(h_out) + first * c->esz,
@@ -786,7 +804,7 @@ static int step_impl(hero_ctx* c, int step, void* d_x, const void* d_temb, void*
       *copied_out = true;
       break;
     } else {
-      HERO_TRY(extrapolate_blocks(c, l, g.n_blocks, d_x, 0, c->elems, k, d));   // the rest of the stack in one pass
+      HERO_TRY(extrapolate_blocks(c, l, g.n_blocks, d_x, 0, c->elems, k, d, in_front));   // the rest in one pass
       break;
     }
   }

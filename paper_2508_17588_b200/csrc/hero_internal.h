@@ -166,6 +166,7 @@ int launch_extrapolate_residual(void* x, const void* ga_prev, const void* ga_las
 // added in the order of the entries, for elements [first, first + n) of every tensor.
 constexpr int kMaxDeepGroup = 32;           // blocks per launch (two entries each)
 struct DeepGroup {
+  int n_plain;                              // 0 or 2: the first entries' `last` is added as it is (a refreshed block's branches)
   int n_entries;
   const void* prev[2 * kMaxDeepGroup];
   const void* last[2 * kMaxDeepGroup];

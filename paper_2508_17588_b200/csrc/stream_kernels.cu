@@ -174,7 +174,8 @@ extrapolate_residual_kernel(T* __restrict__ x, const T* __restrict__ ga_prev, co
 // Eq. 5 for a run of consecutive extrapolated blocks in ONE pass over x: a deep block touches nothing but
 // the residual stream, so x can stay in registers while the blocks' four history tensors stream by.  Per
 // element and block that is 8 bytes read instead of 12 moved (x is read and written once per launch, not
-// once per block), and the sum is rounded to the storage type once.  The adds keep the order of the blocks.
+// once per block), and the sum is rounded to the storage type once.  The adds keep the order of the blocks.  The branches
+// of the last refreshed block in front can come along (n_plain): its residual pass over x is then saved altogether.
 // E entries of the group are in flight per thread: four keep a large pass at the memory's rate (25 GB: 6.6 TB/s); where the
 // elements give every SM less than two blocks the pass is a chain of loads, and sixteen make it shorter (56 entries of
 // 157k elements: 36 -> 14 us).
@@ -188,8 +189,18 @@ __global__ void __launch_bounds__(kStreamThreads) extrapolate_group_kernel(T* __
   const long long stride = (long long)gridDim.x * kStreamThreads;
   for (long long i = (long long)blockIdx.x * kStreamThreads + threadIdx.x; i < n_vec; i += stride) {
     float fx[V::N];
-    ld_stream(xv + i).unpack(fx);
-    for (int e0 = 0; e0 < grp.n_entries; e0 += E) {
+    const V vx = ld_stream(xv + i);
+    if (grp.n_plain) {                     // (both branches of one block)
+      float fa[V::N], ff[V::N];
+      const V va = ld_stream(reinterpret_cast<const V*>(static_cast<const T*>(grp.last[0]) + first) + i);
+      const V vf = ld_stream(reinterpret_cast<const V*>(static_cast<const T*>(grp.last[1]) + first) + i);
+      vx.unpack(fx); va.unpack(fa); vf.unpack(ff);
+#pragma unroll
+      for (int j = 0; j < V::N; ++j) fx[j] = (fx[j] + fa[j]) + ff[j];
+    } else {
+      vx.unpack(fx);
+    }
+    for (int e0 = grp.n_plain; e0 < grp.n_entries; e0 += E) {
       V vp[E], vl[E];
 #pragma unroll
       for (int u = 0; u < E; ++u)
@@ -213,7 +224,8 @@ __global__ void __launch_bounds__(kStreamThreads) extrapolate_group_kernel(T* __
   if (blockIdx.x == 0 && threadIdx.x < n - tail0) {
     const long long i = first + tail0 + threadIdx.x;
     float v = to_f(x[i]);
-    for (int e = 0; e < grp.n_entries; ++e) {
+    for (int e = 0; e < grp.n_plain; ++e) v += to_f(static_cast<const T*>(grp.last[e])[i]);
+    for (int e = grp.n_plain; e < grp.n_entries; ++e) {
       const float a = to_f(static_cast<const T*>(grp.prev[e])[i]), b = to_f(static_cast<const T*>(grp.last[e])[i]);
       v += fmaf(b - a, c, b);
     }

@@ -156,11 +156,15 @@ def test_attention_modes(B, frames, grid_h, grid_w, n_text, heads, ratio_den, ke
     ("bf16", dict(hidden=64, head_dim=64, n_heads=1, ffn_dim=64, n_text=0, ratio_num=1, ratio_den=90)),
     ("bf16", dict(hidden=448, head_dim=64, n_heads=7, ffn_dim=64, deep_collapse=1)),
     ("bf16", dict(hidden=1536, head_dim=64, n_heads=24, ffn_dim=64, batch=1)),
-    ("bf16", dict(hidden=1600, head_dim=64, n_heads=25, ffn_dim=64, batch=1))],
-    ids=["fp32_64", "fp32_768_shared", "fp32_832", "bf16_64_sparse", "bf16_448_collapse", "bf16_1536", "bf16_1600"])
+    ("bf16", dict(hidden=1600, head_dim=64, n_heads=25, ffn_dim=64, batch=1)),
+    # into the deep stack: one refreshed block in front of as many deep ones as a launch holds, and of more
+    ("fp32", dict(hidden=64, head_dim=32, n_heads=2, ffn_dim=64, n_blocks=33, n_shallow=1)),
+    ("fp32", dict(hidden=64, head_dim=32, n_heads=2, ffn_dim=64, n_blocks=36, n_shallow=2))],
+    ids=["fp32_64", "fp32_768_shared", "fp32_832", "bf16_64_sparse", "bf16_448_collapse", "bf16_1536", "bf16_1600",
+         "deep_32", "deep_34"])
 def test_pass_from_block_to_block(dtype, over):
-    cfgd = dict(S.CONFIGS["tiny"], n_blocks=5, n_shallow=3, frames=1, grid_h=9, grid_w=7, seed=43, temb_dim=64, dtype=dtype,
-                full_interval=3, **{**dict(batch=2), **over})
+    cfgd = dict(S.CONFIGS["tiny"], frames=1, grid_h=9, grid_w=7, seed=43, temb_dim=64, dtype=dtype, full_interval=3,
+                **{**dict(batch=2, n_blocks=5, n_shallow=3), **over})
     orc, hero, _ = make_pair(cfgd)
     x_host = S.tokens(cfgd)
     for s in range(7):                                     # full, full, two cached, full, two cached
