@@ -170,7 +170,7 @@ int run_gemm(hero_ctx* c, const void* a, const void* w, const void* bias, int M,
   GemmOut o = out;
   o.weights_settled = 1;               // (behind a kernel of this context, which waited for whatever wrote the weights)
   if (c->cfg.dtype == HERO_DTYPE_BF16) return launch_tc_gemm(a, w, bias, M, Nout, K, o, qk, c->d_status, c->stream);
-  return launch_simt_gemm((const float*)a, (const float*)w, (const float*)bias, M, Nout, K, out, c->stream);
+  return launch_simt_gemm((const float*)a, (const float*)w, (const float*)bias, M, Nout, K, o, c->stream);
 }
 
 int run_attention(hero_ctx* c, const void* q, const void* k, const void* v, void* o, int n_q) {

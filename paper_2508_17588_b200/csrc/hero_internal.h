@@ -130,7 +130,7 @@ struct GemmOut {
   const float* gate;   // optional multiplier [B, gate_ld], indexed by column within the segment
   int gate_ld;
   int act;             // 0 = identity, 1 = GELU-tanh
-  int weights_settled; // W was complete before the kernel in front was placed: its first tiles are fetched without waiting
+  int weights_settled; // W, bias and idx were complete before the kernel in front was placed: no need to wait for that
   float seg0_scale;    // when not 0: factor on the columns of segment 0 (applied after the bias, before rounding)
 };
 
