@@ -380,11 +380,12 @@ int attention_launch(const float* q, const float* k, const float* v, float* o, i
   }));
   const long long groups = (long long)B * heads * ((n_q + kAttQ - 1) / kAttQ);
   const int tiles = (N + kAttK - 1) / kAttK;
-  // Keys over a cluster while that leaves every CTA a tile and the grid within what the chip holds at once: a CTA of four
+  // Keys over a cluster while that shortens the longest run of tiles (a CTA may go without: 144 keys are three tiles, over
+  // four CTAs 8.2 us, over two 12.8) and leaves the grid within what the chip holds at once: a CTA of four
   // warps alone keeps an SM's FMA pipe 40 % busy, two 80 % (310 queries, 1319 keys, 16 heads: 160 CTAs 102 us, 320 83 us).
   const int resident = HD > 64 ? 1 : 3;
   int split = 1;
-  while (split < 8 && split * 2 <= tiles && groups * split * 2 <= (long long)num_sms() * resident * 3 / 4) split *= 2;
+  while (split < 8 && split < tiles && groups * split * 2 <= (long long)num_sms() * resident * 3 / 4) split *= 2;
   if (groups * split > 0x7FFFFFFFll) return HERO_ERR_ARG;
   return launch_kernel(simt_attention_kernel<HD>, (unsigned)(groups * split), 128, Cfg::kSmem, s, (unsigned)split, q, k,
                        v, o, n_q, N, heads, split);
