@@ -263,9 +263,8 @@ int hero_attention_bf16_q_scaled(const void *d_q, const void *d_k, const void *d
  * serving loop that cannot take the device-wide synchronisation cudaMalloc/cudaFree imply, a
  * process whose framework already owns all device memory, code running where allocation is
  * forbidden - calls this instead.  Same arguments and same result (bit for bit); its scratch (the
- * give-up counter and the per-thread-block words through which the fast kernel hands blocks to the
- * fallback kernel) is a fixed 64.25 KiB array inside the library image, present on every GPU that
- * loads the library until the process exits.
+ * give-up counter and one word per thread block that says whether it gave up) is a fixed 64.25 KiB
+ * array inside the library image, present on every GPU that loads the library until the process exits.
  *   - Limit: ceil(n_q / 256) * heads * B <= 16384 (one scratch word per thread block); beyond
  *     that nothing is launched, HERO_ERR_CAP is returned and hero_last_cuda_error() says why.
  *   - The first call on each device resolves the array's device address and sets the kernel's
