@@ -113,7 +113,8 @@ int hero_reset(hero_ctx *ctx);
 void hero_destroy(hero_ctx *ctx);
 const char *hero_strerror(int code);
 /* Synchronise the context's stream and return HERO_ERR_TIMEOUT if any kernel gave up on
- * a bounded wait since the last check, HERO_ERR_CUDA on a CUDA error, else HERO_OK. */
+ * a bounded wait since the last check, HERO_ERR_CUDA on a CUDA error, else HERO_OK.  After a give-up the rows of
+ * that launch are not valid; later launches are unaffected, so a full step makes the context's caches good again. */
 int hero_check_status(hero_ctx *ctx);
 /* Text of the last failing CUDA call on this thread ("" if none). */
 const char *hero_last_cuda_error(void);
@@ -294,7 +295,8 @@ int hero_isolated_status(void *stream);
  * spinning.  This call runs exactly that on purpose, harmlessly: ONE thread block, no TMA, no tensor
  * memory, waits budget_us microseconds (1..100000) through the same helper on a barrier that nobody
  * completes, raises the word and returns.  With ctx given the word and the stream are the context's
- * (the next hero_check_status returns HERO_ERR_TIMEOUT once, then HERO_OK again); with ctx = NULL they
+ * (the next hero_check_status returns HERO_ERR_TIMEOUT once, then HERO_OK again; what the attention of a context keeps
+ * between its thread blocks is left as by a launch that gave up half way, which later calls do not mind); with ctx = NULL they
  * are the isolated calls' word and `stream` (hero_isolated_status reports it the same way). */
 int hero_selftest_wait_timeout(hero_ctx *ctx, int budget_us, void *stream);
 

@@ -72,9 +72,8 @@ struct hero_ctx {
   float* mod = nullptr;                  // [n_blocks, B, n_mod*D] adaLN vectors, one slot per block
   int* pos_ws = nullptr;                 // [n_shallow, idx_cap] every video token's place in those lists, or -1
   int* idx_ws = nullptr;                 // [n_shallow, idx_cap] selection lists of the current step
-  float* att_parts = nullptr;             // bf16: partial results of the attention's cut query groups
-  size_t status_bytes = 0;
-  int* d_status = nullptr;                // word 0: thread blocks that gave up on a wait; from word 4: counters of att_parts
+  AttentionParts att_parts = {};          // bf16: partial results of the attention's cut query groups
+  int* d_status = nullptr;                // word 0: thread blocks that gave up on a wait
   void *x_stage = nullptr, *temb_stage = nullptr;
   int n_full = 0, s_prev = 0, s_last = 0;
   int mode1_n_sel = 0;
@@ -173,14 +172,16 @@ int run_gemm(hero_ctx* c, const void* a, const void* w, const void* bias, int M,
   return launch_simt_gemm((const float*)a, (const float*)w, (const float*)bias, M, Nout, K, o, c->stream);
 }
 
-int run_attention(hero_ctx* c, const void* q, const void* k, const void* v, void* o, int n_q) {
+int run_attention(hero_ctx* c, const void* q, const void* k, const void* v, void* o, int n_q, int n_keys) {
   const hero_config& g = c->cfg;
   LaunchScope scope(c, HERO_PROF_ATTENTION);
-  if (g.dtype == HERO_DTYPE_BF16)
-    return launch_tc_attention(q, k, v, o, g.batch, n_q, c->N, g.n_heads, true, c->att_parts, c->d_status + 4,
-                               c->d_status, nullptr, c->stream);
-  return launch_simt_attention((const float*)q, (const float*)k, (const float*)v, (float*)o, g.batch, n_q, c->N, g.n_heads,
-                               g.head_dim, c->stream);
+  if (g.dtype == HERO_DTYPE_BF16) {
+    if (++c->att_parts.launch == 0) c->att_parts.launch = 1;
+    return launch_tc_attention(q, k, v, o, g.batch, n_q, n_keys, g.n_heads, true, c->att_parts, c->d_status, nullptr,
+                               c->stream);
+  }
+  return launch_simt_attention((const float*)q, (const float*)k, (const float*)v, (float*)o, g.batch, n_q, n_keys,
+                               g.n_heads, g.head_dim, c->stream);
 }
 
 // adaLN vectors of blocks [l0, l1) into their slots of c->mod, at most kMaxModBatch blocks per launch
@@ -300,15 +301,9 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
                 launch_gather_rows(kdst, c->att_list, c->kv_cmp[0], B, N, n_att, D, g.dtype, c->stream));
     HERO_LAUNCH(c, HERO_PROF_GATHER_LN,
                 launch_gather_rows(vdst, c->att_list, c->kv_cmp[1], B, N, n_att, D, g.dtype, c->stream));
-    LaunchScope scope(c, HERO_PROF_ATTENTION);
-    if (g.dtype == HERO_DTYPE_BF16)
-      HERO_TRY(launch_tc_attention(c->ws_q, c->kv_cmp[0], c->kv_cmp[1], c->ws_o, B, n_sel, n_att, g.n_heads, true,
-                                   c->att_parts, c->d_status + 4, c->d_status, nullptr, c->stream));
-    else
-      HERO_TRY(launch_simt_attention((const float*)c->ws_q, (const float*)c->kv_cmp[0], (const float*)c->kv_cmp[1],
-                                     (float*)c->ws_o, B, n_sel, n_att, g.n_heads, g.head_dim, c->stream));
+    HERO_TRY(run_attention(c, c->ws_q, c->kv_cmp[0], c->kv_cmp[1], c->ws_o, n_sel, n_att));
   } else {
-    HERO_TRY(run_attention(c, c->ws_q, kdst, vdst, c->ws_o, n_sel));
+    HERO_TRY(run_attention(c, c->ws_q, kdst, vdst, c->ws_o, n_sel, N));
   }
   GemmOut o_attn = {};
   o_attn.ptr[0] = ga; o_attn.ld[0] = D; o_attn.scatter[0] = 1;
@@ -561,9 +556,12 @@ int hero_init(hero_ctx** out, const hero_config* cfg, const hero_block_weights* 
   A((void**)&c->mod, (size_t)cfg->n_blocks * cfg->batch * c->n_mod * cfg->hidden * sizeof(float));
   A((void**)&c->idx_ws, (size_t)(cfg->n_shallow > 0 ? cfg->n_shallow : 1) * c->idx_cap * sizeof(int));
   A((void**)&c->pos_ws, (size_t)(cfg->n_shallow > 0 ? cfg->n_shallow : 1) * c->idx_cap * sizeof(int));
-  if (cfg->dtype == HERO_DTYPE_BF16) A((void**)&c->att_parts, tc_attention_part_bytes());
-  c->status_bytes = (4 + (cfg->dtype == HERO_DTYPE_BF16 ? tc_attention_part_counters() : 0)) * sizeof(int);
-  A((void**)&c->d_status, c->status_bytes);
+  const size_t count_bytes = tc_attention_part_counters() * sizeof(unsigned long long);
+  if (cfg->dtype == HERO_DTYPE_BF16) {
+    A((void**)&c->att_parts.rows, tc_attention_part_bytes());
+    A((void**)&c->att_parts.count, count_bytes);
+  }
+  A((void**)&c->d_status, 4 * sizeof(int));
   A(&c->x_stage, tensor);
   A(&c->temb_stage, (size_t)cfg->batch * cfg->temb_dim * c->esz);
   if (rc != HERO_OK) { hero_destroy(c); return rc; }
@@ -571,7 +569,8 @@ int hero_init(hero_ctx** out, const hero_config* cfg, const hero_block_weights* 
     cudaError_t er = cudaMemcpy(c->rope_tab, rope_host.data(), rope_host.size() * sizeof(float2), cudaMemcpyHostToDevice);
     if (er != cudaSuccess) { set_cuda_error(er, "cudaMemcpy(rope table)"); hero_destroy(c); return HERO_ERR_CUDA; }
   }
-  cudaError_t e = cudaMemsetAsync(c->d_status, 0, c->status_bytes, c->stream);
+  cudaError_t e = cudaMemsetAsync(c->d_status, 0, 4 * sizeof(int), c->stream);
+  if (e == cudaSuccess && c->att_parts.count) e = cudaMemsetAsync(c->att_parts.count, 0, count_bytes, c->stream);
   if (e != cudaSuccess) { set_cuda_error(e, "cudaMemsetAsync"); hero_destroy(c); return HERO_ERR_CUDA; }
   rc = hero_reset(c);
   if (rc != HERO_OK) { hero_destroy(c); return rc; }
@@ -631,7 +630,7 @@ int hero_check_status(hero_ctx* c) {
   HERO_CUDA_TRY(cudaMemcpyAsync(&st, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   HERO_CUDA_TRY(cudaStreamSynchronize(c->stream));
   if (st != 0) {
-    cudaMemsetAsync(c->d_status, 0, c->status_bytes, c->stream);     // (a block that gave up has not counted its parts in)
+    cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
     return HERO_ERR_TIMEOUT;
   }
   return HERO_OK;
@@ -951,7 +950,7 @@ int hero_attention_bf16(const void* q, const void* k, const void* v, void* o, in
   if (!q || !k || !v || !o) return HERO_ERR_ARG;
   int* st = isolated_status();
   if (!st) return HERO_ERR_NOMEM;
-  return launch_tc_attention(q, k, v, o, B, n_q, N, heads, false, nullptr, nullptr, st, nullptr, (cudaStream_t)stream);
+  return launch_tc_attention(q, k, v, o, B, n_q, N, heads, false, AttentionParts{}, st, nullptr, (cudaStream_t)stream);
 }
 
 int hero_attention_bf16_q_scaled(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N,
@@ -961,7 +960,7 @@ int hero_attention_bf16_q_scaled(const void* q, const void* k, const void* v, vo
   if (!q || !k || !v || !o) return HERO_ERR_ARG;
   int* st = isolated_status();
   if (!st) return HERO_ERR_NOMEM;
-  return launch_tc_attention(q, k, v, o, B, n_q, N, heads, true, nullptr, nullptr, st, nullptr, (cudaStream_t)stream);
+  return launch_tc_attention(q, k, v, o, B, n_q, N, heads, true, AttentionParts{}, st, nullptr, (cudaStream_t)stream);
 }
 
 int hero_attention_bf16_safe(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N, int heads,
@@ -980,12 +979,14 @@ int hero_isolated_status(void* stream) { return poll_isolated_status((cudaStream
 // Self-test of the give-up path: one thread block waits, with a budget of `budget_us` microseconds, on a
 // barrier that nobody will ever complete, through the same bounded-wait helper the tensor-core kernels use;
 // the wait runs out, the block raises the status word and returns.  With a context the word is the
-// context's (hero_check_status then reports HERO_ERR_TIMEOUT once), without one it is the word of the
+// context's (hero_check_status then reports HERO_ERR_TIMEOUT once), and the counters of its attention are left
+// as by a launch whose blocks gave up half way; without one it is the word of the
 // isolated tensor-core calls (hero_isolated_status reports it).
 int hero_selftest_wait_timeout(hero_ctx* c, int budget_us, void* stream) {
   if (budget_us < 1 || budget_us > 100000) return HERO_ERR_ARG;
   int* st = c ? c->d_status : isolated_status();
   if (!st) return HERO_ERR_NOMEM;
+  if (c && c->att_parts.count) HERO_TRY(launch_strand_attention_counters(c->att_parts, c->stream));
   return launch_wait_timeout_selftest(st, budget_us, c ? c->stream : (cudaStream_t)stream);
 }
 

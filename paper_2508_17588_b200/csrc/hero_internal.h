@@ -244,12 +244,20 @@ int launch_tc_gemm(const void* a, const void* w, const void* bias, int M, int No
                    const GemmOut& out, const QkEpilogue* qk, int* d_status, cudaStream_t s);
 // The tensor-core attention serves head_dim 64: a score s enters the softmax as 2^(s * kScoreScaleLog2).
 constexpr float kScoreScaleLog2 = 0.125f * 1.4426950408889634f;   // 1/sqrt(64) * log2(e)
+// Workspace of an attention launch that may cut query groups.
+struct AttentionParts {
+  float* rows;                          // tc_attention_part_bytes()
+  unsigned long long* count;            // tc_attention_part_counters() of them, zero before the first launch
+  unsigned launch;                      // another number, not 0, for every launch on this workspace
+};
 // q_prescaled: Q holds q * kScoreScaleLog2 (the softmax scale folded into the projection)
 int launch_tc_attention(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N,
-                        int heads, bool q_prescaled, float* parts, int* part_count, int* d_status, int* cta_words,
+                        int heads, bool q_prescaled, const AttentionParts& parts, int* d_status, int* cta_words,
                         cudaStream_t s);
-size_t tc_attention_part_bytes();       // workspace of an attention launch that may cut query groups
-size_t tc_attention_part_counters();    // and its counters (ints, zero between launches)
+size_t tc_attention_part_bytes();
+size_t tc_attention_part_counters();
+// (for the self-test of the give-up path)
+int launch_strand_attention_counters(const AttentionParts& parts, cudaStream_t s);
 int launch_tc_attention_safe(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N,
                              int heads, bool q_prescaled, int* d_status, cudaStream_t s);
 long long tc_attention_grid(int B, int n_q, int heads);   // CTAs of one attention launch

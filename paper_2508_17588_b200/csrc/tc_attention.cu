@@ -622,13 +622,27 @@ struct RunIter {
 constexpr int kPartFloats = 8 * 32 * 4 + 32;
 constexpr size_t kSlotFloats = (size_t)kFastSoftmaxWarps * kPartFloats;
 
+// Counts one part in and returns how many of this launch came before it.  A counter carries the number of the launch that
+// last counted in it (upper half): whatever a launch left behind that could not finish (a block that gave up on a wait
+// never counts its parts) is not this launch's count.
+__device__ __forceinline__ int count_part(unsigned long long* counter, unsigned launch) {
+  const unsigned long long none = (unsigned long long)launch << 32;
+  unsigned long long seen = __ldcg(counter);
+  for (;;) {                                       // (goes round only where another part has been counted meanwhile)
+    const unsigned long long before = seen >> 32 == launch ? seen : none;
+    const unsigned long long found = atomicCAS(counter, seen, before + 1);
+    if (found == seen) return (int)(unsigned)before;
+    seen = found;
+  }
+}
+
 // cta_words (may be null): one word per query group, set to 2 where a block gave up on a bounded wait.
 template <bool PRESCALED, AttentionMode MODE>
 __global__ void __launch_bounds__(kFastThreads, 1)
 tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                          const __grid_constant__ CUtensorMap tm_v, __nv_bfloat16* __restrict__ O, int n_q, int N,
-                         int heads, const __grid_constant__ AttentionPlan plan, float* __restrict__ parts,
-                         int* __restrict__ part_count, int* __restrict__ status, int* __restrict__ cta_words) {
+                         int heads, const __grid_constant__ AttentionPlan plan, const __grid_constant__ AttentionParts parts,
+                         int* __restrict__ status, int* __restrict__ cta_words) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   // Two query groups (the next one is fetched while this one is worked on) and the ring; in kCluster, one query group, a
@@ -938,7 +952,7 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       const int c_first = plan.share_of(u0), c_last = plan.share_of(u0 + plan.tiles - 1);
       const int first_slot = 2 * c_first + (plan.share_start(c_first) >= u0 ? 0 : 1);
       {
-        float* const part = parts + (size_t)(block == c_first ? first_slot : 2 * block) * kSlotFloats + sid * kPartFloats;
+        float* const part = parts.rows + (size_t)(block == c_first ? first_slot : 2 * block) * kSlotFloats + sid * kPartFloats;
 #pragma unroll 1
         for (int ch = 0; ch < 2; ++ch) {
           uint32_t r[16];
@@ -955,14 +969,14 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       __threadfence();
       __syncwarp();
       int before = 0;
-      if (lane == 0) before = atomicAdd(part_count + c_first * kFastSoftmaxWarps + sid, 1);
+      if (lane == 0) before = count_part(parts.count + c_first * kFastSoftmaxWarps + sid, parts.launch);
       before = __shfl_sync(0xFFFFFFFFu, before, 0);
       if (before < c_last - c_first) continue;         // the others are not all there yet
       __threadfence();
-      if (lane == 0) part_count[c_first * kFastSoftmaxWarps + sid] = 0;          // for the next launch
+      if (lane == 0) parts.count[c_first * kFastSoftmaxWarps + sid] = 0;         // (launches are numbered from 1)
       l_row = 0.f;
       for (int k = c_first; k <= c_last; ++k)
-        l_row += __ldcg(parts + (size_t)(k == c_first ? first_slot : 2 * k) * kSlotFloats + sid * kPartFloats + 8 * 32 * 4 + lane);
+        l_row += __ldcg(parts.rows + (size_t)(k == c_first ? first_slot : 2 * k) * kSlotFloats + sid * kPartFloats + 8 * 32 * 4 + lane);
       if (!in_range(l_row, qi, run.group)) continue;
 #pragma unroll 1
       for (int ch = 0; ch < 2; ++ch) {
@@ -972,7 +986,7 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
 #pragma unroll 2
         for (int k = c_first; k <= c_last; ++k) {
           const float4* part = reinterpret_cast<const float4*>(
-              parts + (size_t)(k == c_first ? first_slot : 2 * k) * kSlotFloats + sid * kPartFloats);
+              parts.rows + (size_t)(k == c_first ? first_slot : 2 * k) * kSlotFloats + sid * kPartFloats);
           float4 v[4];
 #pragma unroll
           for (int q = 0; q < 4; ++q) v[q] = __ldcg(part + (ch * 4 + q) * 32 + lane);
@@ -1212,13 +1226,24 @@ static PlannedAttention attention_plan(long long groups, int N, bool may_cluster
 size_t tc_attention_part_bytes() { return (size_t)2 * num_sms() * kSlotFloats * sizeof(float); }
 size_t tc_attention_part_counters() { return (size_t)num_sms() * kFastSoftmaxWarps; }
 
+// What a launch leaves in the counters when every block gives up with one part of each group counted in.
+static __global__ void strand_counters_kernel(AttentionParts parts, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) parts.count[i] = ((unsigned long long)parts.launch << 32) + 1;
+}
+int launch_strand_attention_counters(const AttentionParts& parts, cudaStream_t s) {
+  const int n = (int)tc_attention_part_counters();
+  strand_counters_kernel<<<(n + 255) / 256, 256, 0, s>>>(parts, n);
+  HERO_CUDA_TRY(cudaGetLastError());
+  return HERO_OK;
+}
+
 // d_status[0] counts thread blocks that gave up on a wait; cta_words may be null.  q_prescaled: the caller has multiplied Q
 // by log2(e) / sqrt(head_dim) already, so a score IS the exponent of its weight; the kernel then takes 2^s as it stands,
 // with no maximum at all (exact while a row's largest score stays within about +-100, the row sum telling when it did not).
-// parts, part_count (tc_attention_part_bytes, tc_attention_part_counters zeroed ints; both null: groups stay whole) are the
-// caller's for one launch at a time.
+// parts: the caller's for one launch at a time (no rows: groups stay whole).
 int launch_tc_attention(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N, int heads,
-                        bool q_prescaled, float* parts, int* part_count, int* d_status, int* cta_words, cudaStream_t s) {
+                        bool q_prescaled, const AttentionParts& parts, int* d_status, int* cta_words, cudaStream_t s) {
   if (B <= 0 || n_q <= 0) return HERO_OK;
   if (N <= 0 || heads <= 0) return HERO_ERR_ARG;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o)) return HERO_ERR_ALIGN;
@@ -1227,13 +1252,13 @@ int launch_tc_attention(const void* q, const void* k, const void* v, void* o, in
   HERO_TRY(attention_kernel_attributes());
   const long long groups = tc_attention_grid(B, n_q, heads);
   if (groups > 0x7FFFFFFFll / 8) return HERO_ERR_ARG;
-  const PlannedAttention p = attention_plan(groups, N, q_prescaled, q_prescaled && parts != nullptr);
+  const PlannedAttention p = attention_plan(groups, N, q_prescaled, q_prescaled && parts.rows != nullptr);
   return launch_kernel(!q_prescaled ? tc_attention_fast_kernel<false, kWhole>
                        : p.mode == kWhole ? tc_attention_fast_kernel<true, kWhole>
                        : p.mode == kCluster ? tc_attention_fast_kernel<true, kCluster> : tc_attention_fast_kernel<true, kCut>,
                        (unsigned)p.plan.blocks, kFastThreads, kFastSmem, s,
                        p.mode == kCluster ? (unsigned)p.plan.per_span : 1u, tm_q, tm_k, tm_v, (__nv_bfloat16*)o, n_q, N,
-                       heads, p.plan, parts, part_count, d_status, cta_words);
+                       heads, p.plan, parts, d_status, cta_words);
 }
 
 // The safe path alone, as a kernel of its own.
@@ -1323,7 +1348,7 @@ extern "C" int hero_attention_bf16_static(const void* d_q, const void* d_k, cons
   HERO_TRY(static_setup(&scratch));
   // the array still holds the previous call's records: clear the words this grid will use
   HERO_CUDA_TRY(cudaMemsetAsync(scratch, 0, (size_t)(1 + grid) * sizeof(int), s));
-  HERO_TRY(launch_tc_attention(d_q, d_k, d_v, d_o, B, n_q, N, heads, false, nullptr, nullptr, scratch, scratch + 1, s));
+  HERO_TRY(launch_tc_attention(d_q, d_k, d_v, d_o, B, n_q, N, heads, false, AttentionParts{}, scratch, scratch + 1, s));
   if (h_gave_up) {
     HERO_CUDA_TRY(cudaMemcpyAsync(h_gave_up, scratch, sizeof(int), cudaMemcpyDeviceToHost, s));
     HERO_CUDA_TRY(cudaStreamSynchronize(s));

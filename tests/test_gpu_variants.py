@@ -147,6 +147,41 @@ def test_attention_modes(B, frames, grid_h, grid_w, n_text, heads, ratio_den, ke
     hero.close()
 
 
+def cut_block(heads=7, **over):
+    """A block whose attention cuts its last query groups over all blocks of the grid: 25 groups of 6200 rows a head."""
+    cfg = dict(n_blocks=1, n_shallow=1, hidden=heads * 64, n_heads=heads, head_dim=64, ffn_dim=32, temb_dim=8, batch=1, frames=8,
+               grid_h=25, grid_w=31, n_text=0, patch_h=2, patch_w=2, ratio_num=1, ratio_den=8, quota_mode=0,
+               warmup_full_steps=1, full_interval=0, dtype="bf16", has_gate=0, seed=5, **over)
+    hero = H().Hero(cfg, [H().device_weights(S.block_weights(cfg, 0), "bf16")])
+    return hero, to_dev(S.tokens(cfg), "bf16"), to_dev(S.temb(cfg, 0), "bf16")
+
+
+@pytest.mark.parametrize("then", ["nothing", "reset", "check"])
+def test_a_launch_that_gave_up_does_not_reach_into_later_ones(then):
+    """What a cut attention keeps between thread blocks is left as by blocks that gave up half way: the next full pass is
+    what it is without that, whether or not the caller resets the context or asks for its status first."""
+    hero, x0, temb = cut_block()
+    hero.hero_refresh_block(0, x0.clone(), temb)
+    want = hero.hero_state_get(0, "g_attn")
+    hero.hero_check_status()
+    for _ in range(2):
+        hero.hero_refresh_block(0, -2 * x0.flip(1), temb)              # (leaves parts of other values behind)
+        hero.hero_selftest_wait_timeout(50)
+        if then == "reset":
+            hero.hero_reset()
+        if then == "check":
+            with pytest.raises(H().HeroError):
+                hero.hero_check_status()
+        for _ in range(2):
+            hero.hero_refresh_block(0, x0.clone(), temb)
+            assert torch.equal(hero.hero_state_get(0, "g_attn"), want)
+    if then != "check":
+        with pytest.raises(H().HeroError):
+            hero.hero_check_status()
+    hero.hero_check_status()
+    hero.close()
+
+
 @pytest.mark.parametrize("dtype,over", [
     # the pass from block to block: one packet a lane and less, several with the last one partly there, the widest it serves
     # and one beyond; lists of different length from block to block, one list for all, empty lists, a collapsed deep stack
