@@ -468,10 +468,10 @@ constexpr int kFastSoftmaxWarps = 16;            // 2 query tiles x 4 TMEM lane 
 constexpr int kFastThreads = 32 * (kFirstSoftmaxWarp + kFastSoftmaxWarps);   // 20 warps
 constexpr int kHalf = kKT / 2;                   // score columns of a key tile that one thread owns
 constexpr int kXchgFloats = kQTiles * kQT * 2;   // one slot per (query row, column half)
-constexpr int kMaxBad = 64;                      // out-of-range row slices a block keeps a list of
+constexpr int kMaxBad = 64;                      // out-of-range row slices of whole groups that a block keeps a list of
 constexpr size_t kFastBarBytes = 512;
 constexpr size_t kFastSmem = 1024 + 2 * kQTiles * kQBytes + (size_t)kKvStages * kKvStageBytes + kFastBarBytes +
-                             2 * kXchgFloats * sizeof(float) + (kMaxBad + 2) * sizeof(int);
+                             2 * kXchgFloats * sizeof(float) + (kMaxBad + 4) * sizeof(int);
 constexpr float kRowSumLimit = 1.2676506e30f;    // 2^100: a row sum at or beyond it voids the fixed-maximum assumption
 constexpr float kRowSumFloor = 7.8886091e-31f;   // 2^-100: below it a row without a maximum has lost its small terms
 static_assert(kHalf % 16 == 0 && (kHalf / 16) % 2 == 1, "three 16-column reads per half: the ping-pong below ends on ra");
@@ -593,6 +593,7 @@ struct RunIter {
   const AttentionPlan& plan;
   int block, k = 0, u = 0, end = 0;
   __device__ __forceinline__ RunIter(const AttentionPlan& p, int c) : plan(p), block(c) {}
+  __device__ __forceinline__ int number() const { return k - 1; }       // of the current run (all of a share's: the same)
   __device__ __forceinline__ bool next(Run& r) {
     if (MODE != kCut) {                          // one run only
       if (k++) return false;
@@ -666,7 +667,8 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   static_assert((4 + 2 * kKvStages + 4 + 4 + 2 + 8 + kSafeBars) * 8 + 8 <= (int)kFastBarBytes, "barrier block");
   float* xchg = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kFastBarBytes);   // [2][kXchgFloats]
   int* n_bad = reinterpret_cast<int*>(xchg + 2 * kXchgFloats);
-  int* bad = n_bad + 1;                            // [kMaxBad] group * 8 + query tile * 4 + quadrant
+  int* bad_cut = n_bad + 1;                        // [2] a bit per slice (query tile * 4 + quadrant) of the share's runs
+  int* bad = n_bad + 3;                            // [kMaxBad] whole runs: number of the run * 8 + slice
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q_groups = (n_q + kQT * kQTiles - 1) / (kQT * kQTiles);
@@ -685,7 +687,7 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     for (int i = 0; i < kQTiles; ++i) mbar_init(&pv_full[i], 1);
     for (int i = 0; i < 8; ++i) mbar_init(&pair_bar[i], 2);
     *abort_flag = 0;
-    *n_bad = 0;
+    *n_bad = bad_cut[0] = bad_cut[1] = 0;
     mbar_fence_init();
   }
   if (warp == 0 && lane == 0) { tma_prefetch_desc(&tm_q); tma_prefetch_desc(&tm_k); tma_prefetch_desc(&tm_v); }
@@ -697,13 +699,19 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   if (MODE == kCluster) cluster_arrive();              // waited for before anything is sent to another block
   // The row sum tells whether the fixed scaling was good enough (Inf and NaN are caught too; without a maximum the sum must
   // not be vanishingly small either).  If not, the warp's rows are left to the safe path below; of the warps that come to
-  // the same verdict on them, the first half's in the first block records them.
-  auto in_range = [&](float l_row, int qi, int group) -> bool {
+  // the same verdict on them, the first half's in the first block records them.  `run`: which of the block's runs; `part`:
+  // for a part of a group, which of the (at most two) parts in the block's share, else -1.
+  auto in_range = [&](float l_row, int qi, int run, int part) -> bool {
     const bool bad_row = qi < n_q && !(l_row < kRowSumLimit && (!PRESCALED || l_row > kRowSumFloor));
     if (!__any_sync(0xFFFFFFFFu, bad_row)) return true;
     if (lane == 0 && hh == 0 && (MODE != kCluster || block % plan.per_span == 0)) {
-      const int at = atomicAdd(n_bad, 1);
-      if (at < kMaxBad) bad[at] = group * 8 + t_own * 4 + quad;
+      const int slice = t_own * 4 + quad;
+      if (part >= 0) {
+        atomicOr(&bad_cut[part], 1 << slice);
+      } else {
+        const int at = atomicAdd(n_bad, 1);
+        if (at < kMaxBad) bad[at] = run * 8 + slice;
+      }
     }
     return false;
   };
@@ -934,7 +942,7 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         dst = output_of(run.group, qi);
       }
       if (MODE == kWhole || run.n == plan.tiles) {
-        if (in_range(l_row, qi, run.group)) {
+        if (in_range(l_row, qi, it.number(), -1)) {
           const float inv = 1.0f / l_row;
 #pragma unroll
           for (int ch = 0; ch < 2; ++ch) {
@@ -951,8 +959,9 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       const int u0 = (run.group - plan.groups + plan.tail) * plan.tiles;
       const int c_first = plan.share_of(u0), c_last = plan.share_of(u0 + plan.tiles - 1);
       const int first_slot = 2 * c_first + (plan.share_start(c_first) >= u0 ? 0 : 1);
+      const int my_slot = block == c_first ? first_slot : 2 * block;
       {
-        float* const part = parts.rows + (size_t)(block == c_first ? first_slot : 2 * block) * kSlotFloats + sid * kPartFloats;
+        float* const part = parts.rows + (size_t)my_slot * kSlotFloats + sid * kPartFloats;
 #pragma unroll 1
         for (int ch = 0; ch < 2; ++ch) {
           uint32_t r[16];
@@ -977,7 +986,7 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       l_row = 0.f;
       for (int k = c_first; k <= c_last; ++k)
         l_row += __ldcg(parts.rows + (size_t)(k == c_first ? first_slot : 2 * k) * kSlotFloats + sid * kPartFloats + 8 * 32 * 4 + lane);
-      if (!in_range(l_row, qi, run.group)) continue;
+      if (!in_range(l_row, qi, it.number(), my_slot & 1)) continue;
 #pragma unroll 1
       for (int ch = 0; ch < 2; ++ch) {
         float4 sum[4];
@@ -1049,7 +1058,7 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       float l_row = 0.f;                               // (added in rank order, as everything here)
 #pragma unroll
       for (int k = 0; k < S; ++k) l_row += k == rank ? l_cluster : sums[(k < rank ? k : k - 1) * kRows + my_row];
-      if (!in_range(l_row, qi, only_group)) return;    // (all ranks come to the same verdict; the first records it)
+      if (!in_range(l_row, qi, 0, -1)) return;         // (all ranks come to the same verdict; the first records it)
       const float inv = 1.0f / l_row;
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
@@ -1084,25 +1093,25 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   tc_fence_before();
   __syncthreads();
   const int n_marked = *n_bad;
-  if (n_marked > 0 && !*abort_flag) {                  // block-uniform
-    // One group at a time: the listed ones, or, where the list was too short, every group this block had a run of.
-    const bool listed = n_marked <= kMaxBad;
+  if ((n_marked | bad_cut[0] | bad_cut[1]) != 0 && !*abort_flag) {           // block-uniform
+    // One group at a time: the recorded slices, or, where the list was too short, the whole of every whole group.  Of a
+    // group that several blocks share exactly the recorded slices: the others are another block's to write.
     RunIter<MODE> it(plan, block);
     Run run;
     bool used = false;
-    for (int i = 0; listed ? i < n_marked : it.next(run); ++i) {
-      uint32_t mask = ~0u;
-      int group;
-      if (listed) {
-        group = bad[i] >> 3;
-        mask = 0;
-        bool seen = false;
+    int part = 0;
+    while (it.next(run)) {
+      uint32_t mask = 0;
+      if (MODE == kCut && run.n < plan.tiles) {
+        mask = (uint32_t)bad_cut[part++];
+      } else if (n_marked <= kMaxBad) {
         for (int k = 0; k < n_marked; ++k)
-          if (bad[k] >> 3 == group) { mask |= 1u << (bad[k] & 7); seen |= k < i; }
-        if (seen) continue;
+          if (bad[k] >> 3 == it.number()) mask |= 1u << (bad[k] & 7);
       } else {
-        group = run.group;
+        mask = ~0u;
       }
+      if (mask == 0) continue;
+      const int group = run.group;
       const int qg = group % q_groups, bh = group / q_groups;
       if (threadIdx.x == 0) {
         if (used)
@@ -1251,7 +1260,7 @@ int launch_tc_attention(const void* q, const void* k, const void* v, void* o, in
   HERO_TRY(make_attention_maps(q, k, v, B, n_q, N, heads, &tm_q, &tm_k, &tm_v));
   HERO_TRY(attention_kernel_attributes());
   const long long groups = tc_attention_grid(B, n_q, heads);
-  if (groups > 0x7FFFFFFFll / 8) return HERO_ERR_ARG;
+  if (groups > 0x7FFFFFFFll) return HERO_ERR_ARG;
   const PlannedAttention p = attention_plan(groups, N, q_prescaled, q_prescaled && parts.rows != nullptr);
   return launch_kernel(!q_prescaled ? tc_attention_fast_kernel<false, kWhole>
                        : p.mode == kWhole ? tc_attention_fast_kernel<true, kWhole>

@@ -156,6 +156,64 @@ def cut_block(heads=7, **over):
     return hero, to_dev(S.tokens(cfg), "bf16"), to_dev(S.temb(cfg, 0), "bf16")
 
 
+def test_rows_of_cut_groups_are_written_once_when_most_others_are_out_of_range():
+    """Ten whole rounds and twenty cut groups, nearly all rows out of the fixed scaling's range: more than a thread block
+    keeps a list of.  Slices of 32 rows that are in range stay in the cut groups what they are when all rows are, bit for
+    bit, and the whole output repeats itself."""
+    B, heads, N = 2, 30, 16 * 25 * 31
+    D = heads * 64
+    cfg = dict(n_blocks=1, n_shallow=1, hidden=D, n_heads=heads, head_dim=64, ffn_dim=32, temb_dim=8, batch=B, frames=16,
+               grid_h=25, grid_w=31, n_text=0, patch_h=2, patch_w=2, ratio_num=1, ratio_den=2, quota_mode=0,
+               warmup_full_steps=1, full_interval=0, dtype="bf16", has_gate=0, seed=5)
+    g = torch.Generator(device="cuda").manual_seed(11)
+    mk = lambda *s, std=1.0: (torch.randn(*s, device="cuda", generator=g) * std).bfloat16()
+    zero = lambda *s: torch.zeros(*s, device="cuda", dtype=torch.bfloat16)
+    u = torch.randn(heads, 64, device="cuda", generator=g)
+    offset = (2000 * u / u.norm(dim=1, keepdim=True)).view(-1)              # a constant of hundreds on all scores of a row
+    # keys and values of the refreshed rows do not depend on x: the two runs below see the same
+    w = dict(w_mod=zero(4 * D, 8), b_mod=zero(4 * D), w_qkv=zero(3 * D, D), b_qkv=mk(3 * D, std=0.1),
+             w_o=torch.eye(D, device="cuda", dtype=torch.bfloat16), b_o=zero(D), w_1=zero(32, D), b_1=zero(32),
+             w_2=zero(D, 32), b_2=zero(D))
+    w["w_qkv"][:D] = mk(D, D, std=1.5 / D ** 0.5)
+    w["b_qkv"][D:2 * D] = offset.bfloat16()
+    hero, temb = H().Hero(cfg, [w]), mk(B, 8)
+    hero.hero_state_set(0, "k", (torch.randn(B, N, D, device="cuda", generator=g) + offset).bfloat16())
+    hero.hero_state_set(0, "v", mk(B, N, D))
+    for name in ("g_attn", "g_ffn"):
+        hero.hero_state_set(0, name, zero(B, N, D))
+    rows = torch.arange(0, N, 2, device="cuda")
+    n = len(rows)
+    x = mk(B, N, D)
+    calm = (torch.arange(n, device="cuda") // 32 % 4 == 1)                  # their queries are the bias alone
+    x[:, rows[calm]] = 0
+
+    def attention(x):
+        hero.hero_refresh_block(0, x.clone(), temb, rows.int(), n)
+        return hero.hero_state_get(0, "g_attn").cuda()[:, rows]
+
+    got = attention(x)
+    for _ in range(3):
+        assert torch.equal(attention(x), got)
+    all_calm = attention(zero(B, N, D))
+    hero.hero_check_status()
+    q_groups = (n + 255) // 256
+    assert B * heads * q_groups == 10 * 148 + 20
+    cut = calm & (torch.arange(n, device="cuda") >= (q_groups - 20) * 256)  # of the last head of the last item
+    assert torch.equal(got[-1, cut][:, -64:], all_calm[-1, cut][:, -64:])
+    k, v = (hero.hero_state_get(0, name).cuda().view(B, N, D) for name in ("k", "v"))
+    r = x[:, rows].double()
+    a = ((r - r.mean(-1, keepdim=True)) / (r.var(-1, unbiased=False, keepdim=True) + 1e-5).sqrt()).bfloat16().double()
+    q = ((a @ w["w_qkv"][:D].double().T + w["b_qkv"][:D].double()) * 0.125 * 1.4426950408889634).bfloat16()
+    for b, h in ((0, 0), (0, heads - 1), (1, 3), (1, heads - 1)):
+        c = slice(h * 64, h * 64 + 64)
+        p = torch.softmax(q[b, :, c].double() @ k[b, :, c].double().T * 0.6931471805599453, -1)
+        want = p @ v[b, :, c].double()
+        # (a few units of score between the keys on top of the constant: as in test_attention_modes)
+        err = (got[b, :, c].double() - want).norm(dim=-1) / want.norm(dim=-1)
+        assert float(err.max()) <= 2.0 ** -6 and float((got[b, :, c].double() - want).norm() / want.norm()) <= 2.0 ** -7
+    hero.close()
+
+
 @pytest.mark.parametrize("then", ["nothing", "reset", "check"])
 def test_a_launch_that_gave_up_does_not_reach_into_later_ones(then):
     """What a cut attention keeps between thread blocks is left as by blocks that gave up half way: the next full pass is
