@@ -5,9 +5,10 @@
 // all shallow blocks of a step in one launch.  A patch never leaves its band, and the quotas of the patches before a
 // band sum to a closed form, so a warp knows where its part of the list starts without asking anybody; inside the band
 // each lane rebuilds the keys of its token's patch mates from the old ages, ranks the token, and the warp compacts the
-// winners in ascending row order with ballots.  Ages are double-buffered (read old, write new) because a patch spans
-// several grid rows.  Bound by latency (integer work, a few hundred bytes per warp): 2790 tokens in 8 blocks take 5.8 us
-// with a cold cache; one thread block per selected block, walking the tokens 1024 at a time, took 59 us for 17550.
+// winners in ascending row order with ballots.  Bands of more than 32 tokens get a thread block instead, whose warps take
+// 32 tokens each at a time and count their winners for one another (launch_select says when).  Ages are double-buffered
+// (read old, write new) because a patch spans several grid rows.  Bound by latency (integer work, a few hundred bytes per
+// warp) and, where a patch has hundreds of tokens, by the hashes.
 #include "hero_internal.h"
 
 namespace hero {
@@ -41,14 +42,17 @@ __device__ __forceinline__ int band_total_rounded(const SelectGeom& g, int rows)
   return whole * quota(rows * g.patch_w) + (rest ? quota(rows * rest) : 0);
 }
 
-__global__ void __launch_bounds__(kSelWarps * 32) select_kernel(const SelectGeom g, const SelectBatch batch) {
+// LONG: a thread block per band, else a warp.
+template <bool LONG>
+__global__ void __launch_bounds__(LONG ? 1024 : kSelWarps * 32) select_kernel(const SelectGeom g, const SelectBatch batch) {
   stream_order();
+  __shared__ int s_count[2][32];                           // (of this turn and of the one before)
   const int e = blockIdx.y;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int H = g.grid_h, W = g.grid_w, ph = g.patch_h, pw = g.patch_w;
   const int bands_per_frame = (H + ph - 1) / ph;
-  const int band = blockIdx.x * kSelWarps + (threadIdx.x >> 5);
-  if (band >= g.frames * bands_per_frame) return;          // warp-uniform
+  const int band = LONG ? blockIdx.x : blockIdx.x * kSelWarps + warp;
+  if (band >= g.frames * bands_per_frame) return;          // (of whole warps, and never of a warp of a LONG block)
   const uint16_t* __restrict__ ages_in = batch.ages_in[e];
   uint16_t* __restrict__ ages_out = batch.ages_out[e];
   int* __restrict__ idx = batch.idx[e];
@@ -70,8 +74,10 @@ __global__ void __launch_bounds__(kSelWarps * 32) select_kernel(const SelectGeom
     start = t * ((H / ph) * full + tail) + py * full;
   }
   const int n_band = hh * W;
-  for (int base = 0; base < n_band; base += 32) {
-    const int i = base + lane;
+  const int step = LONG ? (int)blockDim.x : 32;
+  int turn = 0;
+  for (int base = 0; base < n_band; base += step, turn ^= 1) {
+    const int i = base + (LONG ? (int)threadIdx.x : lane);
     bool pick = false;
     uint32_t age_v = 0;
     const int v = (int)band_first + i;
@@ -101,13 +107,21 @@ __global__ void __launch_bounds__(kSelWarps * 32) select_kernel(const SelectGeom
       pick = beaten_by < quota;
     }
     const unsigned ballot = __ballot_sync(0xFFFFFFFFu, pick);
+    int before = 0, total = __popc(ballot);                // winners of the warps in front, and of all of them
+    if (LONG) {
+      if (lane == 0) s_count[turn][warp] = total;
+      __syncthreads();
+      const int c = lane < step / 32 ? s_count[turn][lane] : 0;
+      before = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? c : 0);
+      total = __reduce_add_sync(0xFFFFFFFFu, c);
+    }
     if (i < n_band) {
-      const int place = start + __popc(ballot & ((1u << lane) - 1u));
+      const int place = start + before + __popc(ballot & ((1u << lane) - 1u));
       if (pick) idx[place] = g.n_text + v;
       if (pos) pos[v] = pick ? place : -1;
       ages_out[v] = pick ? (uint16_t)0 : (uint16_t)min(age_v + 1u, 65535u);
     }
-    start += __popc(ballot);
+    start += total;
   }
 }
 
@@ -116,9 +130,19 @@ __global__ void __launch_bounds__(kSelWarps * 32) select_kernel(const SelectGeom
 int launch_select(const SelectGeom& g, const SelectBatch& batch, cudaStream_t s) {
   if (batch.n <= 0) return HERO_OK;
   const int bands = g.frames * ((g.grid_h + g.patch_h - 1) / g.patch_h);
-  HERO_TRY(launch_kernel(select_kernel, dim3((unsigned)((bands + kSelWarps - 1) / kSelWarps), (unsigned)batch.n),
-                         kSelWarps * 32, 0, s, 1, g, batch));
-  return HERO_OK;
+  const long long longest = (long long)(g.patch_h < g.grid_h ? g.patch_h : g.grid_h) * g.grid_w;
+  // A warp per band is the better split only where every band is one turn of it, or where there are more tokens than the
+  // chip holds threads and enough bands (16 warps an SM) to fill it.  Measured in us, a block / a warp a band, and in
+  // brackets one block a list, in turns of 1024 tokens (lists x frames x grid, patch): 1 x 1 x 64 x 64, 8 x 8 8.9 / 103 (51),
+  // 64 x 64 2509 / 36621 (2460); 1 x 1 x 2 x 127, 2 x 2 6.9 / 14.6 (7.7); 1 x 1 x 2 x 8775, 2 x 2 39 / 602 (49);
+  // 14 x 13 x 30 x 45, 2 x 2 12.7 / 12.5 (58), 3 x 3 14.7 / 16.7 (72); 14 x 13 x 60 x 90, 2 x 2 29.2 / 22.9 (215);
+  // 14 x 3 x 9 x 11, 2 x 2 (22 tokens a band) 8.4 / 8.1 (8.5).
+  const long long tokens = (long long)g.frames * g.grid_h * g.grid_w * batch.n, sms = num_sms();
+  if (longest > 32 && (tokens <= sms * 2048 || (long long)bands * batch.n < sms * 16))
+    return launch_kernel(select_kernel<true>, dim3((unsigned)bands, (unsigned)batch.n),
+                         longest < 1024 ? (unsigned)((longest + 31) / 32 * 32) : 1024u, 0, s, 1, g, batch);
+  return launch_kernel(select_kernel<false>, dim3((unsigned)((bands + kSelWarps - 1) / kSelWarps), (unsigned)batch.n),
+                       kSelWarps * 32, 0, s, 1, g, batch);
 }
 
 }  // namespace hero

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import hero_oracle as O
 from workloads import synthetic as S
 from tests.util import make_pair, rel_l2, to_dev, to_host
 
@@ -144,6 +145,44 @@ def test_attention_modes(B, frames, grid_h, grid_w, n_text, heads, ratio_den, ke
         # by a few times that); the sum of three bounds with a factor of two for the scores
         assert float(err.max()) <= 2.0 ** -6, (cached, int(err.argmax()))
         assert float((got[:, rows].double() - want).norm() / want.norm()) <= 2.0 ** -7
+    hero.close()
+
+
+@pytest.mark.parametrize("blocks,frames,grid_h,grid_w,patch_h,patch_w,over", [
+    # a band (grid rows of one row of patches) of one turn of a warp, of one token more, of a block's 1024 tokens and more
+    (1, 2, 9, 16, 2, 3, {}), (2, 2, 9, 11, 3, 4, dict(track_mode=1)), (1, 1, 16, 64, 16, 4, {}), (1, 1, 5, 205, 5, 3, {}),
+    (1, 1, 3, 2100, 2, 2, dict(quota_mode=1, ratio_num=1, ratio_den=3)),
+    # patches as large as the grid and larger, one row, one column
+    (1, 2, 33, 37, 40, 50, dict(ratio_num=1, ratio_den=7)), (1, 1, 1, 1500, 1, 7, dict(quota_mode=1)), (1, 3, 70, 1, 70, 1, {}),
+    # more tokens than threads fit the chip, in many bands and in few
+    (10, 4, 128, 80, 2, 2, {}), (8, 1, 9, 4300, 3, 3, {})])
+def test_selection_variants(blocks, frames, grid_h, grid_w, patch_h, patch_w, over):
+    """Lists and ages of all blocks, bit for bit, through calls on one block and through steps (every block at once)."""
+    cfgd = dict(dict(S.CONFIGS["tiny"], hidden=64, n_heads=1, head_dim=64, ffn_dim=4, temb_dim=4, n_blocks=blocks,
+                     n_shallow=blocks, batch=1, n_text=3, frames=frames, grid_h=grid_h, grid_w=grid_w, patch_h=patch_h,
+                     patch_w=patch_w, full_interval=0, warmup_full_steps=1, seed=77), **over)
+    cfg = O.Config.from_dict(cfgd)
+    w = {k: np.zeros(s, np.float32) for k, s in S.weight_shapes(cfgd).items()}
+    hero = H().Hero(cfgd, [H().device_weights(w, "fp32")] * blocks)
+    n_rows = 3 + frames * grid_h * grid_w
+    for l in range(blocks):                                # (caches as after a full pass)
+        for name in ("k", "v", "g_attn", "g_ffn"):
+            hero.hero_state_set(l, name, torch.zeros(1, n_rows, 64))
+    hero.hero_state_set(0, "steps", torch.tensor([1, 0, 0], dtype=torch.int32))
+    ages = [np.zeros(cfg.n_video, np.uint16) for _ in range(blocks)]
+    x, temb = torch.zeros(1, n_rows, 64, device="cuda"), torch.zeros(1, 4, device="cuda")
+    for call in range(3):
+        if call == 2:
+            hero.hero_step(1, x, temb)
+        for l in range(blocks):
+            rows, ages[l] = O.select_tokens(cfg, ages[l], l, call)
+            if call < 2:
+                idx = torch.full((cfg.n_video,), -1, dtype=torch.int32, device="cuda")
+                n = hero.hero_select_tokens(l, idx)
+                got = idx.cpu().numpy()
+                assert n == len(rows) and np.array_equal(got[:n], rows) and (got[n:] == -1).all()
+            assert np.array_equal(hero.hero_state_get(l, "ages").numpy(), ages[l]), (call, l)
+    hero.hero_check_status()
     hero.close()
 
 
