@@ -9,7 +9,7 @@
 // operand of O += P V.  S of tile j+2 is issued right after P V of tile j (same issuer, executed
 // in issue order), so a score tile is normally ready a whole softmax iteration before it is needed.
 //
-// Two kernels share this layout:
+// Two kernels share this layout and these warps:
 //
 //  * tc_attention_fast_kernel, the one that normally does all the work.  20 warps: TMA producer, one
 //    tcgen05.mma issuer warp per query tile (all lanes run the loop, one elected lane issues, so that
@@ -31,8 +31,9 @@
 //    no first-tile exchange, no multiply-add per pair of scores - and is exact while a row's largest score
 //    stays within about +-100; its row sum must then lie in [2^-100, 2^100), else the CTA is marked.
 //  * The safe path (safe_roles) keeps a running maximum that moves whenever a tile exceeds it by 2^8, rescaling the
-//    accumulator in TMEM: 12 warps, one thread per row.  A thread block of the fast kernel whose row sums say that the
-//    range assumption failed recomputes its queries with it before it ends (a second launch for the failed blocks, as it
+//    accumulator in TMEM.  The warps are those of the fast kernel; the two threads of a row trade their halves' maxima for
+//    every key tile.  A thread block of the fast kernel whose row sums say that the range assumption failed recomputes its
+//    queries with it before it ends (a second launch for the failed blocks, as it
 //    used to be, cost every attention 2-4 us at small sizes and 14 us at 1728 blocks for finding nothing to do);
 //    tc_attention_safe_kernel is the same path as a kernel of its own.
 //
@@ -55,10 +56,6 @@
 #include "hero_internal.h"
 #include "tc_common.cuh"
 
-#ifndef HERO_ATT_CHUNK
-#define HERO_ATT_CHUNK 16
-#endif
-
 namespace hero {
 
 int make_tmap_bf16(CUtensorMap* m, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
@@ -72,12 +69,16 @@ constexpr int kQBytes = kQT * kHD * 2;       // 16 KB per query tile
 constexpr int kKBytes = kKT * kHD * 2;       // 12 KB (a multiple of the 1024-byte swizzle atom)
 constexpr int kKvStageBytes = 2 * kKBytes;   // K tile then V tile
 constexpr int kFirstSoftmaxWarp = 4;
-constexpr int kAttThreads = 32 * (kFirstSoftmaxWarp + 4 * kQTiles);   // 12 warps
-constexpr size_t kAttSmem = 1024 + kQTiles * kQBytes + (size_t)kKvStages * kKvStageBytes + 512;
+constexpr int kSoftmaxWarps = 16;            // 2 query tiles x 4 TMEM lane quadrants x 2 column halves
+constexpr int kAttThreads = 32 * (kFirstSoftmaxWarp + kSoftmaxWarps);        // 20 warps
+constexpr int kHalf = kKT / 2;               // score columns of a key tile that one thread owns
+constexpr int kXchgFloats = kQTiles * kQT * 2;   // one slot per (query row, column half)
+constexpr size_t kSafeSmem = 1024 + kQTiles * kQBytes + (size_t)kKvStages * kKvStageBytes + 512 + 2 * kXchgFloats * sizeof(float);
 constexpr uint32_t kTileCols = 256, kColO = 2 * kKT, kAttTmemCols = 512;   // per tile: S0 | S1 | O
 constexpr float kRescaleLog2 = 8.0f;           // the scaling maximum moves only when exceeded by 2^8
 static_assert(2 * kKT + kHD <= (int)kTileCols && kQTiles * kTileCols <= kAttTmemCols, "TMEM layout");
 static_assert(kKBytes % 1024 == 0 && kKT % 16 == 0, "tile shape");
+static_assert(kHalf % 16 == 0 && (kHalf / 16) % 2 == 1, "three 16-column reads per half: half_tile's ping-pong ends on ra");
 
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -91,136 +92,16 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 }
 __device__ __forceinline__ float2 f2(uint32_t a, uint32_t b) { return make_float2(__uint_as_float(a), __uint_as_float(b)); }
 
-// One key tile of one query row.  The kKT scores of the row are read from TMEM in one burst
-// (a single wait for the whole row instead of one per chunk), reduced to their maximum, turned
-// into p = 2^(s*c - m*c) and written back as bf16 pairs over columns [0, kKT/2) of the same
-// buffer.  m_used is the maximum the row's P and accumulator are scaled by: it only moves when
-// this tile exceeds it by more than 2^kRescaleLog2 (always at the first tile), and alpha is then
-// the factor that the sum and the accumulator take.  Returns the row sum of p.
-template <bool MASKED>
-__device__ __forceinline__ float softmax_tile(uint32_t t_buf, int valid, float c, float& m_used, float& alpha,
-                                              bool& grow) {
-  uint32_t s[kKT];
+// 16 output features of one row: accumulator times 1 / row sum, bf16.
+__device__ __forceinline__ void emit16(const uint32_t (&r)[16], float inv, __nv_bfloat16* dst) {
+  uint32_t w[8];
 #pragma unroll
-  for (int ch = 0; ch < kKT / 32; ++ch) tmem_ld32(t_buf + ch * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[ch * 32]));
-  tmem_ld_wait();
-  if (MASKED) {
-#pragma unroll
-    for (int i = 0; i < kKT; ++i)
-      if (i >= valid) s[i] = 0xFF800000u;   // -inf
+  for (int q = 0; q < 8; ++q) {
+    const __nv_bfloat162 pk = __floats2bfloat162_rn(__uint_as_float(r[2 * q]) * inv, __uint_as_float(r[2 * q + 1]) * inv);
+    w[q] = *reinterpret_cast<const uint32_t*>(&pk);
   }
-  float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-  for (int i = 0; i < kKT; i += 8) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) mx[q] = fmaxf(mx[q], fmaxf(__uint_as_float(s[i + 2 * q]), __uint_as_float(s[i + 2 * q + 1])));
-  }
-  const float m_tile = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
-  grow = (m_tile - m_used) * c > kRescaleLog2;                 // true at the first tile (m_used = -inf)
-  const float m_new = grow ? m_tile : m_used;
-  alpha = grow ? ex2((m_used - m_new) * c) : 1.0f;             // 0 at the first tile
-  m_used = m_new;
-  const float neg_mc = -m_new * c;
-  const float2 c2 = make_float2(c, c), nm2 = make_float2(neg_mc, neg_mc);
-  float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-  for (int ch = 0; ch < kKT / 32; ++ch) {
-    uint32_t packed[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {       // pair i = columns 2i, 2i+1 of this 32-column chunk
-      const int col = ch * 32 + 2 * i;
-      const float2 x = __ffma2_rn(f2(s[col], s[col + 1]), c2, nm2);
-      float2 p = make_float2(ex2(x.x), ex2(x.y));
-      if (MASKED) {
-        if (col >= valid) p.x = 0.f;
-        if (col + 1 >= valid) p.y = 0.f;
-      }
-      acc[i & 3] = __fadd2_rn(acc[i & 3], p);
-      const __nv_bfloat162 b = __floats2bfloat162_rn(p.x, p.y);
-      packed[i] = *reinterpret_cast<const uint32_t*>(&b);
-    }
-    tmem_st16(t_buf + ch * 16, packed);
-  }
-  const float2 a01 = __fadd2_rn(acc[0], acc[1]), a23 = __fadd2_rn(acc[2], acc[3]);
-  return (a01.x + a01.y) + (a23.x + a23.y);
-}
-
-// The common case of a key tile, in ONE pass over the row: p = 2^((s - m_used) c) with the maximum
-// the row is already scaled by, the tile's own maximum tracked on the side.  The caller checks the
-// maximum afterwards and falls back to softmax_tile (S is still intact: P is only kept in
-// registers here) in the rare case that it has to move.  Doing without the separate maximum pass
-// matters because that pass issues nothing to the exponential unit for a third of the tile.  The
-// scores are read kCh columns at a time, one read ahead; short reads keep the register count low
-// enough for the compiler to overlap the pairs freely (16 columns measured 4 % faster than 32).
-__device__ __forceinline__ void fused_tile(uint32_t t_buf, float c, float neg_mc, uint32_t (&packed)[kKT / 2],
-                                           float& sum, float& m_tile) {
-  const float2 c2 = make_float2(c, c), nm2 = make_float2(neg_mc, neg_mc);
-  float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  float mx[2] = {-INFINITY, -INFINITY};
-  constexpr int kCh = HERO_ATT_CHUNK;                  // score columns per TMEM read
-  uint32_t ra[kCh], rb[kCh];
-  if (kCh == 32) tmem_ld32(t_buf, *reinterpret_cast<uint32_t(*)[32]>(&ra[0]));
-  else tmem_ld16(t_buf, *reinterpret_cast<uint32_t(*)[16]>(&ra[0]));
-#pragma unroll
-  for (int ch = 0; ch < kKT / kCh; ++ch) {
-    uint32_t(&cur)[kCh] = (ch & 1) ? rb : ra;
-    uint32_t(&nxt)[kCh] = (ch & 1) ? ra : rb;
-    tmem_ld_wait();
-    if (ch + 1 < kKT / kCh) {
-      if (kCh == 32) tmem_ld32(t_buf + (ch + 1) * kCh, *reinterpret_cast<uint32_t(*)[32]>(&nxt[0]));
-      else tmem_ld16(t_buf + (ch + 1) * kCh, *reinterpret_cast<uint32_t(*)[16]>(&nxt[0]));
-    }
-#pragma unroll
-    for (int i = 0; i < kCh / 2; ++i) {
-      const float2 x = __ffma2_rn(f2(cur[2 * i], cur[2 * i + 1]), c2, nm2);
-      const float2 p = make_float2(ex2(x.x), ex2(x.y));
-      acc[i & 3] = __fadd2_rn(acc[i & 3], p);
-      const __nv_bfloat162 b = __floats2bfloat162_rn(p.x, p.y);
-      packed[ch * (kCh / 2) + i] = *reinterpret_cast<const uint32_t*>(&b);
-      mx[i & 1] = max3(mx[i & 1], __uint_as_float(cur[2 * i]), __uint_as_float(cur[2 * i + 1]));
-    }
-  }
-  const float2 a01 = __fadd2_rn(acc[0], acc[1]), a23 = __fadd2_rn(acc[2], acc[3]);
-  sum = (a01.x + a01.y) + (a23.x + a23.y);
-  m_tile = fmaxf(mx[0], mx[1]);
-}
-
-// The two passes of softmax_tile in reads of 16 columns, for a caller that has no registers for a whole row.
-__device__ __forceinline__ float softmax_tile_lean(uint32_t t_buf, int valid, float c, float& m_used, float& alpha,
-                                                   bool& grow) {
-  float m_tile = -INFINITY;
-#pragma unroll 1
-  for (int ch = 0; ch < kKT / 16; ++ch) {
-    uint32_t s[16];
-    tmem_ld16(t_buf + ch * 16, s);
-    tmem_ld_wait();
-#pragma unroll
-    for (int i = 0; i < 16; ++i)
-      if (ch * 16 + i < valid) m_tile = fmaxf(m_tile, __uint_as_float(s[i]));
-  }
-  grow = (m_tile - m_used) * c > kRescaleLog2;
-  const float m_new = grow ? m_tile : m_used;
-  alpha = grow ? ex2((m_used - m_new) * c) : 1.0f;
-  m_used = m_new;
-  const float neg_mc = -m_new * c;
-  float sum = 0.f;
-#pragma unroll 1
-  for (int ch = 0; ch < kKT / 16; ++ch) {              // P of chunk ch goes over columns that were read before
-    uint32_t s[16], packed[8];
-    tmem_ld16(t_buf + ch * 16, s);
-    tmem_ld_wait();
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int col = ch * 16 + 2 * i;
-      const float p0 = col < valid ? ex2(fmaf(__uint_as_float(s[2 * i]), c, neg_mc)) : 0.f;
-      const float p1 = col + 1 < valid ? ex2(fmaf(__uint_as_float(s[2 * i + 1]), c, neg_mc)) : 0.f;
-      sum += p0 + p1;
-      const __nv_bfloat162 b = __floats2bfloat162_rn(p0, p1);
-      packed[i] = *reinterpret_cast<const uint32_t*>(&b);
-    }
-    tmem_st8(t_buf + ch * 8, packed);
-  }
-  return sum;
+  *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+  *reinterpret_cast<uint4*>(dst + 8) = make_uint4(w[4], w[5], w[6], w[7]);
 }
 
 // One thread block's work on the safe path.
@@ -232,22 +113,23 @@ struct SafeWork {
   uint32_t row_mask;             // which 32-row slices (query tile * 4 + quadrant) of the group are written
   uint8_t *s_q, *s_kv;
   uint64_t* bars;                // kSafeBars barriers, set up by safe_init_barriers, never used before
+  float* xchg;                   // [2][kXchgFloats] between the two threads of a row
   volatile int* abort_flag;
   uint32_t tmem_base;
 };
-constexpr int kSafeBars = 1 + 2 * kKvStages + 4 + 4 + 2 * kQTiles;
+constexpr int kSafeBars = 1 + 2 * kKvStages + 4 + 4 + 2 * kQTiles + 4 * kQTiles;
 // The last query group of a (batch, head) may reach into its second tile by no row at all: that tile's
 // issuer and softmax warps then have nothing to do and the K/V stages are released by one issuer alone.
 __device__ __forceinline__ int live_tiles(int qg, int n_q) { return (qg * kQTiles + 1) * kQT < n_q ? kQTiles : 1; }
 __device__ __forceinline__ void safe_init_barriers(uint64_t* bars, int n_tiles) {
   mbar_init(bars, 1);
   for (int i = 0; i < kKvStages; ++i) { mbar_init(bars + 1 + i, 1); mbar_init(bars + 1 + kKvStages + i, n_tiles); }
-  for (int i = 0; i < 4; ++i) { mbar_init(bars + 1 + 2 * kKvStages + i, 1); mbar_init(bars + 5 + 2 * kKvStages + i, 4); }
+  for (int i = 0; i < 4; ++i) { mbar_init(bars + 1 + 2 * kKvStages + i, 1); mbar_init(bars + 5 + 2 * kKvStages + i, 8); }
   for (int i = 0; i < 2 * kQTiles; ++i) mbar_init(bars + 9 + 2 * kKvStages + i, 1);
+  for (int i = 0; i < 4 * kQTiles; ++i) mbar_init(bars + 9 + 2 * kKvStages + 2 * kQTiles + i, 2);
 }
 
-// Warp 0: TMA producer, warps 1 and 2: MMA issuers, warps 4 .. 11: softmax (any others: nothing).
-template <bool LEAN>
+// Warp 0: TMA producer, warps 1 and 2: MMA issuers, warps 4 .. 19: softmax, as in the fast kernel.
 __device__ __forceinline__ void safe_roles(const SafeWork& w) {
   const CUtensorMap &tm_q = *w.tm_q, &tm_k = *w.tm_k, &tm_v = *w.tm_v;
   const int n_q = w.n_q, N = w.N, heads = w.heads, qg = w.qg, h = w.h, b = w.b;
@@ -261,9 +143,10 @@ __device__ __forceinline__ void safe_roles(const SafeWork& w) {
   uint64_t* kv_full = q_full + 1;                  // [kKvStages]           TMA -> both issuers
   uint64_t* kv_empty = kv_full + kKvStages;        // [kKvStages], count 2  both issuers -> TMA
   uint64_t* s_full = kv_empty + kKvStages;         // [qt][parity]  issuer -> softmax: S is ready
-  uint64_t* p_full = s_full + 4;                   // [qt][parity]  softmax -> issuer: P is in TMEM
+  uint64_t* p_full = s_full + 4;                   // [qt][parity]  softmax -> issuer: P is in TMEM (8 warps)
   uint64_t* pv_full = p_full + 4;                  // [qt]          issuer -> softmax: P V of tile j done (phase j)
   uint64_t* pv_last = pv_full + kQTiles;           // [qt]          issuer -> softmax: all P V done
+  uint64_t* pair_bar = pv_last + kQTiles;          // [qt][quadrant] the two warps that share 32 query rows
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_kv = (N + kKT - 1) / kKT;
   const int n_tiles = live_tiles(qg, n_q);
@@ -316,7 +199,8 @@ __device__ __forceinline__ void safe_roles(const SafeWork& w) {
         tc_fence_after();
         const uint32_t buf = t_tile + (uint32_t)(j & 1) * kKT;
 #pragma unroll
-        for (int k = 0; k < kKT / 16; ++k) mma_ts(t_tile + kColO, buf + 8 * k, dv + 128 * k, idesc_pv, (j | k) != 0);
+        for (int k = 0; k < kKT / 16; ++k)         // (each half of the softmax writes P inside its own score columns)
+          mma_ts(t_tile + kColO, buf + (k / 3) * kHalf + (k % 3) * 8, dv + 128 * k, idesc_pv, (j | k) != 0);
         mma_commit(&pv_full[t]);
         if (j == n_kv - 1) mma_commit(&pv_last[t]);
         mma_commit(&kv_empty[st]);               // second arrival comes from the other tile's issuer
@@ -329,45 +213,87 @@ __device__ __forceinline__ void safe_roles(const SafeWork& w) {
         }
       }
     }
-  } else if (warp >= kFirstSoftmaxWarp && ((warp - kFirstSoftmaxWarp) >> 2) < n_tiles) {
+  } else if (warp >= kFirstSoftmaxWarp && (((warp - kFirstSoftmaxWarp) >> 2) & 1) < n_tiles) {
     // ------------------------------------------------------------ softmax
-    const int t = (warp - kFirstSoftmaxWarp) >> 2;     // query tile of this softmax group
+    const int sid = warp - kFirstSoftmaxWarp;
+    const int t = (sid >> 2) & 1, hh = sid >> 3;       // query tile, and which 48 of a tile's 96 score columns
     const int quad = warp & 3;                         // TMEM lane quadrant this warp may touch
+    const int row = quad * 32 + lane;
     const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)t * kTileCols;
-    float m_used = -INFINITY, l_run = 0.f;
+    uint64_t* my_pair = &pair_bar[t * 4 + quad];
+    uint32_t pair_phase = 0;
+    // One value of this thread and its partner's.  (Two exchange buffers in turn: a warp may be one exchange ahead of its
+    // partner, not two.)
+    auto slot = [&]() { return w.xchg + pair_phase * kXchgFloats + (t * kQT + row) * 2; };
+    auto offer = [&](float mine) {
+      slot()[hh] = mine;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(my_pair);
+    };
+    auto take = [&](float2& both) -> bool {
+      if (!mbar_wait_warp(my_pair, pair_phase, abort_flag)) return false;
+      both = make_float2(slot()[0], slot()[1]);
+      pair_phase ^= 1;
+      return true;
+    };
+    float m_used = -INFINITY, l_run = 0.f;             // the maximum that the row's P and accumulator are scaled by
+    float2 both;
     bool ok = true;
     for (int j = 0; j < n_kv; ++j) {
       ok = mbar_wait_warp(&s_full[t * 2 + (j & 1)], (j >> 1) & 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
-      const uint32_t t_buf = lane_base + (uint32_t)(j & 1) * kKT;
-      const int valid = N - j * kKT;                   // keys of this tile that exist (>= 1)
-      const bool ragged = valid < kKT;
-      float alpha = 1.0f, sum;
-      bool grow = true;                                // first and ragged tiles take the two-pass path
-      uint32_t packed[kKT / 2];
-      if (!LEAN && j > 0 && !ragged) {
-        float m_tile;
-        fused_tile(t_buf, c, -m_used * c, packed, sum, m_tile);
-        grow = __any_sync(0xFFFFFFFFu, (m_tile - m_used) * c > kRescaleLog2);
-      }
-      if (grow) {                                      // warp-uniform
-        bool moved;
-        if (LEAN) {
-          sum = softmax_tile_lean(t_buf, valid, c, m_used, alpha, moved);
-          grow = __any_sync(0xFFFFFFFFu, moved);
-        } else {
-          sum = ragged ? softmax_tile<true>(t_buf, valid, c, m_used, alpha, moved)
-                       : softmax_tile<false>(t_buf, valid, c, m_used, alpha, moved);
-        }
-      } else {
+      const uint32_t t_s = lane_base + (uint32_t)(j & 1) * kKT + (uint32_t)hh * kHalf;
+      const int valid = N - j * kKT - hh * kHalf;      // columns of this half that are keys
+      uint32_t s[kHalf];
 #pragma unroll
-        for (int ch = 0; ch < kKT / 32; ++ch)
-          tmem_st16(t_buf + ch * 16, *reinterpret_cast<uint32_t(*)[16]>(&packed[ch * 16]));
+      for (int ch = 0; ch < kHalf / 16; ++ch) tmem_ld16(t_s + ch * 16, *reinterpret_cast<uint32_t(*)[16]>(&s[ch * 16]));
+      tmem_ld_wait();
+      if (valid < kHalf) {                             // warp-uniform
+#pragma unroll
+        for (int i = 0; i < kHalf; ++i)
+          if (i >= valid) s[i] = 0xFF800000u;          // -inf: weight 0 under any finite maximum
       }
+      float mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+      for (int i = 0; i < kHalf; i += 4) {
+        mx[0] = max3(mx[0], __uint_as_float(s[i]), __uint_as_float(s[i + 1]));
+        mx[1] = max3(mx[1], __uint_as_float(s[i + 2]), __uint_as_float(s[i + 3]));
+      }
+      offer(fmaxf(mx[0], mx[1]));
+      // P under the maximum that the row has: where this tile's does not move it, that is all, and the partner's half of
+      // the maximum has arrived meanwhile.
+      const float2 c2 = make_float2(c, c);
+      auto weights = [&]() -> float {
+        const float2 nm2 = make_float2(-m_used * c, -m_used * c);
+        float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+        for (int ch = 0; ch < kHalf / 16; ++ch) {
+          uint32_t pk[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const float2 x = __ffma2_rn(f2(s[ch * 16 + 2 * i], s[ch * 16 + 2 * i + 1]), c2, nm2);
+            const float2 p = make_float2(ex2(x.x), ex2(x.y));
+            acc[i & 1] = __fadd2_rn(acc[i & 1], p);
+            const __nv_bfloat162 bb = __floats2bfloat162_rn(p.x, p.y);
+            pk[i] = *reinterpret_cast<const uint32_t*>(&bb);
+          }
+          tmem_st8(t_s + ch * 8, pk);
+        }
+        const float2 a01 = __fadd2_rn(acc[0], acc[1]);
+        return a01.x + a01.y;
+      };
+      float sum = j > 0 ? weights() : 0.f;
+      if (!(ok = take(both))) break;
+      const float m_tile = fmaxf(both.x, both.y);      // (the same in both threads of the row, and so is what follows)
+      const bool grow = (m_tile - m_used) * c > kRescaleLog2;               // true at the first tile
+      const float alpha = grow ? ex2((m_used - m_tile) * c) : 1.0f;         // 0 at the first tile
+      if (grow) m_used = m_tile;
+      const bool moved = __any_sync(0xFFFFFFFFu, grow);
+      if (j == 0 || moved) sum = weights();
       l_run = fmaf(l_run, alpha, sum);
-      if (j > 0 && grow) {
-        // Rare (warp-uniform): the maximum moved, so the accumulator is scaled down before this tile's
+      if (j > 0 && moved) {
+        // Rare: the maximum moved, so the accumulator is scaled down before this tile's
         // product is added to it - once P V of tile j-1 has completed.  pv_full is only looked at here, yet the
         // parity wait is unambiguous: S of tile j was issued after P V of tile j-2
         // (so that one is complete) and P V of tile j cannot start before this warp's arrival below, hence
@@ -377,16 +303,16 @@ __device__ __forceinline__ void safe_roles(const SafeWork& w) {
         tc_fence_after();
         const float2 a2 = make_float2(alpha, alpha);     // alpha is 1 for rows that did not move
 #pragma unroll
-        for (int ch = 0; ch < kHD / 16; ++ch) {
+        for (int ch = 0; ch < 2; ++ch) {                 // each half 32 of the 64 features
           uint32_t r[16];
-          tmem_ld16(lane_base + kColO + ch * 16, r);
+          tmem_ld16(lane_base + kColO + hh * 32 + ch * 16, r);
           tmem_ld_wait();
 #pragma unroll
           for (int i = 0; i < 16; i += 2) {
             const float2 v = __fmul2_rn(f2(r[i], r[i + 1]), a2);
             r[i] = __float_as_uint(v.x); r[i + 1] = __float_as_uint(v.y);
           }
-          tmem_st16(lane_base + kColO + ch * 16, r);
+          tmem_st16(lane_base + kColO + hh * 32 + ch * 16, r);
         }
       }
       tmem_st_wait();
@@ -394,29 +320,23 @@ __device__ __forceinline__ void safe_roles(const SafeWork& w) {
       __syncwarp();
       if (lane == 0) mbar_arrive(&p_full[t * 2 + (j & 1)]);
     }
+    if (ok) {
+      offer(l_run);
+      ok = take(both);
+    }
     // (Not pv_full: the other warps may still be two tiles behind this one, and its parity cannot tell that.)
     if (ok) ok = mbar_wait_warp(&pv_last[t], 0, abort_flag);
     if (ok) {
       tc_fence_after();
-      const int qi = (qg * kQTiles + t) * kQT + quad * 32 + lane;
-      const float inv = 1.0f / l_run;
-      __nv_bfloat16* dst = O + ((long long)b * n_q + qi) * ((long long)heads * kHD) + h * kHD;
+      const int qi = (qg * kQTiles + t) * kQT + row;
+      const float inv = 1.0f / (both.x + both.y);
+      __nv_bfloat16* dst = O + ((long long)b * n_q + qi) * ((long long)heads * kHD) + h * kHD + hh * 32;
 #pragma unroll
-      for (int ch = 0; ch < kHD / 16; ++ch) {
+      for (int ch = 0; ch < 2; ++ch) {
         uint32_t r[16];
-        tmem_ld16(lane_base + kColO + ch * 16, r);     // warp-collective: every lane loads
+        tmem_ld16(lane_base + kColO + hh * 32 + ch * 16, r);     // warp-collective: every lane loads
         tmem_ld_wait();
-        if (qi < n_q && (row_mask >> (t * 4 + quad) & 1)) {
-          uint32_t w[8];
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const __nv_bfloat162 pk = __floats2bfloat162_rn(__uint_as_float(r[2 * q]) * inv,
-                                                            __uint_as_float(r[2 * q + 1]) * inv);
-            w[q] = *reinterpret_cast<const uint32_t*>(&pk);
-          }
-          *reinterpret_cast<uint4*>(dst + ch * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-          *reinterpret_cast<uint4*>(dst + ch * 16 + 8) = make_uint4(w[4], w[5], w[6], w[7]);
-        }
+        if (qi < n_q && (row_mask >> (t * 4 + quad) & 1)) emit16(r, inv, dst + ch * 16);
       }
     }
   }
@@ -435,6 +355,8 @@ tc_attention_safe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   w.bars = reinterpret_cast<uint64_t*>(w.s_kv + (size_t)kKvStages * kKvStageBytes);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(w.bars + kSafeBars);
   w.abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  w.xchg = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(w.bars) + 512);
+  static_assert(kSafeBars * 8 + 8 <= 512, "barrier block");
   w.c = c;
   w.row_mask = ~0u;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -454,7 +376,7 @@ tc_attention_safe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   tc_fence_after();
   w.tmem_base = *tmem_slot;
   stream_order();
-  safe_roles<false>(w);
+  safe_roles(w);
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && *w.abort_flag) atomicAdd(status, 1);
@@ -464,17 +386,12 @@ tc_attention_safe_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
 // =============================================================================================
 // The fast kernel
 // =============================================================================================
-constexpr int kFastSoftmaxWarps = 16;            // 2 query tiles x 4 TMEM lane quadrants x 2 column halves
-constexpr int kFastThreads = 32 * (kFirstSoftmaxWarp + kFastSoftmaxWarps);   // 20 warps
-constexpr int kHalf = kKT / 2;                   // score columns of a key tile that one thread owns
-constexpr int kXchgFloats = kQTiles * kQT * 2;   // one slot per (query row, column half)
 constexpr int kMaxBad = 64;                      // out-of-range row slices of whole groups that a block keeps a list of
-constexpr size_t kFastBarBytes = 512;
+constexpr size_t kFastBarBytes = 640;
 constexpr size_t kFastSmem = 1024 + 2 * kQTiles * kQBytes + (size_t)kKvStages * kKvStageBytes + kFastBarBytes +
                              2 * kXchgFloats * sizeof(float) + (kMaxBad + 4) * sizeof(int);
 constexpr float kRowSumLimit = 1.2676506e30f;    // 2^100: a row sum at or beyond it voids the fixed-maximum assumption
 constexpr float kRowSumFloor = 7.8886091e-31f;   // 2^-100: below it a row without a maximum has lost its small terms
-static_assert(kHalf % 16 == 0 && (kHalf / 16) % 2 == 1, "three 16-column reads per half: the ping-pong below ends on ra");
 
 // 2^x for two scores on the FMA pipe instead of the special-function unit (Cody-Waite reduction + a cubic).
 // The unit evaluates 16 ex2 per clock per SM and is what bounds this kernel; every pair moved here frees two of
@@ -552,21 +469,6 @@ __device__ __forceinline__ float half_tile(uint32_t t_s, int valid, const float2
   return (a01.x + a01.y) + (a23.x + a23.y);
 }
 
-// (its registers are its own business: a call keeps the fast path's allocation out of it)
-static __device__ __noinline__ void safe_recompute(const SafeWork& w) { safe_roles<true>(w); }
-
-// 16 output features of one row: accumulator times 1 / row sum, bf16.
-__device__ __forceinline__ void emit16(const uint32_t (&r)[16], float inv, __nv_bfloat16* dst) {
-  uint32_t w[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const __nv_bfloat162 pk = __floats2bfloat162_rn(__uint_as_float(r[2 * q]) * inv, __uint_as_float(r[2 * q + 1]) * inv);
-    w[q] = *reinterpret_cast<const uint32_t*>(&pk);
-  }
-  *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-  *reinterpret_cast<uint4*>(dst + 8) = make_uint4(w[4], w[5], w[6], w[7]);
-}
-
 // How one launch's query groups are dealt out.  Block c takes the groups c, c + blocks, ... (`rounds` of them at most), then
 // one share of the key tiles of the remaining `tail` groups, laid end to end and numbered from 0.  These fall into spans of
 // equal length (one group each, or all of them together), every span into `per_span` shares whose lengths differ by one
@@ -621,7 +523,7 @@ struct RunIter {
 // Workspace of a launch that cuts groups: per block two slots (its first and its last run), per slot and softmax warp
 // 32 rows x 32 accumulator columns (eight float4 planes) and the 32 row sums; one counter per block and warp.
 constexpr int kPartFloats = 8 * 32 * 4 + 32;
-constexpr size_t kSlotFloats = (size_t)kFastSoftmaxWarps * kPartFloats;
+constexpr size_t kSlotFloats = (size_t)kSoftmaxWarps * kPartFloats;
 
 // Counts one part in and returns how many of this launch came before it.  A counter carries the number of the launch that
 // last counted in it (upper half): whatever a launch left behind that could not finish (a block that gave up on a wait
@@ -637,22 +539,91 @@ __device__ __forceinline__ int count_part(unsigned long long* counter, unsigned 
   }
 }
 
+// The fast kernel's shared memory.  Two query groups (the next one is fetched while this one is worked on) and the ring; in
+// kCluster, one query group, a shorter ring, and behind it the place for the other blocks' pieces.
+template <AttentionMode MODE>
+struct FastSmem {
+  static constexpr int kStages = MODE == kCluster ? 4 : kKvStages;
+  static constexpr int kQBufs = MODE == kCluster ? 1 : 2;
+  static constexpr int kBars = 2 + 2 + 2 * kKvStages + 4 + 4 + 2 + 8;
+  uint8_t *q, *kv;
+  uint64_t *bars, *safe_bars;                      // (the latter for the safe path, should this block need it)
+  uint32_t* tmem_slot;
+  volatile int* abort_flag;
+  float* xchg;                                     // [2][kXchgFloats]
+  int *n_bad, *bad_cut, *bad;                      // see in_range
+  __device__ __forceinline__ explicit FastSmem(uint8_t* base) {
+    q = base;
+    kv = base + kQBufs * kQTiles * kQBytes;
+    bars = reinterpret_cast<uint64_t*>(base + 2 * kQTiles * kQBytes + (size_t)kKvStages * kKvStageBytes);
+    safe_bars = bars + kBars;
+    tmem_slot = reinterpret_cast<uint32_t*>(safe_bars + kSafeBars);
+    abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    static_assert((kBars + kSafeBars) * 8 + 8 <= (int)kFastBarBytes, "barrier block");
+    xchg = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kFastBarBytes);
+    n_bad = reinterpret_cast<int*>(xchg + 2 * kXchgFloats);
+    bad_cut = n_bad + 1;                           // [2] a bit per slice (query tile * 4 + quadrant) of the share's runs
+    bad = n_bad + 3;                               // [kMaxBad] whole runs: number of the run * 8 + slice
+  }
+};
+
+// The recorded slices once more, on the safe path.  One group at a time: the recorded slices, or, where the list was too
+// short, the whole of every whole group.  Of a group that several blocks share exactly the recorded slices: the others are
+// another block's to write.  (A call of its own: what it needs in registers stays out of the fast path's allocation.)
+template <bool PRESCALED, AttentionMode MODE>
+static __device__ __noinline__ void recompute(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
+                                              __nv_bfloat16* O, int n_q, int N, int heads, const AttentionPlan& plan,
+                                              uint8_t* smem) {
+  const FastSmem<MODE> sm(smem);
+  const int q_groups = (n_q + kQT * kQTiles - 1) / (kQT * kQTiles);
+  const int n_marked = *sm.n_bad;
+  RunIter<MODE> it(plan, blockIdx.x);
+  Run run;
+  bool used = false;
+  int part = 0;
+  while (it.next(run)) {
+    uint32_t mask = 0;
+    if (MODE == kCut && run.n < plan.tiles) {
+      mask = (uint32_t)sm.bad_cut[part++];
+    } else if (n_marked <= kMaxBad) {
+      for (int k = 0; k < n_marked; ++k)
+        if (sm.bad[k] >> 3 == it.number()) mask |= 1u << (sm.bad[k] & 7);
+    } else {
+      mask = ~0u;
+    }
+    if (mask == 0) continue;                       // block-uniform
+    const int qg = run.group % q_groups, bh = run.group / q_groups;
+    if (threadIdx.x == 0) {
+      if (used)
+        for (int k = 0; k < kSafeBars; ++k) mbar_inval(&sm.safe_bars[k]);
+      safe_init_barriers(sm.safe_bars, live_tiles(qg, n_q));
+      mbar_fence_init();
+    }
+    used = true;
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // (kCluster has used the ring through plain stores)
+    __syncthreads();
+    tc_fence_after();
+    safe_roles({&tm_q, &tm_k, &tm_v, O, n_q, N, heads, qg, bh % heads, bh / heads, PRESCALED ? 1.0f : kScoreScaleLog2,
+                mask, sm.q, sm.kv, sm.safe_bars, sm.xchg, sm.abort_flag, *sm.tmem_slot});
+    tc_fence_before();
+    __syncthreads();
+    if (*sm.abort_flag) break;
+  }
+}
+
 // cta_words (may be null): one word per query group, set to 2 where a block gave up on a bounded wait.
 template <bool PRESCALED, AttentionMode MODE>
-__global__ void __launch_bounds__(kFastThreads, 1)
+__global__ void __launch_bounds__(kAttThreads, 1)
 tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                          const __grid_constant__ CUtensorMap tm_v, __nv_bfloat16* __restrict__ O, int n_q, int N,
                          int heads, const __grid_constant__ AttentionPlan plan, const __grid_constant__ AttentionParts parts,
                          int* __restrict__ status, int* __restrict__ cta_words) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  // Two query groups (the next one is fetched while this one is worked on) and the ring; in kCluster, one query group, a
-  // shorter ring, and behind it the place for the other blocks' pieces.
-  constexpr int kStages = MODE == kCluster ? 4 : kKvStages;
-  constexpr int kQBufs = MODE == kCluster ? 1 : 2;
-  uint8_t* s_q = smem;
-  uint8_t* s_kv = smem + kQBufs * kQTiles * kQBytes;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 2 * kQTiles * kQBytes + (size_t)kKvStages * kKvStageBytes);
+  const FastSmem<MODE> sm(smem);
+  constexpr int kStages = FastSmem<MODE>::kStages;
+  uint8_t *const s_q = sm.q, *const s_kv = sm.kv;
+  uint64_t* const bars = sm.bars;
   uint64_t* q_full = bars;                         // [2]           TMA -> both issuers
   uint64_t* q_empty = q_full + 2;                  // [2], count 2  both issuers -> TMA
   uint64_t* kv_full = q_empty + 2;                 // [kKvStages]           TMA -> both issuers
@@ -661,14 +632,10 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   uint64_t* p_full = s_full + 4;                   // [qt][parity]  softmax -> issuer: P is in TMEM (8 warps)
   uint64_t* pv_full = p_full + 4;                  // [qt]          issuer -> softmax: the last P V of a run is done
   uint64_t* pair_bar = pv_full + 2;                // [qt][quadrant] the two warps that share 32 query rows
-  uint64_t* safe_bars = pair_bar + 8;              // for the safe path, should this block need it
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(safe_bars + kSafeBars);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  static_assert((4 + 2 * kKvStages + 4 + 4 + 2 + 8 + kSafeBars) * 8 + 8 <= (int)kFastBarBytes, "barrier block");
-  float* xchg = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kFastBarBytes);   // [2][kXchgFloats]
-  int* n_bad = reinterpret_cast<int*>(xchg + 2 * kXchgFloats);
-  int* bad_cut = n_bad + 1;                        // [2] a bit per slice (query tile * 4 + quadrant) of the share's runs
-  int* bad = n_bad + 3;                            // [kMaxBad] whole runs: number of the run * 8 + slice
+  uint32_t* const tmem_slot = sm.tmem_slot;
+  volatile int* const abort_flag = sm.abort_flag;
+  float* const xchg = sm.xchg;
+  int *const n_bad = sm.n_bad, *const bad_cut = sm.bad_cut, *const bad = sm.bad;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q_groups = (n_q + kQT * kQTiles - 1) / (kQT * kQTiles);
@@ -978,11 +945,11 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
       __threadfence();
       __syncwarp();
       int before = 0;
-      if (lane == 0) before = count_part(parts.count + c_first * kFastSoftmaxWarps + sid, parts.launch);
+      if (lane == 0) before = count_part(parts.count + c_first * kSoftmaxWarps + sid, parts.launch);
       before = __shfl_sync(0xFFFFFFFFu, before, 0);
       if (before < c_last - c_first) continue;         // the others are not all there yet
       __threadfence();
-      if (lane == 0) parts.count[c_first * kFastSoftmaxWarps + sid] = 0;         // (launches are numbered from 1)
+      if (lane == 0) parts.count[c_first * kSoftmaxWarps + sid] = 0;         // (launches are numbered from 1)
       l_row = 0.f;
       for (int k = c_first; k <= c_last; ++k)
         l_row += __ldcg(parts.rows + (size_t)(k == c_first ? first_slot : 2 * k) * kSlotFloats + sid * kPartFloats + 8 * 32 * 4 + lane);
@@ -1092,56 +1059,23 @@ tc_attention_fast_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
   // ---------------------------------------------------------------- rows out of range: once more, on the safe path
   tc_fence_before();
   __syncthreads();
-  const int n_marked = *n_bad;
-  if ((n_marked | bad_cut[0] | bad_cut[1]) != 0 && !*abort_flag) {           // block-uniform
-    // One group at a time: the recorded slices, or, where the list was too short, the whole of every whole group.  Of a
-    // group that several blocks share exactly the recorded slices: the others are another block's to write.
-    RunIter<MODE> it(plan, block);
-    Run run;
-    bool used = false;
-    int part = 0;
-    while (it.next(run)) {
-      uint32_t mask = 0;
-      if (MODE == kCut && run.n < plan.tiles) {
-        mask = (uint32_t)bad_cut[part++];
-      } else if (n_marked <= kMaxBad) {
-        for (int k = 0; k < n_marked; ++k)
-          if (bad[k] >> 3 == it.number()) mask |= 1u << (bad[k] & 7);
-      } else {
-        mask = ~0u;
-      }
-      if (mask == 0) continue;
-      const int group = run.group;
-      const int qg = group % q_groups, bh = group / q_groups;
-      if (threadIdx.x == 0) {
-        if (used)
-          for (int k = 0; k < kSafeBars; ++k) mbar_inval(&safe_bars[k]);
-        safe_init_barriers(safe_bars, live_tiles(qg, n_q));
-        mbar_fence_init();
-      }
-      used = true;
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // (kCluster has used the ring through plain stores)
-      __syncthreads();
-      tc_fence_after();
-      const SafeWork w = {&tm_q, &tm_k, &tm_v, O,    n_q, N,    heads,     qg,         bh % heads, bh / heads,
-                          PRESCALED ? 1.0f : kScoreScaleLog2, mask, s_q, s_kv, safe_bars, abort_flag, tmem_base};
-      safe_recompute(w);
-      tc_fence_before();
-      __syncthreads();
-      if (*abort_flag) break;
-    }
-  }
+  // (What is needed from here on is worked out anew, so that it does not sit in a register until now.)
+  uint32_t smem_again = smem_u32(smem_raw);
+  asm volatile("" : "+r"(smem_again));
+  const FastSmem<MODE> end(static_cast<uint8_t*>(__cvta_shared_to_generic((smem_again + 1023) & ~1023u)));
+  if ((*end.n_bad | end.bad_cut[0] | end.bad_cut[1]) != 0 && !*end.abort_flag)             // block-uniform
+    recompute<PRESCALED, MODE>(tm_q, tm_k, tm_v, O, n_q, N, heads, plan, end.q);
 
   // ---------------------------------------------------------------- teardown
-  if (threadIdx.x == 0 && *abort_flag) {
+  if (threadIdx.x == 0 && *end.abort_flag) {
     atomicAdd(status, 1);
     if (cta_words != nullptr) {
-      RunIter<MODE> it(plan, block);
+      RunIter<MODE> it(plan, blockIdx.x);
       Run run;
       while (it.next(run)) cta_words[run.group] = 2;
     }
   }
-  if (warp == 1) { __syncwarp(); tc_fence_after(); tmem_dealloc(tmem_base, kAttTmemCols); }
+  if (threadIdx.x >> 5 == 1) { __syncwarp(); tc_fence_after(); tmem_dealloc(*end.tmem_slot, kAttTmemCols); }
 }
 
 }  // namespace
@@ -1173,14 +1107,14 @@ static int attention_kernel_attributes() {
   static PerDeviceOnce attr_once;            // the opt-in is a property of the kernel ON a device
   return per_device_once(attr_once, [](int dev) {
     HERO_CUDA_TRY(cudaFuncSetAttribute(tc_attention_safe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kAttSmem));
+                                       (int)kSafeSmem));
     for (auto kernel : {tc_attention_fast_kernel<false, kWhole>, tc_attention_fast_kernel<true, kWhole>,
                         tc_attention_fast_kernel<true, kCluster>, tc_attention_fast_kernel<true, kCut>})
       HERO_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFastSmem));
     for (int split = 2; split <= kMaxSplit; ++split) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3((unsigned)(split * 64));
-      cfg.blockDim = dim3(kFastThreads);
+      cfg.blockDim = dim3(kAttThreads);
       cfg.dynamicSmemBytes = kFastSmem;
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1233,7 +1167,7 @@ static PlannedAttention attention_plan(long long groups, int N, bool may_cluster
 }
 
 size_t tc_attention_part_bytes() { return (size_t)2 * num_sms() * kSlotFloats * sizeof(float); }
-size_t tc_attention_part_counters() { return (size_t)num_sms() * kFastSoftmaxWarps; }
+size_t tc_attention_part_counters() { return (size_t)num_sms() * kSoftmaxWarps; }
 
 // What a launch leaves in the counters when every block gives up with one part of each group counted in.
 static __global__ void strand_counters_kernel(AttentionParts parts, int n) {
@@ -1265,7 +1199,7 @@ int launch_tc_attention(const void* q, const void* k, const void* v, void* o, in
   return launch_kernel(!q_prescaled ? tc_attention_fast_kernel<false, kWhole>
                        : p.mode == kWhole ? tc_attention_fast_kernel<true, kWhole>
                        : p.mode == kCluster ? tc_attention_fast_kernel<true, kCluster> : tc_attention_fast_kernel<true, kCut>,
-                       (unsigned)p.plan.blocks, kFastThreads, kFastSmem, s,
+                       (unsigned)p.plan.blocks, kAttThreads, kFastSmem, s,
                        p.mode == kCluster ? (unsigned)p.plan.per_span : 1u, tm_q, tm_k, tm_v, (__nv_bfloat16*)o, n_q, N,
                        heads, p.plan, parts, d_status, cta_words);
 }
@@ -1281,7 +1215,7 @@ int launch_tc_attention_safe(const void* q, const void* k, const void* v, void* 
   HERO_TRY(attention_kernel_attributes());
   const long long groups = tc_attention_grid(B, n_q, heads);
   if (groups > 0x7FFFFFFFll) return HERO_ERR_ARG;
-  return launch_kernel(tc_attention_safe_kernel, (unsigned)groups, kAttThreads, kAttSmem, s, 1, tm_q, tm_k, tm_v,
+  return launch_kernel(tc_attention_safe_kernel, (unsigned)groups, kAttThreads, kSafeSmem, s, 1, tm_q, tm_k, tm_v,
                        (__nv_bfloat16*)o, n_q, N, heads, q_prescaled ? 1.0f : kScoreScaleLog2, d_status);
 }
 

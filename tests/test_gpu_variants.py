@@ -279,6 +279,25 @@ def test_a_launch_that_gave_up_does_not_reach_into_later_ones(then):
     hero.close()
 
 
+@pytest.mark.parametrize("B,n_q,N,heads", [(2, 300, 1000, 3), (1, 129, 97, 1), (1, 513, 2113, 2)])
+def test_what_a_thread_block_falls_back_to_is_the_exported_path(B, n_q, N, heads):
+    """Rows that the fixed scaling cannot hold (scores rise by far more than 2^100 behind the first 96 keys) come out of
+    the attention and of the running maximum alone the same, bit for bit."""
+    g = torch.Generator(device="cuda").manual_seed(N)
+    mk = lambda *s: torch.randn(*s, device="cuda", generator=g)
+    u = torch.nn.functional.normalize(mk(heads, 64), dim=1).view(-1)
+    q = (mk(B, n_q, heads * 64) + 40 * u).bfloat16()
+    j = torch.arange(N, device="cuda")[:, None]
+    k = (mk(B, N, heads * 64) + (j >= 96) * (40 + 20 * j / N) * u).bfloat16()
+    v, out, safe = mk(B, N, heads * 64).bfloat16(), torch.empty_like(q), torch.empty_like(q)
+    scores = q[:, :, :64].double() @ k[:, :, :64].double().mT * 0.18
+    assert float((scores[:, :, -1] - scores[:, :, :96].amax(-1)).amin()) > 100
+    H().hero_attention_bf16(q, k, v, out, heads)
+    H().hero_attention_bf16_safe(q, k, v, safe, heads)
+    H().hero_isolated_status()
+    assert torch.equal(out, safe)
+
+
 @pytest.mark.parametrize("dtype,over", [
     # the pass from block to block: one packet a lane and less, several with the last one partly there, the widest it serves
     # and one beyond; lists of different length from block to block, one list for all, empty lists, a collapsed deep stack
