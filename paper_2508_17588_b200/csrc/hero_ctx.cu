@@ -72,7 +72,7 @@ struct hero_ctx {
   float* mod = nullptr;                  // [n_blocks, B, n_mod*D] adaLN vectors, one slot per block
   int* pos_ws = nullptr;                 // [n_shallow, idx_cap] every video token's place in those lists, or -1
   int* idx_ws = nullptr;                 // [n_shallow, idx_cap] selection lists of the current step
-  AttentionParts att_parts = {};          // bf16: partial results of the attention's cut query groups
+  AttentionParts att_parts = {};          // partial results of the attention's cut query groups, where it may cut any
   int* d_status = nullptr;                // word 0: thread blocks that gave up on a wait
   void *x_stage = nullptr, *temb_stage = nullptr;
   int n_full = 0, s_prev = 0, s_last = 0;
@@ -557,7 +557,7 @@ int hero_init(hero_ctx** out, const hero_config* cfg, const hero_block_weights* 
   A((void**)&c->idx_ws, (size_t)(cfg->n_shallow > 0 ? cfg->n_shallow : 1) * c->idx_cap * sizeof(int));
   A((void**)&c->pos_ws, (size_t)(cfg->n_shallow > 0 ? cfg->n_shallow : 1) * c->idx_cap * sizeof(int));
   const size_t count_bytes = tc_attention_part_counters() * sizeof(unsigned long long);
-  if (cfg->dtype == HERO_DTYPE_BF16) {
+  if (cfg->dtype == HERO_DTYPE_BF16 && tc_attention_may_cut(cfg->batch, c->N, cfg->n_heads)) {
     A((void**)&c->att_parts.rows, tc_attention_part_bytes());
     A((void**)&c->att_parts.count, count_bytes);
   }

@@ -254,6 +254,7 @@ struct AttentionParts {
 int launch_tc_attention(const void* q, const void* k, const void* v, void* o, int B, int n_q, int N,
                         int heads, bool q_prescaled, const AttentionParts& parts, int* d_status, int* cta_words,
                         cudaStream_t s);
+bool tc_attention_may_cut(int B, int n_rows, int heads);     // with at most n_rows queries and keys
 size_t tc_attention_part_bytes();
 size_t tc_attention_part_counters();
 // (for the self-test of the give-up path)

@@ -1140,6 +1140,7 @@ long long tc_attention_grid(int B, int n_q, int heads) {
 //   * cutting the last round pays from about 64 key tiles on (a part costs some 5 us of fences, counting and adding up):
 //     1755 x 17776 x 48 x 2, 672 groups, 860 -> 851, 4388 x 17776 x 48 x 2, 1728 groups, 2087 -> 2069, the whole 3072-wide
 //     cached step 59.6 -> 58.7 ms; but 2970 x 3196 x 48 x 2 (34 tiles) 295 -> 299 and 2627 x 2627 x 18 x 2 84 -> 90.
+constexpr int kMinCutTiles = 64;
 struct PlannedAttention { AttentionMode mode; AttentionPlan plan; };
 static PlannedAttention attention_plan(long long groups, int N, bool may_cluster, bool may_cut) {
   const long long tiles = (N + kKT - 1) / kKT, sms = num_sms(), tail = groups % sms;
@@ -1157,7 +1158,7 @@ static PlannedAttention attention_plan(long long groups, int N, bool may_cluster
         plan.blocks = (int)(groups * split);
         return {kCluster, plan};
       }
-  if (may_cut && groups > sms && tail > 0 && tiles >= 64 && tail * tiles <= 0x3FFFFFFF) {
+  if (may_cut && groups > sms && tail > 0 && tiles >= kMinCutTiles && tail * tiles <= 0x3FFFFFFF) {
     plan.blocks = (int)sms;
     plan.rounds = (int)(groups / sms);
     spans(1, tail * tiles, sms);
@@ -1166,6 +1167,9 @@ static PlannedAttention attention_plan(long long groups, int N, bool may_cluster
   return {kWhole, plan};
 }
 
+bool tc_attention_may_cut(int B, int n_rows, int heads) {
+  return tc_attention_grid(B, n_rows, heads) > num_sms() && (n_rows + kKT - 1) / kKT >= kMinCutTiles;
+}
 size_t tc_attention_part_bytes() { return (size_t)2 * num_sms() * kSlotFloats * sizeof(float); }
 size_t tc_attention_part_counters() { return (size_t)num_sms() * kSoftmaxWarps; }
 

@@ -253,6 +253,24 @@ def test_rows_of_cut_groups_are_written_once_when_most_others_are_out_of_range()
     hero.close()
 
 
+def test_only_a_context_that_may_cut_groups_pays_for_it():
+    """The cut attention's workspace (20 MB) is allocated where the largest pass can take it, and nowhere else."""
+    def device_bytes(**over):
+        cfg = dict(dict(n_blocks=1, n_shallow=1, hidden=448, n_heads=7, head_dim=64, ffn_dim=32, temb_dim=8, batch=1, frames=8,
+                        grid_h=25, grid_w=31, n_text=0, patch_h=2, patch_w=2, ratio_num=1, ratio_den=8, quota_mode=0,
+                        warmup_full_steps=1, full_interval=0, dtype="bf16", has_gate=0, seed=5), **over)
+        w = {k: torch.zeros(s, device="cuda", dtype=torch.bfloat16) for k, s in S.weight_shapes(cfg).items()}
+        hero = H().Hero(cfg, [w])
+        total = hero.hero_device_bytes()
+        hero.close()
+        n = S.n_rows(cfg)
+        # K, V, two branches, three workspaces and the staged x; FFN rows; lists and counters
+        return total - 2 * cfg["batch"] * n * (8 * cfg["hidden"] + cfg["ffn_dim"])
+    assert device_bytes() > 15 << 20                                       # 175 groups on 148 SMs, 65 key tiles
+    for over in (dict(hidden=320, n_heads=5), dict(frames=7), dict(hidden=64, n_heads=1, frames=1)):
+        assert device_bytes(**over) < 1 << 20, over                        # 125 groups; 57 tiles; neither
+
+
 @pytest.mark.parametrize("then", ["nothing", "reset", "check"])
 def test_a_launch_that_gave_up_does_not_reach_into_later_ones(then):
     """What a cut attention keeps between thread blocks is left as by blocks that gave up half way: the next full pass is
