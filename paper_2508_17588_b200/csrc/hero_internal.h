@@ -21,6 +21,7 @@ void set_cuda_error(cudaError_t e, const char* what);
     cudaError_t e__ = (expr);                                \
     if (e__ != cudaSuccess) {                                \
       ::hero::set_cuda_error(e__, #expr);                    \
+      (void)cudaGetLastError();  /* (it is reported here, not by the caller's next CUDA call) */ \
       return HERO_ERR_CUDA;                                  \
     }                                                        \
   } while (0)

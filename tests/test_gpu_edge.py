@@ -265,6 +265,24 @@ def test_partial_refresh_needs_a_full_pass_or_planted_caches():
     hero.close()
 
 
+def test_a_refused_launch_is_reported_once_and_leaves_no_error_behind():
+    """More rows (8 x 524289) than the fp32 GEMM's grid has places for (65535 tiles of 64): CUDA refuses the launch, the call
+    says so, and the process' next CUDA call finds no error that is not its own."""
+    h = H()
+    cfgd = dict(n_blocks=1, n_shallow=1, hidden=32, n_heads=1, head_dim=32, ffn_dim=4, temb_dim=4, batch=8, frames=1,
+                grid_h=1, grid_w=524289, n_text=0, patch_h=1, patch_w=1, ratio_num=1, ratio_den=4, quota_mode=0,
+                warmup_full_steps=1, full_interval=0, dtype="fp32", has_gate=0, seed=1)
+    w = {k: torch.zeros(s, device="cuda") for k, s in S.weight_shapes(cfgd).items()}
+    hero = h.Hero(cfgd, [w])
+    x, t = torch.zeros(8, 524289, 32, device="cuda"), torch.zeros(8, 4, device="cuda")
+    with pytest.raises(h.HeroError) as e:
+        hero.hero_refresh_block(0, x, t)
+    assert e.value.code == -5
+    assert float((x[0, 0] + 1).sum()) == 32.0
+    hero.hero_check_status()
+    hero.close()
+
+
 def test_a_wait_that_runs_out_is_reported_once_and_the_next_calls_are_healthy():
     """The give-up path, made to happen harmlessly: one thread block waits 50 microseconds on a barrier
     nobody completes, through the helper the tensor-core kernels use; it must raise the status word and
