@@ -1022,6 +1022,13 @@ int launch_gather_ln_modulate(const void* x, const void* add, const int* idx, co
   if (vec_ok && D / per <= 32 * kLnMaxPackets)
     return bf16 ? gather_ln_dispatch<__nv_bfloat16>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s)
                 : gather_ln_dispatch<float>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s);
+  // The widest row, 12288 features, fills the 48 KB a kernel may have without an opt-in; the reduction's words come on top.
+  static PerDeviceOnce once;
+  HERO_TRY(per_device_once(once, [](int) {
+    HERO_CUDA_TRY(cudaFuncSetAttribute(gather_ln_modulate_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 48 * 1024));
+    HERO_CUDA_TRY(cudaFuncSetAttribute(gather_ln_modulate_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 48 * 1024));
+    return HERO_OK;
+  }));
   const size_t smem = (size_t)D * sizeof(float);
   if (bf16)
     HERO_TRY(launch_kernel(gather_ln_modulate_kernel<__nv_bfloat16>, (unsigned)rows, kLnThreads, smem, s, 1,
