@@ -336,7 +336,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-  const int m_tiles = (M + 2 * kBM - 1) / (2 * kBM), n_tiles = (Nout + BN - 1) / BN;
+  const int m_tiles = (M - 1) / (2 * kBM) + 1, n_tiles = (Nout + BN - 1) / BN;
   const int n_tiles_total = m_tiles * n_tiles;
   const int k_blocks = (K + kBK - 1) / kBK;
 
@@ -769,7 +769,7 @@ int launch_pair(const CUtensorMap& tm_a, const CUtensorMap& tm_w, const void* bi
                                        (int)PairCfg<BN>::kSmem));
     return HERO_OK;
   }));
-  const int tiles = ((M + 2 * kBM - 1) / (2 * kBM)) * ((Nout + BN - 1) / BN);
+  const int tiles = ((M - 1) / (2 * kBM) + 1) * ((Nout + BN - 1) / BN);
   const int pairs = tiles < num_sms() / 2 ? tiles : num_sms() / 2;
   QkParam<QK> param;
   if constexpr (QK) static_cast<QkEpilogue&>(param) = qk;
