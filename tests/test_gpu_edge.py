@@ -323,3 +323,69 @@ def test_a_wait_that_runs_out_is_reported_once_and_the_next_calls_are_healthy():
         hero.hero_check_status()
         assert rel_l2(to_host(x), want) <= 3e-2, s
     hero.close()
+
+
+def _small_model(seed, dtype="bf16"):
+    h = H()
+    cfgd = dict(n_blocks=4, n_shallow=2, hidden=256, n_heads=4, head_dim=64, ffn_dim=768, temb_dim=64, batch=2, frames=3,
+                grid_h=9, grid_w=11, n_text=10, patch_h=2, patch_w=2, ratio_num=1, ratio_den=4, quota_mode=0,
+                warmup_full_steps=2, full_interval=3, dtype=dtype, has_gate=1, seed=seed)
+    w = [h.device_weights(S.block_weights(cfgd, l), dtype) for l in range(4)]
+    return cfgd, w, to_dev(S.tokens(cfgd), dtype), [to_dev(S.temb(cfgd, s), dtype) for s in range(6)]
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+def test_weights_rewritten_between_two_steps_are_the_ones_the_next_step_uses(dtype):
+    """Kernels fetch weights before they wait for the kernel in front of them: a step behind a copy into the weights on the
+    same stream sees all of it, in its first block and in its last."""
+    h = H()
+    cfgd, w, x0, temb = _small_model(3, dtype)
+    other = _small_model(4, dtype)[1]
+    want = []
+    for weights in (w, other):
+        hero = h.Hero(cfgd, weights)
+        x = x0.clone()
+        hero.hero_step(0, x, temb[0])
+        want.append(x)
+        hero.close()
+    assert not torch.equal(want[0], want[1])
+    kept = [{k: t.clone() for k, t in block.items()} for block in w]
+    hero = h.Hero(cfgd, w)
+    for turn in range(6):
+        hero.hero_reset()
+        for mine, new in zip(w, kept if turn % 2 else other):
+            for k in mine:
+                mine[k].copy_(new[k])
+        x = x0.clone()
+        hero.hero_step(0, x, temb[0])
+        assert torch.equal(x, want[0 if turn % 2 else 1]), turn
+    hero.close()
+
+
+def test_two_contexts_on_two_streams_at_once():
+    """Their kernels share the chip, tensor memory included; each computes what it does alone."""
+    h = H()
+    models = [_small_model(seed) for seed in (5, 6)]
+    alone, both = [], []
+    for out, streams in ((alone, [torch.cuda.current_stream()] * 2), (both, [torch.cuda.Stream(), torch.cuda.Stream()])):
+        torch.cuda.synchronize()
+        heroes = []
+        for (cfgd, w, x0, temb), st in zip(models, streams):
+            with torch.cuda.stream(st):
+                heroes.append(h.Hero(cfgd, w))
+                out.append([])
+        for rep in range(8):
+            for s in range(6):
+                for hero, (cfgd, w, x0, temb), st, res in zip(heroes, models, streams, out):
+                    with torch.cuda.stream(st):
+                        if s == 0:
+                            hero.hero_reset()
+                        x = x0.clone()
+                        hero.hero_step(s, x, temb[s])
+                        res.append(x)
+        torch.cuda.synchronize()
+        for hero in heroes:
+            hero.hero_check_status()
+            hero.close()
+    for a, b in zip(alone, both):
+        assert len(a) == 48 and all(torch.equal(x, y) for x, y in zip(a, b))
