@@ -20,8 +20,7 @@
  *   - Weight matrices are row-major [out_features, in_features] (K contiguous).
  *     Device pointers must be 16-byte aligned; in bf16 mode hidden and ffn_dim must be
  *     multiples of 32, temb_dim a multiple of 8 and head_dim must be 64.  batch * temb_dim
- *     is at most 12288, and hidden at most 12288 unless the run is bf16 with hidden 1024,
- *     2048, 3072 or 4096 (shared-memory limits of the streaming kernels); hero_init
+ *     and hidden are at most 12288 each (shared memory of the streaming kernels); hero_init
  *     refuses anything else with HERO_ERR_ARG / HERO_ERR_ALIGN.
  *   - All work is enqueued on the CUDA stream given to hero_init; no call
  *     synchronises the device unless stated.  Calls on one context must not
@@ -254,7 +253,9 @@ int hero_attention_bf16_safe(const void *d_q, const void *d_k, const void *d_v, 
  * hero_step and hero_refresh_block use (their QKV projection writes q that way): the kernel then takes
  * 2^score as it stands, with no row maximum at all.  Exact while every row's largest score lies within
  * about +-100 (bf16 and fp32 share the exponent range); a row sum outside [2^-100, 2^100) makes its thread
- * block recompute, as above.  Shapes, layouts and errors as hero_attention_bf16. */
+ * block recompute, as above.  Shapes, layouts and errors as hero_attention_bf16.  (A context's launches over long key
+ * sequences may besides cut the last query groups over all thread blocks, which takes a workspace that this call, which
+ * belongs to nobody, does not have: it keeps groups whole or shares them within a cluster.) */
 int hero_attention_bf16_q_scaled(const void *d_q, const void *d_k, const void *d_v, void *d_o,
                                  int B, int n_q, int N, int heads, void *stream);
 

@@ -37,6 +37,7 @@ constexpr unsigned kAllCaches = 0xFu;
 
 using namespace hero;
 
+constexpr int kMaxSmemFloats = 12288;          // 48 KB
 constexpr int kHostPieces = 8;                 // pieces of x copied back while the next one is computed
 constexpr long long kHostPieceAlign = 4096;    // elements; keeps every piece 16-byte aligned in both dtypes
 
@@ -433,14 +434,9 @@ int validate(const hero_config* g) {
     if (g->head_dim != 32 && g->head_dim != 64 && g->head_dim != 128) return HERO_ERR_ARG;
     if (g->hidden % 4 || g->ffn_dim % 4 || g->temb_dim % 4) return HERO_ERR_ALIGN;
   }
-  // dynamic shared memory the streaming kernels take without an opt-in (48 KB): SiLU(temb) of the whole batch
-  // in the adaLN kernels, one fp32 row in the generic LayerNorm prologue (the bf16 warp-per-row kernel, used
-  // for hidden = 1024 / 2048 / 3072 / 4096, needs none)
-  constexpr long long kPlainSmem = 48 * 1024;
-  if ((long long)g->batch * g->temb_dim * 4 > kPlainSmem) return HERO_ERR_ARG;
-  const bool warp_ln = g->dtype == HERO_DTYPE_BF16 &&
-                       (g->hidden == 1024 || g->hidden == 2048 || g->hidden == 3072 || g->hidden == 4096);
-  if (!warp_ln && (long long)g->hidden * 4 > kPlainSmem) return HERO_ERR_ARG;
+  // dynamic shared memory of the streaming kernels: SiLU(temb) of the whole batch in the adaLN kernels, one fp32 row in the
+  // LayerNorm of rows too wide for a warp's registers (see launch_gather_ln_modulate)
+  if ((long long)g->batch * g->temb_dim > kMaxSmemFloats || g->hidden > kMaxSmemFloats) return HERO_ERR_ARG;
   const long long n_video = (long long)g->frames * g->grid_h * g->grid_w;
   if (n_video + g->n_text > (1ll << 30)) return HERO_ERR_ARG;
   return HERO_OK;
@@ -896,8 +892,7 @@ int hero_gather_ln_modulate(const void* d_x, const void* d_add, const int* d_idx
   if (!d_x || !d_shift || !d_scale || !d_out) return HERO_ERR_ARG;
   if (!aligned16(d_x) || !aligned16(d_out) || (d_add && !aligned16(d_add))) return HERO_ERR_ALIGN;
   if (D % (dtype == HERO_DTYPE_BF16 ? 8 : 4)) return HERO_ERR_ALIGN;
-  const bool warp_ln = dtype == HERO_DTYPE_BF16 && (D == 1024 || D == 2048 || D == 3072 || D == 4096);
-  if (!warp_ln && (long long)D * 4 > 48 * 1024) return HERO_ERR_ARG;      // one fp32 row of shared memory
+  if (D > kMaxSmemFloats) return HERO_ERR_ARG;               // one fp32 row of shared memory
   return launch_gather_ln_modulate(d_x, d_add, d_idx, d_shift, d_scale, mod_ld, d_out, B, N, n_sel, D, 1e-5f, dtype,
                                    (cudaStream_t)stream);
 }
