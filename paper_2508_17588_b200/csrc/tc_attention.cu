@@ -25,11 +25,11 @@
 //    That is exact as long as no later score exceeds the first tile's maximum by more than 2^100
 //    (69 in natural-log units; bf16 and fp32 share their exponent range, so a large p loses no
 //    precision, and the final division by the row sum makes the result independent of the maximum
-//    used).  The row sum tells whether that held; a CTA in which it did not says so in its status word.
+//    used).  The row sum tells whether that held; slices of 32 rows in which it did not go to the safe path.
 //    In the step the QKV projection hands over q already multiplied by log2(e) / sqrt(64), so a score is
 //    the exponent of its weight: that instantiation (PRESCALED) takes p = 2^s as it stands - no maximum,
 //    no first-tile exchange, no multiply-add per pair of scores - and is exact while a row's largest score
-//    stays within about +-100; its row sum must then lie in [2^-100, 2^100), else the CTA is marked.
+//    stays within about +-100; its row sum must then lie in [2^-100, 2^100), else the same.
 //  * The safe path (safe_roles) keeps a running maximum that moves whenever a tile exceeds it by 2^8, rescaling the
 //    accumulator in TMEM.  The warps are those of the fast kernel; the two threads of a row trade their halves' maxima for
 //    every key tile.  A thread block of the fast kernel whose row sums say that the range assumption failed recomputes its
