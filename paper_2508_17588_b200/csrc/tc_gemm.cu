@@ -98,12 +98,6 @@ __device__ __forceinline__ RowOut row_out(const GemmOut& out, int m, int M) {
   return r;
 }
 
-__device__ __forceinline__ void st_global_v8(void* p, const uint32_t* w) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]),
-               "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
-               : "memory");
-}
-
 // Finish NC accumulator columns [n0, n0 + NC) of one row, all of one segment: bias (fp32, staged in shared memory),
 // activation, scale or gate, bf16, full 32-byte sectors per lane (16-byte stores where the destination is not 32-byte
 // aligned or ends inside the columns).

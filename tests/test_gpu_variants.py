@@ -373,3 +373,21 @@ def test_pass_from_block_to_block(dtype, over):
     if sparse:
         assert {0, 1} == {n for step in lengths for n in step}
     hero.close()
+
+
+@pytest.mark.parametrize("B,n_q,N,heads", [(1, 300, 97, 1), (2, 77, 600, 3), (1, 371, 1562, 12), (2, 640, 6200, 30)],
+                         ids=["one_tile", "cluster", "cluster_of_four", "whole"])
+def test_attention_output_at_any_16_byte_boundary(B, n_q, N, heads):
+    """Rows leave in 32-byte stores where the output allows it, else in 16-byte ones: the same values, nothing beside them."""
+    g = torch.Generator(device="cuda").manual_seed(n_q)
+    q, k, v = (torch.randn(B, n, heads * 64, device="cuda", generator=g).bfloat16() for n in (n_q, N, N))
+    q = q * 0.18
+    size = B * n_q * heads * 64
+    outs = []
+    for shift in (16, 8):                                  # elements: 32 bytes, 16 bytes
+        flat = torch.full((size + 32,), 7.0, device="cuda", dtype=torch.bfloat16)
+        H().hero_attention_bf16_q_scaled(q, k, v, flat[shift:shift + size].view(B, n_q, heads * 64), heads)
+        H().hero_isolated_status()
+        assert bool((flat[:shift] == 7.0).all()) and bool((flat[shift + size:] == 7.0).all())
+        outs.append(flat[shift:shift + size].clone())
+    assert torch.equal(outs[0], outs[1])
