@@ -261,12 +261,14 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
     HERO_LAUNCH(c, HERO_PROF_GATHER_LN, launch_gather_rows(host_rows, d_idx, c->ws_o, B, N, n_sel, D, g.dtype, c->stream));
     HERO_LAUNCH(c, HERO_PROF_GATHER_LN,
                 launch_gather_ln_modulate(c->ws_o, nullptr, nullptr, shift1, scale1, mod_ld, c->ws_a, B, n_sel, n_sel, D,
-                                          1e-5f, g.dtype, c->stream));
+                                          1e-5f, g.dtype, kLnModSettled, c->stream));
     HERO_LAUNCH(c, HERO_PROF_GATHER_LN, launch_scatter_rows(c->ws_o, d_idx, d_x, B, N, n_sel, D, g.dtype, c->stream));
   } else {
+    // (in a step only the first block's vectors and list may come from the kernel in front)
     HERO_LAUNCH(c, HERO_PROF_GATHER_LN,
                 launch_gather_ln_modulate(host_rows ? host_rows : d_x, nullptr, d_idx, shift1, scale1, mod_ld, c->ws_a, B,
-                                          N, n_sel, D, 1e-5f, g.dtype, c->stream));
+                                          N, n_sel, D, 1e-5f, g.dtype,
+                                          in_step && block > 0 ? kLnModSettled : kLnNothingSettled, c->stream));
   }
   GemmOut o_qkv = {};
   o_qkv.ptr[0] = c->ws_q; o_qkv.ld[0] = D; o_qkv.scatter[0] = 0;
@@ -312,10 +314,11 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
   o_attn.gate = gate1; o_attn.gate_ld = mod_ld;
   HERO_TRY(run_gemm(c, c->ws_o, w.w_o, w.b_o, M, D, D, o_attn));
 
-  // FFN branch: its input rows are x + G_attn (the residual add is applied to x once, below)
+  // FFN branch: its input rows are x + G_attn (the residual add is applied to x once, below).  Only G_attn is the kernel in
+  // front's; x, list and vectors were there before the projections and the attention.
   HERO_LAUNCH(c, HERO_PROF_GATHER_LN,
               launch_gather_ln_modulate(d_x, ga, d_idx, shift2, scale2, mod_ld, c->ws_a, B, N, n_sel, D, 1e-5f,
-                                        g.dtype, c->stream));
+                                        g.dtype, kLnRowsSettled, c->stream));
   GemmOut o_up = {};
   o_up.ptr[0] = c->ws_u; o_up.ld[0] = F; o_up.scatter[0] = 0;
   o_up.seg_cols = F; o_up.idx = d_idx; o_up.n_sel = n_sel; o_up.n_rows = N; o_up.act = 1;
@@ -894,7 +897,7 @@ int hero_gather_ln_modulate(const void* d_x, const void* d_add, const int* d_idx
   if (D % (dtype == HERO_DTYPE_BF16 ? 8 : 4)) return HERO_ERR_ALIGN;
   if (D > kMaxSmemFloats) return HERO_ERR_ARG;               // one fp32 row of shared memory
   return launch_gather_ln_modulate(d_x, d_add, d_idx, d_shift, d_scale, mod_ld, d_out, B, N, n_sel, D, 1e-5f, dtype,
-                                   (cudaStream_t)stream);
+                                   kLnNothingSettled, (cudaStream_t)stream);
 }
 
 // The isolated tensor-core calls own a status word each; a timeout is reported on the next call.

@@ -222,9 +222,12 @@ int launch_modulation_batch(const void* temb, const ModBatch& batch, int B, int 
 int launch_modulation(const void* temb, const void* w_mod, const void* b_mod, float* mod, int B,
                       int n_out, int E, int dtype, cudaStream_t s);
 // a[m,:] = LN(x[row(m),:] (+ add[row(m),:])) * (1 + scale[b,:]) + shift[b,:]
+// settled: what was complete before the kernel in front on the stream was placed and need not be waited for: nothing, the
+// vectors and the list, or the rows of x as well.
+enum LnSettled { kLnNothingSettled, kLnModSettled, kLnRowsSettled };
 int launch_gather_ln_modulate(const void* x, const void* add, const int* idx, const float* shift,
                               const float* scale, int mod_ld, void* a, int B, int N, int n_sel, int D,
-                              float eps, int dtype, cudaStream_t s);
+                              float eps, int dtype, int settled, cudaStream_t s);
 
 // x = (x + ga) + gf for all rows and the LayerNorm + modulate of the rows that the next
 // block refreshes (pos: as SelectBatch::pos; null: all rows) into a [B, n_sel, D].  Rows as wide as residual_ln_serves.

@@ -589,8 +589,8 @@ gather_ln_modulate_kernel(const T* __restrict__ x, const T* __restrict__ add, co
 __host__ __device__ constexpr int ln_full_chunks(int vpl) {
   return vpl <= 6 ? vpl - 1 : (vpl == 8 ? 6 : (vpl == 10 ? 8 : (vpl == 12 ? 10 : 12)));
 }
-__host__ __device__ constexpr int ln_ctas_per_sm(int vpl) {      // what the registers of a row allow
-  return vpl <= 2 ? 6 : (vpl <= 4 ? 4 : (vpl <= 6 ? 3 : (vpl <= 12 ? 2 : 1)));
+__host__ __device__ constexpr int ln_ctas_per_sm(int vpl, bool one) {      // what the registers of a row allow
+  return vpl <= 2 && !one ? 6 : (vpl <= 4 ? 4 : (vpl <= 6 ? 3 : (vpl <= 12 ? 2 : 1)));
 }
 // One batch item's (1 + scale) and shift into shared memory: [2 * Q][packets] float4.
 template <typename T>
@@ -651,12 +651,14 @@ __device__ __forceinline__ void ln_finish_row(const float (&f)[VPL][Vec<T>::N], 
 }
 
 // (EXACT: the row has exactly 32 * VPL packets, nothing is predicated; the wide rows have no registers to spare for it.)
-template <typename T, int VPL, bool EXACT>
-__global__ void __launch_bounds__(256, ln_ctas_per_sm(VPL))
+// `settled` (launch_gather_ln_modulate) says what was complete before the kernel in front was placed: those loads go out
+// before the wait for that kernel, so that of the chain vectors, list, row, row to add only the last link is left behind it.
+// A row is fetched so early where every warp has one at most (ONE): ahead of a loop it would not stay in registers.
+template <typename T, int VPL, bool EXACT, bool ONE>
+__global__ void __launch_bounds__(256, ln_ctas_per_sm(VPL, ONE))
 gather_ln_modulate_warp_kernel(const T* __restrict__ x, const T* __restrict__ add, const int* __restrict__ idx,
                                const float* __restrict__ shift, const float* __restrict__ scale, int mod_ld,
-                               T* __restrict__ a, int N, int n_sel, int B, int D, float eps) {
-  stream_order();
+                               T* __restrict__ a, int N, int n_sel, int B, int D, float eps, int settled) {
   using V = Vec<T>;
   constexpr int kFull = EXACT ? VPL : ln_full_chunks(VPL);    // chunks of 32 packets that every row it serves has
   const int packets = EXACT ? VPL * 32 : D / V::N;
@@ -664,14 +666,26 @@ gather_ln_modulate_warp_kernel(const T* __restrict__ x, const T* __restrict__ ad
   extern __shared__ float4 s_mod[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = blockIdx.x % B, slot = blockIdx.x / B, slots = gridDim.x / B;
-  ln_stage_modulation<T>(s_mod, scale + (long long)b * mod_ld, shift + (long long)b * mod_ld, packets);
-  for (int i = slot * 8 + warp; i < n_sel; i += slots * 8) {
-    const long long row = (long long)b * N + (idx ? __ldg(idx + i) : i);
-    const V* xr = reinterpret_cast<const V*>(x + row * D);
-    V raw[VPL];
+  const int first = slot * 8 + warp;
+  long long row = 0;
+  V raw[VPL];
+  auto find_row = [&](int i) { row = (long long)b * N + (idx ? __ldg(idx + i) : i); };
+  auto load = [&](const T* from) {
+    const V* r = reinterpret_cast<const V*>(from + row * D);
 #pragma unroll
     for (int c = 0; c < VPL; ++c)
-      if (c < kFull || c * 32 + lane < packets) raw[c].raw = __ldcs(&xr[c * 32 + lane].raw);
+      if (c < kFull || c * 32 + lane < packets) raw[c].raw = __ldcs(&r[c * 32 + lane].raw);
+  };
+  if (settled < kLnModSettled) stream_order();
+  if (ONE && first < n_sel) {                // warp-uniform
+    find_row(first);
+    if (settled == kLnRowsSettled) load(x);
+  }
+  ln_stage_modulation<T>(s_mod, scale + (long long)b * mod_ld, shift + (long long)b * mod_ld, packets);
+  if (settled >= kLnModSettled) stream_order();
+  for (int i = first; i < n_sel; i += slots * 8) {
+    if (!ONE) find_row(i);
+    if (!ONE || settled != kLnRowsSettled) load(x);
     float f[VPL][V::N];
 #pragma unroll
     for (int c = 0; c < VPL; ++c) {
@@ -683,10 +697,7 @@ gather_ln_modulate_warp_kernel(const T* __restrict__ x, const T* __restrict__ ad
       }
     }
     if (add) {
-      const V* ar = reinterpret_cast<const V*>(add + row * D);
-#pragma unroll
-      for (int c = 0; c < VPL; ++c)
-        if (c < kFull || c * 32 + lane < packets) raw[c].raw = __ldcs(&ar[c * 32 + lane].raw);
+      load(add);
 #pragma unroll
       for (int c = 0; c < VPL; ++c) {
         if (c < kFull || c * 32 + lane < packets) {
@@ -698,6 +709,7 @@ gather_ln_modulate_warp_kernel(const T* __restrict__ x, const T* __restrict__ ad
       }
     }
     ln_finish_row<T, VPL, kFull>(f, s_mod, packets, D, eps, lane, a + ((long long)b * n_sel + i) * D);
+    if (ONE) break;
   }
 }
 
@@ -708,31 +720,44 @@ gather_ln_modulate_warp_kernel(const T* __restrict__ x, const T* __restrict__ ad
 // 8 blocks of 5820 x 1024 0.8, of 4 blocks of 1562 x 768 1.1.  A collapsed deep stack's blocks, which add a fp32 sum to the
 // streams of a row, keep the two passes (16 blocks of 5254 x 1152: 4.46 ms apart, 4.47 in one).
 constexpr int rln_ctas_per_sm(int vpl) { return vpl <= 3 ? 3 : 2; }      // what the registers of three rows allow
-template <typename T, int VPL>
+template <typename T, int VPL, bool ONE>
 __global__ void __launch_bounds__(256, rln_ctas_per_sm(VPL))
 residual_ln_kernel(T* __restrict__ x, const T* __restrict__ ga, const T* __restrict__ gf,
                    const int* __restrict__ pos, int n_text, const float* __restrict__ shift, const float* __restrict__ scale,
                    int mod_ld, T* __restrict__ a, int N, int n_sel, int B, int D, float eps) {
-  stream_order();
   using V = Vec<T>;
   constexpr int kFull = ln_full_chunks(VPL);
   const int packets = D / V::N;
   extern __shared__ float4 s_mod[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = blockIdx.x % B, slot = blockIdx.x / B, slots = gridDim.x / B;
-  ln_stage_modulation<T>(s_mod, scale + (long long)b * mod_ld, shift + (long long)b * mod_ld, packets);
-  for (int i = slot * 8 + warp; i < N; i += slots * 8) {
-    const int place = pos == nullptr ? i : (i < n_text ? -1 : __ldg(pos + i - n_text));
-    const long long first = ((long long)b * N + i) * D;
-    V* xr = reinterpret_cast<V*>(x + first);
-    const V* ar = reinterpret_cast<const V*>(ga + first);
-    const V* fr = reinterpret_cast<const V*>(gf + first);
-    V vx[VPL], va[VPL], vf[VPL];
+  // The kernel in front writes gf (the FFN's down-projection).  All else has been complete since before that kernel was
+  // placed (x was last written a block ago, ga three launches ago, the lists and the vectors at the start of the step) and is
+  // fetched before the wait, the rows of x and ga where a warp has one row at most (ONE).
+  int place = 0;
+  V* xr = nullptr;
+  V vx[VPL], va[VPL], vf[VPL];
+  auto load_early = [&](int i) {
+    place = pos == nullptr ? i : (i < n_text ? -1 : __ldg(pos + i - n_text));
+    xr = reinterpret_cast<V*>(x + ((long long)b * N + i) * D);
+    const V* ar = reinterpret_cast<const V*>(ga + ((long long)b * N + i) * D);
 #pragma unroll
     for (int c = 0; c < VPL; ++c)
-      if (c < kFull || c * 32 + lane < packets) {
-        vx[c] = ld_stream(xr + c * 32 + lane); va[c] = ld_stream(ar + c * 32 + lane); vf[c] = ld_stream(fr + c * 32 + lane);
-      }
+      if (c < kFull || c * 32 + lane < packets) { vx[c] = ld_stream(xr + c * 32 + lane); va[c] = ld_stream(ar + c * 32 + lane); }
+  };
+  auto load_late = [&](int i) {
+    const V* fr = reinterpret_cast<const V*>(gf + ((long long)b * N + i) * D);
+#pragma unroll
+    for (int c = 0; c < VPL; ++c)
+      if (c < kFull || c * 32 + lane < packets) vf[c] = ld_stream(fr + c * 32 + lane);
+  };
+  const int first = slot * 8 + warp;
+  if (ONE && first < N) load_early(first);
+  ln_stage_modulation<T>(s_mod, scale + (long long)b * mod_ld, shift + (long long)b * mod_ld, packets);
+  stream_order();
+  for (int i = first; i < N; i += slots * 8) {
+    if (!ONE) load_early(i);
+    load_late(i);
     float f[VPL][V::N];
 #pragma unroll
     for (int c = 0; c < VPL; ++c) {
@@ -750,6 +775,7 @@ residual_ln_kernel(T* __restrict__ x, const T* __restrict__ ga, const T* __restr
       }
     }
     if (place >= 0) ln_finish_row<T, VPL, kFull>(f, s_mod, packets, D, eps, lane, a + ((long long)b * n_sel + place) * D);
+    if (ONE) break;
   }
 }
 
@@ -757,7 +783,8 @@ template <typename T, int VPL>
 int residual_ln_launch(void* x, const void* ga, const void* gf, const int* pos, int n_text, const float* shift,
                        const float* scale, int mod_ld, void* a, int N, int n_sel, int B, int D, float eps, cudaStream_t s) {
   const int resident = (num_sms() * rln_ctas_per_sm(VPL) + B - 1) / B, need = (N + 7) / 8;
-  return launch_kernel(residual_ln_kernel<T, VPL>, (unsigned)((need < resident ? need : resident) * B), 256,
+  return launch_kernel(need <= resident ? residual_ln_kernel<T, VPL, true> : residual_ln_kernel<T, VPL, false>,
+                       (unsigned)((need < resident ? need : resident) * B), 256,
                        (size_t)2 * D * sizeof(float), s, 1, (T*)x, (const T*)ga, (const T*)gf, pos, n_text, shift, scale,
                        mod_ld, (T*)a, N, n_sel, B, D, eps);
 }
@@ -775,30 +802,31 @@ int residual_ln_dispatch(void* x, const void* ga, const void* gf, const int* pos
 
 template <typename T, int VPL>
 int gather_ln_warp(const void* x, const void* add, const int* idx, const float* shift, const float* scale, int mod_ld,
-                   void* a, int N, int n_sel, int B, int D, float eps, cudaStream_t s) {
+                   void* a, int N, int n_sel, int B, int D, float eps, int settled, cudaStream_t s) {
   // the same number of CTAs for every batch item, at most as many as stay resident
-  const int resident = (num_sms() * ln_ctas_per_sm(VPL) + B - 1) / B;
   const int need = (n_sel + 7) / 8;
+  const bool one = VPL < 8 && need <= num_sms() * ln_ctas_per_sm(VPL, true) / B;
+  const int resident = (num_sms() * ln_ctas_per_sm(VPL, one) + B - 1) / B;
   const unsigned grid = (unsigned)((need < resident ? need : resident) * B);
   const size_t smem = (size_t)2 * D * sizeof(float);
-  bool exact = false;
-  if constexpr (VPL >= 8) exact = D == VPL * 32 * Vec<T>::N;
-  if (exact)
-    HERO_TRY(launch_kernel(gather_ln_modulate_warp_kernel<T, VPL, VPL >= 8>, grid, 256, smem, s, 1, (const T*)x,
-                           (const T*)add, idx, shift, scale, mod_ld, (T*)a, N, n_sel, B, D, eps));
-  else
-    HERO_TRY(launch_kernel(gather_ln_modulate_warp_kernel<T, VPL, false>, grid, 256, smem, s, 1, (const T*)x,
-                           (const T*)add, idx, shift, scale, mod_ld, (T*)a, N, n_sel, B, D, eps));
-  return HERO_OK;
+  auto kernel = gather_ln_modulate_warp_kernel<T, VPL, false, false>;
+  if constexpr (VPL >= 8) {
+    if (D == VPL * 32 * Vec<T>::N) kernel = gather_ln_modulate_warp_kernel<T, VPL, true, false>;
+  } else {
+    if (one) kernel = gather_ln_modulate_warp_kernel<T, VPL, false, true>;
+  }
+  return launch_kernel(kernel, grid, 256, smem, s, 1, (const T*)x, (const T*)add, idx, shift, scale, mod_ld, (T*)a, N, n_sel,
+                       B, D, eps, settled);
 }
 
 // Rows of at most 16 packets a lane; wider ones go through shared memory (gather_ln_modulate_kernel).
 constexpr int kLnMaxPackets = 16;
 template <typename T>
 int gather_ln_dispatch(const void* x, const void* add, const int* idx, const float* shift, const float* scale, int mod_ld,
-                       void* a, int N, int n_sel, int B, int D, float eps, cudaStream_t s) {
+                       void* a, int N, int n_sel, int B, int D, float eps, int settled, cudaStream_t s) {
   const int vpl = (D / Vec<T>::N + 31) / 32;
-#define HERO_LN(V) if (vpl <= V) return gather_ln_warp<T, V>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s)
+#define HERO_LN(V) \
+  if (vpl <= V) return gather_ln_warp<T, V>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, D, eps, settled, s)
   HERO_LN(1); HERO_LN(2); HERO_LN(3); HERO_LN(4); HERO_LN(5); HERO_LN(6); HERO_LN(8); HERO_LN(10); HERO_LN(12); HERO_LN(16);
 #undef HERO_LN
   return HERO_ERR_ARG;
@@ -1011,7 +1039,7 @@ int launch_residual_ln(void* x, const void* ga, const void* gf, const int* pos, 
 
 int launch_gather_ln_modulate(const void* x, const void* add, const int* idx, const float* shift,
                               const float* scale, int mod_ld, void* a, int B, int N, int n_sel, int D, float eps,
-                              int dtype, cudaStream_t s) {
+                              int dtype, int settled, cudaStream_t s) {
   const long long rows = (long long)B * n_sel;
   if (rows == 0) return HERO_OK;
   const bool bf16 = dtype == HERO_DTYPE_BF16;
@@ -1020,8 +1048,8 @@ int launch_gather_ln_modulate(const void* x, const void* add, const int* idx, co
   // the warp kernel reads the adaLN vectors as float4: every item's slice starts 16-byte aligned when mod_ld % 4 == 0
   const bool vec_ok = mod_ld % 4 == 0 && ((reinterpret_cast<uintptr_t>(shift) | reinterpret_cast<uintptr_t>(scale)) & 15) == 0;
   if (vec_ok && D / per <= 32 * kLnMaxPackets)
-    return bf16 ? gather_ln_dispatch<__nv_bfloat16>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s)
-                : gather_ln_dispatch<float>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s);
+    return bf16 ? gather_ln_dispatch<__nv_bfloat16>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, D, eps, settled, s)
+                : gather_ln_dispatch<float>(x, add, idx, shift, scale, mod_ld, a, N, n_sel, B, D, eps, settled, s);
   // The widest row, 12288 features, fills the 48 KB a kernel may have without an opt-in; the reduction's words come on top.
   static PerDeviceOnce once;
   HERO_TRY(per_device_once(once, [](int) {
