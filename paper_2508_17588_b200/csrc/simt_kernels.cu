@@ -32,43 +32,55 @@ __device__ __forceinline__ void dot4(float2& acc, const float4& a, const float4&
 }
 
 // ---------------------------------------------------------------------------------------------------------------
-// C[M, Nout] = A[M, K] W[Nout, K]^T + bias.  Tile BM x BN per CTA of 256 threads in KG groups: group g multiplies the
-// g-th 32 of every KG * 32 k (so that a problem of few tiles still keeps all four schedulers of an SM busy), each
-// thread TM x TN outputs, rows ty + i * (BM / TM) and columns tx + j * (BN / TN).  The groups' sums are added in group
-// order.  Three chunks of k in the ring; two CTAs share an SM (eight warps alone keep its FMA pipe 46 % busy): 240 tiles of
-// 64 x 64 x 512 in 42 us, 50 with the registers of one CTA a SM.
+// C[M, Nout] = A[M, K] W[Nout, K]^T + bias.  Tile BM x BN per CTA, in KG groups of threads: group g multiplies the g-th 32
+// of every KG * 32 k, each thread TM x TN outputs, rows ty + i * (BM / TM) and columns tx + j * (BN / TN).  A cluster of
+// `split` CTAs shares a tile where that evens out the SMs' shares, each taking a run of the chunks of k.  The sums of all
+// groups and CTAs go through shared memory (a row of the tile is then stored by neighbouring lanes) and are added in
+// order, groups before CTAs, so that a result does not depend on timing.
 // ---------------------------------------------------------------------------------------------------------------
 constexpr int kGemmPitch = 36;           // floats per staged row of 32
-template <int BM, int BN, int TM, int TN>
+template <int BM, int BN, int TM, int TN, int KG>
 struct SimtCfg {
   static constexpr int kGroupThreads = (BM / TM) * (BN / TN);
-  static constexpr int kGroups = 256 / kGroupThreads;
+  static constexpr int kThreads = KG * kGroupThreads;
   static constexpr int kStages = 3;
-  static constexpr int kStageFloats = kGroups * (BM + BN) * kGemmPitch;
+  static constexpr int kStageFloats = KG * (BM + BN) * kGemmPitch;
+  static constexpr int kSumPitch = BN + 8;                     // (four rows of eight columns: no bank twice)
   static constexpr size_t kSmem = (size_t)kStages * kStageFloats * sizeof(float) + BN * sizeof(float) + BM * sizeof(long long);
-  static_assert((size_t)(kGroups - 1) * BM * BN <= (size_t)kStages * kStageFloats, "the sums of the groups fit in the ring");
+  static_assert((size_t)KG * BM * kSumPitch <= (size_t)kStages * kStageFloats, "the sums of the groups fit in the ring");
+  static_assert(BN + BM <= kThreads, "one thread per column's bias and per row's place");
 };
 
-template <int BM, int BN, int TM, int TN>
-__global__ void __launch_bounds__(256, 2) simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ W,
-                                                        const float* __restrict__ bias, int M, int Nout, int K,
-                                                        const GemmOut out) {
-  using Cfg = SimtCfg<BM, BN, TM, TN>;
-  constexpr int TX = BN / TN, TY = BM / TM, KG = Cfg::kGroups, kChunk = KG * 32;
+__device__ __forceinline__ float4 ld_cluster4(uint32_t cluster_addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(cluster_addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void add4(float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; }
+
+template <int BM, int BN, int TM, int TN, int KG>
+__global__ void __launch_bounds__(SimtCfg<BM, BN, TM, TN, KG>::kThreads, 2)
+simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ W, const float* __restrict__ bias, int M, int Nout,
+                 int K, int split, const GemmOut out) {
+  using Cfg = SimtCfg<BM, BN, TM, TN, KG>;
+  constexpr int TX = BN / TN, TY = BM / TM, kChunk = KG * 32, kThreads = Cfg::kThreads;
   extern __shared__ __align__(16) float ring[];
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const int rank = blockIdx.x % split;
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x / split * BN;
   const int group = threadIdx.x / Cfg::kGroupThreads, lt = threadIdx.x % Cfg::kGroupThreads;
   const int tx = lt % TX, ty = lt / TX;
-  const int chunks = (K + kChunk - 1) / kChunk;
+  const int all_chunks = (K + kChunk - 1) / kChunk;
+  const int first_chunk = all_chunks * rank / split, chunks = all_chunks * (rank + 1) / split - first_chunk;
 
   float* s_bias = ring + Cfg::kStages * Cfg::kStageFloats;
   long long* s_scat = reinterpret_cast<long long*>(s_bias + BN);
   auto load_rows = [&](int chunk, int first, int rows) {       // of the BM rows of A and, behind them, the BN rows of W
     float* st = ring + (chunk % Cfg::kStages) * Cfg::kStageFloats;
     // 16-byte packets: (row, group, packet of 8)
-    for (int e = threadIdx.x; e < rows * KG * 8; e += 256) {
+    for (int e = threadIdx.x; e < rows * KG * 8; e += kThreads) {
       const int p = e & 7, g = (e >> 3) % KG, r = first + (e >> 3) / KG;
-      const int k = chunk * kChunk + g * 32 + p * 4;
+      const int k = (first_chunk + chunk) * kChunk + g * 32 + p * 4;
       const bool is_a = r < BM;
       const int row = is_a ? m0 + r : n0 + r - BM;
       const bool exists = k < K && row < (is_a ? M : Nout);
@@ -128,39 +140,46 @@ __global__ void __launch_bounds__(256, 2) simt_gemm_kernel(const float* __restri
     }
   }
   cp_async_wait<0>();
-  __syncthreads();                         // the ring is free: the other groups hand their sums to group 0
-  if (KG > 1 && group > 0) {
-    float* dst = ring + (group - 1) * BM * BN + lt;
+  __syncthreads();                         // the ring is free: every group lays its sums out in it
+  float* const sums = ring + group * BM * Cfg::kSumPitch;
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-      for (int j = 0; j < TN; ++j) dst[(i * TN + j) * Cfg::kGroupThreads] = acc[i][j].x + acc[i][j].y;
-  }
-  if (KG > 1) __syncthreads();
-  if (group > 0) return;
+    for (int j = 0; j < TN; ++j) sums[(ty + i * TY) * Cfg::kSumPitch + tx + j * TX] = acc[i][j].x + acc[i][j].y;
+  if (split > 1) tc::cluster_sync();
+  else __syncthreads();
+  // Each CTA of the cluster finishes some of the tile's rows, four columns at a time (rows of W, segments and destinations
+  // are multiples of four).
+  const int row0 = BM * rank / split, row1 = BM * (rank + 1) / split;
+  for (int e = row0 * (BN / 4) + threadIdx.x; e < row1 * (BN / 4); e += kThreads) {
+    const int r = e / (BN / 4), c = e % (BN / 4) * 4, n = n0 + c, m = m0 + r;
+    if (m >= M || n >= Nout) continue;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float* at = ring + r * Cfg::kSumPitch + c;
+    if (split == 1) {
 #pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    const int m = m0 + ty + i * TY;
-    if (m >= M) continue;
-    const long long scat = s_scat[ty + i * TY];
+      for (int g = 0; g < KG; ++g) add4(v, *reinterpret_cast<const float4*>(at + g * BM * Cfg::kSumPitch));
+    } else {
+      for (int s = 0; s < split; ++s) {
+        const uint32_t there = tc::cluster_map(tc::smem_u32(at), (uint32_t)s);
 #pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      const int n = n0 + tx + j * TX;
-      if (n >= Nout) continue;
-      float v = acc[i][j].x + acc[i][j].y;
-#pragma unroll
-      for (int g = 1; g < KG; ++g) v += ring[(g - 1) * BM * BN + (i * TN + j) * Cfg::kGroupThreads + lt];
-      const bool s1 = n >= out.seg_cols, s2 = n >= 2 * out.seg_cols;
-      const int col = n - (s2 ? 2 * out.seg_cols : (s1 ? out.seg_cols : 0));
-      v += s_bias[tx + j * TX];
-      if (out.act == 1) v = gelu_tanh(v);
-      if (out.gate) v *= out.gate[(long long)(m / out.n_sel) * out.gate_ld + col];
-      void* const base = s2 ? out.ptr[2] : (s1 ? out.ptr[1] : out.ptr[0]);
-      const long long ld = s2 ? out.ld[2] : (s1 ? out.ld[1] : out.ld[0]);
-      const int scatter = s2 ? out.scatter[2] : (s1 ? out.scatter[1] : out.scatter[0]);
-      static_cast<float*>(base)[(scatter ? scat : (long long)m) * ld + col] = v;
+        for (int g = 0; g < KG; ++g) add4(v, ld_cluster4(there + g * BM * Cfg::kSumPitch * 4));
+      }
     }
+    const bool s1 = n >= out.seg_cols, s2 = n >= 2 * out.seg_cols;
+    const int col = n - (s2 ? 2 * out.seg_cols : (s1 ? out.seg_cols : 0));
+    add4(v, *reinterpret_cast<const float4*>(s_bias + c));
+    if (out.act == 1) v = make_float4(gelu_tanh(v.x), gelu_tanh(v.y), gelu_tanh(v.z), gelu_tanh(v.w));
+    if (out.gate) {
+      const float4 g4 = *reinterpret_cast<const float4*>(out.gate + (long long)(m / out.n_sel) * out.gate_ld + col);
+      v.x *= g4.x; v.y *= g4.y; v.z *= g4.z; v.w *= g4.w;
+    }
+    void* const base = s2 ? out.ptr[2] : (s1 ? out.ptr[1] : out.ptr[0]);
+    const long long ld = s2 ? out.ld[2] : (s1 ? out.ld[1] : out.ld[0]);
+    const int scatter = s2 ? out.scatter[2] : (s1 ? out.scatter[1] : out.scatter[0]);
+    *reinterpret_cast<float4*>(static_cast<float*>(base) + (scatter ? s_scat[r] : (long long)m) * ld + col) = v;
   }
+  if (split > 1) tc::cluster_sync();       // nobody leaves while its sums are being read
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -176,6 +195,7 @@ struct SimtAttCfg {
   static constexpr int kPitch = HD + 4, kPPitch = kAttK + 4;
   static constexpr int kTileFloats = kAttK * kPitch;
   static constexpr int kFloats = kAttQ * kPitch + kAttQ * kPPitch + 3 * kTileFloats + 2 * kAttQ;
+  static_assert(kAttQ * HD <= 3 * kTileFloats, "the merge's rows fit over the tiles");
   static constexpr size_t kSmem = (size_t)kFloats * sizeof(float);
 };
 
@@ -224,12 +244,13 @@ __global__ void __launch_bounds__(128) simt_attention_kernel(const float* __rest
   cp_async_commit();
 
   const float scale = rsqrtf((float)HD);
-  float m_run[kAttRows], l_run[kAttRows], o[kAttRows][CPT];
+  float m_run[kAttRows], l_run[kAttRows];
+  float2 o[kAttRows][CPT / 2];
 #pragma unroll
   for (int i = 0; i < kAttRows; ++i) {
     m_run[i] = -INFINITY; l_run[i] = 0.f;
 #pragma unroll
-    for (int c = 0; c < CPT; ++c) o[i][c] = 0.f;
+    for (int c = 0; c < CPT / 2; ++c) o[i][c] = make_float2(0.f, 0.f);
   }
   for (int t = t0; t < t1; ++t) {
     const int buf = (t - t0) & 1;
@@ -277,7 +298,7 @@ __global__ void __launch_bounds__(128) simt_attention_kernel(const float* __rest
         s_p[(ty * kAttRows + i) * Cfg::kPPitch + tx + 16 * j] = p;
       }
 #pragma unroll
-      for (int c = 0; c < CPT; ++c) o[i][c] *= alpha;
+      for (int c = 0; c < CPT / 2; ++c) o[i][c] = __fmul2_rn(o[i][c], make_float2(alpha, alpha));
     }
     cp_async_wait<1>();
     __syncthreads();                       // V of tile t is there (and a warp's own P rows)
@@ -289,23 +310,22 @@ __global__ void __launch_bounds__(128) simt_attention_kernel(const float* __rest
         p[i] = *reinterpret_cast<const float4*>(s_p + (ty * kAttRows + i) * Cfg::kPPitch + k);
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
-        float v[CPT];
+        float2 v[CPT / 2];
 #pragma unroll
         for (int c = 0; c < CPT; c += (CPT < 4 ? 2 : 4)) {
           const float* src = s_v + (k + kk) * kPitch + (CPT < 4 ? tx * 2 : tx * 4 + 16 * c);
           if constexpr (CPT < 4) {
-            const float2 w = *reinterpret_cast<const float2*>(src);
-            v[0] = w.x; v[1] = w.y;
+            v[0] = *reinterpret_cast<const float2*>(src);
           } else {
             const float4 w = *reinterpret_cast<const float4*>(src);
-            v[c] = w.x; v[c + 1] = w.y; v[c + 2] = w.z; v[c + 3] = w.w;
+            v[c / 2] = make_float2(w.x, w.y); v[c / 2 + 1] = make_float2(w.z, w.w);
           }
         }
 #pragma unroll
         for (int i = 0; i < kAttRows; ++i) {
           const float pk = kk == 0 ? p[i].x : (kk == 1 ? p[i].y : (kk == 2 ? p[i].z : p[i].w));
 #pragma unroll
-          for (int c = 0; c < CPT; ++c) o[i][c] = fmaf(pk, v[c], o[i][c]);
+          for (int c = 0; c < CPT / 2; ++c) o[i][c] = __ffma2_rn(make_float2(pk, pk), v[c], o[i][c]);
         }
       }
     }
@@ -324,7 +344,8 @@ __global__ void __launch_bounds__(128) simt_attention_kernel(const float* __rest
       if (row >= n_q) continue;
       float* dst = O + ((long long)b * n_q + row) * D + h * HD;
 #pragma unroll
-      for (int c = 0; c < CPT; ++c) dst[feature(c)] = o[i][c] / l_run[i];
+      for (int c = 0; c < CPT / 2; ++c)
+        *reinterpret_cast<float2*>(dst + feature(2 * c)) = make_float2(o[i][c].x / l_run[i], o[i][c].y / l_run[i]);
     }
     return;
   }
@@ -335,12 +356,12 @@ __global__ void __launch_bounds__(128) simt_attention_kernel(const float* __rest
   for (int i = 0; i < kAttRows; ++i) {
     const int row = ty * kAttRows + i;
 #pragma unroll
-    for (int c = 0; c < CPT; ++c) s_kv[row * HD + feature(c)] = o[i][c];
+    for (int c = 0; c < CPT / 2; ++c) *reinterpret_cast<float2*>(s_kv + row * HD + feature(2 * c)) = o[i][c];
     if (tx == 0) { s_ml[row] = m_run[i]; s_ml[kAttQ + row] = l_run[i]; }
   }
   tc::cluster_sync();
-  for (int e = threadIdx.x; e < kAttQ / split * HD; e += 128) {
-    const int row = rank * (kAttQ / split) + e / HD, col = e % HD;
+  for (int e = kAttQ * rank / split * HD + threadIdx.x; e < kAttQ * (rank + 1) / split * HD; e += 128) {
+    const int row = e / HD, col = e % HD;
     float m = -INFINITY;
     for (int r = 0; r < split; ++r) m = fmaxf(m, ld_cluster(tc::cluster_map(tc::smem_u32(s_ml + row), r)));
     float l = 0.f, acc = 0.f;
@@ -354,18 +375,19 @@ __global__ void __launch_bounds__(128) simt_attention_kernel(const float* __rest
   tc::cluster_sync();                      // nobody leaves while its rows are being read
 }
 
-template <int BM, int BN, int TM, int TN>
-int gemm_launch(const float* a, const float* w, const float* bias, int M, int Nout, int K, const GemmOut& out,
+template <int BM, int BN, int TM, int TN, int KG>
+int gemm_launch(const float* a, const float* w, const float* bias, int M, int Nout, int K, int split, const GemmOut& out,
                 cudaStream_t s) {
-  using Cfg = SimtCfg<BM, BN, TM, TN>;
+  using Cfg = SimtCfg<BM, BN, TM, TN, KG>;
   static PerDeviceOnce once;
   HERO_TRY(per_device_once(once, [](int) {
-    HERO_CUDA_TRY(cudaFuncSetAttribute(simt_gemm_kernel<BM, BN, TM, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    HERO_CUDA_TRY(cudaFuncSetAttribute(simt_gemm_kernel<BM, BN, TM, TN, KG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)Cfg::kSmem));
     return HERO_OK;
   }));
-  const dim3 grid((Nout + BN - 1) / BN, (M + BM - 1) / BM);
-  HERO_TRY(launch_kernel(simt_gemm_kernel<BM, BN, TM, TN>, grid, 256, Cfg::kSmem, s, 1, a, w, bias, M, Nout, K, out));
+  const dim3 grid((Nout + BN - 1) / BN * split, (M + BM - 1) / BM);
+  HERO_TRY(launch_kernel(simt_gemm_kernel<BM, BN, TM, TN, KG>, grid, Cfg::kThreads, Cfg::kSmem, s, (unsigned)split, a, w,
+                         bias, M, Nout, K, split, out));
   return HERO_OK;
 }
 
@@ -380,12 +402,17 @@ int attention_launch(const float* q, const float* k, const float* v, float* o, i
   }));
   const long long groups = (long long)B * heads * ((n_q + kAttQ - 1) / kAttQ);
   const int tiles = (N + kAttK - 1) / kAttK;
-  // Keys over a cluster while that shortens the longest run of tiles (a CTA may go without: 144 keys are three tiles, over
-  // four CTAs 8.2 us, over two 12.8) and leaves the grid within what the chip holds at once: a CTA of four
-  // warps alone keeps an SM's FMA pipe 40 % busy, two 80 % (310 queries, 1319 keys, 16 heads: 160 CTAs 102 us, 320 83 us).
-  const int resident = HD > 64 ? 1 : 3;
+  // Keys over a cluster of two, four or eight where the chip is then better filled: per SM the CTAs one after the other take
+  // the time of their key tiles plus some for each start and merge (a CTA may go without keys).  us over 1 / 2 / 4 / 8 CTAs:
+  // 310 queries, 1319 keys, 16 heads 102 / 82 / 79 / 82; 8 heads 63 / 59 / 46 / 49; 600 x 1240 x 10 97 / 75 / 77 / 96;
+  // 1319 x 1319 x 16 234 / 253 / 264 / 302; 32 x 144 x 2 11.0 / 12.6 / 7.7 / 7.6.
   int split = 1;
-  while (split < 8 && split < tiles && groups * split * 2 <= (long long)num_sms() * resident * 3 / 4) split *= 2;
+  long long best = -1;
+  for (int c = 1; c <= 8 && (c == 1 || c / 2 < tiles); c *= 2) {
+    const long long per_sm = (groups * c + num_sms() - 1) / num_sms();
+    const long long t = per_sm * ((long long)((tiles + c - 1) / c) * (24 * HD / 64) + 17);
+    if (best < 0 || t < best) { best = t; split = c; }
+  }
   if (groups * split > 0x7FFFFFFFll) return HERO_ERR_ARG;
   return launch_kernel(simt_attention_kernel<HD>, (unsigned)(groups * split), 128, Cfg::kSmem, s, (unsigned)split, q, k,
                        v, o, n_q, N, heads, split);
@@ -396,11 +423,36 @@ int attention_launch(const float* q, const float* k, const float* v, float* o, i
 int launch_simt_gemm(const float* a, const float* w, const float* bias, int M, int Nout, int K, const GemmOut& out,
                      cudaStream_t s) {
   if (M <= 0) return HERO_OK;
-  // 64 x 64 tiles (8 x 4 outputs a thread, two groups) where they give every SM work of its own, else 32 x 32 (4 x 4
-  // outputs, four groups)
-  const long long tiles = (long long)((M + 63) / 64) * ((Nout + 63) / 64);
-  if (tiles >= num_sms()) return gemm_launch<64, 64, 8, 4>(a, w, bias, M, Nout, K, out, s);
-  return gemm_launch<32, 32, 4, 4>(a, w, bias, M, Nout, K, out, s);
+  // Tiles of 64 x 64 (8 x 8 outputs a thread, two groups) or 32 x 32 (4 x 4, four groups), over one CTA or a cluster: what
+  // an SM's CTAs take one after the other, in tenths of a us per chunk of k, and what a launch and an exchange take on top.
+  // (Two CTAs share an SM but hardly run faster for it; clusters of three do not fill the chip.)  Measured, us:
+  //   M x N x K           64: 1     2      3      4      8    32: 1     2      4
+  //   620 x 1536 x 512     34.3   36.6   42.7   36.5   59.7    38.2   46.6   72.4
+  //   620 x 512 x 512      20.1   19.5   16.1   16.9   24.0    17.2   19.4   26.6
+  //   620 x 2048 x 512     48.9   44.9   51.6   49.7   77.1    48.6   62.0   94.8
+  //   620 x 512 x 2048     70.1   65.0   46.6   50.2   49.5    62.0   55.1   58.9
+  //   2638 x 512 x 2048   183.8  154.9  171.8  157.6  178.0   180.1  192.0  219.5
+  //   1200 x 320 x 1280    45.3   42.4   44.9   33.8   46.1    40.1   43.1   53.0
+  //   200 x 256 x 1024     36.4   21.2   17.1   12.5   10.9    12.8    8.9    8.3
+  //   200 x 768 x 256      11.4    8.9   11.3    8.3            6.4   10.0
+  //   32 x 128 x 512       19.3   12.6   10.0    7.7    5.8     7.0    5.5    4.4
+  // With 8 x 4 outputs a thread, the sums stored by one group alone and no clusters: 620 x 1536 x 512 42, 620 x 512 x 2048 62.
+  bool large = false;
+  int split = 1;
+  long long best = -1;
+  for (const bool big : {true, false}) {
+    const int tile = big ? 64 : 32, chunk = big ? 64 : 128;
+    const long long tiles = (long long)((M + tile - 1) / tile) * ((Nout + tile - 1) / tile), chunks = (K + chunk - 1) / chunk;
+    for (int c : {1, 2, 3, 4, 8}) {
+      if (c > chunks) break;
+      const long long slots = c == 3 ? num_sms() * 17 / 20 : num_sms(), per_sm = (tiles * c + slots - 1) / slots;
+      const long long t = big ? per_sm * ((chunks + c - 1) / c * 20 + (c > 1 ? 10 : 0)) + 30
+                              : per_sm * ((chunks + c - 1) / c * 13 + (c > 1 ? 14 : 0)) + 17;
+      if (best < 0 || t < best) { best = t; large = big; split = c; }
+    }
+  }
+  return large ? gemm_launch<64, 64, 8, 8, 2>(a, w, bias, M, Nout, K, split, out, s)
+               : gemm_launch<32, 32, 4, 4, 4>(a, w, bias, M, Nout, K, split, out, s);
 }
 
 int launch_simt_attention(const float* q, const float* k, const float* v, float* o, int B, int n_q, int N, int heads,

@@ -391,3 +391,27 @@ def test_attention_output_at_any_16_byte_boundary(B, n_q, N, heads):
         assert bool((flat[:shift] == 7.0).all()) and bool((flat[shift + size:] == 7.0).all())
         outs.append(flat[shift:shift + size].clone())
     assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("over", [
+    # 64 x 64 tiles whole, over two (FFN up), three (both projections back to the width) in the full pass; the same and 32 x 32
+    # over clusters in the refresh
+    dict(hidden=512, n_heads=8, ffn_dim=2048, grid_h=16, grid_w=19, n_text=5, batch=2),
+    # FFN down over four CTAs: 32 x 32 tiles, the last row tile eight rows; 64 x 64 tiles, K no multiple of a chunk
+    dict(hidden=256, n_heads=4, ffn_dim=1024, grid_h=13, grid_w=15, n_text=5, batch=1),
+    dict(hidden=320, n_heads=5, ffn_dim=1276, grid_h=22, grid_w=26, n_text=25, batch=2, has_gate=1),
+    # one row tile, over eight CTAs' worth of k; nothing to split
+    dict(hidden=64, n_heads=1, ffn_dim=4092, grid_h=5, grid_w=6, n_text=0, batch=1),
+    dict(hidden=192, n_heads=3, ffn_dim=4, grid_h=7, grid_w=50, n_text=1, batch=1)],
+    ids=["width512", "width256", "width320", "long_k", "short_k"])
+def test_fp32_gemm_tiles_and_clusters(over):
+    cfgd = dict(S.CONFIGS["tiny"], n_blocks=1, n_shallow=1, frames=1, seed=43, head_dim=64, **over)
+    orc, hero, _ = make_pair(cfgd)
+    x_host = S.tokens(cfgd)
+    for s in range(3):                                     # two full passes, one refresh
+        temb = S.temb(cfgd, s)
+        want = orc.step(s, x_host, temb)
+        x = to_dev(x_host, "fp32")
+        hero.hero_step(s, x, to_dev(temb, "fp32"))
+        assert rel_l2(to_host(x) - x_host, want - x_host) <= FP32_TOL, s
+    hero.close()
