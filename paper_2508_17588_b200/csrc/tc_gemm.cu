@@ -12,6 +12,7 @@
 
 #include "hero_internal.h"
 #include "tc_common.cuh"
+#include "tc_epilogue.cuh"
 
 namespace hero {
 
@@ -67,36 +68,6 @@ constexpr int kABytes = kBM * kBK * 2;                 // 16 KB
 constexpr int kGemmThreads = 320;                      // producer, issuer, eight epilogue warps
 constexpr int kEpiWarps = 8;                           // two per TMEM lane quadrant, each with half of a tile's columns
 constexpr size_t kAlignSlack = 1024, kBarrierBytes = 512;
-
-__device__ __forceinline__ float gelu_tanh_f(float t) {
-  // 0.5 t (1 + tanh(sqrt(2/pi) (t + 0.044715 t^3))) with the hardware tanh (one special-function
-  // instruction, relative error 2^-11: below the bf16 rounding of the result).  The epilogue shares the
-  // SM's power budget with the tensor core, so every instruction saved here is tensor clock gained.
-  const float t2 = t * t;
-  const float u = t * fmaf(0.0356774081f, t2, 0.7978845608f);
-  float th;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(u));
-  const float h = 0.5f * t;
-  return fmaf(h, th, h);
-}
-
-// Where one accumulator row goes.
-struct RowOut {
-  bool ok;                 // the row exists
-  int m, b;                // row of the compact operand, its batch item
-  long long scat;          // its row in a [B, n_rows] destination
-};
-__device__ __forceinline__ RowOut row_out(const GemmOut& out, int m, int M) {
-  RowOut r;
-  r.ok = m < M;
-  r.m = m; r.b = 0; r.scat = 0;
-  if (r.ok) {
-    r.b = m / out.n_sel;
-    const int li = m - r.b * out.n_sel;
-    r.scat = (long long)r.b * out.n_rows + (out.idx ? __ldg(out.idx + li) : li);
-  }
-  return r;
-}
 
 // Finish NC accumulator columns [n0, n0 + NC) of one row, all of one segment: bias (fp32, staged in shared memory),
 // activation, scale or gate, bf16, full 32-byte sectors per lane (16-byte stores where the destination is not 32-byte
@@ -504,8 +475,9 @@ struct SplitCfg {
   static constexpr int kBBytes = BN * kBK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
   static constexpr int kStages = BN == 128 ? 4 : 6;
-  static constexpr size_t kBiasBytes = kEpiWarps * (BN / 2) * 4;
-  static constexpr int kMaxSplit = BN / 32;                    // a warp finishes at least 16 columns
+  static constexpr int kBiasCols = 64;                         // a warp's columns at most
+  static constexpr size_t kBiasBytes = kEpiWarps * kBiasCols * 4;
+  static constexpr int kMaxSplit = 4;                          // a CTA finishes at least 16 columns
   static constexpr size_t part_bytes(int split) { return (size_t)(split - 1) * (BN / split) * kBM * 4; }
   static constexpr size_t smem(int split) {
     return kAlignSlack + (size_t)kStages * kStageBytes + part_bytes(split) + kBiasBytes + kBarrierBytes;
@@ -517,7 +489,6 @@ __global__ void __launch_bounds__(kGemmThreads)
 tc_gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
                      const __nv_bfloat16* __restrict__ bias, const GemmOut out, const QkParam<QK> qk, int M, int Nout, int K,
                      int split, int* __restrict__ status) {
-  static_assert(!QK || BN == 128, "an epilogue warp's columns are a whole head");
   using Cfg = SplitCfg<BN>;
   constexpr int kStages = Cfg::kStages;
   extern __shared__ uint8_t smem_raw[];
@@ -609,14 +580,19 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
   const int half = (warp - 2) >> 2;
   const int tile_row = quad * 32 + lane;
   const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16);
-  const int width = BN / split;              // columns this CTA finishes: [rank * width, (rank + 1) * width)
-  const int c_first = rank * width + half * (width / 2);       // ... and this warp: width / 2 of them
-  float* s_bias = s_bias_all + (size_t)(warp - 2) * (BN / 2);
+  // This CTA finishes columns [rank * width, (rank + 1) * width) and this warp `mine` of them: half, or, where halves would
+  // be less than a piece of 16 columns or than a head, the first warp of two all of them.
+  const int width = BN / split;
+  const bool alone = QK ? BN == 64 : width < 32;
+  const int mine = alone ? (half == 0 ? width : 0) : width / 2;
+  const int c_first = rank * width + (alone ? 0 : half * (width / 2));
+  constexpr int kBiasCols = Cfg::kBiasCols;
+  float* s_bias = s_bias_all + (size_t)(warp - 2) * kBiasCols;
   RowOut row = {};
   bool ok = true;
   if (warp >= 2) {
     stream_order();
-    stage_bias<BN / 2>(s_bias, bias, nt * BN + c_first, Nout, lane);
+    stage_bias<kBiasCols>(s_bias, bias, nt * BN + c_first, Nout, lane);
     row = row_out(out, mt * kBM + tile_row, M);
     ok = mbar_wait_warp(acc_full, 0, abort_flag);
     if (ok) tc_fence_after();
@@ -645,7 +621,7 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     cluster_sync();                          // every wait above is bounded, so everybody gets here
   }
   if constexpr (QK) {                        // (split is 1: the warp's 64 columns are one head)
-    if (warp >= 2 && ok && nt * BN + c_first < Nout) {
+    if (warp >= 2 && ok && mine > 0 && nt * BN + c_first < Nout) {
       uint32_t r[2][32];
       tmem_ld32(t_row + c_first, r[0]);
       tmem_ld32(t_row + c_first + 32, r[1]);
@@ -653,7 +629,7 @@ tc_gemm_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
       emit_head(r, s_bias, nt * BN + c_first, out, row, qk, row_angles(qk, row, out.n_rows));
     }
   } else if (warp >= 2 && ok) {
-    for (int c = c_first; c < c_first + width / 2; c += 16) {
+    for (int c = c_first; c < c_first + mine; c += 16) {
       const int n0 = nt * BN + c;
       if (n0 >= Nout) break;                 // warp-uniform
       uint32_t r[16];
@@ -723,6 +699,10 @@ int launch_wait_timeout_selftest(int* d_status, int budget_us, cudaStream_t s) {
 //   200 x 1280 x 5120      27.5      24.6      23.0      21.8     25.1     15.4    11.4     19.6    12.6
 //   2300 x 2048 x 2048     16.6      21.8      20.6      20.1     25.9     38.4    72.2     39.3    60.7
 //   7000 x 1536 x 6144     99.1     103.4     125.7     143.8    168.9    181.1   259.5    220.0   315.1
+// 64 columns over four CTAs, where K is long and the tiles are few (CTA 64 over 1 / 2 / 4): 250 x 384 x 1536 7.6 / 5.9 / 4.9,
+// 500 x 512 x 2048 9.4 / 6.9 / 6.1, 60 x 704 x 2112 9.2 / 6.9 / 5.3; 371 x 768 x 3072, whose 36 clusters of four do not all
+// fit, 12.8 / 8.8 / 12.7.  With q/k treatment (pair 256 / pair 128 / CTA 128 / CTA 64): 371 x 2304 x 768 10.4 / 7.3 / 7.3 / 6.2,
+// 614 x 768 x 256 8.0 / 5.9 / 5.3 / 4.3, 700 x 1536 x 512 9.4 / 6.8 / 6.7 / 5.3, 1394 x 3072 x 1024 12.8 / 13.7 / 15.6 / 25.4.
 // ---------------------------------------------------------------------------------------------------------------
 namespace {
 
@@ -745,9 +725,8 @@ GemmPlan plan_gemm(int M, int Nout, int K, bool qk) {
     consider(p.bn, 0, ceil_div(tiles, sms / 2) * kb * p.step + p.fixed);
   }
   for (int bn : {128, 64}) {
-    if (qk && bn != 128) continue;
     const long long tiles = ceil_div(M, kBM) * ceil_div(Nout, bn);
-    const int max_split = qk ? 1 : bn == 128 ? SplitCfg<128>::kMaxSplit : SplitCfg<64>::kMaxSplit;
+    const int max_split = qk ? 1 : SplitCfg<128>::kMaxSplit;
     for (int split = 1; split <= max_split && split <= kb; split *= 2) {
       const long long ctas = tiles * split;
       if (ctas > 0x7FFFFFFFll) continue;
@@ -819,7 +798,9 @@ int launch_tc_gemm(const void* a, const void* w, const void* bias, int M, int No
   }
   if (qk) {
     if (out.seg_cols % 64 || Nout != 3 * out.seg_cols || out.act || out.gate || out.seg0_scale != 0.f) return HERO_ERR_ARG;
-    if (plan.split) return launch_split<128, true>(tm_a, tm_w, bias, out, *qk, M, Nout, K, 1, d_status, s);
+    if (plan.split)
+      return plan.bn == 128 ? launch_split<128, true>(tm_a, tm_w, bias, out, *qk, M, Nout, K, 1, d_status, s)
+                            : launch_split<64, true>(tm_a, tm_w, bias, out, *qk, M, Nout, K, 1, d_status, s);
     return plan.bn == 256 ? launch_pair<256, true>(tm_a, tm_w, bias, out, *qk, M, Nout, K, d_status, s)
                           : launch_pair<128, true>(tm_a, tm_w, bias, out, *qk, M, Nout, K, d_status, s);
   }

@@ -415,3 +415,29 @@ def test_fp32_gemm_tiles_and_clusters(over):
         hero.hero_step(s, x, to_dev(temb, "fp32"))
         assert rel_l2(to_host(x) - x_host, want - x_host) <= FP32_TOL, s
     hero.close()
+
+
+@pytest.mark.parametrize("qk_norm,rope", [(1, 1), (0, 1), (1, 0)])
+@pytest.mark.parametrize("over", [
+    # tiles of 64 columns: a head each, one row tile and several; the same over four CTAs in the other projections
+    dict(hidden=64, n_heads=1, ffn_dim=2048, grid_h=9, grid_w=10, n_text=7, batch=1),
+    dict(hidden=448, n_heads=7, ffn_dim=1792, grid_h=17, grid_w=18, n_text=1, batch=2),
+    # tiles of 128 columns in the full pass
+    dict(hidden=512, n_heads=8, ffn_dim=512, grid_h=25, grid_w=20, n_text=0, batch=2)], ids=["one_head", "7_heads", "wide"])
+def test_qk_treatment_by_tile_width(over, qk_norm, rope):
+    cfgd = dict(S.CONFIGS["tiny"], n_blocks=1, n_shallow=1, frames=1, seed=47, head_dim=64, temb_dim=64, dtype="bf16", rope=rope,
+                qk_norm=qk_norm, **over)
+    orc, hero, _ = make_pair(cfgd)
+    x_host = S.tokens(cfgd)
+    for s in range(3):                                     # two full passes, one refresh
+        temb = S.temb(cfgd, s)
+        orc.step(s, x_host, temb)
+        x = to_dev(x_host, "bf16")
+        hero.hero_step(s, x, to_dev(temb, "bf16"))
+        hero.hero_check_status()
+        # keys and values are one projection of a LayerNormed row away from x: two roundings to bf16 of the inputs of a
+        # K-term sum and one of its result, the latter through the rotation; far below the 2e-2 that a whole block may be off
+        for name, ref in (("k", orc.blocks[0].k_cache), ("v", orc.blocks[0].v_cache)):
+            assert rel_l2(to_host(hero.hero_state_get(0, name)), ref) <= 1e-2, (s, name)
+            ref[...] = to_host(hero.hero_state_get(0, name))
+    hero.close()
