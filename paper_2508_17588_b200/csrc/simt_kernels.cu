@@ -75,17 +75,23 @@ simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ W, const
 
   float* s_bias = ring + Cfg::kStages * Cfg::kStageFloats;
   long long* s_scat = reinterpret_cast<long long*>(s_bias + BN);
-  auto load_rows = [&](int chunk, int first, int rows) {       // of the BM rows of A and, behind them, the BN rows of W
-    float* st = ring + (chunk % Cfg::kStages) * Cfg::kStageFloats;
-    // 16-byte packets: (row, group, packet of 8)
-    for (int e = threadIdx.x; e < rows * KG * 8; e += kThreads) {
-      const int p = e & 7, g = (e >> 3) % KG, r = first + (e >> 3) / KG;
-      const int k = (first_chunk + chunk) * kChunk + g * 32 + p * 4;
-      const bool is_a = r < BM;
-      const int row = is_a ? m0 + r : n0 + r - BM;
-      const bool exists = k < K && row < (is_a ? M : Nout);
-      const float* src = (is_a ? A : W) + (exists ? (long long)row * K + k : 0);
-      cp_async16(st + (g * (BM + BN) + r) * kGemmPitch + p * 4, src, exists);
+  // Chunks come in packets of 16 bytes: a thread fetches packet p of group g's 32 k of every eighth row, whose addresses and
+  // existence it works out once (per packet they were a quarter of the loop's instructions).
+  const int p = threadIdx.x & 7, g = (threadIdx.x >> 3) % KG, r0 = threadIdx.x / (8 * KG);
+  static_assert(kThreads == 64 * KG, "eight rows a round");
+  const int k_first = first_chunk * kChunk + g * 32 + p * 4;
+  const float* const a_src = A + (long long)(m0 + r0) * K + k_first;
+  const float* const w_src = W + (long long)(n0 + r0) * K + k_first;
+  float* const s_dst = ring + (g * (BM + BN) + r0) * kGemmPitch + p * 4;
+  auto load_rows = [&](int chunk, bool weights) {
+    float* dst = s_dst + (chunk % Cfg::kStages) * Cfg::kStageFloats + (weights ? BM * kGemmPitch : 0);
+    const int rows = (weights ? Nout - n0 : M - m0) - r0;      // of which exist those that are multiples of eight below this
+    const bool there = k_first + chunk * kChunk < K;
+    const float* src = (weights ? w_src : a_src) + chunk * kChunk;
+#pragma unroll
+    for (int j = 0; j < (weights ? BN : BM) / 8; ++j) {
+      const bool exists = there && 8 * j < rows;
+      cp_async16(dst + 8 * j * kGemmPitch, exists ? src + (long long)(8 * j) * K : A, exists);
     }
   };
   // What no kernel in front has a hand in, first: the first chunks' weights, the bias and where the rows go (the lists are
@@ -94,7 +100,7 @@ simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ W, const
   auto fetch_ahead = [&]() {
 #pragma unroll
     for (int c = 0; c < Cfg::kStages - 1; ++c)
-      if (c < chunks) load_rows(c, BM, BN);
+      if (c < chunks) load_rows(c, true);
     if (threadIdx.x < BN) {
       const int n = n0 + threadIdx.x;
       s_bias[threadIdx.x] = n < Nout ? __ldg(bias + n) : 0.f;
@@ -116,13 +122,13 @@ simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ W, const
     for (int j = 0; j < TN; ++j) acc[i][j] = make_float2(0.f, 0.f);
 #pragma unroll
   for (int c = 0; c < Cfg::kStages - 1; ++c) {
-    if (c < chunks) load_rows(c, 0, BM);
+    if (c < chunks) load_rows(c, false);
     cp_async_commit();
   }
   for (int c = 0; c < chunks; ++c) {
     cp_async_wait<Cfg::kStages - 2>();
     __syncthreads();                       // chunk c is there for everybody, and nobody reads chunk c - 1 any more
-    if (c + Cfg::kStages - 1 < chunks) load_rows(c + Cfg::kStages - 1, 0, BM + BN);
+    if (c + Cfg::kStages - 1 < chunks) { load_rows(c + Cfg::kStages - 1, false); load_rows(c + Cfg::kStages - 1, true); }
     cp_async_commit();
     const float* sa = ring + (c % Cfg::kStages) * Cfg::kStageFloats + group * (BM + BN) * kGemmPitch;
     const float* sw = sa + BM * kGemmPitch;
@@ -427,7 +433,7 @@ int launch_simt_gemm(const float* a, const float* w, const float* bias, int M, i
   // an SM's CTAs take one after the other, in tenths of a us per chunk of k, and what a launch and an exchange take on top.
   // (Two CTAs share an SM but hardly run faster for it; clusters of three do not fill the chip.)  Measured, us:
   //   M x N x K           64: 1     2      3      4      8    32: 1     2      4
-  //   620 x 1536 x 512     34.3   36.6   42.7   36.5   59.7    38.2   46.6   72.4
+  //   620 x 1536 x 512     34.3   36.6   42.7   36.5   59.7    38.2   46.6   72.4   (before a packet's address was worked out once)
   //   620 x 512 x 512      20.1   19.5   16.1   16.9   24.0    17.2   19.4   26.6
   //   620 x 2048 x 512     48.9   44.9   51.6   49.7   77.1    48.6   62.0   94.8
   //   620 x 512 x 2048     70.1   65.0   46.6   50.2   49.5    62.0   55.1   58.9
