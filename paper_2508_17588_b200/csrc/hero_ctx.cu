@@ -55,9 +55,8 @@ struct hero_ctx {
   void* deep_g[2] = {nullptr, nullptr};
   float* stack_hist[2] = {nullptr, nullptr};
   int stack_last = 0, stack_n = 0, stack_new = 0;
-  // attend_mode 1: compact K/V of the rows a cached step attends to (text + refreshed) and their list
+  // attend_mode 1: compact K/V of the rows a cached step attends to (text + refreshed)
   void* kv_cmp[2] = {nullptr, nullptr};
-  int* att_list = nullptr;
   // hero_step_host: device-to-host copies of finished pieces of x run on this stream, behind the events
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t piece_done[kHostPieces] = {};
@@ -299,11 +298,8 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
   if (g.attend_mode == 1 && !full) {
     // Eq. 3 read literally: the refreshed queries see the refreshed rows (just written) and the text rows
     const int n_att = g.n_text + n_sel;
-    HERO_LAUNCH(c, HERO_PROF_GATHER_LN, launch_attend_list(d_idx, n_sel, g.n_text, c->att_list, c->stream));
-    HERO_LAUNCH(c, HERO_PROF_GATHER_LN,
-                launch_gather_rows(kdst, c->att_list, c->kv_cmp[0], B, N, n_att, D, g.dtype, c->stream));
-    HERO_LAUNCH(c, HERO_PROF_GATHER_LN,
-                launch_gather_rows(vdst, c->att_list, c->kv_cmp[1], B, N, n_att, D, g.dtype, c->stream));
+    HERO_LAUNCH(c, HERO_PROF_GATHER_LN, launch_attend_rows(kdst, vdst, d_idx, c->kv_cmp[0], c->kv_cmp[1], B, N, g.n_text, n_sel,
+                                                           D, g.dtype, c->stream));
     HERO_TRY(run_attention(c, c->ws_q, c->kv_cmp[0], c->kv_cmp[1], c->ws_o, n_sel, n_att));
   } else {
     HERO_TRY(run_attention(c, c->ws_q, kdst, vdst, c->ws_o, n_sel, N));
@@ -533,7 +529,6 @@ int hero_init(hero_ctx** out, const hero_config* cfg, const hero_block_weights* 
   if (cfg->n_shallow < cfg->n_blocks) { A(&c->kv_tmp[0], tensor); A(&c->kv_tmp[1], tensor); }
   if (cfg->attend_mode == 1) {
     A(&c->kv_cmp[0], tensor); A(&c->kv_cmp[1], tensor);
-    A((void**)&c->att_list, (size_t)c->N * sizeof(int));
   }
   std::vector<float2> rope_host;
   if (cfg->rope) {

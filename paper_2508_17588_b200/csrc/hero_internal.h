@@ -201,8 +201,10 @@ struct QkPrepArgs {
   float eps;
 };
 int launch_qk_prep(const QkPrepArgs& a, cudaStream_t s);
-// list[i] = i for i < n_text, list[n_text + i] = idx[i] for i < n_sel (rows a literal Eq. 3 attends to)
-int launch_attend_list(const int* idx, int n_sel, int n_text, int* list, cudaStream_t s);
+// Of K and V [B, N, D] the first n_text rows and the listed ones, compact: [B, n_text + n_sel, D] (what a literal Eq. 3 attends
+// to).  The list was complete before the kernel in front on the stream was placed.
+int launch_attend_rows(const void* k, const void* v, const int* idx, void* k_out, void* v_out, int B, int N, int n_text,
+                       int n_sel, int D, int dtype, cudaStream_t s);
 int launch_gather_rows(const void* src, const int* idx, void* dst, int B, int N, int n_sel, int D,
                        int dtype, cudaStream_t s);
 int launch_scatter_rows(const void* src, const int* idx, void* dst, int B, int N, int n_sel, int D,
