@@ -301,6 +301,12 @@ int hero_isolated_status(void *stream);
  * are the isolated calls' word and `stream` (hero_isolated_status reports it the same way). */
 int hero_selftest_wait_timeout(hero_ctx *ctx, int budget_us, void *stream);
 
+/* ---- what the rules on sizes choose (host arithmetic, no GPU; for tests and for reading a profile) ---- */
+
+/* The fp32 GEMM C[M,N] = A[M,K] W[N,K]^T of a context on a GPU of `sms` SMs: square tiles of *tile (64 or 32) outputs, each
+ * shared by a cluster of *ctas thread blocks along K.  HERO_ERR_ARG where no tile serves so many rows (65535 row tiles of 64). */
+int hero_plan_fp32_gemm(int M, int N, int K, int sms, int *tile, int *ctas);
+
 /* ---- state access for tests and checkpoints -------------------------------- */
 #define HERO_STATE_AGES     0   /* u16[n_video] */
 #define HERO_STATE_CALLS    1   /* int32[1] selection call counter */

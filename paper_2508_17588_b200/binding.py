@@ -27,6 +27,7 @@ EXPORTS = [
     "hero_extrapolate_block", "hero_extrapolate_deep_stack", "hero_step", "hero_step_host", "hero_is_full_step", "hero_extrapolate",
     "hero_gather_rows", "hero_scatter_rows", "hero_gemm_bf16", "hero_attention_bf16", "hero_attention_bf16_safe", "hero_attention_bf16_q_scaled", "hero_attention_bf16_static", "hero_attention_bf16_static_status",
     "hero_isolated_status", "hero_selftest_wait_timeout", "hero_gather_ln_modulate",
+    "hero_plan_fp32_gemm",
     "hero_state_get", "hero_state_set", "hero_second_difference_moments", "hero_extrapolation_error",
 ]
 
@@ -101,6 +102,7 @@ def load() -> C.CDLL:
         "hero_gather_ln_modulate": (i, [vp, vp, vp, vp, vp, i, vp, i, i, i, i, i, vp]),
         "hero_second_difference_moments": (i, [vp, vp, vp, ll, i, vp, vp]),
         "hero_extrapolation_error": (i, [vp, vp, vp, ll, i, i, i, vp, vp]),
+        "hero_plan_fp32_gemm": (i, [i, i, i, i, ip, ip]),
         "hero_state_get": (i, [vp, i, i, vp, ll]),
         "hero_state_set": (i, [vp, i, i, vp, ll]),
     }
@@ -371,6 +373,14 @@ def hero_attention_bf16_static_status(n_records: int = 0):
     _check(load().hero_attention_bf16_static_status(_stream(), C.byref(gave_up), rec if n_records else None, n_records),
            "hero_attention_bf16_static_status")
     return gave_up.value, list(rec)[:n_records]
+
+
+# ---- what the rules on sizes choose (no GPU needed) --------------------------------
+def hero_plan_fp32_gemm(M: int, N: int, K: int, sms: int = 148):
+    """(tile, thread blocks per tile) of a context's fp32 GEMM on a GPU of `sms` SMs."""
+    tile, ctas = C.c_int(), C.c_int()
+    _check(load().hero_plan_fp32_gemm(M, N, K, sms, C.byref(tile), C.byref(ctas)), "hero_plan_fp32_gemm")
+    return tile.value, ctas.value
 
 
 def hero_isolated_status():

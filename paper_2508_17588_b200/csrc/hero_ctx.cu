@@ -983,6 +983,15 @@ int hero_selftest_wait_timeout(hero_ctx* c, int budget_us, void* stream) {
   return launch_wait_timeout_selftest(st, budget_us, c ? c->stream : (cudaStream_t)stream);
 }
 
+// ---------------------------------------------------------------- what the rules on sizes choose
+int hero_plan_fp32_gemm(int M, int N, int K, int sms, int* tile, int* ctas) {
+  if (M <= 0 || N <= 0 || K <= 0 || sms <= 0 || !tile || !ctas) return HERO_ERR_ARG;
+  const SimtGemmPlan plan = plan_simt_gemm(M, N, K, sms);
+  if (!plan.tile) return HERO_ERR_ARG;
+  *tile = plan.tile; *ctas = plan.split;
+  return HERO_OK;
+}
+
 // ---------------------------------------------------------------- state access
 static int state_ptr(hero_ctx* c, int block, int what, void** p, size_t* bytes) {
   const hero_config& g = c->cfg;

@@ -241,6 +241,9 @@ int launch_residual_ln(void* x, const void* ga, const void* gf, const int* pos, 
 // fp32 CUDA-core path (config 1 runs in fp32, where tensor cores would break parity)
 int launch_simt_gemm(const float* a, const float* w, const float* bias, int M, int Nout, int K, const GemmOut& out,
                      cudaStream_t s);
+// Which tile (64 or 32 square) over how many CTAs; tile 0: a problem of more rows than any tile serves.
+struct SimtGemmPlan { int tile, split; };
+SimtGemmPlan plan_simt_gemm(int M, int Nout, int K, int sms);
 int launch_simt_attention(const float* q, const float* k, const float* v, float* o, int B, int n_q, int N, int heads,
                           int head_dim, cudaStream_t s);
 

@@ -38,6 +38,7 @@ __device__ __forceinline__ void dot4(float2& acc, const float4& a, const float4&
 // groups and CTAs go through shared memory (a row of the tile is then stored by neighbouring lanes) and are added in
 // order, groups before CTAs, so that a result does not depend on timing.
 // ---------------------------------------------------------------------------------------------------------------
+constexpr long long kMaxGridY = 65535;   // (the row tiles)
 constexpr int kGemmPitch = 36;           // floats per staged row of 32
 template <int BM, int BN, int TM, int TN, int KG>
 struct SimtCfg {
@@ -426,39 +427,46 @@ int attention_launch(const float* q, const float* k, const float* v, float* o, i
 
 }  // namespace
 
+// Tiles of 64 x 64 (8 x 8 outputs a thread, two groups) or 32 x 32 (4 x 4, four groups), over one CTA or a cluster: what
+// an SM's CTAs take one after the other, in tenths of a us per chunk of k, and what a launch and an exchange take on top.
+// (Two CTAs share an SM but hardly run faster for it; clusters of three do not fill the chip.)  Measured, us:
+//   M x N x K           64: 1     2      3      4      8    32: 1     2      4
+//   620 x 1536 x 512     34.3   36.6   42.7   36.5   59.7    38.2   46.6   72.4   (before a packet's address was worked out once)
+//   620 x 512 x 512      20.1   19.5   16.1   16.9   24.0    17.2   19.4   26.6
+//   620 x 2048 x 512     48.9   44.9   51.6   49.7   77.1    48.6   62.0   94.8
+//   620 x 512 x 2048     70.1   65.0   46.6   50.2   49.5    62.0   55.1   58.9
+//   2638 x 512 x 2048   183.8  154.9  171.8  157.6  178.0   180.1  192.0  219.5
+//   1200 x 320 x 1280    45.3   42.4   44.9   33.8   46.1    40.1   43.1   53.0
+//   200 x 256 x 1024     36.4   21.2   17.1   12.5   10.9    12.8    8.9    8.3
+//   200 x 768 x 256      11.4    8.9   11.3    8.3            6.4   10.0
+//   32 x 128 x 512       19.3   12.6   10.0    7.7    5.8     7.0    5.5    4.4
+// With 8 x 4 outputs a thread, the sums stored by one group alone and no clusters: 620 x 1536 x 512 42, 620 x 512 x 2048 62.
+SimtGemmPlan plan_simt_gemm(int M, int Nout, int K, int sms) {
+  SimtGemmPlan plan = {0, 0};
+  long long best = -1;
+  for (const int tile : {64, 32}) {
+    const bool big = tile == 64;
+    const long long chunk = big ? 64 : 128, chunks = (K + chunk - 1) / chunk, row_tiles = ((long long)M + tile - 1) / tile;
+    const long long tiles = row_tiles * (((long long)Nout + tile - 1) / tile);
+    if (row_tiles > kMaxGridY) continue;             // (a problem of more rows takes the larger tile, up to 4.19 M)
+    for (int c : {1, 2, 3, 4, 8}) {
+      if (c > chunks) break;
+      const long long slots = c == 3 ? sms * 17 / 20 : sms, per_sm = (tiles * c + slots - 1) / slots;
+      const long long t = big ? per_sm * ((chunks + c - 1) / c * 20 + (c > 1 ? 10 : 0)) + 30
+                              : per_sm * ((chunks + c - 1) / c * 13 + (c > 1 ? 14 : 0)) + 17;
+      if (best < 0 || t < best) { best = t; plan = {tile, c}; }
+    }
+  }
+  return plan;
+}
+
 int launch_simt_gemm(const float* a, const float* w, const float* bias, int M, int Nout, int K, const GemmOut& out,
                      cudaStream_t s) {
   if (M <= 0) return HERO_OK;
-  // Tiles of 64 x 64 (8 x 8 outputs a thread, two groups) or 32 x 32 (4 x 4, four groups), over one CTA or a cluster: what
-  // an SM's CTAs take one after the other, in tenths of a us per chunk of k, and what a launch and an exchange take on top.
-  // (Two CTAs share an SM but hardly run faster for it; clusters of three do not fill the chip.)  Measured, us:
-  //   M x N x K           64: 1     2      3      4      8    32: 1     2      4
-  //   620 x 1536 x 512     34.3   36.6   42.7   36.5   59.7    38.2   46.6   72.4   (before a packet's address was worked out once)
-  //   620 x 512 x 512      20.1   19.5   16.1   16.9   24.0    17.2   19.4   26.6
-  //   620 x 2048 x 512     48.9   44.9   51.6   49.7   77.1    48.6   62.0   94.8
-  //   620 x 512 x 2048     70.1   65.0   46.6   50.2   49.5    62.0   55.1   58.9
-  //   2638 x 512 x 2048   183.8  154.9  171.8  157.6  178.0   180.1  192.0  219.5
-  //   1200 x 320 x 1280    45.3   42.4   44.9   33.8   46.1    40.1   43.1   53.0
-  //   200 x 256 x 1024     36.4   21.2   17.1   12.5   10.9    12.8    8.9    8.3
-  //   200 x 768 x 256      11.4    8.9   11.3    8.3            6.4   10.0
-  //   32 x 128 x 512       19.3   12.6   10.0    7.7    5.8     7.0    5.5    4.4
-  // With 8 x 4 outputs a thread, the sums stored by one group alone and no clusters: 620 x 1536 x 512 42, 620 x 512 x 2048 62.
-  bool large = false;
-  int split = 1;
-  long long best = -1;
-  for (const bool big : {true, false}) {
-    const int tile = big ? 64 : 32, chunk = big ? 64 : 128;
-    const long long tiles = (long long)((M + tile - 1) / tile) * ((Nout + tile - 1) / tile), chunks = (K + chunk - 1) / chunk;
-    for (int c : {1, 2, 3, 4, 8}) {
-      if (c > chunks) break;
-      const long long slots = c == 3 ? num_sms() * 17 / 20 : num_sms(), per_sm = (tiles * c + slots - 1) / slots;
-      const long long t = big ? per_sm * ((chunks + c - 1) / c * 20 + (c > 1 ? 10 : 0)) + 30
-                              : per_sm * ((chunks + c - 1) / c * 13 + (c > 1 ? 14 : 0)) + 17;
-      if (best < 0 || t < best) { best = t; large = big; split = c; }
-    }
-  }
-  return large ? gemm_launch<64, 64, 8, 8, 2>(a, w, bias, M, Nout, K, split, out, s)
-               : gemm_launch<32, 32, 4, 4, 4>(a, w, bias, M, Nout, K, split, out, s);
+  const SimtGemmPlan plan = plan_simt_gemm(M, Nout, K, num_sms());
+  if (!plan.tile) return HERO_ERR_ARG;
+  return plan.tile == 64 ? gemm_launch<64, 64, 8, 8, 2>(a, w, bias, M, Nout, K, plan.split, out, s)
+                         : gemm_launch<32, 32, 4, 4, 4>(a, w, bias, M, Nout, K, plan.split, out, s);
 }
 
 int launch_simt_attention(const float* q, const float* k, const float* v, float* o, int B, int n_q, int N, int heads,
