@@ -326,7 +326,8 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
   HERO_TRY(run_gemm(c, c->ws_u, w.w_2, w.b_2, M, D, F, o_dn));
 
   // x = (x + G_attn) + G_ffn for every row: fresh rows and cached rows alike
-  if (c->wait_x_upload) {                  // every row of x is read from here on: the upload has to be complete
+  const bool x_uploading = c->wait_x_upload;
+  if (x_uploading) {                       // every row of x is read from here on: the upload has to be complete
     c->wait_x_upload = false;
     HERO_CUDA_TRY(cudaStreamWaitEvent(c->stream, c->x_uploaded, 0));
   }
@@ -336,7 +337,8 @@ int refresh_block(hero_ctx* c, int block, void* d_x, const void* d_temb, const i
     const float* mod_next = c->mod + (size_t)(block + 1) * B * mod_ld;
     HERO_LAUNCH(c, HERO_PROF_RESIDUAL,
                 launch_residual_ln(d_x, ga, gf, next.pos, g.n_text, mod_next,
-                                   mod_next + D, mod_ld, c->ws_a, B, N, next.n_sel, D, 1e-5f, g.dtype, c->stream));
+                                   mod_next + D, mod_ld, c->ws_a, B, N, next.n_sel, D, 1e-5f, g.dtype, !x_uploading,
+                                   c->stream));
   } else if (collapse) {
     HERO_LAUNCH(c, HERO_PROF_RESIDUAL,
                 launch_residual2_acc(d_x, ga, gf, c->stack_hist[c->stack_new], c->elems, g.dtype, c->stream));

@@ -233,10 +233,13 @@ int launch_gather_ln_modulate(const void* x, const void* add, const int* idx, co
 
 // x = (x + ga) + gf for all rows and the LayerNorm + modulate of the rows that the next
 // block refreshes (pos: as SelectBatch::pos; null: all rows) into a [B, n_sel, D].  Rows as wide as residual_ln_serves.
+// Placed early, it reads all but gf before it waits for the kernel in front, which then has to be the only one on the stream
+// that may still be running, and the writer of gf alone.  early: that holds, and nothing else (an event of another stream)
+// stands between the two launches.
 bool residual_ln_serves(int D, int dtype);
 int launch_residual_ln(void* x, const void* ga, const void* gf, const int* pos, int n_text, const float* shift,
                        const float* scale, int mod_ld, void* a, int B, int N, int n_sel, int D, float eps, int dtype,
-                       cudaStream_t s);
+                       bool early, cudaStream_t s);
 
 // fp32 CUDA-core path (config 1 runs in fp32, where tensor cores would break parity)
 int launch_simt_gemm(const float* a, const float* w, const float* bias, int M, int Nout, int K, const GemmOut& out,

@@ -818,20 +818,23 @@ residual_ln_kernel(T* __restrict__ x, const T* __restrict__ ga, const T* __restr
 
 template <typename T, int VPL>
 int residual_ln_launch(void* x, const void* ga, const void* gf, const int* pos, int n_text, const float* shift,
-                       const float* scale, int mod_ld, void* a, int N, int n_sel, int B, int D, float eps, cudaStream_t s) {
+                       const float* scale, int mod_ld, void* a, int N, int n_sel, int B, int D, float eps, bool early,
+                       cudaStream_t s) {
   const int resident = (num_sms() * rln_ctas_per_sm(VPL) + B - 1) / B, need = (N + 7) / 8;
-  return launch_kernel(need <= resident ? residual_ln_kernel<T, VPL, true> : residual_ln_kernel<T, VPL, false>,
-                       (unsigned)((need < resident ? need : resident) * B), 256,
-                       (size_t)2 * D * sizeof(float), s, 1, (T*)x, (const T*)ga, (const T*)gf, pos, n_text, shift, scale,
-                       mod_ld, (T*)a, N, n_sel, B, D, eps);
+  return launch_kernel_as(early, need <= resident ? residual_ln_kernel<T, VPL, true> : residual_ln_kernel<T, VPL, false>,
+                          (unsigned)((need < resident ? need : resident) * B), 256,
+                          (size_t)2 * D * sizeof(float), s, 1, (T*)x, (const T*)ga, (const T*)gf, pos, n_text, shift, scale,
+                          mod_ld, (T*)a, N, n_sel, B, D, eps);
 }
 constexpr int kResidualLnPackets = 6;        // a lane's packets of three tensors stay in registers up to here
 template <typename T>
 int residual_ln_dispatch(void* x, const void* ga, const void* gf, const int* pos, int n_text, const float* shift,
-                         const float* scale, int mod_ld, void* a, int N, int n_sel, int B, int D, float eps, cudaStream_t s) {
+                         const float* scale, int mod_ld, void* a, int N, int n_sel, int B, int D, float eps, bool early,
+                         cudaStream_t s) {
   const int vpl = (D / Vec<T>::N + 31) / 32;
 #define HERO_RLN(V) \
-  if (vpl <= V) return residual_ln_launch<T, V>(x, ga, gf, pos, n_text, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s)
+  if (vpl <= V) \
+    return residual_ln_launch<T, V>(x, ga, gf, pos, n_text, shift, scale, mod_ld, a, N, n_sel, B, D, eps, early, s)
   HERO_RLN(1); HERO_RLN(2); HERO_RLN(3); HERO_RLN(4); HERO_RLN(5); HERO_RLN(6);
 #undef HERO_RLN
   return HERO_ERR_ARG;
@@ -1065,10 +1068,10 @@ bool residual_ln_serves(int D, int dtype) { return D / (dtype == HERO_DTYPE_BF16
 
 int launch_residual_ln(void* x, const void* ga, const void* gf, const int* pos, int n_text, const float* shift,
                        const float* scale, int mod_ld, void* a, int B, int N, int n_sel, int D, float eps, int dtype,
-                       cudaStream_t s) {
+                       bool early, cudaStream_t s) {
   return dtype == HERO_DTYPE_BF16
-             ? residual_ln_dispatch<__nv_bfloat16>(x, ga, gf, pos, n_text, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s)
-             : residual_ln_dispatch<float>(x, ga, gf, pos, n_text, shift, scale, mod_ld, a, N, n_sel, B, D, eps, s);
+             ? residual_ln_dispatch<__nv_bfloat16>(x, ga, gf, pos, n_text, shift, scale, mod_ld, a, N, n_sel, B, D, eps, early, s)
+             : residual_ln_dispatch<float>(x, ga, gf, pos, n_text, shift, scale, mod_ld, a, N, n_sel, B, D, eps, early, s);
 }
 
 int launch_gather_ln_modulate(const void* x, const void* add, const int* idx, const float* shift,

@@ -375,6 +375,31 @@ def test_pass_from_block_to_block(dtype, over):
     hero.close()
 
 
+@pytest.mark.parametrize("dtype,over", [
+    ("bf16", dict(hidden=1536, head_dim=64, n_heads=24, grid_h=36, grid_w=32, n_text=32)),     # a warp per row, one each
+    ("fp32", dict(hidden=512, head_dim=64, n_heads=8, grid_h=36, grid_w=48, n_text=48)),       # the same
+    ("bf16", dict(hidden=1536, head_dim=64, n_heads=24, grid_h=36, grid_w=33, n_text=0))],     # one row more
+    ids=["bf16", "fp32", "bf16_several_rows"])
+def test_pass_from_block_to_block_behind_an_upload(dtype, over):
+    """A cached step from pinned buffers whose first block is done long before x is on the device: 7 MB travel for 0.14 ms
+    while a dozen rows of a thin block take a third of that.  The pass behind that block sees all of x, bit for bit."""
+    cfgd = dict(S.CONFIGS["tiny"], batch=2, n_blocks=4, n_shallow=3, frames=1, seed=59, temb_dim=64, ffn_dim=64, dtype=dtype,
+                full_interval=0, ratio_num=1, ratio_den=90, **over)
+    weights = [H().device_weights(S.block_weights(cfgd, l), dtype) for l in range(4)]
+    on_device, on_host = H().Hero(cfgd, weights), H().Hero(cfgd, weights)
+    g = torch.Generator(device="cuda").manual_seed(4)
+    for s in range(8):                                     # two full steps, six cached ones, other tokens every time
+        x = torch.randn(2, S.n_rows(cfgd), cfgd["hidden"], device="cuda", generator=g).to(on_device.dt)
+        temb = to_dev(S.temb(cfgd, s), dtype)
+        h_x = x.cpu().pin_memory()
+        on_device.hero_step(s, x, temb)
+        on_host.hero_step_host(s, h_x, temb.cpu().pin_memory())
+        assert torch.equal(h_x, x.cpu()), s
+    for hero in (on_device, on_host):
+        hero.hero_check_status()
+        hero.close()
+
+
 @pytest.mark.parametrize("B,n_q,N,heads", [(1, 300, 97, 1), (2, 77, 600, 3), (1, 371, 1562, 12), (2, 640, 6200, 30)],
                          ids=["one_tile", "cluster", "cluster_of_four", "whole"])
 def test_attention_output_at_any_16_byte_boundary(B, n_q, N, heads):
