@@ -191,8 +191,8 @@ simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ W, const
 
 // ---------------------------------------------------------------------------------------------------------------
 // Flash attention in fp32.  A CTA of 128 threads takes 32 queries of one (batch, head) over a run of keys, 64 at a
-// time (the next K tile and this tile's V in flight: three CTAs then share an SM); a thread owns four query rows (8 row groups) and, of a score tile, the keys tx + 16 j, of
-// the output, HD / 16 features.  Online softmax with a running maximum: no score matrix is stored, P of a warp's own
+// time (the next K tile and this tile's V in flight: three CTAs then share an SM); a thread owns four query rows (8 row
+// groups) and, of a score tile, the keys tx + 16 j, of the output, HD / 16 features.  Online softmax with a running maximum: no score matrix is stored, P of a warp's own
 // rows passes through shared memory.  Where the grid would leave SMs idle the keys are split over a cluster of
 // `split` CTAs, which then merge their (maximum, sum, output) rows through distributed shared memory, in rank order.
 // ---------------------------------------------------------------------------------------------------------------
@@ -204,6 +204,13 @@ struct SimtAttCfg {
   static constexpr int kFloats = kAttQ * kPitch + kAttQ * kPPitch + 3 * kTileFloats + 2 * kAttQ;
   static_assert(kAttQ * HD <= 3 * kTileFloats, "the merge's rows fit over the tiles");
   static constexpr size_t kSmem = (size_t)kFloats * sizeof(float);
+  // Where the compiler's own choice of registers and unrolling loses, us without / with: head dimension 128, of which one CTA's
+  // shared memory fills an SM and which may take 176 registers where it settles for 128 (2 x 8 heads, 1319 x 1319, one CTA a
+  // group 660 / 529; 110 queries, 442 keys over eight 13.2 / 11.9); head dimension 32, whose two features a thread want fewer
+  // keys in flight (310 queries, 1319 keys over eight 10.6 / 9.8; 8 heads, 600 x 1240, one CTA a group 64.1 / 60.7).  At 64
+  // either loses 1 to 2 %.
+  static constexpr int kRegisterCtas = HD > 64 ? 1 : 0;
+  static constexpr int kUnrollPV = HD < 64 ? 2 : 4;
 };
 
 __device__ __forceinline__ float ld_cluster(uint32_t cluster_addr) {
@@ -213,9 +220,9 @@ __device__ __forceinline__ float ld_cluster(uint32_t cluster_addr) {
 }
 
 template <int HD>
-__global__ void __launch_bounds__(128) simt_attention_kernel(const float* __restrict__ Q, const float* __restrict__ Kc,
-                                                             const float* __restrict__ Vc, float* __restrict__ O,
-                                                             int n_q, int N, int heads, int split) {
+__global__ void __launch_bounds__(128, SimtAttCfg<HD>::kRegisterCtas)
+simt_attention_kernel(const float* __restrict__ Q, const float* __restrict__ Kc, const float* __restrict__ Vc,
+                      float* __restrict__ O, int n_q, int N, int heads, int split) {
   stream_order();
   using Cfg = SimtAttCfg<HD>;
   constexpr int kPitch = Cfg::kPitch, CPT = HD / 16;       // output features per thread
@@ -309,7 +316,7 @@ __global__ void __launch_bounds__(128) simt_attention_kernel(const float* __rest
     }
     cp_async_wait<1>();
     __syncthreads();                       // V of tile t is there (and a warp's own P rows)
-#pragma unroll 4
+#pragma unroll Cfg::kUnrollPV
     for (int k = 0; k < kAttK; k += 4) {
       float4 p[kAttRows];
 #pragma unroll
