@@ -994,6 +994,14 @@ int hero_plan_fp32_gemm(int M, int N, int K, int sms, int* tile, int* ctas) {
   return HERO_OK;
 }
 
+int hero_plan_fp32_attention(int B, int n_q, int N, int heads, int head_dim, int sms, int* ctas) {
+  if (B <= 0 || n_q <= 0 || N <= 0 || heads <= 0 || sms <= 0 || !ctas) return HERO_ERR_ARG;
+  if (head_dim != 32 && head_dim != 64 && head_dim != 128) return HERO_ERR_ARG;
+  const long long groups = (long long)B * heads * (((long long)n_q + kSimtAttQ - 1) / kSimtAttQ);
+  *ctas = plan_simt_attention(groups, (int)(((long long)N + kSimtAttK - 1) / kSimtAttK), head_dim, sms);
+  return HERO_OK;
+}
+
 // ---------------------------------------------------------------- state access
 static int state_ptr(hero_ctx* c, int block, int what, void** p, size_t* bytes) {
   const hero_config& g = c->cfg;

@@ -249,6 +249,8 @@ struct SimtGemmPlan { int tile, split; };
 SimtGemmPlan plan_simt_gemm(int M, int Nout, int K, int sms);
 int launch_simt_attention(const float* q, const float* k, const float* v, float* o, int B, int n_q, int N, int heads,
                           int head_dim, cudaStream_t s);
+constexpr int kSimtAttQ = 32, kSimtAttK = 64;                // queries of a group, keys of a tile
+int plan_simt_attention(long long groups, int tiles, int head_dim, int sms);     // CTAs that share a group's keys
 
 // bf16 tensor-core path (tcgen05 + TMEM + TMA)
 int tc_init_driver_api();   // resolves cuTensorMapEncodeTiled once

@@ -196,7 +196,7 @@ simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ W, const
 // rows passes through shared memory.  Where the grid would leave SMs idle the keys are split over a cluster of
 // `split` CTAs, which then merge their (maximum, sum, output) rows through distributed shared memory, in rank order.
 // ---------------------------------------------------------------------------------------------------------------
-constexpr int kAttQ = 32, kAttK = 64, kAttRows = 4;
+constexpr int kAttQ = kSimtAttQ, kAttK = kSimtAttK, kAttRows = 4;
 template <int HD>
 struct SimtAttCfg {
   static constexpr int kPitch = HD + 4, kPPitch = kAttK + 4;
@@ -416,23 +416,56 @@ int attention_launch(const float* q, const float* k, const float* v, float* o, i
   }));
   const long long groups = (long long)B * heads * ((n_q + kAttQ - 1) / kAttQ);
   const int tiles = (N + kAttK - 1) / kAttK;
-  // Keys over a cluster of two, four or eight where the chip is then better filled: per SM the CTAs one after the other take
-  // the time of their key tiles plus some for each start and merge (a CTA may go without keys).  us over 1 / 2 / 4 / 8 CTAs:
-  // 310 queries, 1319 keys, 16 heads 102 / 82 / 79 / 82; 8 heads 63 / 59 / 46 / 49; 600 x 1240 x 10 97 / 75 / 77 / 96;
-  // 1319 x 1319 x 16 234 / 253 / 264 / 302; 32 x 144 x 2 11.0 / 12.6 / 7.7 / 7.6.
-  int split = 1;
-  long long best = -1;
-  for (int c = 1; c <= 8 && (c == 1 || c / 2 < tiles); c *= 2) {
-    const long long per_sm = (groups * c + num_sms() - 1) / num_sms();
-    const long long t = per_sm * ((long long)((tiles + c - 1) / c) * (24 * HD / 64) + 17);
-    if (best < 0 || t < best) { best = t; split = c; }
-  }
+  const int split = plan_simt_attention(groups, tiles, HD, num_sms());
   if (groups * split > 0x7FFFFFFFll) return HERO_ERR_ARG;
   return launch_kernel(simt_attention_kernel<HD>, (unsigned)(groups * split), 128, Cfg::kSmem, s, (unsigned)split, q, k,
                        v, o, n_q, N, heads, split);
 }
 
 }  // namespace
+
+// Keys of a group of 32 queries over a cluster of two, four or eight CTAs where that is sooner done: the estimate, in hundredths
+// of a us, is what the fullest SM's CTAs take for their key tiles (a CTA may go without keys), plus their starts and the merge.
+// How many CTAs that SM gets depends on the cluster: a cluster's CTAs want free SMs of one processing cluster, so that
+// clusters of four double up from 0.7 of the SMs on, first in part, and clusters of eight from 13/16 on.
+// Constants fitted to 490 problems, launches in a row; of 240 others the choice is 0.1 % above the best in the geometric mean and
+// 11 % at most.  Some (heads x queries x keys; us over 1 / 2 / 4 / 8 CTAs, then the choice):
+//   head dimension 32: 8 x 310 x 1319 44.3 / 37.0 / 34.2 / 27.1, 8; 16 x 110 x 442 16.3 / 12.8 / 9.9 / 10.3, 4;
+//     18 x 250 x 500 18.4 / 16.5 / 19.4 / 20.9, 2; 16 x 1319 x 1319 144 / 149 / 154 / 166, 1
+//   head dimension 64: 16 x 310 x 1319 101 / 81 / 78 / 81, 4; 2 x 600 x 1240 59.6 / 35.4 / 28.7 / 26.0, 8;
+//     10 x 600 x 1240 96 / 75 / 78 / 96, 2; 16 x 1319 x 1319 234 / 253 / 264 / 303, 1
+//   head dimension 128, of which an SM holds one: 8 x 310 x 1319 107 / 129 / 108 / 126, 1; 4 x 110 x 442 37.8 / 31.1 / 17.1 / 22.4, 4
+// One time per key tile for every head dimension, and SMs that any cluster fills, came out up to 49 % above a rule that only
+// kept the grid within what the chip holds (2 x 600 x 1240 of 64 over two, 16 x 110 x 442 of 32 over two).
+int plan_simt_attention(long long groups, int tiles, int head_dim, int sms) {
+  struct Cost { int resident, tile[4], further, launch, block, merge[4], crowd; };
+  static const Cost of32 = {4, {207, 289, 503, 543}, 115, 141, 62, {0, 251, 148, 164}, 0};
+  static const Cost of64 = {3, {290, 469, 676, 965}, 215, 213, 70, {0, 428, 236, 223}, 15};
+  static const Cost of128 = {1, {493, 986, 1479, 1972}, 493, 41, 294, {0, 799, 391, 362}, 87};
+  const Cost& cost = head_dim == 32 ? of32 : (head_dim == 64 ? of64 : of128);
+  const bool shared = cost.resident > 1;             // an SM holds several
+  int split = 1;
+  long long best = -1;
+  for (int c = 1, i = 0; c <= 8 && (c == 1 || c / 2 < tiles); c *= 2, ++i) {
+    const long long blocks = groups * c;
+    // the SMs that clusters of this size fill, and twice the blocks of the fullest one
+    const int most = sms * 9 / 10, some = sms * 13 / 16;
+    int full = sms;
+    if (c == 4) full = shared ? sms * 19 / 20 : most;
+    if (c == 8) full = cost.resident > 3 || (shared && blocks <= (long long)cost.resident * most) ? most : some;
+    if (full < 1) full = 1;
+    long long twice = 2 * ((blocks + full - 1) / full);
+    if (c == 4 && shared && blocks <= full) twice = blocks <= sms * 7 / 10 ? 2 : 3;
+    if (c == 8) twice = blocks <= some ? 2 : (twice < 4 ? 4 : twice);
+    if (head_dim == 64 && blocks > sms * 3 / 2 && twice < 6) twice = 6;
+    const long long n = twice / 2;
+    const long long tile = twice == 3 ? (cost.tile[0] + cost.tile[1]) / 2
+                                      : (n <= 4 ? cost.tile[n - 1] : cost.tile[3] + (n - 4) * cost.further);
+    const long long t = (tiles + c - 1) / c * tile + cost.launch + cost.block * twice / 2 + cost.merge[i] * (100 + cost.crowd * (n - 1)) / 100;
+    if (best < 0 || t < best) { best = t; split = c; }
+  }
+  return split;
+}
 
 // Tiles of 64 x 64 (8 x 8 outputs a thread, two groups) or 32 x 32 (4 x 4, four groups), over one CTA or a cluster: what
 // an SM's CTAs take one after the other, in tenths of a us per chunk of k, and what a launch and an exchange take on top.
