@@ -424,10 +424,24 @@ int attention_launch(const float* q, const float* k, const float* v, float* o, i
 
 }  // namespace
 
+// Twice the blocks that the fullest SM gets of `blocks` in clusters of `c`, when an SM holds `resident` at a time.  The CTAs of a
+// cluster want free SMs of one processing cluster: not all SMs are to be had, and clusters of four double up from two thirds of the
+// SMs on, first in part (hence twice), clusters of eight from 13/16 on.
+static long long fullest_sm_twice(long long blocks, int c, int resident, int sms) {
+  const int most = sms * 9 / 10, some = sms * 13 / 16;
+  int full = sms;
+  if (c == 3) full = sms * 13 / 14;
+  if (c == 4) full = resident > 1 ? sms * 19 / 20 : most;
+  if (c == 8) full = resident > 3 || blocks <= (long long)resident * most ? most : some;
+  if (full < 1) full = 1;
+  const long long twice = 2 * ((blocks + full - 1) / full);
+  if (c == 4 && resident > 1 && blocks <= full) return blocks <= sms * 2 / 3 ? 2 : 3;
+  if (c == 8) return blocks <= some ? 2 : (twice < 4 ? 4 : twice);
+  return twice;
+}
+
 // Keys of a group of 32 queries over a cluster of two, four or eight CTAs where that is sooner done: the estimate, in hundredths
 // of a us, is what the fullest SM's CTAs take for their key tiles (a CTA may go without keys), plus their starts and the merge.
-// How many CTAs that SM gets depends on the cluster: a cluster's CTAs want free SMs of one processing cluster, so that
-// clusters of four double up from 0.7 of the SMs on, first in part, and clusters of eight from 13/16 on.
 // Constants fitted to 490 problems, launches in a row; of 240 others the choice is 0.1 % above the best in the geometric mean and
 // 11 % at most.  Some (heads x queries x keys; us over 1 / 2 / 4 / 8 CTAs, then the choice):
 //   head dimension 32: 8 x 310 x 1319 44.3 / 37.0 / 34.2 / 27.1, 8; 16 x 110 x 442 16.3 / 12.8 / 9.9 / 10.3, 4;
@@ -443,20 +457,11 @@ int plan_simt_attention(long long groups, int tiles, int head_dim, int sms) {
   static const Cost of64 = {3, {290, 469, 676, 965}, 215, 213, 70, {0, 428, 236, 223}, 15};
   static const Cost of128 = {1, {493, 986, 1479, 1972}, 493, 41, 294, {0, 799, 391, 362}, 87};
   const Cost& cost = head_dim == 32 ? of32 : (head_dim == 64 ? of64 : of128);
-  const bool shared = cost.resident > 1;             // an SM holds several
   int split = 1;
   long long best = -1;
   for (int c = 1, i = 0; c <= 8 && (c == 1 || c / 2 < tiles); c *= 2, ++i) {
     const long long blocks = groups * c;
-    // the SMs that clusters of this size fill, and twice the blocks of the fullest one
-    const int most = sms * 9 / 10, some = sms * 13 / 16;
-    int full = sms;
-    if (c == 4) full = shared ? sms * 19 / 20 : most;
-    if (c == 8) full = cost.resident > 3 || (shared && blocks <= (long long)cost.resident * most) ? most : some;
-    if (full < 1) full = 1;
-    long long twice = 2 * ((blocks + full - 1) / full);
-    if (c == 4 && shared && blocks <= full) twice = blocks <= sms * 7 / 10 ? 2 : 3;
-    if (c == 8) twice = blocks <= some ? 2 : (twice < 4 ? 4 : twice);
+    long long twice = fullest_sm_twice(blocks, c, cost.resident, sms);
     if (head_dim == 64 && blocks > sms * 3 / 2 && twice < 6) twice = 6;
     const long long n = twice / 2;
     const long long tile = twice == 3 ? (cost.tile[0] + cost.tile[1]) / 2
@@ -467,34 +472,37 @@ int plan_simt_attention(long long groups, int tiles, int head_dim, int sms) {
   return split;
 }
 
-// Tiles of 64 x 64 (8 x 8 outputs a thread, two groups) or 32 x 32 (4 x 4, four groups), over one CTA or a cluster: what
-// an SM's CTAs take one after the other, in tenths of a us per chunk of k, and what a launch and an exchange take on top.
-// (Two CTAs share an SM but hardly run faster for it; clusters of three do not fill the chip.)  Measured, us:
-//   M x N x K           64: 1     2      3      4      8    32: 1     2      4
-//   620 x 1536 x 512     34.3   36.6   42.7   36.5   59.7    38.2   46.6   72.4   (before a packet's address was worked out once)
-//   620 x 512 x 512      20.1   19.5   16.1   16.9   24.0    17.2   19.4   26.6
-//   620 x 2048 x 512     48.9   44.9   51.6   49.7   77.1    48.6   62.0   94.8
-//   620 x 512 x 2048     70.1   65.0   46.6   50.2   49.5    62.0   55.1   58.9
-//   2638 x 512 x 2048   183.8  154.9  171.8  157.6  178.0   180.1  192.0  219.5
-//   1200 x 320 x 1280    45.3   42.4   44.9   33.8   46.1    40.1   43.1   53.0
-//   200 x 256 x 1024     36.4   21.2   17.1   12.5   10.9    12.8    8.9    8.3
-//   200 x 768 x 256      11.4    8.9   11.3    8.3            6.4   10.0
-//   32 x 128 x 512       19.3   12.6   10.0    7.7    5.8     7.0    5.5    4.4
-// With 8 x 4 outputs a thread, the sums stored by one group alone and no clusters: 620 x 1536 x 512 42, 620 x 512 x 2048 62.
+// Tiles of 64 x 64 (8 x 8 outputs a thread, two groups) or 32 x 32 (4 x 4, four groups), over one CTA or a cluster: what the
+// fullest SM's CTAs take for their chunks of k (alone, or two and more side by side, which hardly helps), their start and the
+// exchange, in twice a hundredth of a us.  Fitted to 528 problems; of 220 others the choice (last column) is 0.1 % above the best
+// in the geometric mean and 5 % at most.  us, launches in a row:
+//   M x N x K           64: 1     2      3      4      8    32: 1     2      3      4      8
+//   620 x 1536 x 512     31.6   33.6   39.5   34.1   56.1    34.6   44.9   68.4   68.8         64, 1
+//   620 x 512 x 512      18.4   18.2   15.2   16.1   22.7    16.2   18.5   26.7   25.2         64, 3
+//   620 x 2048 x 512     44.7   41.4   47.8   45.9   72.9    43.8   59.1   89.8   90.7         64, 2
+//   620 x 512 x 2048     62.8   59.3   43.0   46.4   45.1    56.3   50.0   55.5   53.0  69.5   64, 3
+//   2638 x 512 x 2048   165.7  139.9  154.9  143.0  160.2   161.5  171.8  202.6  195.2   271   64, 2
+//   1200 x 320 x 1280    40.7   39.2   41.2   31.2   43.2    36.7   39.2   46.5   47.8  78.4   64, 4
+//   310 x 448 x 1792     55.2   30.5   23.3   28.3   25.8    19.9   19.8   28.4   25.0  33.0   32, 2
+//   200 x 256 x 1024     32.9   19.2   15.6   11.5   10.7    11.9    8.4   10.8    8.6  11.9   32, 2
+//   200 x 768 x 256      10.8    8.4   11.0    8.0            6.9    9.4                       32, 1
+//   32 x 128 x 512       17.2   11.3    9.4    7.3    5.3     6.9    5.5    5.8    4.3         32, 4
 SimtGemmPlan plan_simt_gemm(int M, int Nout, int K, int sms) {
+  struct Cost { int tile, chunk, alone, shared, launch, block, exchange[5]; };
+  static const Cost costs[] = {{64, 64, 180, 159, 302, 26, {0, 56, 92, 65, 117}}, {32, 128, 125, 103, 140, 41, {0, 128, 128, 107, 116}}};
+  static const int ctas[] = {1, 2, 3, 4, 8};
   SimtGemmPlan plan = {0, 0};
   long long best = -1;
-  for (const int tile : {64, 32}) {
-    const bool big = tile == 64;
-    const long long chunk = big ? 64 : 128, chunks = (K + chunk - 1) / chunk, row_tiles = ((long long)M + tile - 1) / tile;
-    const long long tiles = row_tiles * (((long long)Nout + tile - 1) / tile);
+  for (const Cost& cost : costs) {
+    const long long chunks = (K + cost.chunk - 1ll) / cost.chunk, row_tiles = ((long long)M + cost.tile - 1) / cost.tile;
+    const long long tiles = row_tiles * (((long long)Nout + cost.tile - 1) / cost.tile);
     if (row_tiles > kMaxGridY) continue;             // (a problem of more rows takes the larger tile, up to 4.19 M)
-    for (int c : {1, 2, 3, 4, 8}) {
-      if (c > chunks) break;
-      const long long slots = c == 3 ? sms * 17 / 20 : sms, per_sm = (tiles * c + slots - 1) / slots;
-      const long long t = big ? per_sm * ((chunks + c - 1) / c * 20 + (c > 1 ? 10 : 0)) + 30
-                              : per_sm * ((chunks + c - 1) / c * 13 + (c > 1 ? 14 : 0)) + 17;
-      if (best < 0 || t < best) { best = t; plan = {tile, c}; }
+    for (int i = 0; i < 5 && ctas[i] <= chunks; ++i) {
+      const int c = ctas[i];
+      const long long twice = fullest_sm_twice(tiles * c, c, 2, sms);
+      const long long chunk = twice == 2 ? 2 * cost.alone : (twice == 3 ? cost.alone + 2 * cost.shared : twice * cost.shared);
+      const long long t = (chunks + c - 1) / c * chunk + 2 * cost.launch + twice * (cost.block + cost.exchange[i]);
+      if (best < 0 || t < best) { best = t; plan = {cost.tile, c}; }
     }
   }
   return plan;
