@@ -306,6 +306,9 @@ int hero_selftest_wait_timeout(hero_ctx *ctx, int budget_us, void *stream);
 /* The fp32 GEMM C[M,N] = A[M,K] W[N,K]^T of a context on a GPU of `sms` SMs: square tiles of *tile (64 or 32) outputs, each
  * shared by a cluster of *ctas thread blocks along K.  HERO_ERR_ARG where no tile serves so many rows (65535 row tiles of 64). */
 int hero_plan_fp32_gemm(int M, int N, int K, int sms, int *tile, int *ctas);
+/* The bf16 GEMM (of a context and hero_gemm_bf16; qk = 1: a QKV projection that treats q and k rows as well): tiles of *columns
+ * columns, 128 rows in a cluster of *ctas thread blocks that share K, or, *ctas 0, 256 rows on a pair of thread blocks. */
+int hero_plan_bf16_gemm(int M, int N, int K, int qk, int sms, int *columns, int *ctas);
 /* The fp32 attention of a context, n_q queries against N keys: the keys of 32 queries of a head are shared by a cluster of
  * *ctas thread blocks. */
 int hero_plan_fp32_attention(int B, int n_q, int N, int heads, int head_dim, int sms, int *ctas);

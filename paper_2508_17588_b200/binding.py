@@ -27,7 +27,7 @@ EXPORTS = [
     "hero_extrapolate_block", "hero_extrapolate_deep_stack", "hero_step", "hero_step_host", "hero_is_full_step", "hero_extrapolate",
     "hero_gather_rows", "hero_scatter_rows", "hero_gemm_bf16", "hero_attention_bf16", "hero_attention_bf16_safe", "hero_attention_bf16_q_scaled", "hero_attention_bf16_static", "hero_attention_bf16_static_status",
     "hero_isolated_status", "hero_selftest_wait_timeout", "hero_gather_ln_modulate",
-    "hero_plan_fp32_gemm", "hero_plan_fp32_attention",
+    "hero_plan_fp32_gemm", "hero_plan_fp32_attention", "hero_plan_bf16_gemm",
     "hero_state_get", "hero_state_set", "hero_second_difference_moments", "hero_extrapolation_error",
 ]
 
@@ -103,6 +103,7 @@ def load() -> C.CDLL:
         "hero_second_difference_moments": (i, [vp, vp, vp, ll, i, vp, vp]),
         "hero_extrapolation_error": (i, [vp, vp, vp, ll, i, i, i, vp, vp]),
         "hero_plan_fp32_gemm": (i, [i, i, i, i, ip, ip]),
+        "hero_plan_bf16_gemm": (i, [i, i, i, i, i, ip, ip]),
         "hero_plan_fp32_attention": (i, [i, i, i, i, i, i, ip]),
         "hero_state_get": (i, [vp, i, i, vp, ll]),
         "hero_state_set": (i, [vp, i, i, vp, ll]),
@@ -382,6 +383,13 @@ def hero_plan_fp32_gemm(M: int, N: int, K: int, sms: int = 148):
     tile, ctas = C.c_int(), C.c_int()
     _check(load().hero_plan_fp32_gemm(M, N, K, sms, C.byref(tile), C.byref(ctas)), "hero_plan_fp32_gemm")
     return tile.value, ctas.value
+
+
+def hero_plan_bf16_gemm(M: int, N: int, K: int, qk: bool = False, sms: int = 148):
+    """(columns of a tile, thread blocks that share its K; 0: a pair of thread blocks for 256 rows) of the bf16 GEMM."""
+    columns, ctas = C.c_int(), C.c_int()
+    _check(load().hero_plan_bf16_gemm(M, N, K, int(qk), sms, C.byref(columns), C.byref(ctas)), "hero_plan_bf16_gemm")
+    return columns.value, ctas.value
 
 
 def hero_plan_fp32_attention(B: int, n_q: int, N: int, heads: int, head_dim: int, sms: int = 148):

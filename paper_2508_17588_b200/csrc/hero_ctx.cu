@@ -994,6 +994,13 @@ int hero_plan_fp32_gemm(int M, int N, int K, int sms, int* tile, int* ctas) {
   return HERO_OK;
 }
 
+int hero_plan_bf16_gemm(int M, int N, int K, int qk, int sms, int* columns, int* ctas) {
+  if (M <= 0 || N <= 0 || K <= 0 || (qk != 0 && qk != 1) || sms <= 0 || !columns || !ctas) return HERO_ERR_ARG;
+  const TcGemmPlan plan = plan_tc_gemm(M, N, K, qk != 0, sms);
+  *columns = plan.bn; *ctas = plan.split;
+  return HERO_OK;
+}
+
 int hero_plan_fp32_attention(int B, int n_q, int N, int heads, int head_dim, int sms, int* ctas) {
   if (B <= 0 || n_q <= 0 || N <= 0 || heads <= 0 || sms <= 0 || !ctas) return HERO_ERR_ARG;
   if (head_dim != 32 && head_dim != 64 && head_dim != 128) return HERO_ERR_ARG;

@@ -256,6 +256,9 @@ int plan_simt_attention(long long groups, int tiles, int head_dim, int sms);    
 int tc_init_driver_api();   // resolves cuTensorMapEncodeTiled once
 int launch_tc_gemm(const void* a, const void* w, const void* bias, int M, int Nout, int K,
                    const GemmOut& out, const QkEpilogue* qk, int* d_status, cudaStream_t s);
+// Columns of a tile and the CTAs that share its K (0: the kernel on CTA pairs).
+struct TcGemmPlan { int bn, split; };
+TcGemmPlan plan_tc_gemm(int M, int Nout, int K, bool qk, int sms);
 // The tensor-core attention serves head_dim 64: a score s enters the softmax as 2^(s * kScoreScaleLog2).
 constexpr float kScoreScaleLog2 = 0.125f * 1.4426950408889634f;   // 1/sqrt(64) * log2(e)
 // Workspace of an attention launch that may cut query groups.

@@ -730,28 +730,24 @@ int launch_wait_timeout_selftest(int* d_status, int budget_us, cudaStream_t s) {
 //   7000 x 1536 x 6144     99.1     103.4     125.7     143.8    168.9    181.1   259.5    220.0   315.1
 // 64 columns over four CTAs, where K is long and the tiles are few (CTA 64 over 1 / 2 / 4): 250 x 384 x 1536 7.6 / 5.9 / 4.9,
 // 500 x 512 x 2048 9.4 / 6.9 / 6.1, 60 x 704 x 2112 9.2 / 6.9 / 5.3; 371 x 768 x 3072, whose 36 clusters of four do not all
-// fit, 12.8 / 8.8 / 12.7.  With q/k treatment (pair 256 / pair 128 / CTA 128 / CTA 64): 371 x 2304 x 768 10.4 / 7.3 / 7.3 / 6.2,
-// 614 x 768 x 256 8.0 / 5.9 / 5.3 / 4.3, 700 x 1536 x 512 9.4 / 6.8 / 6.7 / 5.3, 1394 x 3072 x 1024 12.8 / 13.7 / 15.6 / 25.4.
+// fit, 12.8 / 8.8 / 12.7.  The more clusters, the longer the exchange, which short K does not pay for: 25 x 2048 x 512 4.7 / 4.7 / 5.2,
+// 60 x 1920 x 640 5.0 / 5.0 / 5.5, but 148 x 512 x 512 4.8 / 4.8 / 4.4.  With q/k treatment (pair 256 / pair 128 / CTA 128 /
+// CTA 64): 371 x 2304 x 768 10.4 / 7.3 / 7.3 / 6.2, 614 x 768 x 256 8.0 / 5.9 / 5.3 / 4.3, 700 x 1536 x 512 9.4 / 6.8 / 6.7 / 5.3,
+// 1394 x 3072 x 1024 12.8 / 13.7 / 15.6 / 25.4.
 // ---------------------------------------------------------------------------------------------------------------
-namespace {
-
-struct GemmPlan { int bn; int split; };        // split 0: the pair kernel
-
-// (qk: only what gives an epilogue warp whole heads)
-GemmPlan plan_gemm(int M, int Nout, int K, bool qk) {
-  const int sms = num_sms();
-  const long long kb = (K + kBK - 1) / kBK;
+TcGemmPlan plan_tc_gemm(int M, int Nout, int K, bool qk, int sms) {
+  const long long kb = ((long long)K + kBK - 1) / kBK;
   auto ceil_div = [](long long a, long long b) { return (a + b - 1) / b; };
-  GemmPlan best = {256, 0};
+  TcGemmPlan best = {256, 0};
   long long best_t = -1;
   auto consider = [&](int bn, int split, long long t) {
     if (best_t < 0 || t < best_t) { best_t = t; best = {bn, split}; }
   };
   struct { int bn, step, fixed; } const pair[] = {{256, 560, 11500}, {224, 510, 10100}, {192, 500, 8000}, {128, 460, 7400}};
   for (const auto& p : pair) {
-    if (qk && p.bn % 128 != 0) continue;
+    if (qk && p.bn % 128 != 0) continue;             // (only what gives an epilogue warp whole heads)
     const long long tiles = ceil_div(M, 2 * kBM) * ceil_div(Nout, p.bn);
-    consider(p.bn, 0, ceil_div(tiles, sms / 2) * kb * p.step + p.fixed);
+    consider(p.bn, 0, ceil_div(tiles, sms < 2 ? 1 : sms / 2) * kb * p.step + p.fixed);
   }
   for (int bn : {128, 64}) {
     const long long tiles = ceil_div(M, kBM) * ceil_div(Nout, bn);
@@ -760,14 +756,17 @@ GemmPlan plan_gemm(int M, int Nout, int K, bool qk) {
       const long long ctas = tiles * split;
       if (ctas > 0x7FFFFFFFll) continue;
       // (clusters of four do not fill the chip: they need four free SMs of one processing cluster)
-      const long long waves = ceil_div(ctas, split == 4 ? sms * 7 / 8 : sms);
+      const long long fours = sms < 2 ? 1 : sms * 7 / 8, waves = ceil_div(ctas, split == 4 ? fours : sms);
       const long long step = bn == 64 ? 390 : 400 + (ctas < 100 ? ctas : 100);
-      const long long exchange = split == 1 ? 0 : (bn == 64 ? 1700 : (split == 2 ? 2000 : 3500));
+      long long exchange = split == 1 ? 0 : (bn == 64 ? 1700 : (split == 2 ? 2000 : 3500));
+      if (bn == 64 && split == 4) exchange += 100 + (ctas > 60 ? 15 * (ctas - 60) : 0);
       consider(bn, split, waves * (ceil_div(kb, split) * step + (bn == 64 ? 4500 : 6300) + exchange));
     }
   }
   return best;
 }
+
+namespace {
 
 template <int BN, bool QK = false>
 int launch_pair(const CUtensorMap& tm_a, const CUtensorMap& tm_w, const void* bias, const GemmOut& out, const QkEpilogue& qk,
@@ -811,7 +810,7 @@ int launch_tc_gemm(const void* a, const void* w, const void* bias, int M, int No
   if (!aligned16(a) || !aligned16(w) || !aligned16(bias)) return HERO_ERR_ALIGN;
   for (int i = 0; i < 3; ++i)
     if (out.ptr[i] && (!aligned16(out.ptr[i]) || out.ld[i] % 8)) return HERO_ERR_ALIGN;
-  const GemmPlan plan = plan_gemm(M, Nout, K, qk != nullptr);
+  const TcGemmPlan plan = plan_tc_gemm(M, Nout, K, qk != nullptr, num_sms());
   CUtensorMap tm_a, tm_w;
   {
     const uint64_t dims[2] = {(uint64_t)K, (uint64_t)M};
