@@ -685,15 +685,18 @@ __device__ __forceinline__ void ln_finish_row(const float (&f)[VPL][Vec<T>::N], 
   }
 }
 
-// (EXACT: the row has exactly 32 * VPL packets, nothing is predicated; the wide rows have no registers to spare for it.)
 // `settled` (launch_gather_ln_modulate) says what was complete before the kernel in front was placed: those loads go out
 // before the wait for that kernel, so that of the chain vectors, list, row, row to add only the last link is left behind it.
-// A row is fetched so early where every warp has one at most (ONE): ahead of a loop it would not stay in registers.  With the
-// same in the pass from block to block and 32-byte stores in the attention, all behind the wait before: schedule of 42 blocks of
-// 614 x 256 2734 -> 2573 us, cached step of 4 blocks of 371 x 768 221 -> 210.
-template <typename T, int VPL, bool EXACT, bool ONE>
-__global__ void __launch_bounds__(256, ln_ctas_per_sm(VPL, ONE))
-gather_ln_modulate_warp_kernel(const T* __restrict__ x, const T* __restrict__ add, const int* __restrict__ idx,
+// A row is fetched so early where every warp has one at most: ahead of a loop it would not stay in registers, and with both in
+// one kernel the loop spills (17776 x 2560 32.4 -> 33.7 us, 150 x 2816 5.3 -> 5.7).  With the same in the pass from block to block
+// and 32-byte stores in the attention, all behind the wait before: schedule of 42 blocks of 614 x 256 2734 -> 2573 us, cached step
+// of 4 blocks of 371 x 768 221 -> 210.
+//
+// Several rows a warp.  (EXACT: the row has exactly 32 * VPL packets, nothing is predicated; the wide rows have no registers to
+// spare for it.)
+template <typename T, int VPL, bool EXACT>
+__global__ void __launch_bounds__(256, ln_ctas_per_sm(VPL, false))
+gather_ln_modulate_rows_kernel(const T* __restrict__ x, const T* __restrict__ add, const int* __restrict__ idx,
                                const float* __restrict__ shift, const float* __restrict__ scale, int mod_ld,
                                T* __restrict__ a, int N, int n_sel, int B, int D, float eps, int settled) {
   using V = Vec<T>;
@@ -703,26 +706,16 @@ gather_ln_modulate_warp_kernel(const T* __restrict__ x, const T* __restrict__ ad
   extern __shared__ float4 s_mod[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = blockIdx.x % B, slot = blockIdx.x / B, slots = gridDim.x / B;
-  const int first = slot * 8 + warp;
-  long long row = 0;
-  V raw[VPL];
-  auto find_row = [&](int i) { row = (long long)b * N + (idx ? __ldg(idx + i) : i); };
-  auto load = [&](const T* from) {
-    const V* r = reinterpret_cast<const V*>(from + row * D);
-#pragma unroll
-    for (int c = 0; c < VPL; ++c)
-      if (c < kFull || c * 32 + lane < packets) raw[c].raw = __ldcs(&r[c * 32 + lane].raw);
-  };
   if (settled < kLnModSettled) stream_order();
-  if (ONE && first < n_sel) {                // warp-uniform
-    find_row(first);
-    if (settled == kLnRowsSettled) load(x);
-  }
   ln_stage_modulation<T>(s_mod, scale + (long long)b * mod_ld, shift + (long long)b * mod_ld, packets);
   if (settled >= kLnModSettled) stream_order();
-  for (int i = first; i < n_sel; i += slots * 8) {
-    if (!ONE) find_row(i);
-    if (!ONE || settled != kLnRowsSettled) load(x);
+  for (int i = slot * 8 + warp; i < n_sel; i += slots * 8) {
+    const long long row = (long long)b * N + (idx ? __ldg(idx + i) : i);
+    const V* xr = reinterpret_cast<const V*>(x + row * D);
+    V raw[VPL];
+#pragma unroll
+    for (int c = 0; c < VPL; ++c)
+      if (c < kFull || c * 32 + lane < packets) raw[c].raw = __ldcs(&xr[c * 32 + lane].raw);
     float f[VPL][V::N];
 #pragma unroll
     for (int c = 0; c < VPL; ++c) {
@@ -734,7 +727,10 @@ gather_ln_modulate_warp_kernel(const T* __restrict__ x, const T* __restrict__ ad
       }
     }
     if (add) {
-      load(add);
+      const V* ar = reinterpret_cast<const V*>(add + row * D);
+#pragma unroll
+      for (int c = 0; c < VPL; ++c)
+        if (c < kFull || c * 32 + lane < packets) raw[c].raw = __ldcs(&ar[c * 32 + lane].raw);
 #pragma unroll
       for (int c = 0; c < VPL; ++c) {
         if (c < kFull || c * 32 + lane < packets) {
@@ -746,8 +742,63 @@ gather_ln_modulate_warp_kernel(const T* __restrict__ x, const T* __restrict__ ad
       }
     }
     ln_finish_row<T, VPL, kFull>(f, s_mod, packets, D, eps, lane, a + ((long long)b * n_sel + i) * D);
-    if (ONE) break;
   }
+}
+
+// One row a warp at most.  What need not be waited for is on its way before the wait; with nothing settled x is, before the
+// vectors are staged (600 x 256 2.21 -> 1.99 us, 4400 x 512 4.34 -> 3.25 against the loop).
+template <typename T, int VPL>
+__global__ void __launch_bounds__(256, ln_ctas_per_sm(VPL, true))
+gather_ln_modulate_row_kernel(const T* __restrict__ x, const T* __restrict__ add, const int* __restrict__ idx,
+                              const float* __restrict__ shift, const float* __restrict__ scale, int mod_ld,
+                              T* __restrict__ a, int N, int n_sel, int B, int D, float eps, int settled) {
+  using V = Vec<T>;
+  constexpr int kFull = ln_full_chunks(VPL);
+  const int packets = D / V::N;
+  extern __shared__ float4 s_mod[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b = blockIdx.x % B, i = blockIdx.x / B * 8 + warp;
+  const bool there = i < n_sel;                               // warp-uniform
+  long long row = 0;
+  V raw[VPL];
+  auto load = [&](const T* from) {
+    const V* r = reinterpret_cast<const V*>(from + row * D);
+#pragma unroll
+    for (int c = 0; c < VPL; ++c)
+      if (c < kFull || c * 32 + lane < packets) raw[c].raw = __ldcs(&r[c * 32 + lane].raw);
+  };
+  if (settled < kLnModSettled) stream_order();
+  if (there) {
+    row = (long long)b * N + (idx ? __ldg(idx + i) : i);
+    if (settled != kLnModSettled) load(x);
+  }
+  ln_stage_modulation<T>(s_mod, scale + (long long)b * mod_ld, shift + (long long)b * mod_ld, packets);
+  if (settled >= kLnModSettled) stream_order();
+  if (!there) return;
+  if (settled == kLnModSettled) load(x);
+  float f[VPL][V::N];
+#pragma unroll
+  for (int c = 0; c < VPL; ++c) {
+    if (c < kFull || c * 32 + lane < packets) {
+      raw[c].unpack(f[c]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < V::N; ++q) f[c][q] = 0.f;
+    }
+  }
+  if (add) {
+    load(add);
+#pragma unroll
+    for (int c = 0; c < VPL; ++c) {
+      if (c < kFull || c * 32 + lane < packets) {
+        float g[V::N];
+        raw[c].unpack(g);
+#pragma unroll
+        for (int q = 0; q < V::N; ++q) f[c][q] += g[q];
+      }
+    }
+  }
+  ln_finish_row<T, VPL, kFull>(f, s_mod, packets, D, eps, lane, a + ((long long)b * n_sel + i) * D);
 }
 
 // The end of one refreshed block and the start of the next in one pass: x = (x + ga) + gf for every row, and the rows that
@@ -849,11 +900,11 @@ int gather_ln_warp(const void* x, const void* add, const int* idx, const float* 
   const int resident = (num_sms() * ln_ctas_per_sm(VPL, one) + B - 1) / B;
   const unsigned grid = (unsigned)((need < resident ? need : resident) * B);
   const size_t smem = (size_t)2 * D * sizeof(float);
-  auto kernel = gather_ln_modulate_warp_kernel<T, VPL, false, false>;
+  auto kernel = gather_ln_modulate_rows_kernel<T, VPL, false>;
   if constexpr (VPL >= 8) {
-    if (D == VPL * 32 * Vec<T>::N) kernel = gather_ln_modulate_warp_kernel<T, VPL, true, false>;
+    if (D == VPL * 32 * Vec<T>::N) kernel = gather_ln_modulate_rows_kernel<T, VPL, true>;
   } else {
-    if (one) kernel = gather_ln_modulate_warp_kernel<T, VPL, false, true>;
+    if (one) kernel = gather_ln_modulate_row_kernel<T, VPL>;
   }
   return launch_kernel(kernel, grid, 256, smem, s, 1, (const T*)x, (const T*)add, idx, shift, scale, mod_ld, (T*)a, N, n_sel,
                        B, D, eps, settled);
