@@ -72,18 +72,32 @@ def test_gather_ln_variants(dtype, B, N, D, n_sel, with_add):
 FP32_TOL = 2e-5
 
 
-@pytest.mark.parametrize("over", [
-    # attention: head dimensions, one query tile and less, keys whole or split over clusters of 2, 4 and 8
-    dict(hidden=128, head_dim=32, n_heads=4, grid_h=5, grid_w=6, n_text=1, batch=1),       # 31 rows: half a key tile
-    dict(hidden=128, head_dim=64, n_heads=2, grid_h=8, grid_w=8, n_text=1, batch=2),       # 65 keys: one in tile two
-    dict(hidden=128, head_dim=128, n_heads=1, grid_h=19, grid_w=23, n_text=5, batch=1),    # 442 keys over four
-    dict(hidden=64, head_dim=64, n_heads=1, grid_h=33, grid_w=31, n_text=22, batch=1),     # 1045 keys over eight
-    # GEMM: 64 x 64 tiles in the full pass, 32 x 32 in the refresh, widths that are no multiple of either
-    dict(hidden=384, head_dim=32, n_heads=12, ffn_dim=1540, grid_h=19, grid_w=23, n_text=5, batch=2, has_gate=1),
-    dict(hidden=192, head_dim=64, n_heads=3, ffn_dim=52, grid_h=31, grid_w=33, n_text=0, batch=2),
-], ids=["half_tile", "65_keys", "hd128_split4", "split8", "wide", "narrow_ffn"])
-def test_fp32_block_variants(over):
+def sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def row_counts(cfgd):
+    """Rows per item of a full pass and of a refresh in quota mode 0."""
+    return S.n_rows(cfgd), (S.n_rows(cfgd) - cfgd["n_text"]) * cfgd["ratio_num"] // cfgd["ratio_den"]
+
+
+@pytest.mark.parametrize("over,splits", [
+    # attention: head dimensions, one query tile and less, keys whole or split over clusters of 2, 4 and 8 (full, refresh)
+    (dict(hidden=128, head_dim=32, n_heads=4, grid_h=5, grid_w=6, n_text=1, batch=1), (1, 1)),       # 31 rows: half a key tile
+    (dict(hidden=128, head_dim=64, n_heads=2, grid_h=8, grid_w=8, n_text=1, batch=2), (1, 1)),       # 65 keys: one in tile two
+    (dict(hidden=128, head_dim=128, n_heads=1, grid_h=19, grid_w=23, n_text=5, batch=1), (8, 8)),    # 7 tiles over eight
+    (dict(hidden=512, head_dim=128, n_heads=4, grid_h=13, grid_w=31, n_text=5, batch=1), (2, 4)),
+    (dict(hidden=64, head_dim=64, n_heads=1, grid_h=33, grid_w=31, n_text=22, batch=1), (4, 8)),
+    (dict(hidden=384, head_dim=32, n_heads=12, grid_h=11, grid_w=31, n_text=5, batch=1), (2, 4)),
+    # widths that are no multiple of a GEMM tile
+    (dict(hidden=384, head_dim=32, n_heads=12, ffn_dim=1540, grid_h=19, grid_w=23, n_text=5, batch=2, has_gate=1), (2, 8)),
+    (dict(hidden=192, head_dim=64, n_heads=3, ffn_dim=52, grid_h=31, grid_w=33, n_text=0, batch=2), (2, 8)),
+], ids=["half_tile", "65_keys", "hd128_eight", "hd128_two_four", "hd64_four_eight", "hd32_two_four", "wide", "narrow_ffn"])
+def test_fp32_block_variants(over, splits):
     cfgd = dict(S.CONFIGS["tiny"], n_blocks=1, n_shallow=1, frames=1, seed=41, **over)
+    n = S.n_rows(cfgd)
+    assert splits == tuple(H().hero_plan_fp32_attention(cfgd["batch"], rows, n, cfgd["n_heads"], cfgd["head_dim"], sms())
+                           for rows in row_counts(cfgd))
     orc, hero, _ = make_pair(cfgd)
     x_host = S.tokens(cfgd)
     for s in range(4):                                     # two full passes, two refreshes
@@ -418,19 +432,30 @@ def test_attention_output_at_any_16_byte_boundary(B, n_q, N, heads):
     assert torch.equal(outs[0], outs[1])
 
 
-@pytest.mark.parametrize("over", [
-    # 64 x 64 tiles whole, over two (FFN up), three (both projections back to the width) in the full pass; the same and 32 x 32
-    # over clusters in the refresh
-    dict(hidden=512, n_heads=8, ffn_dim=2048, grid_h=16, grid_w=19, n_text=5, batch=2),
-    # FFN down over four CTAs: 32 x 32 tiles, the last row tile eight rows; 64 x 64 tiles, K no multiple of a chunk
-    dict(hidden=256, n_heads=4, ffn_dim=1024, grid_h=13, grid_w=15, n_text=5, batch=1),
-    dict(hidden=320, n_heads=5, ffn_dim=1276, grid_h=22, grid_w=26, n_text=25, batch=2, has_gate=1),
-    # one row tile, over eight CTAs' worth of k; nothing to split
-    dict(hidden=64, n_heads=1, ffn_dim=4092, grid_h=5, grid_w=6, n_text=0, batch=1),
-    dict(hidden=192, n_heads=3, ffn_dim=4, grid_h=7, grid_w=50, n_text=1, batch=1)],
-    ids=["width512", "width256", "width320", "long_k", "short_k"])
-def test_fp32_gemm_tiles_and_clusters(over):
+@pytest.mark.parametrize("over,full,refresh", [
+    # (tile, CTAs that share its k) of the QKV, output, up and down projections in the full pass and in the refresh
+    (dict(hidden=512, n_heads=8, ffn_dim=2048, grid_h=16, grid_w=19, n_text=5, batch=2),
+     ((64, 1), (64, 3), (64, 2), (64, 3)), ((32, 1), (32, 1), (32, 1), (32, 3))),
+    # the last row tile eight rows in the full pass, 16 in the refresh
+    (dict(hidden=256, n_heads=4, ffn_dim=1024, grid_h=13, grid_w=15, n_text=5, batch=1),
+     ((32, 1), (32, 1), (32, 1), (32, 2)), ((32, 1), (32, 1), (32, 1), (32, 4))),
+    # k no multiple of a chunk
+    (dict(hidden=320, n_heads=5, ffn_dim=1276, grid_h=22, grid_w=26, n_text=25, batch=2, has_gate=1),
+     ((64, 1), (32, 1), (64, 1), (64, 4)), ((32, 1), (32, 1), (32, 1), (32, 3))),
+    (dict(hidden=384, n_heads=6, ffn_dim=1540, grid_h=8, grid_w=12, n_text=4, batch=1),
+     ((32, 1), (32, 1), (32, 1), (64, 8)), ((32, 3), (32, 3), (32, 1), (32, 8))),
+    # one row tile, long k; one chunk of k with four of its 128 there
+    (dict(hidden=64, n_heads=1, ffn_dim=4092, grid_h=5, grid_w=6, n_text=0, batch=1),
+     ((32, 1), (32, 1), (32, 1), (32, 8)), ((32, 1), (32, 1), (32, 1), (32, 8))),
+    (dict(hidden=192, n_heads=3, ffn_dim=4, grid_h=7, grid_w=50, n_text=1, batch=1),
+     ((32, 1), (32, 1), (32, 1), (32, 1)), ((32, 1), (32, 1), (32, 1), (32, 1)))],
+    ids=["width512", "width256", "width320", "width384", "long_k", "short_k"])
+def test_fp32_gemm_tiles_and_clusters(over, full, refresh):
     cfgd = dict(S.CONFIGS["tiny"], n_blocks=1, n_shallow=1, frames=1, seed=43, head_dim=64, **over)
+    D, F = cfgd["hidden"], cfgd["ffn_dim"]
+    for want, rows in zip((full, refresh), row_counts(cfgd)):
+        assert want == tuple(H().hero_plan_fp32_gemm(cfgd["batch"] * rows, n, k, sms())
+                             for n, k in ((3 * D, D), (D, D), (F, D), (D, F)))
     orc, hero, _ = make_pair(cfgd)
     x_host = S.tokens(cfgd)
     for s in range(3):                                     # two full passes, one refresh
@@ -456,7 +481,7 @@ def test_qk_treatment_by_tile_width(over, qk_norm, rope):
     x_host = S.tokens(cfgd)
     for s in range(3):                                     # two full passes, one refresh
         temb = S.temb(cfgd, s)
-        orc.step(s, x_host, temb)
+        want = orc.step(s, x_host, temb)
         x = to_dev(x_host, "bf16")
         hero.hero_step(s, x, to_dev(temb, "bf16"))
         hero.hero_check_status()
