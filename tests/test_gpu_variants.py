@@ -48,7 +48,10 @@ def test_gemm_tile_variants(M, N, K):
     ("bf16", 3, 2000, 2056, 1900, False), ("bf16", 2, 40, 2816, 17, True), ("bf16", 1, 5000, 4088, 4900, False),
     ("bf16", 1, 20, 4104, 20, True), ("fp32", 2, 3000, 132, 2900, True), ("fp32", 1, 50, 2048, 33, False),
     ("fp32", 1, 5000, 1540, 5000, True), ("fp32", 1, 20, 2052, 20, False), ("bf16", 2, 9, 12288, 5, True),
-    ("fp32", 1, 9, 12288, 9, False)])
+    ("fp32", 1, 9, 12288, 9, False),
+    # one row a warp up to four (rows of two packets a lane and less) and three (five and six) blocks an SM, one more; warps without a row
+    ("bf16", 1, 4800, 64, 4736, True), ("bf16", 1, 4800, 64, 4737, True), ("fp32", 2, 1800, 640, 1776, True),
+    ("fp32", 2, 1800, 640, 1777, True), ("bf16", 3, 50, 1032, 13, True)])
 def test_gather_ln_variants(dtype, B, N, D, n_sel, with_add):
     g = torch.Generator(device="cuda").manual_seed(D + n_sel)
     dt = torch.bfloat16 if dtype == "bf16" else torch.float32
