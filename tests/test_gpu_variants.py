@@ -347,14 +347,23 @@ def test_what_a_thread_block_falls_back_to_is_the_exported_path(B, n_q, N, heads
     ("bf16", dict(hidden=448, head_dim=64, n_heads=7, ffn_dim=64, deep_collapse=1)),
     ("bf16", dict(hidden=1536, head_dim=64, n_heads=24, ffn_dim=64, batch=1)),
     ("bf16", dict(hidden=1600, head_dim=64, n_heads=25, ffn_dim=64, batch=1)),
+    # rows of eight items that a warp has one of at most (448, at three blocks an SM), and one row more: a loop; the last packets
+    # of a row partly there; two blocks an SM, where the limit is 296
+    ("bf16", dict(hidden=64, head_dim=64, n_heads=1, ffn_dim=64, batch=8, grid_h=21, grid_w=21, n_text=7, n_blocks=3, n_shallow=2)),
+    ("bf16", dict(hidden=64, head_dim=64, n_heads=1, ffn_dim=64, batch=8, grid_h=21, grid_w=21, n_text=8, n_blocks=3, n_shallow=2)),
+    ("bf16", dict(hidden=448, head_dim=64, n_heads=7, ffn_dim=64, batch=8, grid_h=21, grid_w=21, n_text=8, n_blocks=3, n_shallow=2,
+                  ratio_num=1, ratio_den=50)),
+    ("fp32", dict(hidden=320, head_dim=64, n_heads=5, ffn_dim=64, batch=8, grid_h=21, grid_w=22, n_text=0, n_blocks=3, n_shallow=2)),
+    ("fp32", dict(hidden=448, head_dim=64, n_heads=7, ffn_dim=64, batch=8, grid_h=17, grid_w=17, n_text=8, n_blocks=2, n_shallow=2)),
     # into the deep stack: one refreshed block in front of as many deep ones as a launch holds, and of more
     ("fp32", dict(hidden=64, head_dim=32, n_heads=2, ffn_dim=64, n_blocks=33, n_shallow=1)),
     ("fp32", dict(hidden=64, head_dim=32, n_heads=2, ffn_dim=64, n_blocks=36, n_shallow=2))],
     ids=["fp32_64", "fp32_768_shared", "fp32_832", "fp32_64_sparse", "bf16_64", "bf16_64_sparse", "bf16_448_collapse",
-         "bf16_1536", "bf16_1600", "deep_32", "deep_34"])
+         "bf16_1536", "bf16_1600", "bf16_64_at_one_row", "bf16_64_loop", "bf16_448_loop_sparse", "fp32_320_loop", "fp32_448_loop",
+         "deep_32", "deep_34"])
 def test_pass_from_block_to_block(dtype, over):
-    cfgd = dict(S.CONFIGS["tiny"], frames=1, grid_h=9, grid_w=7, seed=43, temb_dim=64, dtype=dtype, full_interval=3,
-                **{**dict(batch=2, n_blocks=5, n_shallow=3, ratio_num=3, ratio_den=10), **over})
+    cfgd = dict(S.CONFIGS["tiny"], frames=1, seed=43, temb_dim=64, dtype=dtype, full_interval=3,
+                **{**dict(grid_h=9, grid_w=7, batch=2, n_blocks=5, n_shallow=3, ratio_num=3, ratio_den=10), **over})
     K, sparse = cfgd["n_shallow"], cfgd["ratio_den"] == 90
     orc, hero, _ = make_pair(cfgd)
     for l in range(K):                                     # the blocks' call counters apart, so that their lists differ in length
