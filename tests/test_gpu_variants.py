@@ -480,16 +480,28 @@ def test_fp32_gemm_tiles_and_clusters(over, full, refresh):
 
 
 @pytest.mark.parametrize("qk_norm,rope", [(1, 1), (0, 1), (1, 0)])
-@pytest.mark.parametrize("over", [
-    # tiles of 64 columns: a head each, one row tile and several; the same over four CTAs in the other projections
-    dict(hidden=64, n_heads=1, ffn_dim=2048, grid_h=9, grid_w=10, n_text=7, batch=1),
-    dict(hidden=448, n_heads=7, ffn_dim=1792, grid_h=17, grid_w=18, n_text=1, batch=2),
+@pytest.mark.parametrize("over,qkv,down", [
+    # tiles of 64 columns, a head each: one row tile and several; the down-projection on 64 columns over two and four CTAs
+    (dict(hidden=64, n_heads=1, ffn_dim=2048, grid_h=9, grid_w=10, n_text=7, batch=1), ((64, 1), (64, 1)), ((64, 4), (64, 4))),
+    (dict(hidden=448, n_heads=7, ffn_dim=1792, grid_h=17, grid_w=18, n_text=1, batch=2), ((64, 1), (64, 1)), ((64, 2), (64, 4))),
     # tiles of 128 columns in the full pass
-    dict(hidden=512, n_heads=8, ffn_dim=512, grid_h=25, grid_w=20, n_text=0, batch=2)], ids=["one_head", "7_heads", "wide"])
-def test_qk_treatment_by_tile_width(over, qk_norm, rope):
+    (dict(hidden=512, n_heads=8, ffn_dim=512, grid_h=25, grid_w=20, n_text=0, batch=2), ((128, 1), (64, 1)), ((64, 1), (64, 4)))],
+    ids=["one_head", "7_heads", "wide"])
+def test_qk_treatment_by_tile_width(over, qkv, down, qk_norm, rope):
     cfgd = dict(S.CONFIGS["tiny"], n_blocks=1, n_shallow=1, frames=1, seed=47, head_dim=64, temb_dim=64, dtype="bf16", rope=rope,
                 qk_norm=qk_norm, **over)
-    orc, hero, _ = make_pair(cfgd)
+    D, F = cfgd["hidden"], cfgd["ffn_dim"]
+    rows = [cfgd["batch"] * n for n in row_counts(cfgd)]
+    assert qkv == tuple(H().hero_plan_bf16_gemm(m, 3 * D, D, True, sms()) for m in rows)
+    assert down == tuple(H().hero_plan_bf16_gemm(m, D, F, False, sms()) for m in rows)
+    # scores of a few units, so that the attention says what became of q
+    w = S.block_weights(cfgd, 0)
+    if qk_norm:
+        for name in ("qn_w", "kn_w"):
+            w[name] = S.round_bf16(1.5 * w[name])
+    else:
+        w["w_qkv"][:2 * D] = S.round_bf16(w["w_qkv"][:2 * D] * np.float32(75 / D ** 0.5))
+    orc, hero, _ = make_pair(cfgd, [w])
     x_host = S.tokens(cfgd)
     for s in range(3):                                     # two full passes, one refresh
         temb = S.temb(cfgd, s)
@@ -497,9 +509,15 @@ def test_qk_treatment_by_tile_width(over, qk_norm, rope):
         x = to_dev(x_host, "bf16")
         hero.hero_step(s, x, to_dev(temb, "bf16"))
         hero.hero_check_status()
+        b = orc.blocks[0]
+        blind = b.v_cache.mean(1) @ w["w_o"].astype(np.float64).T + w["b_o"]        # attention that does not look at q
+        assert rel_l2(np.broadcast_to(blind[:, None], b.g[0].shape), b.g[0]) > 0.3
         # keys and values are one projection of a LayerNormed row away from x: two roundings to bf16 of the inputs of a
         # K-term sum and one of its result, the latter through the rotation; far below the 2e-2 that a whole block may be off
-        for name, ref in (("k", orc.blocks[0].k_cache), ("v", orc.blocks[0].v_cache)):
-            assert rel_l2(to_host(hero.hero_state_get(0, name)), ref) <= 1e-2, (s, name)
-            ref[...] = to_host(hero.hero_state_get(0, name))
+        for name, ref, tol in (("k", b.k_cache, 1e-2), ("v", b.v_cache, 1e-2), ("g_attn", b.g[0], 2e-2), ("g_ffn", b.g[1], 2e-2)):
+            got = to_host(hero.hero_state_get(0, name))
+            assert rel_l2(got, ref) <= tol, (s, name)
+            ref[...] = got
+        update = np.linalg.norm(want - x_host)
+        assert np.linalg.norm(to_host(x) - want) <= 2.0 ** -9 * np.linalg.norm(want) + 2e-2 * update, s
     hero.close()
