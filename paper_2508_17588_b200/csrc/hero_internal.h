@@ -60,13 +60,17 @@ int per_device_once(PerDeviceOnce& once, F&& fn) {
 // ---------------------------------------------------------------------------
 // Launches.  Kernels are launched with programmatic stream serialisation: their blocks may be placed while the kernel
 // before them on the stream still runs, so that launch latency, block start and set-up (barriers, TMEM, tensor-map
-// prefetch) are over when that kernel ends.  In return every block of every kernel calls stream_order() before it
-// touches anything another kernel writes or reads:
+// prefetch) are over when that kernel ends.  In return every block of every kernel calls stream_order() before it writes
+// anything and before it reads what the kernel in front writes:
 //   * the wait returns when all earlier work on the stream is complete and visible (the kernel before has itself waited
 //     for its own predecessor, so completion carries over), and
 //   * only then may the next kernel's blocks be placed.  A block that uses tensor memory has to have its columns by
 //     then: a block of the next kernel on the same SM could otherwise take them and hold them until this kernel ends.
 //     (stream_order_wait is the first half alone; the second then happens when the block ends.)
+// So a block that runs finds everything complete up to the kernel before the one in front, and may read that before its wait:
+// the weights of a GEMM (GemmOut::weights_settled), a step's lists and vectors and the rows of x in the LayerNorm kernels
+// (LnSettled, launch_residual_ln), the list of launch_attend_rows.  What a launcher takes for granted stands at its declaration.
+// Work of another stream is not among it: behind a wait for an event, a kernel that reads early is launched as an ordinary one.
 // Measured, all kernels against none (which is the launch order the kernels had before): mini42 schedule (307 rows, 42
 // blocks) 5.36 -> 3.54 ms, width 768 cached step 0.391 -> 0.294, width 1024 cached step 1.156 -> 1.021, fp32 model of width
 // 128 0.141 -> 0.108; the 3072-wide 42-block cached step 59.74 -> 59.39.  Kernels that stream large tensors through more

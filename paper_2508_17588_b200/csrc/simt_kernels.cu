@@ -435,7 +435,7 @@ static long long fullest_sm_twice(long long blocks, int c, int resident, int sms
   if (c == 8) full = resident > 3 || blocks <= (long long)resident * most ? most : some;
   if (full < 1) full = 1;
   const long long twice = 2 * ((blocks + full - 1) / full);
-  if (c == 4 && resident > 1 && blocks <= full) return blocks <= sms * 2 / 3 ? 2 : 3;
+  if (c == 4 && resident > 1 && blocks <= sms) return blocks <= sms * 2 / 3 ? 2 : 3;
   if (c == 8) return blocks <= some ? 2 : (twice < 4 ? 4 : twice);
   return twice;
 }
