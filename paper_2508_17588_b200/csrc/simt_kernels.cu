@@ -511,8 +511,8 @@ SimtGemmPlan plan_simt_gemm(int M, int Nout, int K, int sms) {
 int launch_simt_gemm(const float* a, const float* w, const float* bias, int M, int Nout, int K, const GemmOut& out,
                      cudaStream_t s) {
   if (M <= 0) return HERO_OK;
-  const SimtGemmPlan plan = plan_simt_gemm(M, Nout, K, num_sms());
-  if (!plan.tile) return HERO_ERR_ARG;
+  SimtGemmPlan plan = plan_simt_gemm(M, Nout, K, num_sms());
+  if (!plan.tile) plan = {64, 1};                    // (CUDA refuses the launch and says so)
   return plan.tile == 64 ? gemm_launch<64, 64, 8, 8, 2>(a, w, bias, M, Nout, K, plan.split, out, s)
                          : gemm_launch<32, 32, 4, 4, 4>(a, w, bias, M, Nout, K, plan.split, out, s);
 }
