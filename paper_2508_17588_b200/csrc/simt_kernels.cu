@@ -425,8 +425,9 @@ int attention_launch(const float* q, const float* k, const float* v, float* o, i
 }  // namespace
 
 // Twice the blocks that the fullest SM gets of `blocks` in clusters of `c`, when an SM holds `resident` at a time.  The CTAs of a
-// cluster want free SMs of one processing cluster: not all SMs are to be had, and clusters of four double up from two thirds of the
-// SMs on, first in part (hence twice), clusters of eight from 13/16 on.
+// cluster want free SMs of one processing cluster, so that not all SMs are to be had (of 148, clusters of four with an SM for each
+// CTA fill 132); where an SM holds several, clusters of four double up from two thirds of the SMs on, first in part (hence twice),
+// clusters of eight from 13/16 on.
 static long long fullest_sm_twice(long long blocks, int c, int resident, int sms) {
   const int most = sms * 9 / 10, some = sms * 13 / 16;
   int full = sms;
@@ -442,13 +443,14 @@ static long long fullest_sm_twice(long long blocks, int c, int resident, int sms
 
 // Keys of a group of 32 queries over a cluster of two, four or eight CTAs where that is sooner done: the estimate, in hundredths
 // of a us, is what the fullest SM's CTAs take for their key tiles (a CTA may go without keys), plus their starts and the merge.
-// Constants fitted to 490 problems, launches in a row; of 240 others the choice is 0.1 % above the best in the geometric mean and
+// Constants fitted to 450 problems, launches in a row; of 240 others the choice is 0.1 % above the best in the geometric mean and
 // 11 % at most.  Some (heads x queries x keys; us over 1 / 2 / 4 / 8 CTAs, then the choice):
 //   head dimension 32: 8 x 310 x 1319 44.3 / 37.0 / 34.2 / 27.1, 8; 16 x 110 x 442 16.3 / 12.8 / 9.9 / 10.3, 4;
 //     18 x 250 x 500 18.4 / 16.5 / 19.4 / 20.9, 2; 16 x 1319 x 1319 144 / 149 / 154 / 166, 1
 //   head dimension 64: 16 x 310 x 1319 101 / 81 / 78 / 81, 4; 2 x 600 x 1240 59.6 / 35.4 / 28.7 / 26.0, 8;
 //     10 x 600 x 1240 96 / 75 / 78 / 96, 2; 16 x 1319 x 1319 234 / 253 / 264 / 303, 1
-//   head dimension 128, of which an SM holds one: 8 x 310 x 1319 107 / 129 / 108 / 126, 1; 4 x 110 x 442 37.8 / 31.1 / 17.1 / 22.4, 4
+//   head dimension 128, of which an SM holds one: 8 x 310 x 1319 107 / 129 / 108 / 126, 1;
+//     4 x 110 x 442 37.8 / 31.1 / 17.1 / 22.4, 4
 // One time per key tile for every head dimension, and SMs that any cluster fills, came out up to 49 % above a rule that only
 // kept the grid within what the chip holds (2 x 600 x 1240 of 64 over two, 16 x 110 x 442 of 32 over two).
 int plan_simt_attention(long long groups, int tiles, int head_dim, int sms) {
@@ -462,11 +464,13 @@ int plan_simt_attention(long long groups, int tiles, int head_dim, int sms) {
   for (int c = 1, i = 0; c <= 8 && (c == 1 || c / 2 < tiles); c *= 2, ++i) {
     const long long blocks = groups * c;
     long long twice = fullest_sm_twice(blocks, c, cost.resident, sms);
+    // (of head dimension 64 some SM has three from 1.5 an SM on: 216 blocks take 5.3 us a key tile, 224 6.9)
     if (head_dim == 64 && blocks > sms * 3 / 2 && twice < 6) twice = 6;
     const long long n = twice / 2;
     const long long tile = twice == 3 ? (cost.tile[0] + cost.tile[1]) / 2
                                       : (n <= 4 ? cost.tile[n - 1] : cost.tile[3] + (n - 4) * cost.further);
-    const long long t = (tiles + c - 1) / c * tile + cost.launch + cost.block * twice / 2 + cost.merge[i] * (100 + cost.crowd * (n - 1)) / 100;
+    const long long merge = cost.merge[i] * (100 + cost.crowd * (n - 1)) / 100;
+    const long long t = (tiles + c - 1) / c * tile + cost.launch + cost.block * twice / 2 + merge;
     if (best < 0 || t < best) { best = t; split = c; }
   }
   return split;
@@ -489,7 +493,8 @@ int plan_simt_attention(long long groups, int tiles, int head_dim, int sms) {
 //   32 x 128 x 512       17.2   11.3    9.4    7.3    5.3     6.9    5.5    5.8    4.3         32, 4
 SimtGemmPlan plan_simt_gemm(int M, int Nout, int K, int sms) {
   struct Cost { int tile, chunk, alone, shared, launch, block, exchange[5]; };
-  static const Cost costs[] = {{64, 64, 180, 159, 302, 26, {0, 56, 92, 65, 117}}, {32, 128, 125, 103, 140, 41, {0, 128, 128, 107, 116}}};
+  static const Cost costs[] = {{64, 64, 180, 159, 302, 26, {0, 56, 92, 65, 117}},
+                               {32, 128, 125, 103, 140, 41, {0, 128, 128, 107, 116}}};
   static const int ctas[] = {1, 2, 3, 4, 8};
   SimtGemmPlan plan = {0, 0};
   long long best = -1;
