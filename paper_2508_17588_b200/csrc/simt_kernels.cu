@@ -192,9 +192,10 @@ simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ W, const
 // ---------------------------------------------------------------------------------------------------------------
 // Flash attention in fp32.  A CTA of 128 threads takes 32 queries of one (batch, head) over a run of keys, 64 at a
 // time (the next K tile and this tile's V in flight: three CTAs then share an SM); a thread owns four query rows (8 row
-// groups) and, of a score tile, the keys tx + 16 j, of the output, HD / 16 features.  Online softmax with a running maximum: no score matrix is stored, P of a warp's own
-// rows passes through shared memory.  Where the grid would leave SMs idle the keys are split over a cluster of
-// `split` CTAs, which then merge their (maximum, sum, output) rows through distributed shared memory, in rank order.
+// groups) and, of a score tile, the keys tx + 16 j, of the output, HD / 16 features.  Online softmax with a running maximum: no
+// score matrix is stored, P of a warp's own rows passes through shared memory.  Where the grid would leave SMs idle the keys are
+// split over a cluster of `split` CTAs, which then merge their (maximum, sum, output) rows through distributed shared memory, in
+// rank order.
 // ---------------------------------------------------------------------------------------------------------------
 constexpr int kAttQ = kSimtAttQ, kAttK = kSimtAttK, kAttRows = 4;
 template <int HD>
